@@ -635,7 +635,7 @@ int build_pyramids(reg_ctx *ctx, const Geometry &g, const float *frames, int nf,
     CU(launch_pyramid(frames, nf, fstride, g.W[0], g.H[0], pitch, L, ctx->cfg.storage, o,
                       ctx->means.as<float>() + (size_t)first * L, s));
     ctx->pyr_pairs.push_back({e0, timing_mark(ctx, s)});
-    ctx->last.pyramid_launches += (nonrigid ? 4 : 2) * L;
+    ctx->last.pyramid_launches += pyramid_launches(L, true, o.pad);
     return REG_OK;
 }
 

@@ -130,6 +130,8 @@ struct TileShape {
 // (storage-typed); means[f * levels + l] = mean of level l of frame f (or null).
 cudaError_t launch_pyramid(const float *frames, int N, size_t fstride, int W, int H, int pitch, int levels,
                            int storage, const PyrOut &out, float *means, cudaStream_t s);
+// Kernel launches of one launch_pyramid call.
+int pyramid_launches(int levels, bool means, int pad);
 // tab[l].mean = means[l] for l < L (a slot's level table rows after its pyramid build).
 cudaError_t launch_set_level_means(LevelDesc *tab, const float *means, int L, cudaStream_t s);
 cudaError_t launch_ops(const Params &p, int storage, int cluster, int n_launch_ops,

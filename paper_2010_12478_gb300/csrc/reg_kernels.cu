@@ -1,4 +1,4 @@
-// Device kernels of libreg: pyramid build and the registration operator.
+// Device kernels of libreg: the registration operator.
 //
 // Design (GB300, sm_103a):
 //   * One operator application (A or B, Sec. 2.3.1-2.3.2) runs start to finish
@@ -20,12 +20,11 @@
 //     the cluster rewrites between passes, through L2 (ld/st .cg) with a fence
 //     before each cluster barrier.
 #include <cooperative_groups.h>
-#include <cuda_bf16.h>
-#include <cuda_fp16.h>
 
 #include <cmath>
 
 #include "reg_internal.h"
+#include "reg_dev.cuh"
 #include "reg_f2.cuh"
 
 namespace cg = cooperative_groups;
@@ -36,52 +35,6 @@ constexpr int kWarps = kThreads / 32;
 constexpr int kNM = 8;         // moment slots per reduction (at most 6 are used)
 constexpr int kMaxCluster = 16; // CTAs per operator at most (non-portable cluster size)
 constexpr int kChunk = 32;     // pixels per thread between float-float flushes
-
-// ------------------------------------------------------------------ loads
-template <typename S> __device__ __forceinline__ float ldS(const S *p);
-template <> __device__ __forceinline__ float ldS<float>(const float *p) { return __ldg(p); }
-template <> __device__ __forceinline__ float ldS<__nv_bfloat16>(const __nv_bfloat16 *p)
-{
-    return __bfloat162float(__ldg(p));
-}
-template <> __device__ __forceinline__ float ldS<__half>(const __half *p) { return __half2float(__ldg(p)); }
-
-template <typename S> __device__ __forceinline__ S toS(float v);
-template <> __device__ __forceinline__ float toS<float>(float v) { return v; }
-template <> __device__ __forceinline__ __nv_bfloat16 toS<__nv_bfloat16>(float v) { return __float2bfloat16_rn(v); }
-template <> __device__ __forceinline__ __half toS<__half>(float v) { return __float2half_rn(v); }
-
-// ------------------------------------------------------------------ float-float
-// (hi, lo) += x, exactly up to the final rounding of lo (Knuth's TwoSum).
-__device__ __forceinline__ void ff_acc(float &hi, float &lo, float x)
-{
-    float s = __fadd_rn(hi, x);
-    float bp = __fsub_rn(s, hi);
-    float e = __fadd_rn(__fsub_rn(hi, __fsub_rn(s, bp)), __fsub_rn(x, bp));
-    hi = s;
-    lo = __fadd_rn(lo, e);
-}
-
-// acc += x*y with the exact rounding error of the product kept in err (the error of a
-// product of two floats is exactly representable: fmaf(x, y, -p)).
-__device__ __forceinline__ void acc_prod(float &acc, float &err, float x, float y)
-{
-    const float p = __fmul_rn(x, y);
-    err += fmaf(x, y, -p);
-    acc = __fadd_rn(acc, p);
-}
-
-// (hi, lo) += (h2, l2), renormalised.
-__device__ __forceinline__ void ff_add(float &hi, float &lo, float h2, float l2)
-{
-    float s = __fadd_rn(hi, h2);
-    float bp = __fsub_rn(s, hi);
-    float e = __fadd_rn(__fsub_rn(hi, __fsub_rn(s, bp)), __fsub_rn(h2, bp));
-    e = __fadd_rn(e, __fadd_rn(lo, l2));
-    float h = __fadd_rn(s, e);
-    lo = __fsub_rn(e, __fsub_rn(h, s));
-    hi = h;
-}
 
 // ------------------------------------------------------------------ shared state
 // Step-controller state (FP64), used by thread 0 of each CTA only: kept in shared memory so
@@ -2049,172 +2002,6 @@ __global__ void __launch_bounds__(kThreads) energy_kernel(Params p, const double
     }
 }
 
-// ================================================================== pyramid
-// All kernels take a batch of frames (grid.z or grid.x = frame).  Level pointers address pixel
-// (0, 0) of frame 0; rows are `pitch` elements apart and frames `stride` elements apart.
-// Level 0 in storage type: a CTA of kL0Threads covers kL0Rows rows of kL0Cols columns, each thread
-// kL0Rows x (kL0Cols / kL0Threads) samples with every load issued before the first store.
-constexpr int kL0Threads = 256, kL0Rows = 4, kL0Cols = 1024;
-template <typename S>
-__global__ void __launch_bounds__(kL0Threads) pyr_level0(const float *frames, size_t fstride, int W, int H,
-                                                         int pitch, S *out, size_t ostride, int opitch)
-{
-    constexpr int CB = kL0Cols / kL0Threads;
-    const int c0 = blockIdx.x * kL0Cols + threadIdx.x, r0 = blockIdx.y * kL0Rows;
-    const float *src = frames + blockIdx.z * fstride;
-    S *dst = out + blockIdx.z * ostride;
-    float v[kL0Rows][CB];
-#pragma unroll
-    for (int i = 0; i < kL0Rows; ++i)
-#pragma unroll
-        for (int j = 0; j < CB; ++j) {
-            const int r = r0 + i, c = c0 + j * kL0Threads;
-            v[i][j] = r < H && c < W ? __ldg(src + (size_t)r * pitch + c) : 0.f;
-        }
-#pragma unroll
-    for (int i = 0; i < kL0Rows; ++i)
-#pragma unroll
-        for (int j = 0; j < CB; ++j) {
-            const int r = r0 + i, c = c0 + j * kL0Threads;
-            if (r < H && c < W) dst[(size_t)r * opitch + c] = toS<S>(v[i][j]);
-        }
-}
-
-// Level l+1 from level l: 2x2 box average, last odd row/column clamped.  A thread makes kDnRows
-// samples of one column, every load issued before the first store.
-constexpr int kDnThreads = 128, kDnRows = 8;
-template <typename S>
-__global__ void __launch_bounds__(kDnThreads) pyr_down(const S *src, size_t sstride, int spitch, int W, int H,
-                                                       S *dst, size_t dstride, int dpitch)
-{
-    const int w2 = (W + 1) / 2, h2 = (H + 1) / 2;
-    const int c = blockIdx.x * kDnThreads + threadIdx.x, rb = blockIdx.y * kDnRows;
-    if (c >= w2) return;
-    src += blockIdx.z * sstride;
-    dst += blockIdx.z * dstride;
-    const int c0 = 2 * c, c1 = min(2 * c + 1, W - 1);
-    float v[kDnRows];
-#pragma unroll
-    for (int k = 0; k < kDnRows; ++k) {
-        v[k] = 0.f;
-        const int r = rb + k;
-        if (r < h2) {
-            const int r0 = 2 * r, r1 = min(2 * r + 1, H - 1);
-            v[k] = ((ldS<S>(src + (size_t)r0 * spitch + c0) + ldS<S>(src + (size_t)r0 * spitch + c1)) +
-                    ldS<S>(src + (size_t)r1 * spitch + c0)) + ldS<S>(src + (size_t)r1 * spitch + c1);
-        }
-    }
-#pragma unroll
-    for (int k = 0; k < kDnRows; ++k)
-        if (rb + k < h2) dst[(size_t)(rb + k) * dpitch + c] = toS<S>(0.25f * v[k]);
-}
-
-// Border of `pad` samples around a W x H level (pitch W + 2 pad) holding the level's mean (frame
-// f's at mean[f * mstride]): beyond its border a frame is taken to be its mean.  Thread t covers one
-// border sample, the top and bottom bands first, then the left and right bands.
-template <typename S>
-__global__ void pyr_border(S *lvl, size_t stride, int W, int H, int pad, const float *mean, int mstride)
-{
-    const int pitch = W + 2 * pad;
-    const int bands = 2 * pad * pitch, sides = 2 * pad * H;
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= bands + sides) return;
-    lvl += blockIdx.z * stride;
-    int r, c;
-    if (t < bands) {
-        const int q = t / pitch;                      // 0 .. 2 pad - 1
-        r = q < pad ? q - pad : H + (q - pad);        // -pad .. -1, then H .. H + pad - 1
-        c = t - q * pitch - pad;                      // -pad .. W + pad - 1
-    } else {
-        const int u = t - bands, q = u / H;           // 0 .. 2 pad - 1
-        r = u - q * H;
-        c = q < pad ? q - pad : W + (q - pad);
-    }
-    lvl[(ptrdiff_t)r * pitch + c] = toS<S>(mean[(size_t)blockIdx.z * mstride]);
-}
-
-// The quadratic B-spline model at the pixel centres: the separable filter (1/8, 3/4, 1/8) of a
-// bordered level (its border, the level's mean, supplies the outer taps), with the operations of
-// sample_q at a zero offset, so that a frame registered to itself matches bit for bit.  Written
-// as a plain W x H level.  A thread walks kSmoothRows rows down one column and carries the
-// horizontal filter of the rows above and at the current one, so each output row reads one row
-// of three taps.
-constexpr int kSmoothRows = 16;
-template <typename S>
-__global__ void pyr_smooth(const S *src, size_t sstride, int spitch, int W, int H, S *dst, size_t dstride)
-{
-    const int c = blockIdx.x * blockDim.x + threadIdx.x, r0 = blockIdx.y * kSmoothRows;
-    if (c >= W || r0 >= H) return;
-    const S *p = src + blockIdx.z * sstride + (ptrdiff_t)r0 * spitch + c;
-    S *q = dst + blockIdx.z * dstride + (size_t)r0 * W + c;
-    // the horizontal filter of row r0 + k of the bordered level (k = -1 .. kSmoothRows)
-    auto hrow = [&](int k) {
-        const S *x = p + (ptrdiff_t)k * spitch;
-        return fmaf(0.125f, ldS<S>(x + 1), fmaf(0.75f, ldS<S>(x), 0.125f * ldS<S>(x - 1)));
-    };
-    float a = hrow(-1), b = hrow(0);
-#pragma unroll
-    for (int k = 0; k < kSmoothRows; ++k) {
-        if (r0 + k >= H) break;
-        const float d = hrow(k + 1);
-        q[(size_t)k * W] = toS<S>(fmaf(0.125f, d, fmaf(0.75f, b, 0.125f * a)));
-        a = b;
-        b = d;
-    }
-}
-
-// Mean of one level of each frame (one CTA per frame), deterministic float-float sum.
-template <typename S>
-__global__ void __launch_bounds__(kThreads) level_mean(const S *img, size_t stride, int W, int H, int pitch,
-                                                       float *mean, int mstride)
-{
-    __shared__ float2 ws[kWarps];
-    img += blockIdx.x * stride;
-    const int n = W * H;
-    float hi = 0.f, lo = 0.f;
-    for (int base = 0; base < n; base += kThreads * kChunk) {
-        // a thread's kChunk samples of the chunk, loaded first, then summed in index order
-        float x[kChunk];
-#pragma unroll
-        for (int k = 0; k < kChunk; ++k) {
-            const int i = base + threadIdx.x + k * kThreads;
-            x[k] = 0.f;
-            if (i < n) {
-                const int r = i / W;
-                x[k] = ldS<S>(img + (size_t)r * pitch + (i - r * W));
-            }
-        }
-        float a = 0.f;
-#pragma unroll
-        for (int k = 0; k < kChunk; ++k) a += x[k];
-        ff_acc(hi, lo, a);
-    }
-    for (int off = 16; off > 0; off >>= 1) {
-        float h2 = __shfl_xor_sync(0xffffffffu, hi, off), l2 = __shfl_xor_sync(0xffffffffu, lo, off);
-        ff_add(hi, lo, h2, l2);
-    }
-    if ((threadIdx.x & 31) == 0) ws[threadIdx.x >> 5] = make_float2(hi, lo);
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        float h = 0.f, l = 0.f;
-        for (int k = 0; k < kWarps; ++k) ff_add(h, l, ws[k].x, ws[k].y);
-        mean[(size_t)blockIdx.x * mstride] = (float)(((double)h + (double)l) / (double)n);
-    }
-}
-
-// The level means of a freshly built pyramid into its rows of a level table.
-__global__ void set_level_means_kernel(LevelDesc *tab, const float *means, int L)
-{
-    const int l = threadIdx.x;
-    if (l < L) tab[l].mean = means[l];
-}
-
-cudaError_t launch_set_level_means(LevelDesc *tab, const float *means, int L, cudaStream_t s)
-{
-    set_level_means_kernel<<<1, 32, 0, s>>>(tab, means, L);
-    return cudaGetLastError();
-}
-
 // Composition of two control grids at the control points (standalone entry point).
 __global__ void grid_compose_kernel(const float2 *q1, const float2 *q2, Grid G, float2 *out)
 {
@@ -2262,63 +2049,6 @@ __global__ void grid_from_dense_kernel(const float *u, int W, int H, Grid G, flo
 }
 
 // ================================================================== host launchers
-template <typename S>
-static cudaError_t pyramid_t(const float *frames, int N, size_t fstride, int W, int H, int pitch, int levels,
-                             const PyrOut &o, float *means, cudaStream_t s)
-{
-    S *lv[kMaxLevels];
-    int w = W, h = H;
-    for (int l = 0; l < levels; ++l) {
-        lv[l] = (S *)o.raw[l] + level_origin(w, o.pad);
-        w = (w + 1) / 2;
-        h = (h + 1) / 2;
-    }
-    pyr_level0<S><<<dim3((W + kL0Cols - 1) / kL0Cols, (H + kL0Rows - 1) / kL0Rows, N), kL0Threads, 0, s>>>(
-        frames, fstride, W, H, pitch, lv[0], o.raw_stride[0], level_pitch(W, o.pad));
-    w = W; h = H;
-    for (int l = 0; l + 1 < levels; ++l) {
-        int w2 = (w + 1) / 2, h2 = (h + 1) / 2;
-        pyr_down<S><<<dim3((w2 + kDnThreads - 1) / kDnThreads, (h2 + kDnRows - 1) / kDnRows, N), kDnThreads, 0, s>>>(
-            lv[l], o.raw_stride[l], level_pitch(w, o.pad), w, h, lv[l + 1], o.raw_stride[l + 1], level_pitch(w2, o.pad));
-        w = w2; h = h2;
-    }
-    w = W; h = H;
-    for (int l = 0; l < levels; ++l) {
-        if (means)
-            level_mean<S><<<N, kThreads, 0, s>>>(lv[l], o.raw_stride[l], w, h, level_pitch(w, o.pad), means + l,
-                                                 levels);
-        if (o.pad > 0) {
-            const int nb = 2 * o.pad * level_pitch(w, o.pad) + 2 * o.pad * h;
-            pyr_border<S><<<dim3((nb + 127) / 128, 1, N), 128, 0, s>>>(lv[l], o.raw_stride[l], w, h, o.pad,
-                                                                       means + l, levels);
-            if (o.smooth[l])
-                pyr_smooth<S><<<dim3((w + 127) / 128, (h + kSmoothRows - 1) / kSmoothRows, N), 128, 0, s>>>(
-                    lv[l], o.raw_stride[l], level_pitch(w, o.pad), w, h, (S *)o.smooth[l], o.smooth_stride[l]);
-        }
-        w = (w + 1) / 2;
-        h = (h + 1) / 2;
-    }
-    return cudaGetLastError();
-}
-
-cudaError_t launch_pyramid(const float *frames, int N, size_t fstride, int W, int H, int pitch, int levels,
-                           int storage, const PyrOut &out, float *means, cudaStream_t s)
-{
-    if (out.pad != 0) {
-        // the smoothed levels read the 3x3 window of a bordered level; the border holds the mean
-        if (out.pad < 1 || !means) return cudaErrorInvalidValue;
-    } else {
-        for (int l = 0; l < levels; ++l)
-            if (out.smooth[l]) return cudaErrorInvalidValue;
-    }
-    switch (storage) {
-    case REG_F32: return pyramid_t<float>(frames, N, fstride, W, H, pitch, levels, out, means, s);
-    case REG_BF16: return pyramid_t<__nv_bfloat16>(frames, N, fstride, W, H, pitch, levels, out, means, s);
-    case REG_F16: return pyramid_t<__half>(frames, N, fstride, W, H, pitch, levels, out, means, s);
-    }
-    return cudaErrorInvalidValue;
-}
-
 // Dynamic shared memory of the nonrigid kernels (layout of grid_layout).
 static size_t grid_smem(const Params &p, int cluster)
 {
