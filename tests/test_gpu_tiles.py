@@ -1,0 +1,78 @@
+"""Sizes at which the tiles, strips and chunks of the kernels end: one row or column past a tile, fewer
+rows than CTAs, frames narrower than a warp, series of a few frames, against the oracle.
+
+Bounds as for the same steps at ordinary sizes: levels and registered frames a few FP32 roundings of
+values of order 1, energies 1e-6 relative, gradients 2e-4 of their largest entry.
+"""
+import numpy as np
+import pytest
+import torch
+
+import oracle as O
+from paper_2010_12478_gb300 import binding as B
+from paper_2010_12478_gb300 import synth
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def built():
+    from paper_2010_12478_gb300 import build
+    build.build()
+    assert torch.cuda.is_available(), "GPU tests need a CUDA device"
+
+
+@pytest.mark.parametrize("shape", [(8, 512), (9, 513), (7, 511), (17, 1025), (3, 3), (600, 31)])
+@pytest.mark.parametrize("storage", ["f32", "bf16", "f16"])
+def test_pyramid_levels_at_tile_edges(shape, storage):
+    H, W = shape
+    img = np.random.default_rng(2).uniform(0, 1, size=(H, W)).astype(np.float32)
+    h2, w2 = (H + 1) // 2, (W + 1) // 2
+    dt = {"f32": torch.float32, "bf16": torch.bfloat16, "f16": torch.float16}[storage]
+    out = torch.full((H * W + h2 * w2,), -7.0, dtype=dt, device="cuda")
+    B.Context(B.Config()).pyramid(torch.from_numpy(img).cuda(), 2, storage, out)
+    got = out.float().cpu().numpy().astype(np.float64)
+    l0, l1 = got[:H * W].reshape(H, W), got[H * W:].reshape(h2, w2)
+    assert np.array_equal(l0, torch.from_numpy(img).to(dt).double().numpy())
+    tol = {"f32": 3e-7, "bf16": 8e-3, "f16": 1e-3}[storage]
+    np.testing.assert_allclose(l1, O.downsample(l0), rtol=tol, atol=tol)
+
+
+@pytest.mark.parametrize("shape", [(17, 33), (65, 513), (240, 37), (3, 129), (129, 3)])
+@pytest.mark.parametrize("far", [0.0, 40.0])
+def test_energy_and_gradient_at_strip_edges(shape, far):
+    # far: every sample beyond the template's border on one side of the frame, so the mean that stands
+    # there (the border of a level, its model at the pixel centres) carries the energy
+    H, W = shape
+    rng = np.random.default_rng(11)
+    R, T = (rng.uniform(0, 1, size=(H, W)).astype(np.float32) for _ in range(2))
+    g = O.grid_for(W, H)
+    c = rng.uniform(-0.5, 0.5, size=(2, g.ny, g.nx))
+    c[0] += far * np.linspace(0.0, 1.0, g.nx)[None, :]
+    cd = torch.from_numpy(np.ascontiguousarray(c.transpose(1, 2, 0)).astype(np.float32)).cuda()
+    gd = torch.zeros((g.ny, g.nx, 2), device="cuda")
+    dR, dT = torch.from_numpy(R).cuda(), torch.from_numpy(T).cuda()
+    E = B.Context(B.Config(mode="nonrigid")).energy_grid(dR, dT, cd, gd)
+    Eo, go = O.grid_energy(R, T, 0, g, cd.cpu().numpy().transpose(2, 0, 1).astype(np.float64), 2.0)
+    assert abs(E - Eo) <= 1e-6 * abs(Eo)
+    np.testing.assert_allclose(gd.cpu().numpy().transpose(2, 0, 1), go, atol=2e-4 * np.abs(go).max())
+    th = [0.01, 0.3 + 0.2 * far, -0.2]
+    E, gr = B.Context(B.Config()).energy_rigid(dR, dT, th)
+    Eo, gro = O.rigid_energy(R, T, th)
+    assert abs(E - Eo) <= 1e-6 * abs(Eo)
+    assert np.abs(gr - gro).max() <= 1e-4 * max(1.0, np.abs(gro).max())
+
+
+@pytest.mark.parametrize("N", [1, 2, 5, 65, 131])
+def test_registered_mean_over_any_number_of_frames(N):
+    # the frames of a chunk, and so the number of chunks, follow from the sizes
+    F = synth.make_series(synth.SeriesSpec(N, 70, 133, step=2.0, snr=(10.0, 10.0), seed=4)).frames
+    rng = np.random.default_rng(N)
+    els = [(0, k + 1, *(float(v) for v in rng.uniform(-1, 1, 3) * (0.02, 6.0, 6.0))) for k in range(N - 1)]
+    mean = torch.empty((70, 133), device="cuda")
+    out = torch.empty((N, 70, 133), device="cuda")
+    B.Context(B.Config()).warp(F.cuda(), elems=els, out=out, mean=mean)
+    want, wmean = O.register_series(F.numpy().astype(np.float64), "rigid",
+                                    [np.array(e[2:], np.float32).astype(np.float64) for e in els])
+    assert np.abs(out.cpu().numpy() - want).max() <= 1e-5
+    assert np.abs(mean.cpu().numpy() - wmean).max() <= 1e-5
