@@ -32,6 +32,7 @@ constexpr int kConsumers = 8;              // consumer warps; one more warp prod
 constexpr int kRun = 16;                   // frames summed in FP32 before the float-float fold
 constexpr int kWinX = 12, kWinY = 8;       // control points under a tile (spacing >= 8)
 constexpr int kWThreads = 32 * (kConsumers + 1);
+constexpr int kCtasPerSm = 3;              // 70 KB of shared memory each
 constexpr unsigned kBoxBytes = kBW * kBH * 4;
 constexpr unsigned kMaxTap = kBW * kBH - kBW - 2;   // largest top-left tap index in a box
 
@@ -421,7 +422,7 @@ __device__ __forceinline__ void fold(float2 &hi, float2 &lo, float2 &run)
 }
 
 template <int MODE, bool WINDOW>
-__global__ void __launch_bounds__(kWThreads, 3) warp_kernel(const WarpArgs a, const __grid_constant__ CUtensorMap tmap)
+__global__ void __launch_bounds__(kWThreads, kCtasPerSm) warp_kernel(const WarpArgs a, const __grid_constant__ CUtensorMap tmap)
 {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     WarpSmem &sm = *reinterpret_cast<WarpSmem *>(smem_raw);
@@ -602,14 +603,37 @@ EncodeTiled encoder()
 
 }  // namespace
 
-int warp_chunk_frames()
+// Frames per chunk.  A block takes the frames of one chunk at one tile, so the grid is tiles x
+// chunks; with a fixed 64 frames, 256 frames of 512x512 made 512 blocks for the 456 that are resident
+// at once, and the second wave ran nearly empty (219 us a call with frames and mean out, 196 us with 7 chunks of 37
+// frames in two full waves).  The rule takes the chunk whose waves x (frames + kChunkCost) is least, the larger
+// of equals: kChunkCost stands for the pipeline's fill and the chunk's partial sums, in frames, and
+// keeps the chunks of a long series near 64.  It depends on the sizes alone, so a series' mean does
+// not depend on which outputs a call asks for.
+constexpr int kMaxChunk = 64, kChunkCost = 4;
+static int warp_chunk_frames(int N, int W, int H)
 {
-    return 64;
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+        sms = 152;
+    const long long tiles = (long long)((W + kTW - 1) / kTW) * ((H + kTH - 1) / kTH), slots = (long long)kCtasPerSm * sms;
+    const int top = N < kMaxChunk ? N : kMaxChunk;
+    int best = top;
+    long long least = -1;
+    for (int c = top; c >= 1; --c) {
+        const long long blocks = tiles * ((N + c - 1) / c), cost = (blocks + slots - 1) / slots * (c + kChunkCost);
+        if (least < 0 || cost < least) {
+            least = cost;
+            best = c;
+        }
+    }
+    return best;
 }
 
 size_t warp_workspace_bytes(int N, int W, int H, bool mean)
 {
-    const size_t chunks = (size_t)(N + warp_chunk_frames() - 1) / warp_chunk_frames();
+    const int chunk = warp_chunk_frames(N, W, H);
+    const size_t chunks = (size_t)(N + chunk - 1) / chunk;
     size_t b = 256 * (((size_t)N * sizeof(float4) + 255) / 256);
     if (mean) b += chunks * (size_t)W * H * sizeof(float2);
     return b;
@@ -617,7 +641,7 @@ size_t warp_workspace_bytes(int N, int W, int H, bool mean)
 
 cudaError_t launch_warp(const WarpJob &j, cudaStream_t s, int *used_tma)
 {
-    const int chunk = warp_chunk_frames();
+    const int chunk = warp_chunk_frames(j.N, j.W, j.H);
     const int chunks = (j.N + chunk - 1) / chunk;
     WarpArgs a;
     memset(&a, 0, sizeof(a));
