@@ -131,18 +131,19 @@ typedef struct {
     double step_cap;      /* largest step, pixels of the current level */
     double lambda;        /* regulariser weight (REG_NONRIGID) */
     int    storage;       /* REG_F32, REG_BF16 or REG_F16 pyramid storage */
-    int    cluster;       /* CTAs cooperating on one operator (1,2,4,8,16); 0 = auto */
+    int    cluster;       /* CTAs cooperating on one operator (1,2,4,8,16); 0 = auto.  Raised where a
+                             control grid does not fit the shared memory of so few */
     int    workers;       /* persistent executor: operator slots in flight; 0 = auto */
     size_t mem_budget;    /* stream service: device bytes it may hold; 0 = unlimited */
     int    grid;          /* REG_NONRIGID control-grid spacing in finest pixels; 0 = auto (16,
                              doubled until at most 65 points per axis); a multiple of 2^(levels-1) */
     int    metric;        /* REG_NONRIGID scalar product of the gradient flow: REG_METRIC_GAUSS_NEWTON
                              (default), REG_METRIC_MEAN or REG_METRIC_H1 */
-    int    unroll;        /* REG_NONRIGID energy passes: pixels in flight per lane (2 or 4); 0 = auto
+    int    unroll;        /* REG_NONRIGID passes: pixels in flight per lane (2 or 4); 0 = auto
                              (the autotuned value, else 4) */
-    int    ctas_per_sm;   /* REG_NONRIGID operator kernels: register budget sized for 3 or 4 CTAs
-                             per SM (80 or 64 registers a thread); 0 = auto (the autotuned value,
-                             else 4 for 16-CTA operators and 3 below) */
+    int    ctas_per_sm;   /* REG_NONRIGID register form, 3 or 4; 0 = auto (3).  Accepted and recorded
+                             for saved shapes; both name the one form there is, 128 registers a
+                             thread and two CTAs per SM */
     double sigma;         /* REG_METRIC_H1: smoothing length in control-grid spacings (>= 0; default 1) */
     double tol_coarse;    /* stop at every level above the finest: tol_coarse x tol_grad (a coarse
                              level only supplies the next level's initial guess); in [1, 1e6],
@@ -417,9 +418,8 @@ int reg_stream_close(reg_stream_t *s);
  * storage type and executor, by timing reg_scan on `frames` (each candidate twice, after one
  * untimed run; nonrigid scans are timed without dense fields, whose kernel costs the same for
  * every candidate) and keeping the fastest:
- *   1. CTAs per operator (rows of each pyramid level per CTA): 1, 2, 4, 8 and 16, for
- *      REG_NONRIGID each with either register form (3 or 4 CTAs per SM);
- *   2. REG_NONRIGID, at the chosen pair: pixels per lane of the energy passes (4, then 2).
+ *   1. CTAs per operator (rows of each pyramid level per CTA): 1, 2, 4, 8 and 16;
+ *   2. REG_NONRIGID, at the chosen size: pixels per lane of the passes (4, then 2).
  * Fields of cfg that are set (cluster, unroll, ctas_per_sm > 0) are not tuned.  Later reg_scan
  * calls on the context with a matching shape (same W, H, mode, storage, executor and
  * floor(log2 N)) use the choice for every field the config leaves at 0.  Arguments as reg_scan;
@@ -459,7 +459,7 @@ typedef struct {
                                   of the B phase (same method as op_kernel_ms) */
     int32_t cluster;           /* launch shape of the last operator launch: CTAs per operator, */
     int32_t unroll;            /* energy-pass pixels per lane (0 for REG_RIGID), */
-    int32_t ctas_per_sm;       /* and the register form (CTAs per SM it is sized for) */
+    int32_t ctas_per_sm;       /* and the register form */
     int32_t h2d_path;          /* host frames staged by: 0 none (device frames), 1 cudaMemcpyAsync,
                                   2 the SMs reading mapped page-locked memory */
     double  h2d_ms;            /* with timing: device time of that staging (0 for device frames) */

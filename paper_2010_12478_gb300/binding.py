@@ -174,8 +174,8 @@ class Config:
     grid: int = 0
     metric: int = 1               # nonrigid scalar product: 1 Gauss-Newton diagonal, 0 mean over control
                                   # points, 2 H1 (identity + sigma^2 grid Laplacian)
-    unroll: int = 0               # nonrigid energy passes: pixels per lane (2, 4); 0 = tuned or 4
-    ctas_per_sm: int = 0          # nonrigid register form (3, 4); 0 = tuned or by CTAs per operator
+    unroll: int = 0               # nonrigid passes: pixels per lane (2, 4); 0 = tuned or 4
+    ctas_per_sm: int = 0          # nonrigid register form (3, 4: one and the same); 0 = 3
     sigma: float = 1.0            # metric 2 (H1): smoothing length in control-grid spacings
     tol_coarse: float = 10.0      # stop factor at every level above the finest
 

@@ -697,7 +697,7 @@ void note_shape(reg_ctx *ctx, const Params &p, int C)
 {
     ctx->last.cluster = C;
     ctx->last.unroll = p.cfg.mode == REG_NONRIGID ? (p.unroll == 2 ? 2 : 4) : 0;
-    ctx->last.ctas_per_sm = p.cfg.mode == REG_NONRIGID ? (p.minb > 0 ? p.minb : (C >= 16 ? 4 : 3)) : 4;
+    ctx->last.ctas_per_sm = p.cfg.mode == REG_NONRIGID ? (p.minb > 0 ? p.minb : 3) : 4;
 }
 
 int pow2_floor(int v)
@@ -895,7 +895,7 @@ int execute(reg_ctx *ctx, const ScanPlan &plan, Params &p, int exec, const TileS
     if (exec == REG_EXEC_LEVEL) {
         for (int dpt = 0; dpt < n_depth; ++dpt) {
             int b = plan.depth_start[dpt], e = plan.depth_start[dpt + 1];
-            int C = tuned.cluster > 0 ? tuned.cluster : auto_cluster(ctx, e - b);
+            const int C = fit_cluster(p, tuned.cluster > 0 ? tuned.cluster : auto_cluster(ctx, e - b));
             note_shape(ctx, p, C);
             int chunk = std::max(1, e - b);
             for (int q = b; q < e; q += chunk) {
@@ -911,7 +911,7 @@ int execute(reg_ctx *ctx, const ScanPlan &plan, Params &p, int exec, const TileS
     if (exec == REG_EXEC_PLAIN) {
         CHECK(ensure_pool(ctx));
         CHECK(ensure_op_events(ctx, n_ops));
-        const int C = tuned.cluster > 0 ? tuned.cluster : 8;
+        const int C = fit_cluster(p, tuned.cluster > 0 ? tuned.cluster : 8);
         note_shape(ctx, p, C);
         const int t0 = timing_mark(ctx, s);
         CHECK(launch_plain(ctx, plan, p, C, s));
@@ -922,7 +922,7 @@ int execute(reg_ctx *ctx, const ScanPlan &plan, Params &p, int exec, const TileS
     if (exec == REG_EXEC_GRAPH) {
         CHECK(ensure_pool(ctx));
         CHECK(ensure_op_events(ctx, n_ops));
-        const int C = tuned.cluster > 0 ? tuned.cluster : 8;
+        const int C = fit_cluster(p, tuned.cluster > 0 ? tuned.cluster : 8);
         note_shape(ctx, p, C);
         // The graph bakes in the kernel arguments (workspace pointers, config) and the
         // dependency edges; the descriptors themselves are read from device memory when it runs.
@@ -1059,7 +1059,7 @@ int execute(reg_ctx *ctx, const ScanPlan &plan, Params &p, int exec, const TileS
             long long ms = atoll(t);
             if (ms > 0) p.queue.timeout_ns = ms * 1000 * 1000;
         }
-        const int C = tuned.cluster > 0 ? tuned.cluster : 8;
+        const int C = fit_cluster(p, tuned.cluster > 0 ? tuned.cluster : 8);
         note_shape(ctx, p, C);
         int workers = ctx->cfg.workers;
         if (workers <= 0) {
@@ -1546,7 +1546,7 @@ extern "C" int reg_pairwise(reg_ctx_t *ctx, const float *R, const float *T, int 
             CU(cudaStreamSynchronize(s));
         }
     }
-    int C = ctx->cfg.cluster > 0 ? ctx->cfg.cluster : 8;
+    const int C = fit_cluster(p, ctx->cfg.cluster > 0 ? ctx->cfg.cluster : 8);
     p.op_base = 0;
     p.unroll = ctx->cfg.unroll;
     p.minb = ctx->cfg.ctas_per_sm;
@@ -1737,32 +1737,24 @@ extern "C" int reg_autotune(reg_ctx_t *ctx, const float *frames, int N, int W, i
     TileShape bestT;
     int rc = REG_OK;
     float best_ms = 1e30f;
-    // 1. CTAs per operator (nonrigid: with either register form), at the default pixels per lane
+    // 1. CTAs per operator, at the default pixels per lane
     const bool nonrigid = saved.mode == REG_NONRIGID;
     const int clusters[] = {1, 2, 4, 8, 16};
     for (int c : clusters) {
         if (saved.cluster > 0 && c != saved.cluster) continue;
-        bool stop = false;
-        for (int mb : {3, 4}) {
-            if (!nonrigid && mb == 4) continue;
-            if (nonrigid && saved.ctas_per_sm > 0 && mb != saved.ctas_per_sm) continue;
-            ctx->cfg.cluster = c;
-            if (nonrigid) ctx->cfg.ctas_per_sm = mb;
-            float ms;
-            rc = trial(ms);
-            if (rc != REG_OK) { stop = true; break; }   // e.g. a cluster size the device cannot schedule
-            if (ms < best_ms) {
-                best_ms = ms;
-                bestT.cluster = c;
-                bestT.minb = nonrigid ? mb : 0;
-            }
+        ctx->cfg.cluster = c;
+        float ms;
+        rc = trial(ms);
+        if (rc != REG_OK) break;   // e.g. a cluster size the device cannot schedule
+        if (ms < best_ms) {
+            best_ms = ms;
+            bestT.cluster = c;
+            bestT.minb = !nonrigid ? 0 : saved.ctas_per_sm > 0 ? saved.ctas_per_sm : 3;
         }
-        if (stop) break;
     }
     // 2. nonrigid: the other pixels per lane at that shape
     if (bestT.cluster > 0 && nonrigid) {
         ctx->cfg.cluster = bestT.cluster;
-        ctx->cfg.ctas_per_sm = bestT.minb;
         bestT.unroll = saved.unroll > 0 ? saved.unroll : 4;
         if (saved.unroll == 0) {
             ctx->cfg.unroll = 2;

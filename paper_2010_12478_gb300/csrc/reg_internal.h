@@ -109,9 +109,8 @@ struct Params {
     float2 *node_grid;         // nonrigid: [n_nodes][gny * gnx] control values (finest px)
     const float *mock_us;      // mock operator (kModeMock): duration of each operator, microseconds
     const float *h1q;          // REG_METRIC_H1: the control grid's cosine bases and eigenvalues (Qx, Qy, lx, ly)
-    int unroll;                // nonrigid energy passes: pixels in flight per lane (2 or 4; 0 = 4)
-    int minb;                  // nonrigid register form: CTAs per SM (3 or 4; 0 = 4 at 16 CTAs per
-                               // operator, else 3)
+    int unroll;                // nonrigid passes: pixels in flight per lane (2 or 4; 0 = 4)
+    int minb;                  // nonrigid register form as configured (3 or 4; 0 = 3); one kernel serves both
     int gnx, gny, gs;          // nonrigid control grid: points per axis and spacing (finest px)
     int n_nodes;
     OpStats *stats;            // [n_ops]
@@ -120,7 +119,7 @@ struct Params {
 };
 
 // Launch shape of the operator kernels (0 = not chosen): CTAs per operator, energy-pass pixels
-// per lane, and register form (CTAs per SM the kernel's register budget is sized for).
+// per lane, and register form.
 struct TileShape {
     int cluster = 0, unroll = 0, minb = 0;
 };
@@ -134,6 +133,9 @@ cudaError_t launch_pyramid(const float *frames, int N, size_t fstride, int W, in
 int pyramid_launches(int levels, bool means, int pad);
 // tab[l].mean = means[l] for l < L (a slot's level table rows after its pyramid build).
 cudaError_t launch_set_level_means(LevelDesc *tab, const float *means, int L, cudaStream_t s);
+// CTAs per operator for a launch that asks for `cluster`: more where an operator's control grid does
+// not fit the shared memory of so few.
+int fit_cluster(const Params &p, int cluster);
 cudaError_t launch_ops(const Params &p, int storage, int cluster, int n_launch_ops,
                        cudaStream_t s);
 cudaError_t launch_persistent(const Params &p, int storage, int cluster, int workers,

@@ -5,20 +5,19 @@
 //     inside ONE thread-block cluster: every level, every gradient-flow
 //     iteration and every Armijo trial.  The C CTAs of the cluster split the
 //     rows of each pyramid level; their partial sums meet through distributed
-//     shared memory, so an iteration costs one cluster barrier and never a
+//     shared memory, so an iteration costs cluster barriers and never a
 //     kernel launch or a grid-wide synchronisation.
-//   * Per pixel the work is FP32 (warp, bilinear sample, derivative, moment
-//     products).  Sums are accumulated per thread in FP32 over chunks of 32
-//     pixels, then carried as float-float pairs (error-free transformations on
-//     the FP32 pipes: GB300's FP64 rate is a small fraction of FP32) through the
-//     warp and CTA stages, and in FP64 across the cluster.  Reduction order is
-//     fixed, so results are bitwise reproducible for a given cluster size.
+//   * Per pixel the work is FP32 (warp, sample, derivative, moment products).
+//     Sums are accumulated per thread in FP32 over runs of 8 pixels, then carried
+//     as float-float pairs (error-free transformations on the FP32 pipes: GB300's
+//     FP64 rate is a small fraction of FP32) through the warp and CTA stages, and
+//     in FP64 across the cluster.  Reduction order is fixed, so results are bitwise
+//     reproducible for a given cluster size.
 //   * The step controller (NCC from the moments, gradient, Armijo test, step
 //     size, stop rules) is FP64 and runs on thread 0 of every CTA of the
 //     cluster on identical totals, so all CTAs take identical decisions.
-//   * Images are read through the read-only path; the nonrigid fields, which
-//     the cluster rewrites between passes, through L2 (ld/st .cg) with a fence
-//     before each cluster barrier.
+//   * Images are read through the read-only path; the nonrigid model's control
+//     values live in shared memory.
 #include <cooperative_groups.h>
 
 #include <cmath>
@@ -32,7 +31,7 @@ namespace cg = cooperative_groups;
 namespace reg {
 
 constexpr int kWarps = kThreads / 32;
-constexpr int kNM = 8;         // moment slots per reduction (at most 6 are used)
+constexpr int kNM = 16;        // sums per reduction at most
 constexpr int kMaxCluster = 16; // CTAs per operator at most (non-portable cluster size)
 constexpr int kChunk = 32;     // pixels per thread between float-float flushes
 
@@ -50,7 +49,7 @@ struct RigidCtl {
 };
 
 struct FieldCtl {
-    double E, tau, tau_pend, tau_acc, slope, P, Nc, sr, srr, invP, invNc;
+    double E, tau, tau_acc, slope, P, Nc, sr, srr, invP, invNc;
     double a, b, rbar, tbar;      // NCC terms at the current field
     double ta, tb, trbar, ttbar;  // at the trial field
     int degen, tdegen;
@@ -72,6 +71,8 @@ struct Smem {
     float2 warp[kWarps][kNM];   // per-warp (hi, lo) partials
     double part[2][kMaxCluster][kNM];   // every CTA's partials, pushed here by each CTA
     double tot[kNM];            // cluster totals
+    unsigned wmax[kWarps], pmax[2][kMaxCluster];   // bits of the per-warp and per-CTA maxima
+    double tmax;
     float pm[16];               // pass parameters broadcast by thread 0
     int action;
     int idata[4];
@@ -81,62 +82,75 @@ struct Smem {
     };
 };
 
-// Reduce NM per-thread float-float partials over the cluster into sm.tot.
-// If MAXLAST, slot NM-1 holds a non-negative value combined by max (hi only).
-template <int NM, bool MAXLAST>
-__device__ __forceinline__ void cluster_reduce(float (&hi)[NM], float (&lo)[NM], Smem &sm,
-                                               int &buf, const cg::cluster_group &cl, bool fence)
+// Reduce NM per-thread float-float sums over the cluster into sm.tot, in a fixed order, and with MAXV
+// the largest of a non-negative value into sm.tmax.  Within a warp the sums are exchanged by halves,
+// so a lane carries one of them after log2 steps (9 pair additions for 8 sums instead of 40); the
+// warps', then the CTAs' partials of a sum are shared out over the lanes and folded the same way.
+// Every CTA pushes its partials into every CTA's shared memory (remote stores do not wait; the cluster
+// barrier makes them visible) and adds the same values in the same order: identical totals.
+template <int NM, bool MAXV>
+__device__ __forceinline__ void cluster_reduce(const float (&hi)[NM], const float (&lo)[NM], float mx, Smem &sm,
+                                               int &buf, const cg::cluster_group &cl)
 {
-    static_assert(NM <= kNM, "reduction slots");
+    static_assert(NM <= kNM && kWarps == 8, "reduction slots");
+    constexpr int kLog = NM <= 8 ? 3 : 4, N2 = 1 << kLog, kParts = 32 / N2;   // lanes that share a sum
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+    float h[N2], l[N2];
 #pragma unroll
-    for (int m = 0; m < NM; ++m) {
+    for (int m = 0; m < N2; ++m) { h[m] = m < NM ? hi[m] : 0.f; l[m] = m < NM ? lo[m] : 0.f; }
 #pragma unroll
-        for (int off = 16; off > 0; off >>= 1) {
-            float h2 = __shfl_xor_sync(0xffffffffu, hi[m], off);
-            float l2 = __shfl_xor_sync(0xffffffffu, lo[m], off);
-            if (MAXLAST && m == NM - 1) hi[m] = fmaxf(hi[m], h2);
-            else ff_add(hi[m], lo[m], h2, l2);
+    for (int o = 16, n = N2 / 2; o >= 1; o >>= 1, n >>= 1) {
+        if (n >= 1) {
+            const bool up = lane & o;
+#pragma unroll
+            for (int m = 0; m < n; ++m) {
+                const float h2 = __shfl_xor_sync(0xffffffffu, up ? h[m] : h[m + n], o);
+                const float l2 = __shfl_xor_sync(0xffffffffu, up ? l[m] : l[m + n], o);
+                h[m] = up ? h[m + n] : h[m];
+                l[m] = up ? l[m + n] : l[m];
+                ff_add(h[m], l[m], h2, l2);
+            }
+        } else {
+            const float h2 = __shfl_xor_sync(0xffffffffu, h[0], o), l2 = __shfl_xor_sync(0xffffffffu, l[0], o);
+            ff_add(h[0], l[0], h2, l2);
         }
     }
-    if (lane == 0) {
-#pragma unroll
-        for (int m = 0; m < NM; ++m) sm.warp[w][m] = make_float2(hi[m], lo[m]);
+    if (lane % kParts == 0) sm.warp[w][lane / kParts] = make_float2(h[0], l[0]);
+    if constexpr (MAXV) {
+        const unsigned m = __reduce_max_sync(0xffffffffu, __float_as_uint(mx));   // non-negative: bits order as values
+        if (lane == 0) sm.wmax[w] = m;
     }
     __syncthreads();
-    const unsigned C = cl.num_blocks(), me = cl.block_rank();
-    if (tid < NM) {
-        float h = 0.f, l = 0.f;
-        for (int k = 0; k < kWarps; ++k) {
-            float2 v = sm.warp[k][tid];
-            if (MAXLAST && tid == NM - 1) h = fmaxf(h, v.x);
-            else ff_add(h, l, v.x, v.y);
+    const int C = cl.num_blocks(), me = cl.block_rank();
+    const int m = lane % N2, q = lane / N2;   // warp 0: lane's sum, and which share of its parts
+    if (w == 0) {
+        float2 v = sm.warp[q][m];
+#pragma unroll
+        for (int k = q + kParts; k < kWarps; k += kParts) ff_add(v.x, v.y, sm.warp[k][m].x, sm.warp[k][m].y);
+#pragma unroll
+        for (int o = N2; o < 32; o <<= 1) {
+            const float h2 = __shfl_xor_sync(0xffffffffu, v.x, o), l2 = __shfl_xor_sync(0xffffffffu, v.y, o);
+            ff_add(v.x, v.y, h2, l2);
         }
-        // push this CTA's partial into slot `me` of every CTA of the cluster (remote stores do
-        // not wait; the cluster barrier below makes them visible)
-        const double v = (double)h + (double)l;
-        for (unsigned r = 0; r < C; ++r) *cl.map_shared_rank(&sm.part[buf][me][tid], r) = v;
+        const double t = (double)v.x + (double)v.y;
+        for (int r = q; r < C; r += kParts) *cl.map_shared_rank(&sm.part[buf][me][m], r) = t;
+    } else if (MAXV && w == 1) {
+        const unsigned v = __reduce_max_sync(0xffffffffu, lane < kWarps ? sm.wmax[lane] : 0u);
+        if (lane < C) *cl.map_shared_rank(&sm.pmax[buf][me], lane) = v;
     }
-    if (fence) __threadfence();
     cl.sync();
-    if (tid < NM) {
-        // every CTA adds the same values in rank order: identical totals everywhere
-        double s = 0.0;
-        for (unsigned r = 0; r < C; ++r) {
-            const double v = sm.part[buf][r][tid];
-            if (MAXLAST && tid == NM - 1) s = fmax(s, v);
-            else s = __dadd_rn(s, v);
-        }
-        sm.tot[tid] = s;
+    if (w == 0) {
+        double s = q < C ? sm.part[buf][q][m] : 0.0;
+        for (int r = q + kParts; r < C; r += kParts) s = __dadd_rn(s, sm.part[buf][r][m]);
+#pragma unroll
+        for (int o = N2; o < 32; o <<= 1) s = __dadd_rn(s, __shfl_xor_sync(0xffffffffu, s, o));
+        if (lane < N2) sm.tot[m] = s;
+    } else if (MAXV && w == 1) {
+        const unsigned v = __reduce_max_sync(0xffffffffu, lane < C ? sm.pmax[buf][lane] : 0u);
+        if (lane == 0) sm.tmax = (double)__uint_as_float(v);
     }
     buf ^= 1;
     __syncthreads();
-}
-
-__device__ __forceinline__ void cluster_barrier(const cg::cluster_group &cl)
-{
-    __threadfence();
-    cl.sync();
 }
 
 // ------------------------------------------------------------------ NCC (FP64)
@@ -205,39 +219,7 @@ __device__ __forceinline__ void strip_rows(int H, int rank, int C, int &r0, int 
     r1 = min(H, r0 + per);
 }
 
-// Iterate the pixels of rows [r0, r1): f(r, c) per pixel; flush_fast() after every
-// kFast pixels of this thread and flush() after every kChunk pixels (and at the end).
-constexpr int kFast = 8;
-template <typename F, typename G, typename Q>
-__device__ __forceinline__ void for_pixels2(int W, int r0, int r1, F &&f, Q &&flush_fast, G &&flush)
-{
-    const int tid = threadIdx.x;
-    int i = r0 * W + tid;
-    const int end = r1 * W;
-    int r = i / W, c = i - r * W;
-    const int dr = kThreads / W, dc = kThreads - dr * W;
-    while (i < end) {
-#pragma unroll 1
-        for (int q = 0; q < kChunk / kFast && i < end; ++q) {
-#pragma unroll 1
-            for (int k = 0; k < kFast && i < end; ++k) {
-                f(r, c);
-                i += kThreads;
-                c += dc; r += dr;
-                if (c >= W) { c -= W; r += 1; }
-            }
-            flush_fast();
-        }
-        flush();
-    }
-}
-
-template <typename F, typename G>
-__device__ __forceinline__ void for_pixels(int W, int r0, int r1, F &&f, G &&flush)
-{
-    for_pixels2(W, r0, r1, f, []() {}, flush);
-}
-
+constexpr int kFast = 8;   // pixels of a thread in one FP32 run before the float-float fold
 // Row-major traversal for the fused evaluation passes: warp w walks rows r0 + w, r0 + w + kWarps,
 // ...; in a row, lane l takes columns l + 32 u (u < U) per step, so each thread has U independent
 // samples in flight and a warp's loads stay coalesced.  row(r) runs once per row; px(r, c) per
@@ -255,35 +237,6 @@ __device__ __forceinline__ void for_rows(int W, int r0, int r1, RowF &&row, PixF
             if (c0 + 32 * (U - 1) < W) {
 #pragma unroll
                 for (int u = 0; u < U; ++u) px(r, c0 + 32 * u);
-            } else {
-#pragma unroll
-                for (int u = 0; u < U; ++u)
-                    if (c0 + 32 * u < W) px(r, c0 + 32 * u);
-            }
-            cnt += U;
-            if ((cnt & (kFast - 1)) == 0) flush_fast();
-            if ((cnt & (kChunk - 1)) == 0) flush();
-        }
-    }
-    flush_fast();
-    flush();
-}
-
-// for_rows with the pixels of a step taken in pairs: px2(r, c, c + 32) for columns 32 apart (U
-// even); a row's partial last step goes pixel by pixel through px(r, c).
-template <int U, typename RowF, typename Pix2F, typename PixF, typename Q, typename G>
-__device__ __forceinline__ void for_rows2(int W, int r0, int r1, RowF &&row, Pix2F &&px2, PixF &&px, Q &&flush_fast,
-                                          G &&flush)
-{
-    static_assert(kFast % U == 0 && U % 2 == 0, "U even, dividing kFast");
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    int cnt = 0;
-    for (int r = r0 + warp; r < r1; r += kWarps) {
-        row(r);
-        for (int c0 = lane; c0 < W; c0 += 32 * U) {
-            if (c0 + 32 * (U - 1) < W) {
-#pragma unroll
-                for (int u = 0; u < U; u += 2) px2(r, c0 + 32 * u, c0 + 32 * u + 32);
             } else {
 #pragma unroll
                 for (int u = 0; u < U; ++u)
@@ -328,114 +281,6 @@ __device__ __forceinline__ float sample_at(const S *T, int W, int H, int Tp, int
         dty = cly ? 0.f : (bot - top);
     }
     return fmaf(fy, bot, gy * top);
-}
-
-// Bilinear value (no derivative) of an fp32 field read through L2, at (xi + vx, yi + vy).
-__device__ __forceinline__ float sample_cg(const float *F, int W, int H, int xi, int yi, float vx, float vy)
-{
-    vx = fminf(fmaxf(vx, -1.0e6f), 1.0e6f);
-    vy = fminf(fmaxf(vy, -1.0e6f), 1.0e6f);
-    const float flx = floorf(vx), fly = floorf(vy);
-    int x = xi + (int)flx, y = yi + (int)fly;
-    float fx = vx - flx, fy = vy - fly;
-    if (x < 0) { x = 0; fx = 0.f; } else if (x > W - 2) { x = W - 2; fx = 1.f; }
-    if (y < 0) { y = 0; fy = 0.f; } else if (y > H - 2) { y = H - 2; fy = 1.f; }
-    const float *row = F + (size_t)y * W + x;
-    float t00 = __ldcg(row), t01 = __ldcg(row + 1), t10 = __ldcg(row + W), t11 = __ldcg(row + W + 1);
-    float gx = 1.f - fx;
-    float top = fmaf(fx, t01, gx * t00);
-    float bot = fmaf(fx, t11, gx * t10);
-    return fmaf(fy, bot, (1.f - fy) * top);
-}
-
-// Quadratic B-spline model of the samples of T (storage S) at p = (xi + vx, yi + vy), with the
-// samples beyond the border equal to the level's mean: the image model of the nonrigid energy,
-// continuously differentiable everywhere.  With n the nearest sample and t = p - n in
-// [-1/2, 1/2) per axis, the three taps n - 1, n, n + 1 carry the weights (1/2 - t)^2 / 2,
-// 3/4 - t^2, (1/2 + t)^2 / 2 and, for the derivative, t - 1/2, -2 t, t + 1/2.  T addresses
-// pixel (0, 0) of a level stored with a border of kPad >= 3 samples holding its mean (row pitch
-// Tp): n clamped to [-2, W + 1] x [-2, H + 1] keeps the window inside the border, and a window
-// clamped there lies wholly in the border, as the true one does: the mean-extended model for any p.
-template <typename S, bool DERIV>
-__device__ __forceinline__ float sample_q(const S *T, int W, int H, int Tp, int xi, int yi, float vx, float vy,
-                                          float &dtx, float &dty)
-{
-    // nearest sample n = floor(v + 1/2), t = v - n: within rounding of [-1/2, 1/2) (at a tie either
-    // window gives the same value and derivative, the model being C1).  A NaN or huge offset
-    // converts to 0 or a saturated integer, the sum wraps, and the clamp keeps the window inside
-    // the border whatever the offset.
-    const float fnx = floorf(vx + 0.5f), fny = floorf(vy + 0.5f);
-    const float tx = vx - fnx, ty = vy - fny;
-    int nx = (int)((unsigned)xi + (unsigned)__float2int_rz(fnx));
-    int ny = (int)((unsigned)yi + (unsigned)__float2int_rz(fny));
-    nx = min(max(nx, -2), W + 1);
-    ny = min(max(ny, -2), H + 1);
-    const S *p0 = T + (ptrdiff_t)(ny - 1) * Tp + nx;
-    const S *p1 = p0 + Tp, *p2 = p1 + Tp;
-    // weights (1/2 - t)^2 / 2, 3/4 - t^2, (1/2 + t)^2 / 2; the last is the first plus t
-    const float ax = 0.5f - tx, ay = 0.5f - ty;
-    const float wx0 = (0.5f * ax) * ax, wx1 = fmaf(-tx, tx, 0.75f), wx2 = wx0 + tx;
-    const float wy0 = (0.5f * ay) * ay, wy1 = fmaf(-ty, ty, 0.75f), wy2 = wy0 + ty;
-    const float t00 = ldS<S>(p0 - 1), t01 = ldS<S>(p0), t02 = ldS<S>(p0 + 1);
-    const float t10 = ldS<S>(p1 - 1), t11 = ldS<S>(p1), t12 = ldS<S>(p1 + 1);
-    const float t20 = ldS<S>(p2 - 1), t21 = ldS<S>(p2), t22 = ldS<S>(p2 + 1);
-    const float a0 = fmaf(wx2, t02, fmaf(wx1, t01, wx0 * t00));
-    const float a1 = fmaf(wx2, t12, fmaf(wx1, t11, wx0 * t10));
-    const float a2 = fmaf(wx2, t22, fmaf(wx1, t21, wx0 * t20));
-    if (DERIV) {
-        // derivative weights t - 1/2, -2 t, t + 1/2
-        const float m2x = -2.f * tx, bx = 0.5f + tx;
-        const float b0 = fmaf(bx, t02, fmaf(m2x, t01, -ax * t00));
-        const float b1 = fmaf(bx, t12, fmaf(m2x, t11, -ax * t10));
-        const float b2 = fmaf(bx, t22, fmaf(m2x, t21, -ax * t20));
-        dtx = fmaf(wy2, b2, fmaf(wy1, b1, wy0 * b0));
-        dty = fmaf(0.5f + ty, a2, fmaf(-2.f * ty, a1, -ay * a0));
-    }
-    return fmaf(wy2, a2, fmaf(wy1, a1, wy0 * a0));
-}
-
-// Two samples of the model at once, pixel a in the .x and pixel b in the .y of every float2: the
-// steps of sample_q with each floating-point operation done on both in one packed FP32x2
-// instruction (each lane rounded as the scalar operation, so the values equal two sample_q calls).
-template <typename S, bool DERIV>
-__device__ __forceinline__ float2 sample_q2(const S *T, int W, int H, int Tp, int2 xi, int2 yi, float2 vx, float2 vy,
-                                            float2 &dtx, float2 &dty)
-{
-    const float2 h = make_float2(0.5f, 0.5f);
-    const float2 px = __fadd2_rn(vx, h), py = __fadd2_rn(vy, h);
-    const float2 fnx = make_float2(floorf(px.x), floorf(px.y)), fny = make_float2(floorf(py.x), floorf(py.y));
-    const float2 tx = __fadd2_rn(vx, make_float2(-fnx.x, -fnx.y)), ty = __fadd2_rn(vy, make_float2(-fny.x, -fny.y));
-    const int nxa = min(max((int)((unsigned)xi.x + (unsigned)__float2int_rz(fnx.x)), -2), W + 1);
-    const int nxb = min(max((int)((unsigned)xi.y + (unsigned)__float2int_rz(fnx.y)), -2), W + 1);
-    const int nya = min(max((int)((unsigned)yi.x + (unsigned)__float2int_rz(fny.x)), -2), H + 1);
-    const int nyb = min(max((int)((unsigned)yi.y + (unsigned)__float2int_rz(fny.y)), -2), H + 1);
-    const S *pa = T + (ptrdiff_t)(nya - 1) * Tp + nxa, *pb = T + (ptrdiff_t)(nyb - 1) * Tp + nxb;
-    const float2 ax = __fadd2_rn(h, make_float2(-tx.x, -tx.y)), ay = __fadd2_rn(h, make_float2(-ty.x, -ty.y));
-    const float2 wx0 = __fmul2_rn(__fmul2_rn(h, ax), ax), wy0 = __fmul2_rn(__fmul2_rn(h, ay), ay);
-    const float2 q34 = make_float2(0.75f, 0.75f);
-    const float2 wx1 = __ffma2_rn(make_float2(-tx.x, -tx.y), tx, q34), wy1 = __ffma2_rn(make_float2(-ty.x, -ty.y), ty, q34);
-    const float2 wx2 = __fadd2_rn(wx0, tx), wy2 = __fadd2_rn(wy0, ty);
-    float2 tr[3][3];
-#pragma unroll
-    for (int r = 0; r < 3; ++r)
-#pragma unroll
-        for (int k = 0; k < 3; ++k) tr[r][k] = make_float2(ldS<S>(pa + r * Tp + k - 1), ldS<S>(pb + r * Tp + k - 1));
-    float2 a[3];
-#pragma unroll
-    for (int r = 0; r < 3; ++r) a[r] = __ffma2_rn(wx2, tr[r][2], __ffma2_rn(wx1, tr[r][1], __fmul2_rn(wx0, tr[r][0])));
-    if (DERIV) {
-        // derivative weights t - 1/2, -2 t, t + 1/2
-        const float2 m2 = make_float2(-2.f, -2.f);
-        const float2 nax = make_float2(-ax.x, -ax.y), bx = __fadd2_rn(h, tx);
-        float2 b[3];
-#pragma unroll
-        for (int r = 0; r < 3; ++r)
-            b[r] = __ffma2_rn(bx, tr[r][2], __ffma2_rn(__fmul2_rn(m2, tx), tr[r][1], __fmul2_rn(nax, tr[r][0])));
-        dtx = __ffma2_rn(wy2, b[2], __ffma2_rn(wy1, b[1], __fmul2_rn(wy0, b[0])));
-        dty = __ffma2_rn(__fadd2_rn(h, ty), a[2], __ffma2_rn(__fmul2_rn(m2, ty), a[1],
-                                                                 __fmul2_rn(make_float2(-ay.x, -ay.y), a[0])));
-    }
-    return __ffma2_rn(wy2, a[2], __ffma2_rn(wy1, a[1], __fmul2_rn(wy0, a[0])));
 }
 
 // ================================================================== rigid
@@ -493,7 +338,7 @@ __device__ void eval_rigid_energy(const Lvl &L, int r0, int r1, const float *pm,
             if constexpr (RSTAT) { lo[4] += e4; e4 = 0.f; }
         },
         []() {});
-    cluster_reduce<NM, false>(hi, lo, sm, buf, cl, false);
+    cluster_reduce<NM, false>(hi, lo, 0.f, sm, buf, cl);
 }
 
 // Gradient pass at a point whose NCC terms are known (from the energy pass or the accepted
@@ -548,10 +393,10 @@ __device__ void eval_rigid_grad(const Lvl &L, int r0, int r1, const float *pm, S
 #pragma unroll
             for (int m = 0; m < NM; ++m) { ff_acc(hi[m], lo[m], a[m]); a[m] = 0.f; }
         });
-    cluster_reduce<NM, false>(hi, lo, sm, buf, cl, false);
+    cluster_reduce<NM, false>(hi, lo, 0.f, sm, buf, cl);
 }
 
-enum Action { kActGrad = 0, kActTrial = 1, kActDone = 2, kActEnergy = 3, kActField = 4, kActMetric = 5 };
+enum Action { kActGrad = 0, kActTrial = 1, kActDone = 2, kActEnergy = 3 };
 
 
 __device__ void rigid_params(const double *th, float *pm)
@@ -758,9 +603,28 @@ __device__ void run_rigid(const Params &p, const OpDesc &op, int op_index, Smem 
 // Free-form field: u(x) bilinear in control values c_j on a grid of spacing s
 // (finest-level pixels), points (jx s, jy s).  At level l a pixel x sits at
 // finest coordinate X = 2^l x + (2^l - 1)/2, and the level works on c in its
-// own pixels (c / 2^l).  Every CTA of the cluster holds the whole grid in
-// shared memory: c (current), d (descent direction), mt (scalar product) and gp
-// (this CTA's partial gradient); a trial's values c + tau d are formed where read.
+// own pixels (c / 2^l).
+//
+// One pass over a level's pixels gives everything an evaluation needs: the moments of the energy
+// and, per control point, the sums from which the gradient follows once the moments are known.
+// With F = P dE/dTw = aP (t - r) + (b - a) P t + kappa (r, t the shifted samples, kappa =
+// (a rbar - b tbar) P), the gradient of the data term is
+//     sum_x w_j F dT/dp = aP sum w_j (t - r) dT/dp + (b - a) P sum w_j t dT/dp + kappa sum w_j dT/dp,
+// three sums per point and axis that do not depend on the moments.  The second coefficient is
+// small where the energy is (b = NCC sqrt(S'_rr / S'_tt) a), so the split loses no precision to
+// cancellation; identical frames give t - r = 0, b = a and kappa = 0 exactly.  An accepted trial
+// (three in four and more) thus costs one pass over the pixels, not one for the energy and one for
+// the gradient, and a level starts with one pass, which also gives the Gauss-Newton scalar product.
+// The gradient sums of a rejected trial are dropped.  With separate passes a scan of 256 frames of
+// 512x512 took 28.4 ms and a pair 1,031 us (8 CTAs per operator); fused, with two packed columns a lane
+// and sliding windows, 16.5 ms and 513 us, and what bounds the pass is the latency of its loads and of
+// dependent packed steps (39 % issue, 16 warps per SM).
+//
+// A CTA of the cluster holds the control rows of its own band of cell rows and one row on either
+// side, assembles the gradient at its own rows (the first one with the last partial row of the CTA
+// above, read from its shared memory), and hands the direction of its edge rows to its neighbours.
+// With the whole grid in every CTA, each assembled all of it (13,000 cycles of an iteration's 230,000
+// at 512x512, most of one at 128x128) and 26 KB a CTA were taken from the L1 cache.
 
 struct Grid {
     int nx, ny, s;   // points per axis, spacing in finest pixels
@@ -773,264 +637,543 @@ struct GridLvl {
     float pl;        // 2^l
 };
 
-// Cell and weights of level pixel (x, y); matches the clamped cell choice of the oracle.
-__device__ __forceinline__ void grid_cell(const Grid &G, const GridLvl &L, int x, int y, int &ix, int &iy,
-                                          float &wx, float &wy)
+__device__ __forceinline__ GridLvl grid_level(const Grid &G, const Lvl &L, int l)
 {
-    float gx = fmaf(L.pl, (float)x, L.off) * L.scale_inv;
-    float gy = fmaf(L.pl, (float)y, L.off) * L.scale_inv;
-    gx = fminf(gx, (float)(G.nx - 1));
-    gy = fminf(gy, (float)(G.ny - 1));
-    ix = min((int)gx, G.nx - 2);
-    iy = min((int)gy, G.ny - 2);
-    wx = gx - (float)ix;
-    wy = gy - (float)iy;
-}
-
-__device__ __forceinline__ float2 grid_eval(const float2 *c, int nx, int ix, int iy, float wx, float wy)
-{
-    const float2 a = c[iy * nx + ix], b = c[iy * nx + ix + 1], e = c[(iy + 1) * nx + ix], f = c[(iy + 1) * nx + ix + 1];
-    const float gx = 1.f - wx, gy = 1.f - wy;
-    float2 u;
-    u.x = fmaf(wy, fmaf(wx, f.x, gx * e.x), gy * fmaf(wx, b.x, gx * a.x));
-    u.y = fmaf(wy, fmaf(wx, f.y, gx * e.y), gy * fmaf(wx, b.y, gx * a.y));
-    return u;
-}
-
-// Rows and band of control-cell rows owned by a CTA: cell rows [k q, (k+1) q), q = ceil((ny-1)/C);
-// level pixel rows of those cells (the last CTA also takes rows clamped into the last cell row).
-// Partial-gradient buffer of one CTA: the control rows of its band of cell rows, [cr0, cr1].
-__host__ __device__ __forceinline__ int grid_band_elems(int gnx, int gny, int C)
-{
-    return ((gny - 1 + C - 1) / C + 1) * gnx;
-}
-
-// Dynamic shared memory of the nonrigid kernels, in float2 units: c, d, mt (whole grid each; mt the
-// flow's scalar product per control point and axis, or with the H1 product its right-hand side),
-// with the H1 product two more whole-grid buffers t and u for its solve, the band of partial
-// gradients, then (16-byte aligned) one row of gnx - 1 float4 per warp: the control values of the
-// warp's pixel row interpolated along y, (u_j, u_{j+1} - u_j).
-struct GridLayout {
-    int c, d, mt, t, u, gp, crow;
-};
-__host__ __device__ __forceinline__ GridLayout grid_layout(int gnx, int gny, int C, bool h1)
-{
-    const int Nc = gnx * gny;
-    GridLayout g;
-    g.c = 0;
-    g.d = Nc;
-    g.mt = 2 * Nc;
-    int o = 3 * Nc;
-    g.t = h1 ? o : -1;
-    g.u = h1 ? o + Nc : -1;
-    if (h1) o += 2 * Nc;
-    g.gp = o;
-    o += grid_band_elems(gnx, gny, C);
-    g.crow = o + (o & 1);
+    GridLvl g;
+    g.W = L.W; g.H = L.H; g.l = l;
+    g.pl = ldexpf(1.f, l);
+    g.off = 0.5f * (g.pl - 1.f);
+    g.scale_inv = 1.f / (float)G.s;
     return g;
 }
 
-__device__ __forceinline__ void grid_rows(const Grid &G, const GridLvl &L, int rank, int C, int &cr0, int &cr1,
-                                          int &r0, int &r1)
+// Cell rows of one CTA at most: rank k owns cell rows [k q, (k+1) q).
+__host__ __device__ __forceinline__ int band_cells(int gny, int C)
 {
-    const int cells = G.ny - 1;
-    const int q = (cells + C - 1) / C;
-    cr0 = min(cells, rank * q);
-    cr1 = min(cells, cr0 + q);
-    const int sl = G.s >> L.l;   // cell height in level pixels
-    r0 = min(L.H, cr0 * sl);
-    r1 = (cr1 == cells) ? L.H : min(L.H, cr1 * sl);
-    if (cr0 == cr1) r0 = r1 = L.H;
+    return (gny - 1 + C - 1) / C;
 }
 
-// Energy moments of the field ct = c + tau d (TRIAL; else ct = c): slots 0 St, 1 Stt, 2 Srt, with
-// RSTAT (first pass of a level) 3 Sr, 4 Srr; slot 5 = sum over control edges |dct|^2 (rank 0 only,
-// so the cluster sum counts it once).  Each warp first interpolates the control values of its row
-// along y into crow (u_j and u_{j+1} - u_j for the nx - 1 cells), so a pixel only interpolates
-// along x.  The trial values are formed where they are read, fmaf(tau, d_j, c_j), the expression
-// an accepted step stores into c.
-template <typename S, bool RSTAT, int U, bool TRIAL>
-__device__ void grid_energy_pass(const Lvl &L, const Grid &G, const GridLvl &GL, const float2 *c, const float2 *d,
-                                 float tau, float4 *crow_all, int r0, int r1, Smem &sm, int &buf,
-                                 const cg::cluster_group &cl)
+// The rows of a CTA: cell rows [cr0, cr1); control rows [cr0, own1) are its own (the last band
+// owns the grid's last row too); rows [h0, h1) are held in shared memory.
+struct Band {
+    int q, cr0, cr1, own1, h0, h1;
+};
+
+__device__ __forceinline__ Band grid_band(const Grid &G, int rank, int C)
 {
-    auto ct = [&](int j) {
+    const int cells = G.ny - 1;
+    Band b;
+    b.q = band_cells(G.ny, C);
+    b.cr0 = min(cells, rank * b.q);
+    b.cr1 = min(cells, b.cr0 + b.q);
+    const bool any = b.cr0 < b.cr1;
+    b.own1 = any ? (b.cr1 == cells ? G.ny : b.cr1) : b.cr0;
+    b.h0 = any ? max(0, b.cr0 - 1) : b.cr0;
+    b.h1 = any ? min(G.ny, b.own1 + 1) : b.cr0;
+    return b;
+}
+
+// How a pass splits a band's pixels among the warps.  A strip is up to 32 columns: those of g = 32 / sl
+// whole cells (sl the cell width at the level), or from 32 columns a cell on a chunk of one cell; a
+// column past the last cell, which a frame of 2^k + 1 columns has, is a strip of its own.  A warp's
+// task is two neighbouring strips, a column of each per lane, over the rows of a segment: m cell
+// rows, or one h-th of a cell row.  Every strip of every segment has slots of its own for its sums
+// (m + 1 control rows of g + 1 points, 8 floats each), so no two warps add to one place and the
+// order is fixed.  Long segments are best (a control row inside one is reduced over the lanes once, not
+// twice), short ones where there are too few strips for the warps: the rule takes the least number of
+// rounds x (pixel rows + about two rows' time per reduction).
+struct PassGeom {
+    int sl, g, chunks;    // cell width, cells per strip, strips per cell (wide cells)
+    int ns, nst;          // strips of cells, strips
+    int m, h, ph;         // cell rows per segment, pieces per cell row, pixel rows per piece
+    int nseg;
+};
+
+__host__ __device__ inline PassGeom pass_geom(int sl, int ncx, int q, bool over)
+{
+    PassGeom P;
+    P.sl = sl;
+    P.g = sl < 32 ? 32 / sl : 1;
+    P.chunks = (sl + 31) / 32;
+    P.ns = sl < 32 ? (ncx + P.g - 1) / P.g : ncx * P.chunks;
+    P.nst = P.ns + (over ? 1 : 0);
+    const int pairs = (P.nst + 1) / 2;
+    int least = -1;
+    for (int k = 1; k < 2 * q; k *= 2) {
+        const int m = (q + k - 1) / k, nseg = (q + m - 1) / m;
+        const int cost = (pairs * nseg + kWarps - 1) / kWarps * (m * sl + 2 * m + 4);
+        if (least < 0 || cost < least) {
+            least = cost;
+            P.m = m; P.h = 1; P.ph = sl; P.nseg = nseg;
+        }
+    }
+    for (int h = 2; h <= 8 && sl / h >= 2; h *= 2) {
+        const int ph = (sl + h - 1) / h;
+        const int cost = (pairs * q * h + kWarps - 1) / kWarps * (ph + 6);
+        if (cost < least) {
+            least = cost;
+            P.m = 1; P.h = h; P.ph = ph; P.nseg = q * h;
+        }
+    }
+    return P;
+}
+
+constexpr int kSlot = 8;   // floats per slot: (t - r, t, 1) x (x, y), then dT^2 x (x, y)
+__host__ __device__ __forceinline__ size_t slot_floats(const PassGeom &P)
+{
+    return (size_t)P.nseg * P.nst * (P.m + 1) * (P.g + 1) * kSlot;
+}
+
+// Dynamic shared memory of the nonrigid kernels, in float2 units: c, d, mt (the held rows; mt the
+// flow's scalar product per control point and axis), two staged halo rows of d, then the slots.
+// With the H1 product mt is the right-hand side of its solve on the whole grid, and the two work
+// grids t and u of the solve lie in the place of the slots, which it has read by then.
+struct GridLayout {
+    int c, d, mt, halo, slots;
+};
+__host__ __device__ __forceinline__ GridLayout grid_layout(int gnx, int gny, int C, bool h1)
+{
+    const int q = band_cells(gny, C);
+    const int rows = q + 2 < gny ? q + 2 : gny;
+    GridLayout g;
+    g.c = 0;
+    g.d = rows * gnx;
+    g.mt = 2 * rows * gnx;
+    g.halo = g.mt + (h1 ? gny : rows) * gnx;
+    g.slots = g.halo + 2 * gnx;
+    g.slots += g.slots & 1;
+    return g;
+}
+
+// Sum 16 per-lane values over aligned segments of SEG lanes by halving exchanges (8 + 4 + 2 + 1
+// shuffles and a butterfly for SEG = 32): on return a lane holds the segment's totals of the values
+// first .. first + 15 / SEG (fixed order, so deterministic).
+template <int SEG> struct SegSum {
+    static constexpr int kHeld = SEG >= 16 ? 1 : 16 / SEG;
+    float v[kHeld];
+    int first;
+};
+template <int SEG>
+__device__ __forceinline__ SegSum<SEG> seg_sum16(float (&v)[16], int lane)
+{
+    SegSum<SEG> o;
+    o.first = 0;
+#pragma unroll
+    for (int w = SEG / 2, n = 8; w >= 1; w >>= 1, n >>= 1) {
+        if (n >= 1) {
+            const bool up = lane & w;
+#pragma unroll
+            for (int k = 0; k < n; ++k) {
+                const float send = up ? v[k] : v[k + n], keep = up ? v[k + n] : v[k];
+                v[k] = keep + __shfl_xor_sync(0xffffffffu, send, w);
+            }
+            o.first += up ? n : 0;
+        } else {
+            v[0] += __shfl_xor_sync(0xffffffffu, v[0], w);
+        }
+    }
+#pragma unroll
+    for (int k = 0; k < SegSum<SEG>::kHeld; ++k) o.v[k] = v[k];
+    return o;
+}
+
+// One control row's sums of a strip into its slots (points 0 .. last + 1 of the strip; slot[p kSlot]).
+// v: the lane's column, already weighted along x: entries 0-7 for the point left of its cell k, 8-15
+// for the point right of it; ncomp entries of each are written.  A point between two cells gets
+// the left cell's share after the right cell's.
+template <int SEG>
+__device__ __forceinline__ void emit_row(float (&v)[16], int lane, int k, int last, float *slot, int ncomp)
+{
+    const SegSum<SEG> s = seg_sum16<SEG>(v, lane);
+    const bool writer = k <= last && (SEG < 32 || (lane & 1) == 0);
+#pragma unroll
+    for (int i = 0; i < SegSum<SEG>::kHeld; ++i) {
+        const int id = s.first + i, side = id >> 3, comp = id & 7;
+        if (writer && comp < ncomp && (side == 0 || k == last)) slot[(k + side) * kSlot + comp] = s.v[i];
+    }
+    if (SEG == 32) return;
+    __syncwarp();
+#pragma unroll
+    for (int i = 0; i < SegSum<SEG>::kHeld; ++i) {
+        const int id = s.first + i, side = id >> 3, comp = id & 7;
+        if (writer && comp < ncomp && side == 1 && k < last) slot[(k + 1) * kSlot + comp] += s.v[i];
+    }
+}
+
+__device__ __forceinline__ void emit_any(int sl, bool whole, float (&v)[16], int lane, int k, int last, float *slot,
+                                         int ncomp)
+{
+    if (whole) emit_row<32>(v, lane, k, last, slot, ncomp);   // a strip of one cell
+    else if (sl == 16) emit_row<16>(v, lane, k, last, slot, ncomp);
+    else if (sl == 8) emit_row<8>(v, lane, k, last, slot, ncomp);
+    else if (sl == 4) emit_row<4>(v, lane, k, last, slot, ncomp);
+    else if (sl == 2) emit_row<2>(v, lane, k, last, slot, ncomp);
+    else if (sl == 1) emit_row<1>(v, lane, k, last, slot, ncomp);
+    else
+        // a cell width that is no power of two: cell by cell over the whole warp
+        for (int q = 0; q <= last; ++q) {
+            float x[16];
+#pragma unroll
+            for (int i = 0; i < 16; ++i) x[i] = k == q ? v[i] : 0.f;
+            const SegSum<32> s = seg_sum16<32>(x, lane);
+            const int side = s.first >> 3, comp = s.first & 7;
+            float *p = slot + (q + side) * kSlot + comp;
+            if ((lane & 1) == 0 && comp < ncomp) *p = side == 0 && q > 0 ? *p + s.v[0] : s.v[0];
+            __syncwarp();
+        }
+}
+
+// Value and twice the gradient of the B-spline model for two samples (.x and .y) from their 3 x 3
+// windows t (rows, then columns) at offsets (tx, ty) in [-1/2, 1/2] from the middle sample.  Along an
+// axis the taps' weights (1/2 - t)^2 / 2, 3/4 - t^2, (1/2 + t)^2 / 2 are taken as a polynomial in t,
+//     S + t/2 (D1 + t D2),   S = (t0 + t2) / 8 + 3/4 t1,   D1 = t2 - t0,   D2 = t0 - 2 t1 + t2,
+// its derivative as (D1 + 2 t D2) / 2: S, D1 and D2 of a tap row serve every window that holds it.
+struct TapRow {
+    float2 S, D1, D2;
+};
+__device__ __forceinline__ TapRow tap_row(float2 t0, float2 t1, float2 t2)
+{
+    const float2 s = __fadd2_rn(t0, t2);
+    return TapRow{__ffma2_rn(f2(0.125f), s, __fmul2_rn(f2(0.75f), t1)), f2sub(t2, t0), __ffma2_rn(f2(-2.f), t1, s)};
+}
+__device__ __forceinline__ float2 bspline2(const TapRow &r0, const TapRow &r1, const TapRow &r2, float2 tx, float2 ty,
+                                           float2 &dtx2, float2 &dty2)
+{
+    const float2 hx = __fmul2_rn(f2(0.5f), tx), hy = __fmul2_rn(f2(0.5f), ty);
+    const float2 x2 = __fadd2_rn(tx, tx), y2 = __fadd2_rn(ty, ty);
+    const float2 a0 = __ffma2_rn(hx, __ffma2_rn(tx, r0.D2, r0.D1), r0.S), b0 = __ffma2_rn(x2, r0.D2, r0.D1);
+    const float2 a1 = __ffma2_rn(hx, __ffma2_rn(tx, r1.D2, r1.D1), r1.S), b1 = __ffma2_rn(x2, r1.D2, r1.D1);
+    const float2 a2 = __ffma2_rn(hx, __ffma2_rn(tx, r2.D2, r2.D1), r2.S), b2 = __ffma2_rn(x2, r2.D2, r2.D1);
+    const TapRow a = tap_row(a0, a1, a2), b = tap_row(b0, b1, b2);
+    dtx2 = __ffma2_rn(hy, __ffma2_rn(ty, b.D2, b.D1), b.S);
+    dty2 = __ffma2_rn(y2, a.D2, a.D1);
+    return __ffma2_rn(hy, __ffma2_rn(ty, a.D2, a.D1), a.S);
+}
+
+// x rounded to the nearest integer by adding and subtracting 1.5 2^23: the sum's low bits are the
+// integer (kRoundBits + n), with no conversion instruction.  Beyond 2^22 the bits are no longer the
+// integer, but they are far above or below every pixel, and so is the position.
+constexpr float kRound = 12582912.f;
+constexpr unsigned kRoundBits = 0x4B400000u;
+constexpr int kRunRows = 16;   // rows of a straight run at most; half of it is tried next
+
+// One pass at c (START: a level's first) or at the trial c + tau d: the moments into sm.tot (slots
+// 0 St, 1 Stt, 2 Srt, with START 3 Sr, 4 Srr; 5: sum over control edges of |dct|^2) and the gradient
+// sums into the slots.  The trial values are formed where they are read, fmaf(tau, d_j, c_j), the
+// expression an accepted step stores into c.
+//
+// Two columns a lane, every floating-point step on both in one packed instruction.  Where the sample
+// positions of every column of the warp move down by one row per row (a straight run: the rounded
+// displacement is constant, as it is over most of a smooth field), the window slides: a row loads one
+// tap row and keeps two, R rows' loads in flight together.  Elsewhere each row loads its own window.
+// A sum of products takes one rounding per product (fmaf), in runs of at most 8 pixels carried on in
+// float-float.
+template <typename S, bool START, int R>
+__device__ void grid_pass(const Lvl &L, const Grid &G, const GridLvl &GL, const PassGeom &P, const Band &B,
+                          const float2 *c, const float2 *d, float tau, float *slots, Smem &sm, int &buf,
+                          const cg::cluster_group &cl)
+{
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int ncx = G.nx - 1, ncy = G.ny - 1, sl = P.sl, pairs = (P.nst + 1) / 2;
+    const S *Rp = (const S *)L.R, *T = (const S *)L.T;
+    const float2 ncR = f2(-L.cR), dw = f2(GL.pl * GL.scale_inv);
+    auto ct = [&](int row, int col) {   // control value of the point evaluated
+        const int j = (row - B.h0) * G.nx + col;
         const float2 a = c[j];
-        if constexpr (TRIAL) {
+        if constexpr (START) {
+            return a;
+        } else {
             const float2 b = d[j];
             return make_float2(fmaf(tau, b.x, a.x), fmaf(tau, b.y, a.y));
-        } else {
-            return a;
         }
     };
-    const S *R = (const S *)L.R, *T = (const S *)L.T;
-    constexpr int NM = 6;
-    float hi[NM], lo[NM];
-    // per-lane partial sums of the current kFast pixels, in pairs (.x and .y: the two pixels of a
-    // packed step); e: the exact rounding errors of the products of slots 1, 2 and 4
-    float2 a[5], e1 = make_float2(0.f, 0.f), e2 = e1, e4 = e1;
+    constexpr int NM = START ? 5 : 3;
+    float2 hi2[NM], lo2[NM], a[NM];
 #pragma unroll
-    for (int m = 0; m < NM; ++m) { hi[m] = 0.f; lo[m] = 0.f; }
+    for (int i = 0; i < NM; ++i) hi2[i] = lo2[i] = a[i] = f2(0.f);
+
+    for (int task = warp; task < pairs * P.nseg; task += kWarps) {
+        const int seg = task / pairs, strip0 = 2 * (task - seg * pairs);
+        const int grp = seg / P.h, piece = seg - grp * P.h;
+        const int ca = B.cr0 + grp * P.m, cb = min(ca + P.m, B.cr1);
+        if (ca >= cb) continue;
+        // this lane's column of either strip; an idle lane repeats the last column and counts for nothing
+        int xc[2], cell[2], kl[2], last[2];
+        float wx[2];
+        bool act[2];
 #pragma unroll
-    for (int m = 0; m < 5; ++m) a[m] = make_float2(0.f, 0.f);
-    const int lane = threadIdx.x & 31;
-    float4 *crow = crow_all + (threadIdx.x >> 5) * (G.nx - 1);
-    const S *Rrow = R;
-    auto row = [&](int r) {
-        Rrow = R + (size_t)r * L.Rp;
-        const float gyf = fminf(fmaf(GL.pl, (float)r, GL.off) * GL.scale_inv, (float)(G.ny - 1));
-        const int iy = min((int)gyf, G.ny - 2);
-        const float wy = gyf - (float)iy, hy = 1.f - wy;
-        __syncwarp();
-        for (int j = lane; j < G.nx - 1; j += 32) {
-            const float2 a0 = ct(iy * G.nx + j), a1 = ct((iy + 1) * G.nx + j);
-            const float2 b0 = ct(iy * G.nx + j + 1), b1 = ct((iy + 1) * G.nx + j + 1);
-            const float ux0 = fmaf(wy, a1.x, hy * a0.x), uy0 = fmaf(wy, a1.y, hy * a0.y);
-            const float ux1 = fmaf(wy, b1.x, hy * b0.x), uy1 = fmaf(wy, b1.y, hy * b0.y);
-            crow[j] = make_float4(ux0, uy0, ux1 - ux0, uy1 - uy0);
+        for (int u = 0; u < 2; ++u) {
+            const int strip = strip0 + u;
+            const bool over = strip == P.ns;      // the column past the last cell
+            const int cell0 = over ? ncx - 1 : sl < 32 ? strip * P.g : strip / P.chunks;
+            const int c0 = min(cell0, ncx - 1);
+            last[u] = over || sl >= 32 ? 0 : min(P.g, ncx - c0) - 1;
+            kl[u] = over || sl >= 32 ? 0 : lane / sl;
+            const int xs = over ? ncx * sl : sl < 32 ? c0 * sl : c0 * sl + (strip - cell0 * P.chunks) * 32;
+            const int xe = over ? L.W : min(L.W, min(c0 * sl + (last[u] + 1) * sl, xs + 32));
+            act[u] = strip < P.nst && xs + lane < xe && kl[u] <= last[u];
+            cell[u] = c0 + min(kl[u], last[u]);
+            xc[u] = min(xs + lane, L.W - 1);
+            wx[u] = fminf(fmaf(GL.pl, (float)xc[u], GL.off) * GL.scale_inv, (float)ncx) - (float)cell[u];
+            if (!act[u]) { xc[u] = min(cell[u] * sl, L.W - 1); wx[u] = 0.f; }
         }
-        __syncwarp();
-    };
-    const float2 ncr = make_float2(-L.cR, -L.cR);
-    // two pixels (r, ca) and (r, cb) with displacements (ux.x, uy.x) and (ux.y, uy.y)
-    auto pixel2 = [&](int r, int ca, int cb, float2 ux, float2 uy) {
-        float2 dtx, dty;
-        const float2 tw = sample_q2<S, false>(T, L.W, L.H, L.Tp, make_int2(ca, cb), make_int2(r, r), ux, uy, dtx, dty);
-        const float2 rv = __fadd2_rn(make_float2(ldS<S>(Rrow + ca), ldS<S>(Rrow + cb)), ncr);
-        const float2 tv = __fadd2_rn(tw, ncr);
-        a[0] = __fadd2_rn(a[0], tv);
-        acc_prod2(a[1], e1, tv, tv);
-        acc_prod2(a[2], e2, rv, tv);
-        if constexpr (RSTAT) {
-            a[3] = __fadd2_rn(a[3], rv);
-            acc_prod2(a[4], e4, rv, rv);
-        }
-    };
-    // one pixel (a row's ragged end), into the .x partial sums
-    auto pixel = [&](int r, int c, float ux, float uy) {
-        float dtx, dty;
-        const float tw = sample_q<S, false>(T, L.W, L.H, L.Tp, c, r, ux, uy, dtx, dty);
-        const float rv = ldS<S>(Rrow + c) - L.cR;
-        const float tv = tw - L.cR;
-        a[0].x += tv;
-        acc_prod(a[1].x, e1.x, tv, tv);
-        acc_prod(a[2].x, e2.x, rv, tv);
-        if constexpr (RSTAT) {
-            a[3].x += rv;
-            acc_prod(a[4].x, e4.x, rv, rv);
-        }
-    };
-    auto flush_fast = [&]() {
-#pragma unroll
-        for (int m = 0; m < (RSTAT ? 5 : 3); ++m) {
-            ff_acc(hi[m], lo[m], a[m].x + a[m].y);
-            a[m] = make_float2(0.f, 0.f);
-        }
-        lo[1] += e1.x + e1.y; lo[2] += e2.x + e2.y;
-        e1 = make_float2(0.f, 0.f); e2 = e1;
-        if constexpr (RSTAT) { lo[4] += e4.x + e4.y; e4 = e1; }
-    };
-    // A lane's columns are 32 apart.  When the cell width sl at this level is a power of two
-    // dividing 32, the spacing a power of two and no column reaches the grid's last line, every
-    // column of a lane has the same offset in its cell: the weight along x is fixed per lane and
-    // the cell index is a shift.  Both are exact, so the values equal the general form's.
-    const int sl = G.s >> GL.l;
-    const bool fast = sl >= 1 && sl <= 32 && (sl & (sl - 1)) == 0 && (sl << GL.l) == G.s &&
-                      fmaf(GL.pl, (float)(L.W - 1), GL.off) * GL.scale_inv < (float)(G.nx - 1);
-    if (fast) {
-        const int lgl = 31 - __clz(sl);
-        const float wxl = fmaf(GL.pl, (float)(lane & (sl - 1)), GL.off) * GL.scale_inv;
-        const float2 wxl2 = make_float2(wxl, wxl);
-        for_rows2<U>(
-            L.W, r0, r1, row,
-            [&](int r, int ca, int cb) {
-                const float4 qa = crow[ca >> lgl], qb = crow[cb >> lgl];
-                pixel2(r, ca, cb, __ffma2_rn(wxl2, make_float2(qa.z, qb.z), make_float2(qa.x, qb.x)),
-                       __ffma2_rn(wxl2, make_float2(qa.w, qb.w), make_float2(qa.y, qb.y)));
-            },
-            [&](int r, int c) {
-                const float4 q = crow[c >> lgl];
-                pixel(r, c, fmaf(wxl, q.z, q.x), fmaf(wxl, q.w, q.y));
-            },
-            flush_fast, []() {});
-    } else {
-        auto cellx = [&](int c, float &wx) {
-            const float gxf = fminf(fmaf(GL.pl, (float)c, GL.off) * GL.scale_inv, (float)(G.nx - 1));
-            const int ix = min((int)gxf, G.nx - 2);
-            wx = gxf - (float)ix;
-            return crow[ix];
+        auto column = [&](int row, float2 &tx, float2 &ty) {   // displacement of a control row at the two columns
+            const float2 p0 = ct(row, cell[0]), p1 = ct(row, cell[0] + 1), q0 = ct(row, cell[1]), q1 = ct(row, cell[1] + 1);
+            tx = make_float2(fmaf(wx[0], p1.x - p0.x, p0.x), fmaf(wx[1], q1.x - q0.x, q0.x));
+            ty = make_float2(fmaf(wx[0], p1.y - p0.y, p0.y), fmaf(wx[1], q1.y - q0.y, q0.y));
         };
-        for_rows2<U>(
-            L.W, r0, r1, row,
-            [&](int r, int ca, int cb) {
-                float wa, wb;
-                const float4 qa = cellx(ca, wa), qb = cellx(cb, wb);
-                const float2 w2 = make_float2(wa, wb);
-                pixel2(r, ca, cb, __ffma2_rn(w2, make_float2(qa.z, qb.z), make_float2(qa.x, qb.x)),
-                       __ffma2_rn(w2, make_float2(qa.w, qb.w), make_float2(qa.y, qb.y)));
-            },
-            [&](int r, int c) {
-                float wx;
-                const float4 q = cellx(c, wx);
-                pixel(r, c, fmaf(wx, q.z, q.x), fmaf(wx, q.w, q.y));
-            },
-            flush_fast, []() {});
+        const S *ra = Rp + xc[0], *rb = Rp + xc[1];
+        float2 sF[4], sT[4], s1[4], sM[4];   // top x, top y, bottom x, bottom y
+#pragma unroll
+        for (int i = 0; i < 4; ++i) sF[i] = sT[i] = s1[i] = sM[i] = f2(0.f);
+        float2 tx, ty;
+        column(ca, tx, ty);
+        auto flush = [&]() {
+#pragma unroll
+            for (int i = 0; i < NM; ++i) {
+                ff_acc2(hi2[i], lo2[i], make_float2(act[0] ? a[i].x : 0.f, act[1] ? a[i].y : 0.f));
+                a[i] = f2(0.f);
+            }
+        };
+        // one pixel of either column; wy: the weight of the control row below
+        auto pixel = [&](const TapRow &t0, const TapRow &t1, const TapRow &t2, float2 fx, float2 fy, float2 r, float2 wy) {
+            float2 dx2, dy2;
+            const float2 t = __fadd2_rn(bspline2(t0, t1, t2, fx, fy, dx2, dy2), ncR);
+            a[0] = __fadd2_rn(a[0], t);
+            a[1] = __ffma2_rn(t, t, a[1]);
+            a[2] = __ffma2_rn(r, t, a[2]);
+            if constexpr (START) {
+                a[3] = __fadd2_rn(a[3], r);
+                a[4] = __ffma2_rn(r, r, a[4]);
+            }
+            const float2 F = f2sub(t, r);
+            const float2 wb = __fmul2_rn(f2(0.5f), wy), wt = f2sub(f2(0.5f), wb);   // half of wy and 1 - wy
+            const float2 g[4] = {__fmul2_rn(wt, dx2), __fmul2_rn(wt, dy2), __fmul2_rn(wb, dx2), __fmul2_rn(wb, dy2)};
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                sF[i] = __ffma2_rn(F, g[i], sF[i]);
+                sT[i] = __ffma2_rn(t, g[i], sT[i]);
+                s1[i] = __fadd2_rn(s1[i], g[i]);
+                if constexpr (START) sM[i] = __ffma2_rn(g[i], g[i], sM[i]);
+            }
+        };
+        // the window of one row of one column, anywhere: clamped into the level's border
+        auto window = [&](float m_x, float m_y, int x, int y) {
+            const int wxn = min(max((int)(__float_as_uint(m_x) - kRoundBits + (unsigned)x), -2), L.W + 1);
+            const int wyn = min(max((int)(__float_as_uint(m_y) - kRoundBits + (unsigned)y), -2), L.H + 1);
+            return T + (ptrdiff_t)(wyn - 1) * L.Tp + wxn;
+        };
+        auto row = [&](const S *qa, const S *qb) {
+            return tap_row(make_float2(ldS<S>(qa - 1), ldS<S>(qb - 1)), make_float2(ldS<S>(qa), ldS<S>(qb)),
+                           make_float2(ldS<S>(qa + 1), ldS<S>(qb + 1)));
+        };
+        for (int cy = ca; cy <= cb; ++cy) {
+            if (cy < cb) {
+                float2 bx, by;
+                column(cy + 1, bx, by);
+                const float2 ex = f2sub(bx, tx), ey = f2sub(by, ty);
+                const float cyf = (float)cy;
+                const int yc = min(L.H, (cy + 1) * sl), y1 = cy == ncy - 1 ? L.H : yc;
+                int y = min(y1, cy * sl + piece * P.ph);
+                const int ye = piece == P.h - 1 ? y1 : min(y1, y + P.ph);
+                while (y < ye) {
+                    // the weight of the control row below; a row past the last cell row lies on it
+                    const float2 w0 = f2(y < yc ? fmaf(GL.pl, (float)y, GL.off) * GL.scale_inv - cyf : 1.f);
+                    const float2 v0x = __ffma2_rn(w0, ex, tx), v0y = __ffma2_rn(w0, ey, ty);
+                    const float2 m0x = __fadd2_rn(v0x, f2(kRound)), m0y = __fadd2_rn(v0y, f2(kRound));
+                    const int nxa = (int)(__float_as_uint(m0x.x) - kRoundBits + (unsigned)xc[0]);
+                    const int nxb = (int)(__float_as_uint(m0x.y) - kRoundBits + (unsigned)xc[1]);
+                    const int nya = (int)(__float_as_uint(m0y.x) - kRoundBits + (unsigned)y);
+                    const int nyb = (int)(__float_as_uint(m0y.y) - kRoundBits + (unsigned)y);
+                    // a straight run of n rows: the rounded displacement is the same in its first and its last
+                    // row, and so in every one between (it is monotonic along a column of a cell)
+                    auto straight = [&](int n) {
+                        const float2 w1 = __ffma2_rn(f2((float)(n - 1)), dw, w0);
+                        const float2 m1x = __fadd2_rn(__ffma2_rn(w1, ex, tx), f2(kRound));
+                        const float2 m1y = __fadd2_rn(__ffma2_rn(w1, ey, ty), f2(kRound));
+                        const unsigned diff = (__float_as_uint(m1x.x) ^ __float_as_uint(m0x.x)) |
+                                              (__float_as_uint(m1x.y) ^ __float_as_uint(m0x.y)) |
+                                              (__float_as_uint(m1y.x) ^ __float_as_uint(m0y.x)) |
+                                              (__float_as_uint(m1y.y) ^ __float_as_uint(m0y.y));
+                        return (bool)__all_sync(0xffffffffu, diff == 0u && (unsigned)(nxa + 2) <= (unsigned)(L.W + 3) &&
+                                                                 (unsigned)(nxb + 2) <= (unsigned)(L.W + 3) &&
+                                                                 nya >= -2 && nya + n <= L.H + 2 && nyb >= -2 &&
+                                                                 nyb + n <= L.H + 2);
+                    };
+                    const int left = min(ye, yc) - y;
+                    int n = min(left, kRunRows);
+                    bool run = n > 1 && straight(n);
+                    if (!run && n > kRunRows / 2) {
+                        n = kRunRows / 2;
+                        run = straight(n);
+                    }
+                    const S *rya = ra + (ptrdiff_t)y * L.Rp, *ryb = rb + (ptrdiff_t)y * L.Rp;
+                    if (run) {
+                        const S *qa = T + (ptrdiff_t)(nya - 1) * L.Tp + nxa, *qb = T + (ptrdiff_t)(nyb - 1) * L.Tp + nxb;
+                        const float2 ox = f2sub(tx, f2sub(m0x, f2(kRound))), oy = f2sub(ty, f2sub(m0y, f2(kRound)));
+                        TapRow t0 = row(qa, qb);
+                        qa += L.Tp; qb += L.Tp;
+                        TapRow t1 = row(qa, qb);
+                        float2 w = w0;
+                        int k = 0;
+                        for (; k + R <= n; k += R) {
+                            float2 r[R], q[R][3];
+#pragma unroll
+                            for (int i = 0; i < R; ++i) {
+                                qa += L.Tp; qb += L.Tp;
+#pragma unroll
+                                for (int j = 0; j < 3; ++j) q[i][j] = make_float2(ldS<S>(qa + j - 1), ldS<S>(qb + j - 1));
+                                r[i] = make_float2(ldS<S>(rya), ldS<S>(ryb));
+                                rya += L.Rp; ryb += L.Rp;
+                            }
+#pragma unroll
+                            for (int i = 0; i < R; ++i) {
+                                const float2 wy = i == 0 ? w : __ffma2_rn(f2((float)i), dw, w);
+                                const TapRow t2 = tap_row(q[i][0], q[i][1], q[i][2]);
+                                pixel(t0, t1, t2, __ffma2_rn(wy, ex, ox), __ffma2_rn(wy, ey, oy), __fadd2_rn(r[i], ncR), wy);
+                                t0 = t1;
+                                t1 = t2;
+                            }
+                            w = __ffma2_rn(f2((float)R), dw, w);
+                            if ((k & (kFast - R)) == kFast - R) flush();
+                        }
+                        for (; k < n; ++k) {   // what R does not divide
+                            qa += L.Tp; qb += L.Tp;
+                            const TapRow t2 = row(qa, qb);
+                            const float2 r = make_float2(ldS<S>(rya), ldS<S>(ryb));
+                            rya += L.Rp; ryb += L.Rp;
+                            pixel(t0, t1, t2, __ffma2_rn(w, ex, ox), __ffma2_rn(w, ey, oy), __fadd2_rn(r, ncR), w);
+                            t0 = t1;
+                            t1 = t2;
+                            w = __fadd2_rn(w, dw);
+                        }
+                    } else {
+                        // every row loads its own window
+                        n = min(n, kRunRows / 2);
+                        if (n < 1) n = 1;
+#pragma unroll 2
+                        for (int k = 0; k < n; ++k) {
+                            const float2 wy = __ffma2_rn(f2((float)k), dw, w0);
+                            const float2 vx = __ffma2_rn(wy, ex, tx), vy = __ffma2_rn(wy, ey, ty);
+                            const float2 mx = __fadd2_rn(vx, f2(kRound)), my = __fadd2_rn(vy, f2(kRound));
+                            const S *qa = window(mx.x, my.x, xc[0], y + k), *qb = window(mx.y, my.y, xc[1], y + k);
+                            const float2 r = make_float2(ldS<S>(rya), ldS<S>(ryb));
+                            rya += L.Rp; ryb += L.Rp;
+                            const TapRow t0 = row(qa, qb), t1 = row(qa + L.Tp, qb + L.Tp),
+                                         t2 = row(qa + 2 * (ptrdiff_t)L.Tp, qb + 2 * (ptrdiff_t)L.Tp);
+                            pixel(t0, t1, t2, f2sub(vx, f2sub(mx, f2(kRound))), f2sub(vy, f2sub(my, f2(kRound))),
+                                  __fadd2_rn(r, ncR), wy);
+                        }
+                    }
+                    flush();
+                    y += n;
+                }
+                tx = bx;
+                ty = by;
+            }
+            // control row cy: what the cell row above it left and the top sums of the one below
+#pragma unroll 1
+            for (int u = 0; u < 2; ++u) {
+                const int strip = strip0 + u;
+                if (strip >= P.nst) break;
+                const bool on = u ? act[1] : act[0];
+                const float w = u ? wx[1] : wx[0];
+                const float lw = on ? 1.f - w : 0.f, rw = on ? w : 0.f;
+                float v[16];
+#pragma unroll
+                for (int i = 0; i < 2; ++i) {
+                    const float f = u ? sF[i].y : sF[i].x, t = u ? sT[i].y : sT[i].x, o = u ? s1[i].y : s1[i].x;
+                    const float m = START ? (u ? sM[i].y : sM[i].x) : 0.f;
+                    v[i] = lw * f; v[8 + i] = rw * f;
+                    v[2 + i] = lw * t; v[10 + i] = rw * t;
+                    v[4 + i] = lw * o; v[12 + i] = rw * o;
+                    v[6 + i] = lw * lw * m; v[14 + i] = rw * rw * m;
+                }
+                float *slot = slots + ((size_t)(seg * P.nst + strip) * (P.m + 1) + (cy - ca)) * (P.g + 1) * kSlot;
+                emit_any(sl, sl >= 32 || strip == P.ns, v, lane, u ? kl[1] : kl[0], u ? last[1] : last[0], slot,
+                         START ? 8 : 6);
+            }
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
+                sF[i] = sF[2 + i]; sF[2 + i] = f2(0.f);
+                sT[i] = sT[2 + i]; sT[2 + i] = f2(0.f);
+                s1[i] = s1[2 + i]; s1[2 + i] = f2(0.f);
+                sM[i] = sM[2 + i]; sM[2 + i] = f2(0.f);
+            }
+        }
     }
-    if (cl.block_rank() == 0) {
-        const int Nc = G.nx * G.ny;
+    float hi[6], lo[6];
+#pragma unroll
+    for (int i = 0; i < 6; ++i) {
+        hi[i] = i < NM ? hi2[i].x : 0.f;
+        lo[i] = i < NM ? lo2[i].x : 0.f;
+        if (i < NM) ff_add(hi[i], lo[i], hi2[i].y, lo2[i].y);
+    }
+    // the regulariser's edges from this CTA's own rows: to the right and down
+    {
         float e = 0.f;
         int k = 0;
-        for (int j = threadIdx.x; j < Nc; j += kThreads) {
-            const int jx = j % G.nx;
-            const float2 v = ct(j);
-            if (jx + 1 < G.nx) {
-                const float2 w = ct(j + 1);
+        for (int j = threadIdx.x; j < (B.own1 - B.cr0) * G.nx; j += kThreads) {
+            const int row = B.cr0 + j / G.nx, col = j % G.nx;
+            const float2 v = ct(row, col);
+            if (col + 1 < G.nx) {
+                const float2 w = ct(row, col + 1);
                 e = fmaf(w.x - v.x, w.x - v.x, fmaf(w.y - v.y, w.y - v.y, e));
             }
-            if (j + G.nx < Nc) {
-                const float2 w = ct(j + G.nx);
+            if (row + 1 < G.ny) {
+                const float2 w = ct(row + 1, col);
                 e = fmaf(w.x - v.x, w.x - v.x, fmaf(w.y - v.y, w.y - v.y, e));
             }
             if (++k == kFast) { ff_acc(hi[5], lo[5], e); e = 0.f; k = 0; }
         }
         ff_acc(hi[5], lo[5], e);
     }
-    cluster_reduce<NM, false>(hi, lo, sm, buf, cl, false);
+    cluster_reduce<6, false>(hi, lo, 0.f, sm, buf, cl);
 }
 
-// Sum eight per-lane values over aligned segments of S lanes (S = 8, 16 or 32) by halving
-// exchanges: on return every lane holds its segment's total of value index 4 B1 + 2 B2 + B3, where
-// B1, B2, B3 are the lane's bits at S/2, S/4 and S/8 (the same in the S/8 lanes sharing them).
-// 2 log2(S) + 1 shuffles for S = 32 instead of 40; fixed order, so deterministic.
-template <int S>
-__device__ __forceinline__ float seg_reduce_scatter8(const float (&v)[8], int lane)
+// Sums of control point (cr0 + i, jx) over the slots that one CTA with nr cell rows wrote: entries
+// first .. first + N - 1, segment by segment and strip by strip.
+template <int N>
+__device__ __forceinline__ void slot_sum(const float *slots, const PassGeom &P, int ncx, int nr, int i, int jx,
+                                         int first, float (&o)[N])
 {
-    constexpr int o1 = S / 2, o2 = S / 4, o3 = S / 8;
-    const bool b1 = lane & o1, b2 = lane & o2, b3 = lane & o3;
-    float a4[4];
+    const int ga = i > 0 ? (i - 1) / P.m : 0, gb = i < nr ? i / P.m : (nr - 1) / P.m;
+    auto add = [&](int seg, int strip, int row, int pt) {
+        const float *s = slots + (((size_t)(seg * P.nst + strip) * (P.m + 1) + row) * (P.g + 1) + pt) * kSlot + first;
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        const float send = b1 ? v[k] : v[k + 4], keep = b1 ? v[k + 4] : v[k];
-        a4[k] = keep + __shfl_xor_sync(0xffffffffu, send, o1);
-    }
-    float a2[2];
-#pragma unroll
-    for (int k = 0; k < 2; ++k) {
-        const float send = b2 ? a4[k] : a4[k + 2], keep = b2 ? a4[k + 2] : a4[k];
-        a2[k] = keep + __shfl_xor_sync(0xffffffffu, send, o2);
-    }
-    const float send = b3 ? a2[0] : a2[1], keep = b3 ? a2[1] : a2[0];
-    float t = keep + __shfl_xor_sync(0xffffffffu, send, o3);
-#pragma unroll
-    for (int o = o3 / 2; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-    return t;
+        for (int k = 0; k < N; k += 2) {
+            const float2 v = *(const float2 *)(s + k);
+            o[k] += v.x;
+            o[k + 1] += v.y;
+        }
+    };
+    const int st = jx / P.g, pt = jx - st * P.g;
+    for (int grp = ga; grp <= gb; ++grp)
+        for (int piece = 0; piece < P.h; ++piece) {
+            const int seg = grp * P.h + piece, row = i - grp * P.m;
+            if (P.sl < 32) {
+                if (pt == 0 && jx > 0) add(seg, st - 1, row, P.g);
+                if (st < P.ns) add(seg, st, row, pt);
+            } else {
+                for (int q = 0; q < P.chunks; ++q) {
+                    if (jx > 0) add(seg, (jx - 1) * P.chunks + q, row, 1);
+                    if (jx < ncx) add(seg, jx * P.chunks + q, row, 0);
+                }
+            }
+            if (P.nst > P.ns && jx >= ncx - 1) add(seg, P.ns, row, jx - (ncx - 1));
+        }
 }
 
-// Value index a lane holds after seg_reduce_scatter8<S>, and whether it is the segment's writer.
-template <int S>
-__device__ __forceinline__ int seg_index8(int lane)
+// The same over the whole grid: this CTA's slots, and at its first row the last partial row of the
+// CTA above.
+template <int N>
+__device__ __forceinline__ void point_sum(const float *slots, const float *above, const PassGeom &P, const Band &B,
+                                          int ncx, int row, int jx, int first, float (&o)[N])
 {
-    return ((lane & (S / 2)) ? 4 : 0) + ((lane & (S / 4)) ? 2 : 0) + ((lane & (S / 8)) ? 1 : 0);
+#pragma unroll
+    for (int k = 0; k < N; ++k) o[k] = 0.f;
+    if (row == B.cr0 && above) slot_sum<N>(above, P, ncx, B.q, B.q, jx, first, o);
+    slot_sum<N>(slots, P, ncx, B.cr1 - B.cr0, row - B.cr0, jx, first, o);
 }
 
 // Buffers of the H1 scalar product (B null: another product): B the right-hand side -Nc dE/dc,
@@ -1105,389 +1248,116 @@ __device__ void h1_solve(const H1Bufs &h, int nx, int ny)
     __syncthreads();
 }
 
-// Gradient pass at c: this CTA's cells in four parity phases (no two cells of a phase share a
-// corner, so each corner is updated by one warp at a time, in a fixed order); then every CTA
-// assembles the whole gradient from the (at most two) CTAs whose band holds each control row,
-// and forms d = -(Nc/P) [sum F grad T w + lambda sum_nbrs (c_j - c_k)], F = P dE/dTw.
-// d = -M^-1 grad E with the scalar product mt.  pm: aP, bP, rbar, tbar, lambda.  Returns
-// sum_j m_j |d_j|^2 (float-float, in sm.tot[0]), max |d_j|^2 (sm.tot[1]), and with the direction
-// d held before the call, <d_old, d_old - d>_M (sm.tot[2]) and |d_old - d|_M^2 (sm.tot[3]);
-// identical in every CTA.
-//
-// METRIC: instead of the gradient, the flow's scalar product at c (the level's initial control
-// values): per control point and axis m = dk sum_x w_j(x)^2 (dT/dp)^2 + rk n_j (pm[0] = dk =
-// 1/(P var T), pm[1] = rk = lambda/P, n_j the neighbours of j), normalised by the mean of all
-// 2 Nc values and floored at 1e-3 of it, written to mt.
-template <typename S, bool METRIC>
-__device__ void grid_grad_pass(const Lvl &L, const Grid &G, const GridLvl &GL, const float2 *c, float2 *d,
-                               float2 *mt, float2 *gp, const float *pm, int cr0, int cr1, Smem &sm,
-                               const cg::cluster_group &cl, const H1Bufs &h1)
+// The flow's scalar product at c, from the pass's squared-derivative sums: per own control point and
+// axis m = dk sum_x w_j(x)^2 (dT/dp)^2 + rk n_j (dk = 1/(P var T), rk = lambda/P, n_j the neighbours
+// of j), normalised by the mean of all 2 Nc values and floored at 1e-3 of it, written to mt.
+__device__ void grid_metric(const Grid &G, const PassGeom &P, const Band &B, const float *slots, const float *above,
+                            float2 *mt, float dk, float rk, Smem &sm, int &buf, const cg::cluster_group &cl)
 {
-    const S *R = (const S *)L.R, *T = (const S *)L.T;
-    const float aP = pm[0], bP = pm[1], rb = pm[2], tb = pm[3], lam = pm[4];
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int Nc = G.nx * G.ny, ncx = G.nx - 1, ncy = G.ny - 1;
-    const int sl = G.s >> GL.l;
-    const int lg = 31 - __clz(max(sl, 1));   // log2 of sl when sl is a power of two (the fast path below)
-    // fast path: cell width a power of two dividing 32, spacing a power of two
-    const bool pow2 = sl >= 1 && sl <= 32 && (sl & (sl - 1)) == 0 && (sl << GL.l) == G.s;
-    const float dwy = (float)(32 >> lg) * GL.pl * GL.scale_inv;   // weight step between a lane's rows
-    // cells of width 16 or 8: G = 32 / sl cells per warp (below)
-    const int grp = (pow2 && (sl == 16 || sl == 8)) ? 32 / sl : 1;
-    float *gpf = (float *)gp;   // band-local: control row cr0 + i at gp[i nx .. (i + 1) nx)
-    for (int j = tid; j < (cr1 - cr0 + 1) * G.nx; j += kThreads) gp[j] = make_float2(0.f, 0.f);
-    __syncthreads();
-    for (int phase = 0; phase < 4; ++phase) {
-        const int px = phase & 1, py = phase >> 1;
-        const int first_row = cr0 + ((py - cr0) % 2 + 2) % 2;
-        const int rows = first_row < cr1 ? (cr1 - first_row + 1) / 2 : 0;
-        const int cols = (ncx - px + 1) / 2;
-        // cells taken G at a time by a warp (all but a last column narrower than sl), then the rest
-        // one per warp
-        const bool has_last = ncx - 1 - px >= 0 && ((ncx - 1 - px) & 1) == 0;
-        const int gcols = grp > 1 ? cols - ((has_last && L.W - (ncx - 1) * sl != sl) ? 1 : 0) : 0;
-        const int gpr = (gcols + grp - 1) / grp;   // groups per phase row
-        const int ngroup = rows * gpr, rc = cols - gcols;
-        for (int q = warp; q < ngroup + rows * rc; q += kWarps) {
-            if (q < ngroup) {
-                // lane: column lane mod sl of cell k = lane / sl of the group, through all its rows;
-                // weights and x-interpolated control values as in the single-cell form below
-                const int ri = q / gpr, ci = (q - ri * gpr) * grp + (lane >> lg);
-                const bool valid = ci < gcols;
-                const int cyy = first_row + 2 * ri, cxx = px + 2 * min(ci, gcols - 1);
-                const int x = cxx * sl + (lane & (sl - 1));
-                const int y0 = cyy * sl, y1 = (cyy == ncy - 1) ? L.H : min(L.H, y0 + sl);
-                const int j0 = cyy * G.nx + cxx;
-                const float2 c00 = c[j0], c01 = c[j0 + 1], c10 = c[j0 + G.nx], c11 = c[j0 + G.nx + 1];
-                const float wx = fminf(fmaf(GL.pl, (float)x, GL.off) * GL.scale_inv, (float)(G.nx - 1)) - (float)cxx;
-                const float tx = fmaf(wx, c01.x - c00.x, c00.x), ty = fmaf(wx, c01.y - c00.y, c00.y);
-                const float bx = fmaf(wx, c11.x - c10.x, c10.x), by = fmaf(wx, c11.y - c10.y, c10.y);
-                const float ex = bx - tx, ey = by - ty;
-                const float wmax = (float)(G.ny - 1 - cyy), dw1 = GL.pl * GL.scale_inv;
-                float wyk = GL.off * GL.scale_inv;   // g(y0) - cyy, exact
-                float st_x = 0.f, st_y = 0.f, sb_x = 0.f, sb_y = 0.f;
-#pragma unroll 4
-                for (int y = y0; y < y1; ++y) {
-                    const float wy = fminf(wyk, wmax);
-                    wyk += dw1;
-                    float dtx, dty;
-                    const float tw = sample_q<S, true>(T, L.W, L.H, L.Tp, x, y, fmaf(wy, ex, tx), fmaf(wy, ey, ty),
-                                                       dtx, dty);
-                    const float hy = 1.f - wy;
-                    if constexpr (METRIC) {
-                        (void)tw;
-                        const float gx = dtx * dtx, gy = dty * dty, hy2 = hy * hy, wy2 = wy * wy;
-                        st_x = fmaf(hy2, gx, st_x); st_y = fmaf(hy2, gy, st_y);
-                        sb_x = fmaf(wy2, gx, sb_x); sb_y = fmaf(wy2, gy, sb_y);
-                    } else {
-                        const float rv = ldS<S>(R + (size_t)y * L.Rp + x) - L.cR;
-                        const float tv = tw - L.cR;
-                        const float F = -__fsub_rn(__fmul_rn(aP, rv - rb), __fmul_rn(bP, tv - tb));
-                        const float gx = F * dtx, gy = F * dty;
-                        st_x = fmaf(hy, gx, st_x); st_y = fmaf(hy, gy, st_y);
-                        sb_x = fmaf(wy, gx, sb_x); sb_y = fmaf(wy, gy, sb_y);
-                    }
-                }
-                const float hx = METRIC ? (1.f - wx) * (1.f - wx) : 1.f - wx, vx = METRIC ? wx * wx : wx;
-                const float m = valid ? 1.f : 0.f;
-                float acc[8] = {m * hx * st_x, m * hx * st_y, m * vx * st_x, m * vx * st_y,
-                                m * hx * sb_x, m * hx * sb_y, m * vx * sb_x, m * vx * sb_y};
-                const float tot = sl == 16 ? seg_reduce_scatter8<16>(acc, lane) : seg_reduce_scatter8<8>(acc, lane);
-                const bool writer = sl == 16 ? (lane & 1) == 0 : true;
-                if (valid && writer) {
-                    const int vi = sl == 16 ? seg_index8<16>(lane) : seg_index8<8>(lane);
-                    const int corner = vi >> 1;
-                    const int jc = (cyy + (corner >> 1) - cr0) * G.nx + cxx + (corner & 1);
-                    gpf[2 * jc + (vi & 1)] += tot;
-                }
-                continue;
-            }
-            const int r = q - ngroup;
-            const int cyy = first_row + 2 * (r / rc), cxx = px + 2 * (gcols + r % rc);
-            const int x0 = cxx * sl, x1 = (cxx == ncx - 1) ? L.W : min(L.W, x0 + sl);
-            const int y0 = cyy * sl, y1 = (cyy == ncy - 1) ? L.H : min(L.H, y0 + sl);
-            const int w = x1 - x0, npx = w * (y1 - y0);
-            const int j0 = cyy * G.nx + cxx;
-            const float2 c00 = c[j0], c01 = c[j0 + 1], c10 = c[j0 + G.nx], c11 = c[j0 + G.nx + 1];
-            const float2 dtop = make_float2(c01.x - c00.x, c01.y - c00.y);
-            const float2 dbot = make_float2(c11.x - c10.x, c11.y - c10.y);
-            float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-            if (w == sl && pow2) {
-                // Full-width cell whose width (a power of two) divides the warp: every lane keeps one column
-                // (x = x0 + lane mod sl) and walks rows 32/sl apart, so the weight along x and
-                // the x-interpolated control values are fixed per lane; the y weights are summed
-                // and the x weights applied once at the end (the bilinear weight factorises).
-                // With a power-of-two spacing the weights are exact dyadic values, so the weight
-                // along y advances by a constant and equals the per-row formula
-                // min(g(y), ny - 1) - cyy, g(y) = (2^l y + off) / s.
-                const int x = x0 + (lane & (sl - 1)), dy = 32 >> lg;
-                const float wx = fminf(fmaf(GL.pl, (float)x, GL.off) * GL.scale_inv, (float)(G.nx - 1)) - (float)cxx;
-                const float tx = fmaf(wx, dtop.x, c00.x), ty = fmaf(wx, dtop.y, c00.y);
-                const float bx = fmaf(wx, dbot.x, c10.x), by = fmaf(wx, dbot.y, c10.y);
-                const float ex = bx - tx, ey = by - ty;
-                const float wmax = (float)(G.ny - 1 - cyy);
-                float wyk = fmaf(GL.pl, (float)(lane >> lg), GL.off) * GL.scale_inv;
-                float st_x = 0.f, st_y = 0.f, sb_x = 0.f, sb_y = 0.f;
-#pragma unroll 4
-                for (int y = y0 + (lane >> lg); y < y1; y += dy) {
-                    const float wy = fminf(wyk, wmax);
-                    wyk += dwy;
-                    float dtx, dty;
-                    const float tw = sample_q<S, true>(T, L.W, L.H, L.Tp, x, y, fmaf(wy, ex, tx), fmaf(wy, ey, ty),
-                                                       dtx, dty);
-                    const float hy = 1.f - wy;
-                    if constexpr (METRIC) {
-                        // squared weights: w^2 = hx^2 hy^2 factorises like w
-                        (void)tw;
-                        const float gx = dtx * dtx, gy = dty * dty, hy2 = hy * hy, wy2 = wy * wy;
-                        st_x = fmaf(hy2, gx, st_x); st_y = fmaf(hy2, gy, st_y);
-                        sb_x = fmaf(wy2, gx, sb_x); sb_y = fmaf(wy2, gy, sb_y);
-                    } else {
-                        const float rv = ldS<S>(R + (size_t)y * L.Rp + x) - L.cR;
-                        const float tv = tw - L.cR;
-                        // F = P dE/dTw = -(aP (r - rbar) - bP (t - tbar)), no contraction
-                        const float F = -__fsub_rn(__fmul_rn(aP, rv - rb), __fmul_rn(bP, tv - tb));
-                        const float gx = F * dtx, gy = F * dty;
-                        st_x = fmaf(hy, gx, st_x); st_y = fmaf(hy, gy, st_y);
-                        sb_x = fmaf(wy, gx, sb_x); sb_y = fmaf(wy, gy, sb_y);
-                    }
-                }
-                const float hx = METRIC ? (1.f - wx) * (1.f - wx) : 1.f - wx, vx = METRIC ? wx * wx : wx;
-                acc[0] = hx * st_x; acc[1] = hx * st_y; acc[2] = vx * st_x; acc[3] = vx * st_y;
-                acc[4] = hx * sb_x; acc[5] = hx * sb_y; acc[6] = vx * sb_x; acc[7] = vx * sb_y;
-            } else
-            for (int i = lane; i < npx; i += 32) {
-                const int y = y0 + i / w, x = x0 + i % w;
-                const float gxf = fminf(fmaf(GL.pl, (float)x, GL.off) * GL.scale_inv, (float)(G.nx - 1));
-                const float gyf = fminf(fmaf(GL.pl, (float)y, GL.off) * GL.scale_inv, (float)(G.ny - 1));
-                const float wx = gxf - (float)cxx, wy = gyf - (float)cyy;
-                const float tx = fmaf(wx, dtop.x, c00.x), ty = fmaf(wx, dtop.y, c00.y);
-                const float bx = fmaf(wx, dbot.x, c10.x), by = fmaf(wx, dbot.y, c10.y);
-                const float ux = fmaf(wy, bx - tx, tx), uy = fmaf(wy, by - ty, ty);
-                float dtx, dty;
-                const float tw = sample_q<S, true>(T, L.W, L.H, L.Tp, x, y, ux, uy, dtx, dty);
-                float gx, gy;
-                if constexpr (METRIC) {
-                    (void)tw;
-                    gx = dtx * dtx;
-                    gy = dty * dty;
-                } else {
-                    const float rv = ldS<S>(R + (size_t)y * L.Rp + x) - L.cR;
-                    const float tv = tw - L.cR;
-                    // F = P dE/dTw = -(aP (r - rbar) - bP (t - tbar)), no contraction
-                    const float F = -__fsub_rn(__fmul_rn(aP, rv - rb), __fmul_rn(bP, tv - tb));
-                    gx = F * dtx;
-                    gy = F * dty;
-                }
-                const float hx = 1.f - wx, hy = 1.f - wy;
-                float w00 = hx * hy, w01 = wx * hy, w10 = hx * wy, w11 = wx * wy;
-                if constexpr (METRIC) { w00 *= w00; w01 *= w01; w10 *= w10; w11 *= w11; }
-                acc[0] = fmaf(w00, gx, acc[0]); acc[1] = fmaf(w00, gy, acc[1]);
-                acc[2] = fmaf(w01, gx, acc[2]); acc[3] = fmaf(w01, gy, acc[3]);
-                acc[4] = fmaf(w10, gx, acc[4]); acc[5] = fmaf(w10, gy, acc[5]);
-                acc[6] = fmaf(w11, gx, acc[6]); acc[7] = fmaf(w11, gy, acc[7]);
-            }
-            const float tot8 = seg_reduce_scatter8<32>(acc, lane);
-            if ((lane & 3) == 0) {
-                const int vi = seg_index8<32>(lane);
-                const int corner = vi >> 1;
-                const int jc = (cyy + (corner >> 1) - cr0) * G.nx + cxx + (corner & 1);
-                gpf[2 * jc + (vi & 1)] += tot8;
-            }
-        }
-        __syncthreads();
+    const int n = (B.own1 - B.cr0) * G.nx;
+    float hi[1] = {0.f}, lo[1] = {0.f};
+    for (int j = threadIdx.x; j < n; j += kThreads) {
+        const int i = j / G.nx, jx = j - i * G.nx, row = B.cr0 + i;
+        float s[2];
+        point_sum<2>(slots, above, P, B, G.nx - 1, row, jx, 6, s);
+        const float nb = (float)((jx > 0) + (jx + 1 < G.nx) + (row > 0) + (row + 1 < G.ny));
+        const float2 m = make_float2(fmaf(dk, s[0], rk * nb), fmaf(dk, s[1], rk * nb));
+        mt[(row - B.h0) * G.nx + jx] = m;
+        ff_acc(hi[0], lo[0], m.x + m.y);
     }
-    cl.sync();   // every CTA's partial gradient is complete and visible in the cluster
-    const int C = cl.num_blocks();
-    const int q = (ncy + C - 1) / C;
+    cluster_reduce<1, false>(hi, lo, 0.f, sm, buf, cl);
+    const double mean = sm.tot[0] / (2.0 * (G.nx * G.ny));
+    const float inv = mean > 0.0 ? (float)(1.0 / mean) : 0.f;
+    for (int j = threadIdx.x; j < n; j += kThreads) {
+        float2 &m = mt[(B.cr0 - B.h0) * G.nx + j];
+        m = mean > 0.0 ? make_float2(fmaxf(m.x * inv, 1e-3f), fmaxf(m.y * inv, 1e-3f)) : make_float2(1.f, 1.f);
+    }
+}
+
+// The descent direction d = -M^-1 grad E at c with the scalar product mt, from the pass's gradient
+// sums: dE/dc_j = (1/P) [aP sF + bmaP sT + kappa s1 + lambda sum_nbrs (c_j - c_k)] (pm: aP, (b - a) P,
+// kappa, lambda), at the own rows and, through the neighbours' staged rows, at the held ones.  Leaves
+// sum_j m_j |d_j|^2 in sm.tot[0], with the direction d held before the call <d_old, d_old - d>_M in
+// sm.tot[1] and |d_old - d|_M^2 in sm.tot[2], max |d_j|^2 in sm.tmax; identical in every CTA.
+__device__ void grid_direction(const Grid &G, const Lvl &L, const PassGeom &P, const Band &B, const float2 *c,
+                               float2 *d, float2 *mt, float2 *halo, const float *slots, const float *above,
+                               const float *pm, Smem &sm, int &buf, const cg::cluster_group &cl, const H1Bufs &h1)
+{
+    const int Nc = G.nx * G.ny, n = (B.own1 - B.cr0) * G.nx, rank = cl.block_rank();
+    const float aP = pm[0], bmaP = pm[1], kappa = pm[2], lam = pm[3];
     const float scale = -(float)Nc / ((float)L.W * (float)L.H);
-    if constexpr (METRIC) {
-        // m_j = dk sum w^2 dT^2 + rk n_j per axis, then its mean over all 2 Nc values
-        const float dk = pm[0], rk = pm[1];
-        float mh = 0.f, ml = 0.f, mrun = 0.f;
-        int kk = 0;
-        for (int j = tid; j < Nc; j += kThreads) {
-            const int jy = j / G.nx, jx = j - jy * G.nx;
-            const int rlo = jy > 0 ? min(C - 1, (jy - 1) / max(q, 1)) : 0;
-            const int rhi = min(C - 1, jy / max(q, 1));
-            float2 h = *cl.map_shared_rank(gp + (jy - min(ncy, rlo * q)) * G.nx + jx, rlo);
-            if (rhi != rlo) {
-                const float2 h2 = *cl.map_shared_rank(gp + (jy - min(ncy, rhi * q)) * G.nx + jx, rhi);
-                h.x += h2.x;
-                h.y += h2.y;
-            }
-            const float nb = (float)((jx > 0) + (jx + 1 < G.nx) + (jy > 0) + (jy + 1 < G.ny));
-            const float2 m = make_float2(fmaf(dk, h.x, rk * nb), fmaf(dk, h.y, rk * nb));
-            mt[j] = m;
-            mrun += m.x + m.y;
-            if (++kk == kFast) { ff_acc(mh, ml, mrun); mrun = 0.f; kk = 0; }
-        }
-        ff_acc(mh, ml, mrun);
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) {
-            const float h2 = __shfl_xor_sync(0xffffffffu, mh, off), l2 = __shfl_xor_sync(0xffffffffu, ml, off);
-            ff_add(mh, ml, h2, l2);
-        }
-        if (lane == 0) sm.warp[warp][0] = make_float2(mh, ml);
-        __syncthreads();
-        if (tid == 0) {
-            float h = 0.f, l = 0.f;
-            for (int w2 = 0; w2 < kWarps; ++w2) ff_add(h, l, sm.warp[w2][0].x, sm.warp[w2][0].y);
-            sm.tot[0] = ((double)h + (double)l) / (2.0 * Nc);
-        }
-        __syncthreads();
-        const double mean = sm.tot[0];
-        const float inv = mean > 0.0 ? (float)(1.0 / mean) : 0.f;
-        for (int j = tid; j < Nc; j += kThreads) {
-            const float2 m = mt[j];
-            mt[j] = mean > 0.0 ? make_float2(fmaxf(m.x * inv, 1e-3f), fmaxf(m.y * inv, 1e-3f)) : make_float2(1.f, 1.f);
-        }
-        // no CTA may overwrite its band (next gradient pass) while a peer still reads it
-        cl.sync();
-        return;
-    }
-    float ssh = 0.f, ssl = 0.f, mx = 0.f, run = 0.f;
-    // <d_prev, d_prev - d> and |d_prev - d|^2 for the first trial step (d still holds d_prev)
-    float nmh = 0.f, nml = 0.f, dnh = 0.f, dnl = 0.f, nrun = 0.f, drun = 0.f;
-    int k = 0;
-    constexpr int kBatch = 4;   // points per thread whose remote loads are in flight together
+    float hi[3] = {0.f, 0.f, 0.f}, lo[3] = {0.f, 0.f, 0.f}, mx = 0.f;
+    // -Nc dE/dc at own point j (row i of the own rows)
+    auto rhs = [&](int i, int jx) {
+        const int row = B.cr0 + i, k = (row - B.h0) * G.nx + jx;
+        float s[6];
+        point_sum<6>(slots, above, P, B, G.nx - 1, row, jx, 0, s);
+        const float gx = fmaf(aP, s[0], fmaf(bmaP, s[2], kappa * s[4]));
+        const float gy = fmaf(aP, s[1], fmaf(bmaP, s[3], kappa * s[5]));
+        const float2 cj = c[k];
+        float lx = 0.f, ly = 0.f;
+        if (jx > 0)         { const float2 v = c[k - 1];    lx += cj.x - v.x; ly += cj.y - v.y; }
+        if (jx + 1 < G.nx)  { const float2 v = c[k + 1];    lx += cj.x - v.x; ly += cj.y - v.y; }
+        if (row > 0)        { const float2 v = c[k - G.nx]; lx += cj.x - v.x; ly += cj.y - v.y; }
+        if (row + 1 < G.ny) { const float2 v = c[k + G.nx]; lx += cj.x - v.x; ly += cj.y - v.y; }
+        return make_float2(scale * fmaf(lam, lx, gx), scale * fmaf(lam, ly, gy));
+    };
     if (h1.B) {
-        // H1 product: b = scale (lambda lap + g) = -Nc dE/dc into B, d = M^-1 b into U; then
+        // H1 product: b = -Nc dE/dc into B of every CTA, d = M^-1 b into U by every CTA; then
         // |d|_M^2 = d.b, and for the first trial <d_prev, y>_M, |y|_M^2 with y = d_prev - d, M y
         // taken as the stencil y + s2 Lg y
-        for (int j = tid; j < Nc; j += kThreads) {
-            const int jy = j / G.nx, jx = j - jy * G.nx;
-            const int rlo = jy > 0 ? min(C - 1, (jy - 1) / max(q, 1)) : 0;
-            const int rhi = min(C - 1, jy / max(q, 1));
-            float2 g = *cl.map_shared_rank(gp + (jy - min(ncy, rlo * q)) * G.nx + jx, rlo);
-            if (rhi != rlo) {
-                const float2 w2 = *cl.map_shared_rank(gp + (jy - min(ncy, rhi * q)) * G.nx + jx, rhi);
-                g.x += w2.x;
-                g.y += w2.y;
-            }
-            const float2 cj = c[j];
-            float lx = 0.f, ly = 0.f;
-            if (jx > 0)        { const float2 v = c[j - 1];    lx += cj.x - v.x; ly += cj.y - v.y; }
-            if (jx + 1 < G.nx) { const float2 v = c[j + 1];    lx += cj.x - v.x; ly += cj.y - v.y; }
-            if (jy > 0)        { const float2 v = c[j - G.nx]; lx += cj.x - v.x; ly += cj.y - v.y; }
-            if (jy + 1 < G.ny) { const float2 v = c[j + G.nx]; lx += cj.x - v.x; ly += cj.y - v.y; }
-            h1.B[j] = make_float2(scale * fmaf(lam, lx, g.x), scale * fmaf(lam, ly, g.y));
+        for (int j = threadIdx.x; j < n; j += kThreads) {
+            const int i = j / G.nx, jx = j - i * G.nx;
+            const float2 b = rhs(i, jx);
+            for (unsigned r = 0; r < cl.num_blocks(); ++r) *cl.map_shared_rank(h1.B + (B.cr0 + i) * G.nx + jx, r) = b;
         }
-        __syncthreads();
+        cl.sync();   // B is complete, and no CTA reads another's slots any more (T and U lie there)
         h1_solve(h1, G.nx, G.ny);
-        auto yv = [&](int i) {
-            const float2 a = d[i], b = h1.U[i];
+        auto yv = [&](int row, int jx) {
+            const float2 a = d[(row - B.h0) * G.nx + jx], b = h1.U[row * G.nx + jx];
             return make_float2(a.x - b.x, a.y - b.y);
         };
-        for (int j = tid; j < Nc; j += kThreads) {
-            const int jy = j / G.nx, jx = j - jy * G.nx;
-            const float2 dj = h1.U[j], bj = h1.B[j], dold = d[j], y = yv(j);
+        for (int j = threadIdx.x; j < n; j += kThreads) {
+            const int i = j / G.nx, jx = j - i * G.nx, row = B.cr0 + i;
+            const float2 dj = h1.U[row * G.nx + jx], bj = h1.B[row * G.nx + jx], dold = d[(row - B.h0) * G.nx + jx];
+            const float2 y = yv(row, jx);
             float lx = 0.f, ly = 0.f;
-            if (jx > 0)        { const float2 v = yv(j - 1);    lx += y.x - v.x; ly += y.y - v.y; }
-            if (jx + 1 < G.nx) { const float2 v = yv(j + 1);    lx += y.x - v.x; ly += y.y - v.y; }
-            if (jy > 0)        { const float2 v = yv(j - G.nx); lx += y.x - v.x; ly += y.y - v.y; }
-            if (jy + 1 < G.ny) { const float2 v = yv(j + G.nx); lx += y.x - v.x; ly += y.y - v.y; }
+            if (jx > 0)         { const float2 v = yv(row, jx - 1); lx += y.x - v.x; ly += y.y - v.y; }
+            if (jx + 1 < G.nx)  { const float2 v = yv(row, jx + 1); lx += y.x - v.x; ly += y.y - v.y; }
+            if (row > 0)        { const float2 v = yv(row - 1, jx); lx += y.x - v.x; ly += y.y - v.y; }
+            if (row + 1 < G.ny) { const float2 v = yv(row + 1, jx); lx += y.x - v.x; ly += y.y - v.y; }
             const float myx = fmaf(h1.s2, lx, y.x), myy = fmaf(h1.s2, ly, y.y);
-            run = fmaf(dj.x, bj.x, fmaf(dj.y, bj.y, run));
-            nrun = fmaf(dold.x, myx, fmaf(dold.y, myy, nrun));
-            drun = fmaf(y.x, myx, fmaf(y.y, myy, drun));
+            ff_acc(hi[0], lo[0], fmaf(dj.x, bj.x, dj.y * bj.y));
+            ff_acc(hi[1], lo[1], fmaf(dold.x, myx, dold.y * myy));
+            ff_acc(hi[2], lo[2], fmaf(y.x, myx, y.y * myy));
             mx = fmaxf(mx, fmaf(dj.x, dj.x, dj.y * dj.y));
-            if (++k == kFast) {
-                ff_acc(ssh, ssl, run); run = 0.f;
-                ff_acc(nmh, nml, nrun); nrun = 0.f;
-                ff_acc(dnh, dnl, drun); drun = 0.f;
-                k = 0;
-            }
         }
         __syncthreads();   // every d_prev was read before d is replaced
-        for (int j = tid; j < Nc; j += kThreads) d[j] = h1.U[j];
-    } else
-    for (int j0 = tid; j0 < Nc; j0 += kBatch * kThreads) {
-        float2 gb[kBatch];
-#pragma unroll
-        for (int b = 0; b < kBatch; ++b) {
-            const int j = j0 + b * kThreads;
-            gb[b] = make_float2(0.f, 0.f);
-            if (j < Nc) {
-                const int jy = j / G.nx;
-                // bands: rank r owns cell rows [r q, (r+1) q) and so control rows [r q, (r+1) q]
-                const int rlo = jy > 0 ? min(C - 1, (jy - 1) / max(q, 1)) : 0;
-                const int rhi = min(C - 1, jy / max(q, 1));
-                const int jx = j - jy * G.nx;
-                const float2 v = *cl.map_shared_rank(gp + (jy - min(ncy, rlo * q)) * G.nx + jx, rlo);
-                gb[b].x += v.x;
-                gb[b].y += v.y;
-                if (rhi != rlo) {
-                    const float2 w2 = *cl.map_shared_rank(gp + (jy - min(ncy, rhi * q)) * G.nx + jx, rhi);
-                    gb[b].x += w2.x;
-                    gb[b].y += w2.y;
-                }
-            }
-        }
-#pragma unroll
-        for (int b = 0; b < kBatch; ++b) {
-        const int j = j0 + b * kThreads;
-        if (j >= Nc) break;
-        const int jy = j / G.nx, jx = j - jy * G.nx;
-        const float2 g = gb[b];
-        const float2 cj = c[j];
-        float lx = 0.f, ly = 0.f;
-        if (jx > 0)        { const float2 v = c[j - 1];    lx += cj.x - v.x; ly += cj.y - v.y; }
-        if (jx + 1 < G.nx) { const float2 v = c[j + 1];    lx += cj.x - v.x; ly += cj.y - v.y; }
-        if (jy > 0)        { const float2 v = c[j - G.nx]; lx += cj.x - v.x; ly += cj.y - v.y; }
-        if (jy + 1 < G.ny) { const float2 v = c[j + G.nx]; lx += cj.x - v.x; ly += cj.y - v.y; }
-        // d = -M^-1 grad E with the level's scalar product M (per axis)
-        const float2 mj = mt[j];
-        float2 dj;
-        dj.x = scale * fmaf(lam, lx, g.x) / mj.x;
-        dj.y = scale * fmaf(lam, ly, g.y) / mj.y;
-        const float2 dold = d[j];
-        d[j] = dj;
-        const float qd = fmaf(dj.x, dj.x, dj.y * dj.y);
+        for (int j = threadIdx.x; j < (B.h1 - B.h0) * G.nx; j += kThreads) d[j] = h1.U[B.h0 * G.nx + j];
+        cluster_reduce<3, true>(hi, lo, mx, sm, buf, cl);
+        return;
+    }
+    // The edge rows go to the neighbours' halo rows (0: the row above the own ones, 1: the row below),
+    // not to their d, which a slower neighbour may still read for its accepted step.
+    for (int j = threadIdx.x; j < n; j += kThreads) {
+        const int i = j / G.nx, jx = j - i * G.nx, row = B.cr0 + i, k = (row - B.h0) * G.nx + jx;
+        const float2 b = rhs(i, jx), mj = mt[k], dold = d[k];
+        const float2 dj = make_float2(b.x / mj.x, b.y / mj.y);
+        d[k] = dj;
+        if (i == 0 && B.cr0 > 0) *cl.map_shared_rank(halo + G.nx + jx, rank - 1) = dj;
+        if (row == B.cr1 - 1 && B.own1 < G.ny) *cl.map_shared_rank(halo + jx, rank + 1) = dj;
         const float yx = dold.x - dj.x, yy = dold.y - dj.y;
-        run = fmaf(mj.x * dj.x, dj.x, fmaf(mj.y * dj.y, dj.y, run));
-        nrun = fmaf(mj.x * dold.x, yx, fmaf(mj.y * dold.y, yy, nrun));
-        drun = fmaf(mj.x * yx, yx, fmaf(mj.y * yy, yy, drun));
-        mx = fmaxf(mx, qd);
-        if (++k == kFast) {
-            ff_acc(ssh, ssl, run); run = 0.f;
-            ff_acc(nmh, nml, nrun); nrun = 0.f;
-            ff_acc(dnh, dnl, drun); drun = 0.f;
-            k = 0;
-        }
-        }
+        ff_acc(hi[0], lo[0], fmaf(mj.x * dj.x, dj.x, mj.y * dj.y * dj.y));
+        ff_acc(hi[1], lo[1], fmaf(mj.x * dold.x, yx, mj.y * dold.y * yy));
+        ff_acc(hi[2], lo[2], fmaf(mj.x * yx, yx, mj.y * yy * yy));
+        mx = fmaxf(mx, fmaf(dj.x, dj.x, dj.y * dj.y));
     }
-    ff_acc(ssh, ssl, run);
-    ff_acc(nmh, nml, nrun);
-    ff_acc(dnh, dnl, drun);
-    // block reduction (identical in every CTA: same inputs, same order)
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-        float h2 = __shfl_xor_sync(0xffffffffu, ssh, off), l2 = __shfl_xor_sync(0xffffffffu, ssl, off);
-        ff_add(ssh, ssl, h2, l2);
-        h2 = __shfl_xor_sync(0xffffffffu, nmh, off); l2 = __shfl_xor_sync(0xffffffffu, nml, off);
-        ff_add(nmh, nml, h2, l2);
-        h2 = __shfl_xor_sync(0xffffffffu, dnh, off); l2 = __shfl_xor_sync(0xffffffffu, dnl, off);
-        ff_add(dnh, dnl, h2, l2);
-        mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, off));
+    cluster_reduce<3, true>(hi, lo, mx, sm, buf, cl);
+    for (int j = threadIdx.x; j < 2 * G.nx; j += kThreads) {
+        const bool below = j >= G.nx;
+        const int row = below ? B.own1 : B.cr0 - 1;
+        if (B.cr0 < B.own1 && row >= 0 && row < G.ny) d[(row - B.h0) * G.nx + (below ? j - G.nx : j)] = halo[j];
     }
-    if (lane == 0) {
-        sm.warp[warp][0] = make_float2(ssh, ssl);
-        sm.warp[warp][1] = make_float2(mx, 0.f);
-        sm.warp[warp][2] = make_float2(nmh, nml);
-        sm.warp[warp][3] = make_float2(dnh, dnl);
-    }
-    __syncthreads();
-    if (tid < 4 && tid != 1) {
-        float h = 0.f, l = 0.f;
-        for (int w2 = 0; w2 < kWarps; ++w2) ff_add(h, l, sm.warp[w2][tid].x, sm.warp[w2][tid].y);
-        sm.tot[tid] = (double)h + (double)l;
-    } else if (tid == 1) {
-        float m = 0.f;
-        for (int w2 = 0; w2 < kWarps; ++w2) m = fmaxf(m, sm.warp[w2][1].x);
-        sm.tot[1] = (double)m;
-    }
-    __syncthreads();
 }
 
 __device__ double field_energy(FieldCtl &k, const Config &cfg, const double *tot, bool trial)
@@ -1500,73 +1370,72 @@ __device__ double field_energy(FieldCtl &k, const Config &cfg, const double *tot
     return E;
 }
 
-// Gradient-pass parameters from the current NCC terms: aP, bP, rbar, tbar, lambda.
+// Parameter slots of the nonrigid passes: gradient coefficients aP, (b - a) P, (a rbar - b tbar) P
+// and lambda; the scalar product's 1/(P var T) and lambda/P; the next trial's step.
+enum FieldParam { kPmA = 0, kPmB = 1, kPmK = 2, kPmLam = 3, kPmDk = 4, kPmRk = 5, kPmTau = 6 };
+
+// Gradient coefficients from the current NCC terms; a == b and rbar == tbar give exact zeros.
 __device__ void field_grad_params(const FieldCtl &k, const Config &cfg, float *pm)
 {
-    pm[0] = (float)(k.a * k.P);
-    pm[1] = (float)(k.b * k.P);
-    pm[2] = (float)k.rbar;
-    pm[3] = (float)k.tbar;
-    pm[4] = (float)cfg.lambda;
+    pm[kPmA] = (float)(k.a * k.P);
+    pm[kPmB] = (float)(__dsub_rn(k.b, k.a) * k.P);
+    pm[kPmK] = (float)(__dsub_rn(__dmul_rn(k.a, k.rbar), __dmul_rn(k.b, k.tbar)) * k.P);
+    pm[kPmLam] = (float)cfg.lambda;
 }
 
-// Thread-0 controller of the nonrigid level loop (same rules as the rigid one): ENERGY at level
-// start, GRAD = gradient pass, TRIAL = Armijo trial at c + tau d.  pm[0] of a trial is tau.
-__device__ int field_step(FieldCtl &k, const Config &cfg, const double *tot, int action, float *pm)
+// Thread-0 controller of the nonrigid level loop (same rules as the rigid one).  field_eval decides
+// on a pass's moments: the level's first point, an accepted trial (`accepted` = 1) or a rejected
+// one, whose shorter step it leaves in pm[kPmTau]; kActGrad asks for the direction there.
+__device__ int field_eval(FieldCtl &k, const Config &cfg, const double *tot, bool start, float *pm, int &accepted)
 {
-    if (action == kActEnergy) {
+    accepted = 0;
+    if (start) {
         k.sr = tot[3]; k.srr = tot[4];
         k.E = field_energy(k, cfg, tot, false);
-        if (cfg.metric == 1) {
-            // the level's scalar product at its initial control values: 1/(P var T) and lambda/P
-            const double vt = (tot[1] - tot[0] * tot[0] * k.invP) * k.invP;
-            pm[0] = vt > 0.0 ? (float)(k.invP / vt) : 0.f;
-            pm[1] = (float)(cfg.lambda * k.invP);
-            return kActMetric;
-        }
+        // the level's scalar product at its initial control values: 1/(P var T) and lambda/P
+        const double vt = (tot[1] - tot[0] * tot[0] * k.invP) * k.invP;
+        pm[kPmDk] = vt > 0.0 ? (float)(k.invP / vt) : 0.f;
+        pm[kPmRk] = (float)(cfg.lambda * k.invP);
         field_grad_params(k, cfg, pm);
         return kActGrad;
     }
-    if (action == kActMetric) {
-        field_grad_params(k, cfg, pm);
-        return kActGrad;
-    }
-    if (action == kActGrad) {
-        k.evals += 1;
-        if (k.iters >= cfg.max_iter) { k.stop = REG_STOP_MAXIT; return kActDone; }
-        // |g| = sqrt(ss / Nc) and the largest control step dmax = sqrt(tot[1]): compared squared
-        const double ss = tot[0], dmax2 = tot[1];
-        k.slope = -ss * k.invNc;
-        if (!(ss * k.invNc >= k.tolg * k.tolg)) { k.stop = REG_STOP_GRAD; return kActDone; }
-        // the metric (mean over control points) is a common factor of tot[2] and tot[3]
-        if (k.have_prev) k.tau = bb_tau(k.tau, k.tau_acc, tot[2], tot[3]);
-        if (k.tau * k.tau * dmax2 > cfg.step_cap * cfg.step_cap) k.tau = cfg.step_cap / sqrt(dmax2);
-        k.nrej = 0;
-        pm[0] = (float)k.tau;
-        return kActTrial;
-    }
-    // trial
     const double Et = field_energy(k, cfg, tot, true);
     k.evals += 1;
     if (Et <= k.E + cfg.armijo_c * k.tau * k.slope) {
+        accepted = 1;   // c is advanced by the trial's step
         k.iters += 1;
         const double Eold = k.E;
-        k.tau_pend = (double)(float)k.tau;
-        k.tau_acc = k.tau_pend;   // the step applied: c + (float)tau d
+        k.tau_acc = (double)(float)k.tau;   // the step applied: c + (float)tau d
         k.have_prev = 1;
         k.tau = next_tau(k.E, k.slope, k.tau, Et, true);
         k.E = Et;
         k.a = k.ta; k.b = k.tb; k.rbar = k.trbar; k.tbar = k.ttbar; k.degen = k.tdegen;
         if (Eold - Et <= cfg.tol_rel_e * fabs(Eold)) { k.stop = REG_STOP_REL; return kActDone; }
         field_grad_params(k, cfg, pm);
-        return kActGrad;   // c is advanced to ct before the gradient pass
+        return kActGrad;
     }
     k.rejects += 1;
     k.nrej += 1;
     k.tau = next_tau(k.E, k.slope, k.tau, Et, false);
-    k.tau_pend = 0.0;
     if (k.nrej > cfg.max_rejects) { k.stop = REG_STOP_LS; return kActDone; }
-    pm[0] = (float)k.tau;
+    pm[kPmTau] = (float)k.tau;
+    return kActTrial;
+}
+
+// The stop tests at a point whose direction is known, and the first trial's step.
+__device__ int field_grad(FieldCtl &k, const Config &cfg, const double *tot, double dmax2, float *pm)
+{
+    k.evals += 1;
+    if (k.iters >= cfg.max_iter) { k.stop = REG_STOP_MAXIT; return kActDone; }
+    // |g| = sqrt(ss / Nc) and the largest control step dmax: compared squared
+    const double ss = tot[0];
+    k.slope = -ss * k.invNc;
+    if (!(ss * k.invNc >= k.tolg * k.tolg)) { k.stop = REG_STOP_GRAD; return kActDone; }
+    // the metric (mean over control points) is a common factor of the two sums
+    if (k.have_prev) k.tau = bb_tau(k.tau, k.tau_acc, tot[1], tot[2]);
+    if (k.tau * k.tau * dmax2 > cfg.step_cap * cfg.step_cap) k.tau = cfg.step_cap / sqrt(dmax2);
+    k.nrej = 0;
+    pm[kPmTau] = (float)k.tau;
     return kActTrial;
 }
 
@@ -1586,7 +1455,7 @@ __device__ __forceinline__ float2 grid_eval_global(const float2 *q, const Grid &
     return u;
 }
 
-template <typename S, int U>
+template <typename S, int R>
 __device__ void run_nonrigid(const Params &p, const OpDesc &op, int op_index, Smem &sm, float2 *gbuf,
                              const cg::cluster_group &cl)
 {
@@ -1598,11 +1467,12 @@ __device__ void run_nonrigid(const Params &p, const OpDesc &op, int op_index, Sm
     const int Nc = G.nx * G.ny;
     const bool h1 = cfg.metric == REG_METRIC_H1;
     const GridLayout lay = grid_layout(G.nx, G.ny, C, h1);
-    float2 *c = gbuf + lay.c, *d = gbuf + lay.d, *mt = gbuf + lay.mt, *gp = gbuf + lay.gp;
-    float4 *crow = (float4 *)(gbuf + lay.crow);
-    // H1 product: mt holds the right-hand side of its solve
-    const H1Bufs hb{h1 ? mt : nullptr, h1 ? gbuf + lay.t : nullptr, h1 ? gbuf + lay.u : nullptr, p.h1q,
-                    (float)(cfg.sigma * cfg.sigma)};
+    const Band B = grid_band(G, rank, C);
+    const int held = (B.h1 - B.h0) * G.nx, first = B.h0 * G.nx;   // points held, and the first of them
+    float2 *c = gbuf + lay.c, *d = gbuf + lay.d, *mt = gbuf + lay.mt, *halo = gbuf + lay.halo;
+    float *slots = (float *)(gbuf + lay.slots);
+    const float *above = rank > 0 && B.cr0 < B.cr1 ? cl.map_shared_rank(slots, rank - 1) : nullptr;
+    const H1Bufs hb{h1 ? mt : nullptr, (float2 *)slots, (float2 *)slots + Nc, p.h1q, (float)(cfg.sigma * cfg.sigma)};
     int buf = 0;
     // initial control values (finest px), scaled to the coarsest level
     {
@@ -1610,20 +1480,20 @@ __device__ void run_nonrigid(const Params &p, const OpDesc &op, int op_index, Sm
         if (op.left >= 0) {
             // B's initial guess phi_jk o phi_ij at the control points (Sec. 2.3.2)
             const float2 *q1 = p.node_grid + (size_t)Nc * op.left, *q2 = p.node_grid + (size_t)Nc * op.right;
-            for (int j = tid; j < Nc; j += kThreads) {
-                const int jy = j / G.nx, jx = j - jy * G.nx;
-                const float2 a = __ldcg(q1 + j);
+            for (int j = tid; j < held; j += kThreads) {
+                const int jy = (first + j) / G.nx, jx = first + j - jy * G.nx;
+                const float2 a = __ldcg(q1 + first + j);
                 const float2 u = grid_eval_global(q2, G, (float)(jx * G.s) + a.x, (float)(jy * G.s) + a.y);
                 c[j] = make_float2(sc * (a.x + u.x), sc * (a.y + u.y));
             }
         } else if (op.init_node >= 0) {
             const float2 *q = p.node_grid + (size_t)Nc * op.init_node;
-            for (int j = tid; j < Nc; j += kThreads) {
-                const float2 a = __ldcg(q + j);
+            for (int j = tid; j < held; j += kThreads) {
+                const float2 a = __ldcg(q + first + j);
                 c[j] = make_float2(sc * a.x, sc * a.y);
             }
         } else {
-            for (int j = tid; j < Nc; j += kThreads) c[j] = make_float2(0.f, 0.f);
+            for (int j = tid; j < held; j += kThreads) c[j] = make_float2(0.f, 0.f);
         }
     }
     FieldCtl &k = sm.fctl;
@@ -1635,74 +1505,68 @@ __device__ void run_nonrigid(const Params &p, const OpDesc &op, int op_index, Sm
     int stops[kMaxLevels], iters[kMaxLevels], evals[kMaxLevels];
     for (int l = Lc - 1; l >= 0; --l) {
         const Lvl L = level_of(p, op.ref, op.tmpl, l);
-        GridLvl GL;
-        GL.W = L.W; GL.H = L.H; GL.l = l;
-        GL.pl = ldexpf(1.f, l);
-        GL.off = 0.5f * (GL.pl - 1.f);
-        GL.scale_inv = 1.f / (float)G.s;
-        int cr0, cr1, r0, r1;
-        grid_rows(G, GL, rank, C, cr0, cr1, r0, r1);
-        for (int j = tid; j < Nc; j += kThreads) mt[j] = make_float2(1.f, 1.f);
+        const GridLvl GL = grid_level(G, L, l);
+        const PassGeom P = pass_geom(G.s >> l, G.nx - 1, B.q, L.W > (G.nx - 1) * (G.s >> l));
+        if (cfg.metric == REG_METRIC_MEAN)
+            for (int j = tid; j < held; j += kThreads) mt[j] = make_float2(1.f, 1.f);
         if (tid == 0) {
             k.P = (double)L.W * (double)L.H;
             k.invP = 1.0 / k.P;
             k.tau = cfg.tau0;
-            k.tau_pend = 0.0;
             k.have_prev = 0;
             k.iters = 0; k.evals = 0; k.stop = REG_STOP_MAXIT;
             // a coarse level only supplies the next level's initial guess: a looser stop
             k.tolg = cfg.tol_grad * (l > 0 ? cfg.tol_coarse : 1.0);
-            sm.action = kActEnergy;
-        }
-        for (;;) {
-            __syncthreads();
-            const int act = sm.action;
-            if (act == kActDone) break;
-            float pm[5];
-#pragma unroll
-            for (int q = 0; q < 5; ++q) pm[q] = sm.pm[q];
-            if (act == kActEnergy) {
-                grid_energy_pass<S, true, U, false>(L, G, GL, c, d, 0.f, crow, r0, r1, sm, buf, cl);
-            } else if (act == kActTrial) {
-                grid_energy_pass<S, false, U, true>(L, G, GL, c, d, pm[0], crow, r0, r1, sm, buf, cl);
-            } else if (act == kActMetric) {
-                grid_grad_pass<S, true>(L, G, GL, c, d, mt, gp, pm, cr0, cr1, sm, cl, hb);
-            } else {
-                grid_grad_pass<S, false>(L, G, GL, c, d, mt, gp, pm, cr0, cr1, sm, cl, hb);
-            }
-            if (tid == 0) {
-                const int next = field_step(k, cfg, sm.tot, act, sm.pm);
-                sm.action = next;
-                sm.idata[0] = (act == kActTrial && k.tau_pend != 0.0) ? 1 : 0;   // accepted: c <- ct
-            }
-            __syncthreads();
-            if (sm.idata[0]) {
-                // the accepted trial: c + tau d with the trial's tau, as the trial pass formed it
-                for (int j = tid; j < Nc; j += kThreads) {
-                    const float2 a = c[j], b = d[j];
-                    c[j] = make_float2(fmaf(pm[0], b.x, a.x), fmaf(pm[0], b.y, a.y));
-                }
-                __syncthreads();
-                if (tid == 0) { sm.idata[0] = 0; k.tau_pend = 0.0; }
-            }
-        }
-        if (tid == 0) { stops[l] = k.stop; iters[l] = k.iters; evals[l] = k.evals; }
-        if (l > 0) {
-            for (int j = tid; j < Nc; j += kThreads) c[j] = make_float2(2.f * c[j].x, 2.f * c[j].y);
         }
         __syncthreads();
+        for (bool start = true;; start = false) {
+            const float tau = sm.pm[kPmTau];   // not read by a level's first pass
+            if (start) grid_pass<S, true, R>(L, G, GL, P, B, c, d, 0.f, slots, sm, buf, cl);
+            else grid_pass<S, false, R>(L, G, GL, P, B, c, d, tau, slots, sm, buf, cl);
+            if (tid == 0) sm.action = field_eval(k, cfg, sm.tot, start, sm.pm, sm.idata[0]);
+            __syncthreads();
+            const int act = sm.action;
+            if (sm.idata[0]) {
+                // the accepted trial, as the pass formed it
+                for (int j = tid; j < held; j += kThreads) {
+                    const float2 a = c[j], b = d[j];
+                    c[j] = make_float2(fmaf(tau, b.x, a.x), fmaf(tau, b.y, a.y));
+                }
+                __syncthreads();
+            }
+            if (act == kActDone) break;
+            if (act == kActTrial) continue;
+            float pm[6];
+#pragma unroll
+            for (int q = 0; q < 6; ++q) pm[q] = sm.pm[q];
+            if (start && cfg.metric == REG_METRIC_GAUSS_NEWTON)
+                grid_metric(G, P, B, slots, above, mt, pm[kPmDk], pm[kPmRk], sm, buf, cl);
+            grid_direction(G, L, P, B, c, d, mt, halo, slots, above, pm, sm, buf, cl, hb);
+            if (tid == 0) sm.action = field_grad(k, cfg, sm.tot, sm.tmax, sm.pm);
+            __syncthreads();
+            if (sm.action == kActDone) break;
+        }
+        if (tid == 0) { stops[l] = k.stop; iters[l] = k.iters; evals[l] = k.evals; }
+        __syncthreads();
+        if (l > 0)
+            for (int j = tid; j < held; j += kThreads) c[j] = make_float2(2.f * c[j].x, 2.f * c[j].y);
     }
-    if (rank == 0) {
-        float2 *o = p.node_grid + (size_t)Nc * op.out;
-        for (int j = tid; j < Nc; j += kThreads) __stcg(o + j, c[j]);
+    // the result: every CTA its own rows; the mean displacement over all points
+    float hi[2] = {0.f, 0.f}, lo[2] = {0.f, 0.f};
+    float2 *o = p.node_grid + (size_t)Nc * op.out + (size_t)B.cr0 * G.nx;
+    for (int j = tid; j < (B.own1 - B.cr0) * G.nx; j += kThreads) {
+        const float2 v = c[(B.cr0 - B.h0) * G.nx + j];
+        __stcg(o + j, v);
+        ff_acc(hi[0], lo[0], v.x);
+        ff_acc(hi[1], lo[1], v.y);
     }
+    __threadfence();   // before the cluster's first CTA publishes the node
+    cluster_reduce<2, false>(hi, lo, 0.f, sm, buf, cl);
     if (tid == 0 && rank == 0) {
-        double mx = 0.0, my = 0.0;
-        for (int j = 0; j < Nc; ++j) { mx += c[j].x; my += c[j].y; }
-        double *o = p.node_theta + 3 * op.out;
-        o[0] = 0.0;
-        o[1] = mx / Nc;
-        o[2] = my / Nc;
+        double *th = p.node_theta + 3 * op.out;
+        th[0] = 0.0;
+        th[1] = sm.tot[0] / Nc;
+        th[2] = sm.tot[1] / Nc;
         OpStats &st = p.stats[op_index];
         st.i = op.ref;
         st.k = op.tmpl;
@@ -1715,7 +1579,7 @@ __device__ void run_nonrigid(const Params &p, const OpDesc &op, int op_index, Sm
         st.rejects = k.rejects;
         st.status = kDevOk;
         st.energy = k.E;
-        st.theta[0] = o[0]; st.theta[1] = o[1]; st.theta[2] = o[2];
+        st.theta[0] = th[0]; st.theta[1] = th[1]; st.theta[2] = th[2];
     }
 }
 
@@ -1773,13 +1637,14 @@ __device__ void run_op(const Params &p, int op_index, Smem &sm, float2 *gbuf, co
     }
     if constexpr (MODE == REG_RIGID) run_rigid<S>(p, op, op_index, sm, cl);
     else if constexpr (MODE == kModeMock) run_mock(p, op, op_index, cl);
-    else run_nonrigid<S, U>(p, op, op_index, sm, gbuf, cl);
+    else run_nonrigid<S, U / 2>(p, op, op_index, sm, gbuf, cl);
 }
 
-// Batched launch: cluster q of the grid runs operator op_base + q.  MINB: CTAs per SM the
-// register budget is sized for (the nonrigid kernels come in a 3-CTA form without spills and a
-// 4-CTA form with a few spilled registers, faster once the clusters are large).  U: pixels in
-// flight per lane in the nonrigid energy passes (2 or 4, the tile shape reg_autotune chooses).
+// Batched launch: cluster q of the grid runs operator op_base + q.  MINB: CTAs per SM the register
+// budget is sized for.  The nonrigid kernels take 128 registers a thread, two CTAs per SM: at 80 (three
+// CTAs) the pass spills in its pixel loop, and a scan of 1,024 frames of 512x512 took 97 ms instead of
+// 76 (8 CTAs per operator).  U: pixels in flight per lane in the nonrigid passes (2 or 4, the tile shape
+// reg_autotune chooses): two columns of one or two rows.
 template <int MODE, typename S, int MINB, int U = 4>
 __global__ void __launch_bounds__(kThreads, MINB) op_kernel(Params p)
 {
@@ -1977,22 +1842,24 @@ __global__ void __launch_bounds__(kThreads) energy_kernel(Params p, const double
         const Grid G{p.gnx, p.gny, p.gs};
         const int Nc = G.nx * G.ny;
         const GridLayout lay = grid_layout(G.nx, G.ny, C, false);
-        float2 *c = gbuf + lay.c, *d = gbuf + lay.d, *mt = gbuf + lay.mt, *gp = gbuf + lay.gp;
-        float4 *crow = (float4 *)(gbuf + lay.crow);
-        for (int j = tid; j < Nc; j += kThreads) { c[j] = cgrid[j]; mt[j] = make_float2(1.f, 1.f); }
+        const Band B = grid_band(G, rank, C);
+        float2 *c = gbuf + lay.c, *d = gbuf + lay.d, *mt = gbuf + lay.mt, *halo = gbuf + lay.halo;
+        float *slots = (float *)(gbuf + lay.slots);
+        const float *above = rank > 0 && B.cr0 < B.cr1 ? cl.map_shared_rank(slots, rank - 1) : nullptr;
+        for (int j = tid; j < (B.h1 - B.h0) * G.nx; j += kThreads) {
+            c[j] = cgrid[B.h0 * G.nx + j];
+            d[j] = make_float2(0.f, 0.f);
+            mt[j] = make_float2(1.f, 1.f);
+        }
         __syncthreads();
-        GridLvl GL;
-        GL.W = L.W; GL.H = L.H; GL.l = 0; GL.pl = 1.f; GL.off = 0.f; GL.scale_inv = 1.f / (float)G.s;
-        int cr0, cr1, r0, r1;
-        grid_rows(G, GL, rank, C, cr0, cr1, r0, r1);
-        grid_energy_pass<S, true, 4, false>(L, G, GL, c, c, 0.f, crow, r0, r1, sm, buf, cl);
+        const GridLvl GL = grid_level(G, L, 0);
+        const PassGeom P = pass_geom(G.s, G.nx - 1, B.q, L.W > (G.nx - 1) * G.s);
+        grid_pass<S, true, 2>(L, G, GL, P, B, c, d, 0.f, slots, sm, buf, cl);
         FieldCtl &k = sm.fctl;
         if (tid == 0) {
             memset(&k, 0, sizeof(k));
             k.P = (double)L.W * L.H;
             k.invP = 1.0 / k.P;
-            k.Nc = Nc;
-            k.invNc = 1.0 / k.Nc;
             k.sr = sm.tot[3]; k.srr = sm.tot[4];
             const double E = field_energy(k, p.cfg, sm.tot, false);
             if (first) out[0] = E;
@@ -2000,12 +1867,14 @@ __global__ void __launch_bounds__(kThreads) energy_kernel(Params p, const double
         }
         __syncthreads();
         if (grad_c) {
-            float pm[5];
-            for (int q = 0; q < 5; ++q) pm[q] = sm.pm[q];
-            grid_grad_pass<S, false>(L, G, GL, c, d, mt, gp, pm, cr0, cr1, sm, cl, H1Bufs{});
+            float pm[4];
+            for (int q = 0; q < 4; ++q) pm[q] = sm.pm[q];
+            grid_direction(G, L, P, B, c, d, mt, halo, slots, above, pm, sm, buf, cl, H1Bufs{});
             // d = -Nc dE/dc (unit scalar product)
             const float s = -1.f / (float)Nc;
-            for (int j = rank * kThreads + tid; j < Nc; j += C * kThreads) grad_c[j] = make_float2(s * d[j].x, s * d[j].y);
+            const float2 *own = d + (B.cr0 - B.h0) * G.nx;
+            for (int j = tid; j < (B.own1 - B.cr0) * G.nx; j += kThreads)
+                grad_c[B.cr0 * G.nx + j] = make_float2(s * own[j].x, s * own[j].y);
         }
     }
     cl.sync();   // no CTA leaves while a peer may still read its shared memory
@@ -2062,8 +1931,23 @@ __global__ void grid_from_dense_kernel(const float *u, int W, int H, Grid G, flo
 static size_t grid_smem(const Params &p, int cluster)
 {
     if (p.cfg.mode != REG_NONRIGID) return 0;
-    return sizeof(float2) * (size_t)grid_layout(p.gnx, p.gny, cluster, p.cfg.metric == REG_METRIC_H1).crow +
-           sizeof(float4) * (size_t)kWarps * (p.gnx - 1);
+    const bool h1 = p.cfg.metric == REG_METRIC_H1;
+    size_t slots = h1 ? sizeof(float2) * 2 * (size_t)p.gnx * p.gny : 0;
+    for (int l = 0; l < p.cfg.levels; ++l)
+        for (const bool over : {false, true}) {   // the frame's width decides, which is not known here
+            const size_t b = sizeof(float) * slot_floats(pass_geom(p.gs >> l, p.gnx - 1, band_cells(p.gny, cluster), over));
+            if (b > slots) slots = b;
+        }
+    return sizeof(float2) * (size_t)grid_layout(p.gnx, p.gny, cluster, h1).slots + slots;
+}
+
+// The largest grids do not fit the few CTAs of a small cluster: from the size asked for, the first
+// whose control state and slots leave room for the static part.
+int fit_cluster(const Params &p, int cluster)
+{
+    constexpr size_t kMost = 227 * 1024 - sizeof(Smem) - 256;
+    while (cluster < kMaxCluster && grid_smem(p, cluster) > kMost) cluster *= 2;
+    return cluster;
 }
 
 template <typename K>
@@ -2095,32 +1979,26 @@ static cudaError_t launch_cluster(K kernel, int blocks, int cluster, cudaStream_
 
 typedef void (*OpKernelFn)(Params);
 
-// The nonrigid kernel for a storage type, launch form, register form and energy-pass unroll.
+// The nonrigid kernel for a storage type, launch form and energy-pass unroll.
 template <typename S>
-static OpKernelFn nonrigid_fn(bool persistent, bool minb4, int unroll)
+static OpKernelFn nonrigid_fn(bool persistent, int unroll)
 {
-    const bool u2 = unroll == 2;
-    if (persistent) {
-        if (minb4) return u2 ? persistent_kernel<REG_NONRIGID, S, 4, 2> : persistent_kernel<REG_NONRIGID, S, 4, 4>;
-        return u2 ? persistent_kernel<REG_NONRIGID, S, 3, 2> : persistent_kernel<REG_NONRIGID, S, 3, 4>;
-    }
-    if (minb4) return u2 ? op_kernel<REG_NONRIGID, S, 4, 2> : op_kernel<REG_NONRIGID, S, 4, 4>;
-    return u2 ? op_kernel<REG_NONRIGID, S, 3, 2> : op_kernel<REG_NONRIGID, S, 3, 4>;
+    if (persistent) return unroll == 2 ? persistent_kernel<REG_NONRIGID, S, 2, 2> : persistent_kernel<REG_NONRIGID, S, 2, 4>;
+    return unroll == 2 ? op_kernel<REG_NONRIGID, S, 2, 2> : op_kernel<REG_NONRIGID, S, 2, 4>;
 }
 
-static OpKernelFn nonrigid_kernel(int storage, bool persistent, bool minb4, int unroll)
+static OpKernelFn nonrigid_kernel(int storage, bool persistent, int unroll)
 {
     switch (storage) {
-    case REG_F32: return nonrigid_fn<float>(persistent, minb4, unroll);
-    case REG_BF16: return nonrigid_fn<__nv_bfloat16>(persistent, minb4, unroll);
-    case REG_F16: return nonrigid_fn<__half>(persistent, minb4, unroll);
+    case REG_F32: return nonrigid_fn<float>(persistent, unroll);
+    case REG_BF16: return nonrigid_fn<__nv_bfloat16>(persistent, unroll);
+    case REG_F16: return nonrigid_fn<__half>(persistent, unroll);
     }
     return nullptr;
 }
 
 cudaError_t launch_ops(const Params &p, int storage, int cluster, int n_launch_ops, cudaStream_t s)
 {
-    const bool minb4 = p.minb > 0 ? p.minb == 4 : cluster >= 16;   // nonrigid register form
     const int blocks = n_launch_ops * cluster;
     if (p.cfg.mode == kModeMock) return launch_cluster(op_kernel<kModeMock, float, 8>, blocks, cluster, s, p);
     if (p.cfg.mode == REG_RIGID) {
@@ -2130,7 +2008,7 @@ cudaError_t launch_ops(const Params &p, int storage, int cluster, int n_launch_o
         case REG_F16: return launch_cluster(op_kernel<REG_RIGID, __half, 4>, blocks, cluster, s, p);
         }
     } else {
-        OpKernelFn k = nonrigid_kernel(storage, false, minb4, p.unroll);
+        OpKernelFn k = nonrigid_kernel(storage, false, p.unroll);
         if (k) return launch_cluster(k, blocks, cluster, s, p);
     }
     return cudaErrorInvalidValue;
@@ -2138,7 +2016,6 @@ cudaError_t launch_ops(const Params &p, int storage, int cluster, int n_launch_o
 
 cudaError_t launch_persistent(const Params &p, int storage, int cluster, int workers, cudaStream_t s)
 {
-    const bool minb4 = p.minb > 0 ? p.minb == 4 : cluster >= 16;   // nonrigid register form
     const int blocks = workers * cluster;
     if (p.cfg.mode == kModeMock) return launch_cluster(persistent_kernel<kModeMock, float, 8>, blocks, cluster, s, p);
     if (p.cfg.mode == REG_RIGID) {
@@ -2148,7 +2025,7 @@ cudaError_t launch_persistent(const Params &p, int storage, int cluster, int wor
         case REG_F16: return launch_cluster(persistent_kernel<REG_RIGID, __half, 4>, blocks, cluster, s, p);
         }
     } else {
-        OpKernelFn k = nonrigid_kernel(storage, true, minb4, p.unroll);
+        OpKernelFn k = nonrigid_kernel(storage, true, p.unroll);
         if (k) return launch_cluster(k, blocks, cluster, s, p);
     }
     return cudaErrorInvalidValue;
@@ -2180,7 +2057,6 @@ static int resident_clusters(K kernel, int cluster, const Params &p)
 
 int persistent_resident_clusters(const Params &p, int storage, int cluster)
 {
-    const bool minb4 = p.minb > 0 ? p.minb == 4 : cluster >= 16;   // nonrigid register form
     int n = -1;
     if (p.cfg.mode == kModeMock) {
         n = resident_clusters(persistent_kernel<kModeMock, float, 8>, cluster, p);
@@ -2191,7 +2067,7 @@ int persistent_resident_clusters(const Params &p, int storage, int cluster)
         case REG_F16: n = resident_clusters(persistent_kernel<REG_RIGID, __half, 4>, cluster, p); break;
         }
     } else {
-        OpKernelFn k = nonrigid_kernel(storage, true, minb4, p.unroll);
+        OpKernelFn k = nonrigid_kernel(storage, true, p.unroll);
         if (k) n = resident_clusters(k, cluster, p);
     }
     if (n < 0) cudaGetLastError();

@@ -152,7 +152,7 @@ __global__ void __launch_bounds__(32 * kMeanWarps) level_means(Levels<S> L, floa
 
 // Border and B-spline model of every level (grid.y = level, grid.z = frame).  Beyond its border a
 // frame is taken to be its mean: a border of `pad` samples holds it, in storage type.  The model at
-// the pixel centres is the separable filter (1/8, 3/4, 1/8), with the operations of sample_q at a
+// the pixel centres is the separable filter (1/8, 3/4, 1/8), with the operations of bspline2 at a
 // zero offset, so that a frame registered to itself matches bit for bit; it is written as a plain
 // W x H level.  The first nsb blocks of a level make the model: a thread walks kSmoothRows rows down
 // one column and carries the horizontal filter of the rows above and at the current one, so each
@@ -196,14 +196,14 @@ __global__ void __launch_bounds__(kFinishThreads) pyr_finish(Levels<S> L, int pa
         const bool in = r >= 0 && r < H;
         const S *x = p + (ptrdiff_t)min(max(r, 0), H - 1) * pitch;
         const float t0 = in && c > 0 ? ldS<S>(x - 1) : m, t1 = in ? ldS<S>(x) : m, t2 = in && c + 1 < W ? ldS<S>(x + 1) : m;
-        return fmaf(0.125f, t2, fmaf(0.75f, t1, 0.125f * t0));
+        return fmaf(0.125f, t0 + t2, 0.75f * t1);
     };
     float a = hrow(-1), b = hrow(0);
 #pragma unroll
     for (int k = 0; k < kSmoothRows; ++k) {
         if (r0 + k >= H) break;
         const float d = hrow(k + 1);
-        q[(size_t)k * W] = toS<S>(fmaf(0.125f, d, fmaf(0.75f, b, 0.125f * a)));
+        q[(size_t)k * W] = toS<S>(fmaf(0.125f, a + d, 0.75f * b));
         a = b;
         b = d;
     }

@@ -172,7 +172,8 @@ int launch_op(Service *sv, reg_stream *s, int e, const OpDesc &op, cudaEvent_t e
         return REG_ECUDA;
     Params p = stream_params(s);
     p.op_base = e;
-    const int C = host_config(s->ctx).cluster > 0 ? host_config(s->ctx).cluster : (op.left >= 0 ? kClusterB : kClusterA);
+    const int want = host_config(s->ctx).cluster > 0 ? host_config(s->ctx).cluster : (op.left >= 0 ? kClusterB : kClusterA);
+    const int C = fit_cluster(p, want);
     if (launch_ops(p, s->storage, C, 1, ls) != cudaSuccess) return REG_ECUDA;
     if (cudaMemcpyAsync(s->h_theta + 3 * e, s->theta + 3 * e, 3 * sizeof(double), cudaMemcpyDeviceToHost, ls) !=
         cudaSuccess)

@@ -76,3 +76,58 @@ def test_registered_mean_over_any_number_of_frames(N):
                                     [np.array(e[2:], np.float32).astype(np.float64) for e in els])
     assert np.abs(out.cpu().numpy() - want).max() <= 1e-5
     assert np.abs(mean.cpu().numpy() - wmean).max() <= 1e-5
+
+
+@pytest.mark.parametrize("shape", [(65, 129), (100, 97), (33, 160)])
+@pytest.mark.parametrize("grid", [1, 2, 4, 20, 32, 40, 64])
+def test_gradient_for_every_kind_of_cell_width(shape, grid):
+    # strips of many cells, of one cell, of a part of one; widths that divide a warp and that do not; the
+    # column and row past the last cell (129 = 2^7 + 1)
+    H, W = shape
+    if grid <= 2:
+        H, W = 33, 41   # as many points as shared memory holds
+    rng = np.random.default_rng(21)
+    R, T = (rng.uniform(0, 1, size=(H, W)).astype(np.float32) for _ in range(2))
+    g = O.grid_for(W, H, grid)
+    c = rng.uniform(-0.9, 0.9, size=(g.ny, g.nx, 2)).astype(np.float32)
+    gd = torch.zeros((g.ny, g.nx, 2), device="cuda")
+    E = B.Context(B.Config(mode="nonrigid", grid=grid)).energy_grid(
+        torch.from_numpy(R).cuda(), torch.from_numpy(T).cuda(), torch.from_numpy(c).cuda(), gd)
+    Eo, go = O.grid_energy(R, T, 0, g, c.transpose(2, 0, 1).astype(np.float64), 2.0)
+    assert abs(E - Eo) <= 1e-6 * abs(Eo)
+    np.testing.assert_allclose(gd.cpu().numpy().transpose(2, 0, 1), go, atol=2e-4 * np.abs(go).max())
+
+
+@pytest.mark.parametrize("cluster", [1, 2, 4, 8, 16])
+@pytest.mark.parametrize("levels,grid,metric", [(1, 16, 1), (3, 16, 1), (2, 24, 0), (2, 16, 2)])
+def test_pair_for_every_band_split(cluster, levels, grid, metric):
+    # bands of many, one and no cell rows per CTA, cell widths down to 4, each scalar product: three steps
+    # per level take both sides through the same trials, so only rounding separates their end points
+    # (a gradient off by 1e-6 of itself, steps of at most half a pixel: far below 1e-3 px)
+    spec = synth.SeriesSpec(2, 107, 140, step=1.0, field_amp=1.0, snr=(10.0, 10.0), seed=8)
+    F = synth.make_series(spec).frames
+    cfg = B.Config(mode="nonrigid", cluster=cluster, levels=levels, grid=grid, metric=metric, max_iter=3)
+    out = torch.empty((2, 107, 140), device="cuda")
+    _, st = B.Context(cfg).pairwise(F[0].cuda(), F[1].cuda(), field_out=out)
+    oc = O.Config(levels=levels, max_iter=3, max_rejects=cfg.max_rejects, tol_grad=cfg.tol_grad,
+                  tol_rel_e=cfg.tol_rel_e, armijo_c=cfg.armijo_c, tau0=cfg.tau0, step_cap=cfg.step_cap, lam=cfg.lam,
+                  mode="nonrigid", grid=grid, metric=metric, sigma=cfg.sigma, tol_coarse=cfg.tol_coarse)
+    F = F.numpy()
+    c_o, st_o = O.register_nonrigid(O.pyramid(F[0], levels), O.pyramid(F[1], levels), None, oc)
+    assert O.max_px_error(out.cpu().numpy(), c_o, 107, 140, "nonrigid", grid) <= 1e-3
+    assert st["iters"] == list(st_o.iters) and st["evals"] == list(st_o.evals)
+    assert abs(st["energy"] - st_o.energy) <= 1e-6 * abs(st_o.energy)
+
+
+def test_a_grid_too_large_for_one_cta_takes_more():
+    # 65 x 65 points: one CTA cannot hold the control state and its slots; the results are those of a
+    # cluster that can
+    F = synth.make_series(synth.SeriesSpec(2, 513, 513, step=1.0, field_amp=1.0, snr=(10.0, 10.0), seed=9),
+                          device="cuda").frames
+    outs = []
+    for cluster in (1, 16):
+        ctx = B.Context(B.Config(mode="nonrigid", grid=8, cluster=cluster, max_iter=2))
+        outs.append(torch.empty((2, 513, 513), device="cuda"))
+        ctx.pairwise(F[0], F[1], field_out=outs[-1])
+        assert ctx.last_timing()["cluster"] >= cluster
+    assert float((outs[0] - outs[1]).abs().max()) <= 1e-4
