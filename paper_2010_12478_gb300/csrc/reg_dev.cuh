@@ -36,15 +36,6 @@ __device__ __forceinline__ void ff_acc(float &hi, float &lo, float x)
     lo = __fadd_rn(lo, e);
 }
 
-// acc += x*y with the exact rounding error of the product kept in err (the error of a
-// product of two floats is exactly representable: fmaf(x, y, -p)).
-__device__ __forceinline__ void acc_prod(float &acc, float &err, float x, float y)
-{
-    const float p = __fmul_rn(x, y);
-    err += fmaf(x, y, -p);
-    acc = __fadd_rn(acc, p);
-}
-
 // (hi, lo) += (h2, l2), renormalised.
 __device__ __forceinline__ void ff_add(float &hi, float &lo, float h2, float l2)
 {

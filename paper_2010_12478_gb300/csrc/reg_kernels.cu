@@ -33,7 +33,6 @@ namespace reg {
 constexpr int kWarps = kThreads / 32;
 constexpr int kNM = 16;        // sums per reduction at most
 constexpr int kMaxCluster = 16; // CTAs per operator at most (non-portable cluster size)
-constexpr int kChunk = 32;     // pixels per thread between float-float flushes
 
 // ------------------------------------------------------------------ shared state
 // Step-controller state (FP64), used by thread 0 of each CTA only: kept in shared memory so
@@ -43,13 +42,12 @@ struct RigidCtl {
     double E, tau, slope, sr, srr, m0, P, cx, cy, invP, inv_m0;
     double tau_acc;                // length of the last accepted step (along dp)
     double a, b, rbar, tbar;       // NCC terms at th
-    double ta, tb, trbar, ttbar;   // at the trial point tt
     int nrej, iters, evals, stop, rejects, have_prev;
     double tolg;   // the level's stop tolerance (tol_grad, times tol_coarse above the finest level)
 };
 
 struct FieldCtl {
-    double E, tau, tau_acc, slope, P, Nc, sr, srr, invP, invNc;
+    double E, tau, tau_acc, slope, P, Nc, sr, srr, stt, invP, invNc;
     double a, b, rbar, tbar;      // NCC terms at the current field
     double ta, tb, trbar, ttbar;  // at the trial field
     int degen, tdegen;
@@ -156,6 +154,7 @@ __device__ __forceinline__ void cluster_reduce(const float (&hi)[NM], const floa
 // ------------------------------------------------------------------ NCC (FP64)
 struct Ncc {
     double ncc, a, b, rbar, tbar;   // means of the shifted samples
+    double stt;                     // S'_TT
     int degenerate;
 };
 
@@ -176,18 +175,25 @@ __device__ __forceinline__ double rsqrt_nr(double q)
     return y;
 }
 
-// NCC and its gradient coefficients from the shifted sums (invP = 1/P, formed once per level).
-// Explicit round-to-nearest operations keep the result independent of FMA contraction; when
-// S'_rt == S'_rr == S'_tt (T o phi equals R up to the shift: identical inputs) the result is
-// exactly NCC = 1 with a == b, so the gradient vanishes exactly.
-__device__ Ncc ncc_terms(double P, double invP, double sr, double st, double srr, double stt, double srt)
+// NCC and its gradient coefficients from the shifted sums (invP = 1/P, formed once per level) of r and
+// of the difference e = t - r: sum r, sum e, sum r^2, sum e^2, sum r e.  With S'_TT = S'_RR + 2 S'_RE
+// + S'_EE and S'_RT = S'_RR + S'_RE the rounding of the FP32 sums enters 1 - NCC, about (S'_EE - S'_RE^2
+// / S'_RR) / (2 S'_RR), relative to its own size; sums of t^2 and r t enter it relative to 1, which
+// left 1.8e-8 in an energy of 1e-3 (a noiseless lattice, every run of pixels rounded alike).
+// Explicit round-to-nearest operations keep the result independent of FMA contraction; e = 0 everywhere
+// (T o phi equals R up to the shift: identical inputs) is exactly NCC = 1 with a == b, so the gradient
+// vanishes exactly.
+__device__ Ncc ncc_terms(double P, double invP, double sr, double se, double srr, double see, double sre)
 {
     Ncc o;
     const double Srr = __dsub_rn(srr, __dmul_rn(__dmul_rn(sr, sr), invP));
-    const double Stt = __dsub_rn(stt, __dmul_rn(__dmul_rn(st, st), invP));
-    const double Srt = __dsub_rn(srt, __dmul_rn(__dmul_rn(sr, st), invP));
+    const double See = __dsub_rn(see, __dmul_rn(__dmul_rn(se, se), invP));
+    const double Sre = __dsub_rn(sre, __dmul_rn(__dmul_rn(sr, se), invP));
+    const double Srt = __dadd_rn(Srr, Sre);
+    const double Stt = __dadd_rn(Srt, __dadd_rn(Sre, See));
+    o.stt = Stt;
     o.rbar = __dmul_rn(sr, invP);
-    o.tbar = __dmul_rn(st, invP);
+    o.tbar = __dmul_rn(__dadd_rn(sr, se), invP);
     if (Srr < 1e-12 * P || Stt < 1e-12 * P) {
         o.ncc = 0.0; o.a = 0.0; o.b = 0.0; o.degenerate = 1;
         return o;
@@ -220,37 +226,6 @@ __device__ __forceinline__ void strip_rows(int H, int rank, int C, int &r0, int 
 }
 
 constexpr int kFast = 8;   // pixels of a thread in one FP32 run before the float-float fold
-// Row-major traversal for the fused evaluation passes: warp w walks rows r0 + w, r0 + w + kWarps,
-// ...; in a row, lane l takes columns l + 32 u (u < U) per step, so each thread has U independent
-// samples in flight and a warp's loads stay coalesced.  row(r) runs once per row; px(r, c) per
-// pixel; flush_fast() after every kFast pixels of a thread, flush() after every kChunk (and at
-// the end).  U must divide kFast.
-template <int U, typename RowF, typename PixF, typename Q, typename G>
-__device__ __forceinline__ void for_rows(int W, int r0, int r1, RowF &&row, PixF &&px, Q &&flush_fast, G &&flush)
-{
-    static_assert(kFast % U == 0, "U must divide kFast");
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    int cnt = 0;
-    for (int r = r0 + warp; r < r1; r += kWarps) {
-        row(r);
-        for (int c0 = lane; c0 < W; c0 += 32 * U) {
-            if (c0 + 32 * (U - 1) < W) {
-#pragma unroll
-                for (int u = 0; u < U; ++u) px(r, c0 + 32 * u);
-            } else {
-#pragma unroll
-                for (int u = 0; u < U; ++u)
-                    if (c0 + 32 * u < W) px(r, c0 + 32 * u);
-            }
-            cnt += U;
-            if ((cnt & (kFast - 1)) == 0) flush_fast();
-            if ((cnt & (kChunk - 1)) == 0) flush();
-        }
-    }
-    flush_fast();
-    flush();
-}
-
 // Bilinear sample of T (storage S, pitch Tp) at p = (xi + vx, yi + vy) with clamp-to-edge,
 // where (xi, yi) is an integer pixel and (vx, vy) a small FP32 offset.  Splitting the
 // position keeps the FP32 fractional part exact to the precision of the offset, not
@@ -283,120 +258,184 @@ __device__ __forceinline__ float sample_at(const S *T, int W, int H, int Tp, int
     return fmaf(fy, bot, gy * top);
 }
 
+// x rounded to the nearest integer by adding and subtracting 1.5 2^23: the sum's low bits are the
+// integer (kRoundBits + n), with no conversion instruction.  Beyond 2^22 the bits are no longer the
+// integer, but they are far above or below every pixel, and so is the position.
+constexpr float kRound = 12582912.f;
+constexpr unsigned kRoundBits = 0x4B400000u;
+
 // ================================================================== rigid
-// Energy pass moment slots: 0 St, 1 Stt, 2 Srt (t = T(phi(x)) - cR, r = R(x) - cR), and with
-// RSTAT (first pass of a level) 3 Sr, 4 Srr.
-template <typename S, bool RSTAT>
-__device__ void eval_rigid_energy(const Lvl &L, int r0, int r1, const float *pm, Smem &sm, int &buf,
-                                  const cg::cluster_group &cl)
+// One pass over a level's rows [r0, r1) at (cos(alpha) - 1, sin(alpha), translation) gives the moments
+// of the energy and the sums the gradient follows from: with the shifted samples t = T(phi(x)) - cR,
+// r = R(x) - cR, F = P dE/dTw = aP (t - r) + (b - a) P t + kappa as in the nonrigid pass, and g_k =
+// grad T(phi(x)) . dphi/dtheta_k, k = alpha, Gx, Gy.  Sums in sm.tot, e = t - r: 0 sum e, 1 sum e^2,
+// 2 sum r e, with START (a level's first pass) 3 sum r, 4 sum r^2; 5 + k sum e g_k; 8 + k sum t g_k;
+// 11 + k sum g_k.
+//
+// Two columns a lane in packed steps, as in the nonrigid pass: a warp's task is 64 columns over a
+// segment of rows, and in a straight run (the cell of every column's sample moves down by one row per
+// row) a row loads one tap row and keeps the other.  In a run a column beyond the left or right edge
+// keeps its clamped cell; runs that reach the top or bottom edge go row by row through sample_at.
+constexpr int kRigidSums = 14, kRigidRows = 4;   // rows whose loads are in flight together
+template <typename S, bool START>
+__device__ void rigid_pass(const Lvl &L, int r0, int r1, const float *pm, Smem &sm, int &buf,
+                           const cg::cluster_group &cl)
 {
-    constexpr int NM = RSTAT ? 5 : 3;
+    constexpr int NS = START ? 5 : 3;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     // pm: cos(alpha) - 1, sin(alpha), fractional translation (x, y), integer translation (x, y)
-    const float cm1 = pm[0], sa = pm[1], gfx = pm[2], gfy = pm[3];
+    const float cm1 = pm[0], sa = pm[1], gfx = pm[2], gfy = pm[3], ca = 1.f + cm1;
     const int gix = (int)pm[4], giy = (int)pm[5];
     const float cx = 0.5f * (float)(L.W - 1), cy = 0.5f * (float)(L.H - 1);
     const S *R = (const S *)L.R, *T = (const S *)L.T;
-    float hi[NM], lo[NM], a[NM];
-    float e1 = 0.f, e2 = 0.f, e4 = 0.f;   // exact product rounding errors of slots 1, 2, 4
+    const float2 ncR = f2(-L.cR), one = f2(1.f);
+    float2 mh[NS], ml[NS], m[NS];   // moments: float-float sums and the current run, per column
+    float gh[9], gl[9];             // gradient sums: float-float, and the current run
+    float2 g[9];
 #pragma unroll
-    for (int m = 0; m < NM; ++m) { hi[m] = 0.f; lo[m] = 0.f; a[m] = 0.f; }
-    // per-row terms of phi(x) - x - integer translation (small, so FP32 keeps ~1e-7 relative)
-    float bx = 0.f, by = 0.f;
-    const S *Rrow = R;
-    int yi = 0;
-    for_rows<4>(
-        L.W, r0, r1,
-        [&](int r) {
-            const float yc = (float)r - cy;
-            bx = fmaf(-sa, yc, gfx);
-            by = fmaf(cm1, yc, gfy);
-            Rrow = R + (size_t)r * L.Rp;
-            yi = r + giy;
-        },
-        [&](int r, int c) {
-            (void)r;
-            const float xc = (float)c - cx;
-            float dtx, dty;
-            const float tw = sample_at<S, false>(T, L.W, L.H, L.Tp, c + gix, yi, fmaf(cm1, xc, bx),
-                                                 fmaf(sa, xc, by), dtx, dty);
-            const float rv = ldS<S>(Rrow + c) - L.cR;
-            const float tv = tw - L.cR;
-            a[0] += tv;
-            acc_prod(a[1], e1, tv, tv);
-            acc_prod(a[2], e2, rv, tv);
-            if constexpr (RSTAT) {
-                a[3] += rv;
-                acc_prod(a[4], e4, rv, rv);
+    for (int i = 0; i < NS; ++i) mh[i] = ml[i] = m[i] = f2(0.f);
+#pragma unroll
+    for (int i = 0; i < 9; ++i) { gh[i] = gl[i] = 0.f; g[i] = f2(0.f); }
+    // rows split so that the warps' tasks even out: the least rounds x (rows + the window's first row)
+    const int strips = (L.W + 63) / 64, rows = r1 - r0;
+    int nseg = 1, least = 0x7fffffff;
+    for (int k = 1; k <= 8; k *= 2) {
+        const int cost = (strips * k + kWarps - 1) / kWarps * ((rows + k - 1) / k + 2);
+        if (cost < least) { least = cost; nseg = k; }
+    }
+    const int per = (rows + nseg - 1) / nseg;
+    for (int task = warp; task < strips * nseg; task += kWarps) {
+        const int seg = task / strips, x0 = 64 * (task - seg * strips);
+        int y = r0 + seg * per;
+        const int ye = min(r1, y + per);
+        const bool acta = x0 + lane < L.W, actb = x0 + 32 + lane < L.W;
+        const int xa = acta ? x0 + lane : x0, xb = actb ? x0 + 32 + lane : x0;   // an idle column counts for nothing
+        const float2 xc = make_float2((float)xa - cx, (float)xb - cx);
+        auto flush = [&]() {
+#pragma unroll
+            for (int i = 0; i < NS; ++i) {
+                ff_acc2(mh[i], ml[i], make_float2(acta ? m[i].x : 0.f, actb ? m[i].y : 0.f));
+                m[i] = f2(0.f);
             }
-        },
-        [&]() {
-            // short FP32 runs plus the exact product errors keep 1 - NCC accurate to ~1e-9
 #pragma unroll
-            for (int m = 0; m < NM; ++m) { ff_acc(hi[m], lo[m], a[m]); a[m] = 0.f; }
-            lo[1] += e1; lo[2] += e2;
-            e1 = 0.f; e2 = 0.f;
-            if constexpr (RSTAT) { lo[4] += e4; e4 = 0.f; }
-        },
-        []() {});
-    cluster_reduce<NM, false>(hi, lo, 0.f, sm, buf, cl);
+            for (int i = 0; i < 9; ++i) {
+                ff_acc(gh[i], gl[i], (acta ? g[i].x : 0.f) + (actb ? g[i].y : 0.f));
+                g[i] = f2(0.f);
+            }
+        };
+        // displacement without the integer translation at row y (small, so FP32 keeps ~1e-7 relative)
+        auto shift = [&](int row, float2 &vx, float2 &vy, float &yc) {
+            yc = (float)row - cy;
+            vx = __ffma2_rn(f2(cm1), xc, f2(fmaf(-sa, yc, gfx)));
+            vy = __ffma2_rn(f2(sa), xc, f2(fmaf(cm1, yc, gfy)));
+        };
+        auto pixel = [&](float2 tw, float2 dx, float2 dy, float2 rv, float yc) {
+            const float2 t = __fadd2_rn(tw, ncR), r = __fadd2_rn(rv, ncR), F = f2sub(t, r);
+            m[0] = __fadd2_rn(m[0], F);
+            m[1] = __ffma2_rn(F, F, m[1]);
+            m[2] = __ffma2_rn(r, F, m[2]);
+            if constexpr (START) {
+                m[3] = __fadd2_rn(m[3], r);
+                m[4] = __ffma2_rn(r, r, m[4]);
+            }
+            // dphi/dalpha = Rot'(alpha) (x - c) = (-sa xc - ca yc, ca xc - sa yc)
+            const float2 px = __ffma2_rn(f2(-sa), xc, f2(-ca * yc)), py = __ffma2_rn(f2(ca), xc, f2(-sa * yc));
+            const float2 q[3] = {__ffma2_rn(dy, py, __fmul2_rn(dx, px)), dx, dy};
+#pragma unroll
+            for (int i = 0; i < 3; ++i) {
+                g[i] = __ffma2_rn(F, q[i], g[i]);
+                g[3 + i] = __ffma2_rn(t, q[i], g[3 + i]);
+                g[6 + i] = __fadd2_rn(g[6 + i], q[i]);
+            }
+        };
+        while (y < ye) {
+            float2 v0x, v0y, v1x, v1y;
+            float yc;
+            const int n = min(ye - y, kFast);
+            shift(y, v0x, v0y, yc);
+            shift(y + n - 1, v1x, v1y, yc);
+            const float2 m0x = f2add_down(v0x, f2(kRound)), m0y = f2add_down(v0y, f2(kRound));
+            const float2 m1x = f2add_down(v1x, f2(kRound)), m1y = f2add_down(v1y, f2(kRound));
+            const unsigned diff = (__float_as_uint(m0x.x) ^ __float_as_uint(m1x.x)) | (__float_as_uint(m0x.y) ^ __float_as_uint(m1x.y)) |
+                                  (__float_as_uint(m0y.x) ^ __float_as_uint(m1y.x)) | (__float_as_uint(m0y.y) ^ __float_as_uint(m1y.y));
+            // the cells of the first row; |displacement| < 2^22, as the rounding needs
+            const int ua = xa + gix + (int)(__float_as_uint(m0x.x) - kRoundBits), ub = xb + gix + (int)(__float_as_uint(m0x.y) - kRoundBits);
+            const int wa = y + giy + (int)(__float_as_uint(m0y.x) - kRoundBits), wb = y + giy + (int)(__float_as_uint(m0y.y) - kRoundBits);
+            const bool near = fabsf(v0x.x) < 4.0e6f && fabsf(v0x.y) < 4.0e6f && fabsf(v0y.x) < 4.0e6f && fabsf(v0y.y) < 4.0e6f;
+            const bool ok = diff == 0u && near && wa >= 0 && wa + n <= L.H - 1 && wb >= 0 && wb + n <= L.H - 1;
+            const S *pa = R + (ptrdiff_t)y * L.Rp + xa, *pb = R + (ptrdiff_t)y * L.Rp + xb;
+            if (__all_sync(0xffffffffu, ok)) {
+                const bool edge = __any_sync(0xffffffffu, (unsigned)ua > (unsigned)(L.W - 2) || (unsigned)ub > (unsigned)(L.W - 2));
+                const S *qa = T + (ptrdiff_t)wa * L.Tp + min(max(ua, 0), L.W - 2), *qb = T + (ptrdiff_t)wb * L.Tp + min(max(ub, 0), L.W - 2);
+                const float2 nx = f2sub(m0x, f2(kRound)), ny = f2sub(m0y, f2(kRound));
+                // a tap row's sample and difference; beyond the right edge the last sample, at weight 0
+                const bool ra = ua > L.W - 2, rb = ub > L.W - 2;
+                auto tap = [&](float2 l, float2 r, float2 &t, float2 &d) {
+                    d = f2sub(r, l);
+                    t = edge ? make_float2(ra ? r.x : l.x, rb ? r.y : l.y) : l;
+                };
+                float2 t0, d0;
+                tap(make_float2(ldS<S>(qa), ldS<S>(qb)), make_float2(ldS<S>(qa + 1), ldS<S>(qb + 1)), t0, d0);
+                for (int k = 0; k < n; k += kRigidRows) {
+                    float2 q[kRigidRows][2], r[kRigidRows];
+#pragma unroll
+                    for (int i = 0; i < kRigidRows; ++i) {
+                        if (k + i < n) { qa += L.Tp; qb += L.Tp; }   // the last rows of a short run repeat
+                        q[i][0] = make_float2(ldS<S>(qa), ldS<S>(qb));
+                        q[i][1] = make_float2(ldS<S>(qa + 1), ldS<S>(qb + 1));
+                        r[i] = make_float2(ldS<S>(pa), ldS<S>(pb));
+                        if (k + i + 1 < n) { pa += L.Rp; pb += L.Rp; }
+                    }
+#pragma unroll
+                    for (int i = 0; i < kRigidRows; ++i) {
+                        if (k + i >= n) break;
+                        float2 vx, vy;
+                        shift(y + k + i, vx, vy, yc);
+                        float2 fx = f2sub(vx, nx), on = one;
+                        const float2 fy = f2sub(vy, ny);
+                        if (edge) {
+                            // beyond an edge: its sample, and no derivative along x (on the last column
+                            // itself, fx = 0, the cell's own)
+                            on = make_float2(ua < 0 || ua > L.W - 1 || (ua == L.W - 1 && fx.x > 0.f) ? 0.f : 1.f,
+                                             ub < 0 || ub > L.W - 1 || (ub == L.W - 1 && fx.y > 0.f) ? 0.f : 1.f);
+                            fx = make_float2(ua < 0 || ra ? 0.f : fx.x, ub < 0 || rb ? 0.f : fx.y);
+                        }
+                        float2 t1, d1;
+                        tap(q[i][0], q[i][1], t1, d1);
+                        const float2 top = __ffma2_rn(fx, d0, t0), dy = f2sub(__ffma2_rn(fx, d1, t1), top);
+                        const float2 dx = __fmul2_rn(on, __ffma2_rn(fy, f2sub(d1, d0), d0));
+                        pixel(__ffma2_rn(fy, dy, top), dx, dy, r[i], yc);
+                        t0 = t1;
+                        d0 = d1;
+                    }
+                }
+            } else {
+                for (int k = 0; k < n; ++k) {
+                    float2 vx, vy, dx, dy, tw;
+                    shift(y + k, vx, vy, yc);
+                    tw.x = sample_at<S, true>(T, L.W, L.H, L.Tp, xa + gix, y + k + giy, vx.x, vy.x, dx.x, dy.x);
+                    tw.y = sample_at<S, true>(T, L.W, L.H, L.Tp, xb + gix, y + k + giy, vx.y, vy.y, dx.y, dy.y);
+                    pixel(tw, dx, dy, make_float2(ldS<S>(pa), ldS<S>(pb)), yc);
+                    pa += L.Rp; pb += L.Rp;
+                }
+            }
+            flush();
+            y += n;
+        }
+    }
+    float hi[kRigidSums], lo[kRigidSums];
+#pragma unroll
+    for (int i = 0; i < 5; ++i) {
+        hi[i] = i < NS ? mh[i].x : 0.f;
+        lo[i] = i < NS ? ml[i].x : 0.f;
+        if (i < NS) ff_add(hi[i], lo[i], mh[i].y, ml[i].y);
+    }
+#pragma unroll
+    for (int i = 0; i < 9; ++i) { hi[5 + i] = gh[i]; lo[5 + i] = gl[i]; }
+    cluster_reduce<kRigidSums, false>(hi, lo, 0.f, sm, buf, cl);
 }
 
-// Gradient pass at a point whose NCC terms are known (from the energy pass or the accepted
-// trial at the same point): slots k = 0..2 sum F(x) g_k(x), F = P dE/dTw =
-// -(aP (r - rbar) - bP (t - tbar)), g_k = grad T(phi(x)) . dphi/dtheta_k.
-// pm[6..9] = aP, bP, rbar, tbar (rbar, tbar: means of the shifted samples).
-template <typename S>
-__device__ void eval_rigid_grad(const Lvl &L, int r0, int r1, const float *pm, Smem &sm, int &buf,
-                                const cg::cluster_group &cl)
-{
-    constexpr int NM = 3;
-    const float cm1 = pm[0], sa = pm[1], gfx = pm[2], gfy = pm[3];
-    const int gix = (int)pm[4], giy = (int)pm[5];
-    const float aP = pm[6], bP = pm[7], rb = pm[8], tb = pm[9];
-    const float ca = 1.f + cm1;
-    const float cx = 0.5f * (float)(L.W - 1), cy = 0.5f * (float)(L.H - 1);
-    const S *R = (const S *)L.R, *T = (const S *)L.T;
-    float hi[NM], lo[NM], a[NM];
-#pragma unroll
-    for (int m = 0; m < NM; ++m) { hi[m] = 0.f; lo[m] = 0.f; a[m] = 0.f; }
-    float bx = 0.f, by = 0.f, gax = 0.f, gay = 0.f;
-    const S *Rrow = R;
-    int yi = 0;
-    for_rows<4>(
-        L.W, r0, r1,
-        [&](int r) {
-            const float yc = (float)r - cy;
-            bx = fmaf(-sa, yc, gfx);
-            by = fmaf(cm1, yc, gfy);
-            gax = -sa * yc;   // terms in yc of dphi/dalpha = Rot'(alpha) (x - c)
-            gay = ca * yc;
-            Rrow = R + (size_t)r * L.Rp;
-            yi = r + giy;
-        },
-        [&](int r, int c) {
-            (void)r;
-            const float xc = (float)c - cx;
-            float dtx, dty;
-            const float tw = sample_at<S, true>(T, L.W, L.H, L.Tp, c + gix, yi, fmaf(cm1, xc, bx),
-                                                fmaf(sa, xc, by), dtx, dty);
-            const float rv = ldS<S>(Rrow + c) - L.cR;
-            const float tv = tw - L.cR;
-            // no contraction: identical r and t give F == 0 exactly
-            const float F = -__fsub_rn(__fmul_rn(aP, rv - rb), __fmul_rn(bP, tv - tb));
-            const float g0 = fmaf(dty, fmaf(ca, xc, gax), -dtx * fmaf(sa, xc, gay));
-            a[0] = fmaf(F, g0, a[0]);
-            a[1] = fmaf(F, dtx, a[1]);
-            a[2] = fmaf(F, dty, a[2]);
-        },
-        []() {},
-        [&]() {
-#pragma unroll
-            for (int m = 0; m < NM; ++m) { ff_acc(hi[m], lo[m], a[m]); a[m] = 0.f; }
-        });
-    cluster_reduce<NM, false>(hi, lo, 0.f, sm, buf, cl);
-}
-
-enum Action { kActGrad = 0, kActTrial = 1, kActDone = 2, kActEnergy = 3 };
+enum Action { kActGrad = 0, kActTrial = 1, kActDone = 2 };
 
 
 __device__ void rigid_params(const double *th, float *pm)
@@ -413,15 +452,6 @@ __device__ void rigid_params(const double *th, float *pm)
     pm[5] = (float)fmax(-4.0e6, fmin(4.0e6, iy));
 }
 
-__device__ void rigid_grad_params(const RigidCtl &k, float *pm)
-{
-    rigid_params(k.th, pm);
-    pm[6] = (float)(k.a * k.P);
-    pm[7] = (float)(k.b * k.P);
-    pm[8] = (float)k.rbar;
-    pm[9] = (float)k.tbar;
-}
-
 // Step-size rule of the line search: Armijo backtracking with safeguarded quadratic
 // interpolation (Nocedal and Wright, Numerical Optimization, Sec. 3.5).  tq minimises the
 // parabola through E(0) = E, E'(0) = slope and E(tau) = Et; a rejected trial retries at tq
@@ -436,65 +466,66 @@ __device__ __forceinline__ double next_tau(double E, double slope, double tau, d
     return accepted ? fmin(fmax(tq, 0.5 * tau), 4.0 * tau) : fmin(fmax(tq, 0.1 * tau), 0.5 * tau);
 }
 
-// Thread-0 controller after an ENERGY (level start), GRAD or TRIAL pass.  Returns the next
-// action and writes its parameters.  Same rules as the oracle's level loop.
-__device__ int rigid_step(RigidCtl &k, const Config &cfg, const double *tot, int action, float *pm)
+// Gradient at the point of a pass from its sums and the point's NCC terms: dE/dtheta_k = a sum (t - r)
+// g_k + (b - a) sum t g_k + (a rbar - b tbar) sum g_k; a == b and rbar == tbar give exact zeros.
+__device__ void rigid_gradient(const RigidCtl &k, const double *tot, double *g)
 {
-    if (action == kActEnergy) {
+    const double bma = __dsub_rn(k.b, k.a), kap = __dsub_rn(__dmul_rn(k.a, k.rbar), __dmul_rn(k.b, k.tbar));
+    for (int q = 0; q < 3; ++q) g[q] = k.a * tot[5 + q] + bma * tot[8 + q] + kap * tot[11 + q];
+}
+
+// Thread-0 controller after a pass at a level's start or at a trial point: the energy there, the Armijo
+// test, and where the point is taken the stop tests, the direction and the next trial.  Returns the
+// next action and writes its parameters.  Same rules as the oracle's level loop.
+__device__ int rigid_step(RigidCtl &k, const Config &cfg, const double *tot, bool start, float *pm)
+{
+    if (start) {
         k.sr = tot[3];
         k.srr = tot[4];
-        const Ncc n = ncc_terms(k.P, k.invP, k.sr, tot[0], k.srr, tot[1], tot[2]);
-        k.E = n.degenerate ? 1.0 : __dsub_rn(1.0, n.ncc);
-        k.a = n.a; k.b = n.b; k.rbar = n.rbar; k.tbar = n.tbar;
-        rigid_grad_params(k, pm);
-        return kActGrad;
     }
-    if (action == kActGrad) {
-        double g[3];
-        for (int q = 0; q < 3; ++q) g[q] = tot[q] * k.invP;
-        k.evals += 1;
-        if (k.iters >= cfg.max_iter) { k.stop = REG_STOP_MAXIT; return kActDone; }
-        k.d[0] = -g[0] * k.inv_m0; k.d[1] = -g[1]; k.d[2] = -g[2];
-        k.slope = g[0] * k.d[0] + g[1] * k.d[1] + g[2] * k.d[2];
-        // |g|_M = sqrt(-slope); the tests compare squares (no square root unless the cap applies)
-        const double gn2 = -k.slope;
-        if (!(gn2 >= k.tolg * k.tolg)) { k.stop = REG_STOP_GRAD; return kActDone; }
-        if (k.have_prev) {
-            double num = 0.0, den = 0.0;
-            for (int q = 0; q < 3; ++q) {
-                const double w = q == 0 ? k.m0 : 1.0, y = k.dp[q] - k.d[q];
-                num += w * k.dp[q] * y;
-                den += w * y * y;
-            }
-            k.tau = bb_tau(k.tau, k.tau_acc, num, den);
-        }
-        if (k.tau * k.tau * gn2 > cfg.step_cap * cfg.step_cap) k.tau = cfg.step_cap / sqrt(gn2);
-        k.nrej = 0;
-        for (int q = 0; q < 3; ++q) k.tt[q] = k.th[q] + k.tau * k.d[q];
-        rigid_params(k.tt, pm);
-        return kActTrial;
-    }
-    // trial
     const Ncc n = ncc_terms(k.P, k.invP, k.sr, tot[0], k.srr, tot[1], tot[2]);
     const double Et = n.degenerate ? 1.0 : __dsub_rn(1.0, n.ncc);
-    k.evals += 1;
-    if (Et <= k.E + cfg.armijo_c * k.tau * k.slope) {
+    if (!start) {
+        k.evals += 1;
+        if (!(Et <= k.E + cfg.armijo_c * k.tau * k.slope)) {
+            k.rejects += 1;
+            k.nrej += 1;
+            k.tau = next_tau(k.E, k.slope, k.tau, Et, false);
+            if (k.nrej > cfg.max_rejects) { k.stop = REG_STOP_LS; return kActDone; }
+            for (int q = 0; q < 3; ++q) k.tt[q] = k.th[q] + k.tau * k.d[q];
+            rigid_params(k.tt, pm);
+            return kActTrial;
+        }
         for (int q = 0; q < 3; ++q) { k.th[q] = k.tt[q]; k.dp[q] = k.d[q]; }
         k.tau_acc = k.tau;
         k.have_prev = 1;
         k.iters += 1;
-        const double Eold = k.E;
         k.tau = next_tau(k.E, k.slope, k.tau, Et, true);
-        k.E = Et;
-        k.a = n.a; k.b = n.b; k.rbar = n.rbar; k.tbar = n.tbar;
-        if (Eold - Et <= cfg.tol_rel_e * fabs(Eold)) { k.stop = REG_STOP_REL; return kActDone; }
-        rigid_grad_params(k, pm);
-        return kActGrad;
     }
-    k.rejects += 1;
-    k.nrej += 1;
-    k.tau = next_tau(k.E, k.slope, k.tau, Et, false);
-    if (k.nrej > cfg.max_rejects) { k.stop = REG_STOP_LS; return kActDone; }
+    const double Eold = k.E;
+    k.E = Et;
+    k.a = n.a; k.b = n.b; k.rbar = n.rbar; k.tbar = n.tbar;
+    if (!start && Eold - Et <= cfg.tol_rel_e * fabs(Eold)) { k.stop = REG_STOP_REL; return kActDone; }
+    double g[3];
+    rigid_gradient(k, tot, g);
+    k.evals += 1;
+    if (k.iters >= cfg.max_iter) { k.stop = REG_STOP_MAXIT; return kActDone; }
+    k.d[0] = -g[0] * k.inv_m0; k.d[1] = -g[1]; k.d[2] = -g[2];
+    k.slope = g[0] * k.d[0] + g[1] * k.d[1] + g[2] * k.d[2];
+    // |g|_M = sqrt(-slope); the tests compare squares (no square root unless the cap applies)
+    const double gn2 = -k.slope;
+    if (!(gn2 >= k.tolg * k.tolg)) { k.stop = REG_STOP_GRAD; return kActDone; }
+    if (k.have_prev) {
+        double num = 0.0, den = 0.0;
+        for (int q = 0; q < 3; ++q) {
+            const double w = q == 0 ? k.m0 : 1.0, y = k.dp[q] - k.d[q];
+            num += w * k.dp[q] * y;
+            den += w * y * y;
+        }
+        k.tau = bb_tau(k.tau, k.tau_acc, num, den);
+    }
+    if (k.tau * k.tau * gn2 > cfg.step_cap * cfg.step_cap) k.tau = cfg.step_cap / sqrt(gn2);
+    k.nrej = 0;
     for (int q = 0; q < 3; ++q) k.tt[q] = k.th[q] + k.tau * k.d[q];
     rigid_params(k.tt, pm);
     return kActTrial;
@@ -560,19 +591,17 @@ __device__ void run_rigid(const Params &p, const OpDesc &op, int op_index, Smem 
             // a coarse level only supplies the next level's initial guess: a looser stop
             k.tolg = cfg.tol_grad * (l > 0 ? cfg.tol_coarse : 1.0);
             rigid_params(k.th, sm.pm);
-            sm.action = kActEnergy;
+            sm.action = kActTrial;
         }
-        for (;;) {
+        for (bool start = true;; start = false) {
             __syncthreads();
-            const int act = sm.action;
-            if (act == kActDone) break;
-            float pm[10];
+            if (sm.action == kActDone) break;
+            float pm[6];
 #pragma unroll
-            for (int q = 0; q < 10; ++q) pm[q] = sm.pm[q];
-            if (act == kActEnergy) eval_rigid_energy<S, true>(L, r0, r1, pm, sm, buf, cl);
-            else if (act == kActGrad) eval_rigid_grad<S>(L, r0, r1, pm, sm, buf, cl);
-            else eval_rigid_energy<S, false>(L, r0, r1, pm, sm, buf, cl);
-            if (tid == 0) sm.action = rigid_step(k, cfg, sm.tot, act, sm.pm);
+            for (int q = 0; q < 6; ++q) pm[q] = sm.pm[q];
+            if (start) rigid_pass<S, true>(L, r0, r1, pm, sm, buf, cl);
+            else rigid_pass<S, false>(L, r0, r1, pm, sm, buf, cl);
+            if (tid == 0) sm.action = rigid_step(k, cfg, sm.tot, start, sm.pm);
         }
         if (tid == 0) {
             stops[l] = k.stop; iters[l] = k.iters; evals[l] = k.evals;
@@ -850,15 +879,10 @@ __device__ __forceinline__ float2 bspline2(const TapRow &r0, const TapRow &r1, c
     return __ffma2_rn(hy, __ffma2_rn(ty, a.D2, a.D1), a.S);
 }
 
-// x rounded to the nearest integer by adding and subtracting 1.5 2^23: the sum's low bits are the
-// integer (kRoundBits + n), with no conversion instruction.  Beyond 2^22 the bits are no longer the
-// integer, but they are far above or below every pixel, and so is the position.
-constexpr float kRound = 12582912.f;
-constexpr unsigned kRoundBits = 0x4B400000u;
 constexpr int kRunRows = 16;   // rows of a straight run at most; half of it is tried next
 
-// One pass at c (START: a level's first) or at the trial c + tau d: the moments into sm.tot (slots
-// 0 St, 1 Stt, 2 Srt, with START 3 Sr, 4 Srr; 5: sum over control edges of |dct|^2) and the gradient
+// One pass at c (START: a level's first) or at the trial c + tau d: the moments into sm.tot (e =
+// t - r: 0 sum e, 1 sum e^2, 2 sum r e, with START 3 sum r, 4 sum r^2; 5: sum over control edges of |dct|^2) and the gradient
 // sums into the slots.  The trial values are formed where they are read, fmaf(tau, d_j, c_j), the
 // expression an accepted step stores into c.
 //
@@ -939,14 +963,14 @@ __device__ void grid_pass(const Lvl &L, const Grid &G, const GridLvl &GL, const 
         auto pixel = [&](const TapRow &t0, const TapRow &t1, const TapRow &t2, float2 fx, float2 fy, float2 r, float2 wy) {
             float2 dx2, dy2;
             const float2 t = __fadd2_rn(bspline2(t0, t1, t2, fx, fy, dx2, dy2), ncR);
-            a[0] = __fadd2_rn(a[0], t);
-            a[1] = __ffma2_rn(t, t, a[1]);
-            a[2] = __ffma2_rn(r, t, a[2]);
+            const float2 F = f2sub(t, r);
+            a[0] = __fadd2_rn(a[0], F);
+            a[1] = __ffma2_rn(F, F, a[1]);
+            a[2] = __ffma2_rn(r, F, a[2]);
             if constexpr (START) {
                 a[3] = __fadd2_rn(a[3], r);
                 a[4] = __ffma2_rn(r, r, a[4]);
             }
-            const float2 F = f2sub(t, r);
             const float2 wb = __fmul2_rn(f2(0.5f), wy), wt = f2sub(f2(0.5f), wb);   // half of wy and 1 - wy
             const float2 g[4] = {__fmul2_rn(wt, dx2), __fmul2_rn(wt, dy2), __fmul2_rn(wb, dx2), __fmul2_rn(wb, dy2)};
 #pragma unroll
@@ -1362,7 +1386,8 @@ __device__ void grid_direction(const Grid &G, const Lvl &L, const PassGeom &P, c
 
 __device__ double field_energy(FieldCtl &k, const Config &cfg, const double *tot, bool trial)
 {
-    Ncc n = ncc_terms(k.P, k.invP, k.sr, tot[0], k.srr, tot[1], tot[2]);
+    const Ncc n = ncc_terms(k.P, k.invP, k.sr, tot[0], k.srr, tot[1], tot[2]);
+    k.stt = n.stt;
     double Ed = n.degenerate ? 1.0 : __dsub_rn(1.0, n.ncc);
     double E = Ed + 0.5 * cfg.lambda * tot[5] * k.invP;
     if (trial) { k.ta = n.a; k.tb = n.b; k.trbar = n.rbar; k.ttbar = n.tbar; k.tdegen = n.degenerate; }
@@ -1393,7 +1418,7 @@ __device__ int field_eval(FieldCtl &k, const Config &cfg, const double *tot, boo
         k.sr = tot[3]; k.srr = tot[4];
         k.E = field_energy(k, cfg, tot, false);
         // the level's scalar product at its initial control values: 1/(P var T) and lambda/P
-        const double vt = (tot[1] - tot[0] * tot[0] * k.invP) * k.invP;
+        const double vt = k.stt * k.invP;
         pm[kPmDk] = vt > 0.0 ? (float)(k.invP / vt) : 0.f;
         pm[kPmRk] = (float)(cfg.lambda * k.invP);
         field_grad_params(k, cfg, pm);
@@ -1828,16 +1853,15 @@ __global__ void __launch_bounds__(kThreads) energy_kernel(Params p, const double
         __syncthreads();
         int r0, r1;
         strip_rows(L.H, rank, C, r0, r1);
-        float pm[10];
+        float pm[6];
         for (int q = 0; q < 6; ++q) pm[q] = sm.pm[q];
-        eval_rigid_energy<S, true>(L, r0, r1, pm, sm, buf, cl);
-        if (tid == 0) rigid_step(k, p.cfg, sm.tot, kActEnergy, sm.pm);
-        if (first) out[0] = k.E;
-        __syncthreads();
-        for (int q = 0; q < 10; ++q) pm[q] = sm.pm[q];
-        eval_rigid_grad<S>(L, r0, r1, pm, sm, buf, cl);
-        if (first)
-            for (int q = 0; q < 3; ++q) out[1 + q] = sm.tot[q] / k.P;
+        rigid_pass<S, true>(L, r0, r1, pm, sm, buf, cl);
+        if (first) {
+            const Ncc n = ncc_terms(k.P, k.invP, sm.tot[3], sm.tot[0], sm.tot[4], sm.tot[1], sm.tot[2]);
+            k.a = n.a; k.b = n.b; k.rbar = n.rbar; k.tbar = n.tbar;
+            out[0] = n.degenerate ? 1.0 : __dsub_rn(1.0, n.ncc);
+            rigid_gradient(k, sm.tot, out + 1);
+        }
     } else {
         const Grid G{p.gnx, p.gny, p.gs};
         const int Nc = G.nx * G.ny;
@@ -2003,9 +2027,9 @@ cudaError_t launch_ops(const Params &p, int storage, int cluster, int n_launch_o
     if (p.cfg.mode == kModeMock) return launch_cluster(op_kernel<kModeMock, float, 8>, blocks, cluster, s, p);
     if (p.cfg.mode == REG_RIGID) {
         switch (storage) {
-        case REG_F32: return launch_cluster(op_kernel<REG_RIGID, float, 4>, blocks, cluster, s, p);
-        case REG_BF16: return launch_cluster(op_kernel<REG_RIGID, __nv_bfloat16, 4>, blocks, cluster, s, p);
-        case REG_F16: return launch_cluster(op_kernel<REG_RIGID, __half, 4>, blocks, cluster, s, p);
+        case REG_F32: return launch_cluster(op_kernel<REG_RIGID, float, 2>, blocks, cluster, s, p);
+        case REG_BF16: return launch_cluster(op_kernel<REG_RIGID, __nv_bfloat16, 2>, blocks, cluster, s, p);
+        case REG_F16: return launch_cluster(op_kernel<REG_RIGID, __half, 2>, blocks, cluster, s, p);
         }
     } else {
         OpKernelFn k = nonrigid_kernel(storage, false, p.unroll);
@@ -2020,9 +2044,9 @@ cudaError_t launch_persistent(const Params &p, int storage, int cluster, int wor
     if (p.cfg.mode == kModeMock) return launch_cluster(persistent_kernel<kModeMock, float, 8>, blocks, cluster, s, p);
     if (p.cfg.mode == REG_RIGID) {
         switch (storage) {
-        case REG_F32: return launch_cluster(persistent_kernel<REG_RIGID, float, 4>, blocks, cluster, s, p);
-        case REG_BF16: return launch_cluster(persistent_kernel<REG_RIGID, __nv_bfloat16, 4>, blocks, cluster, s, p);
-        case REG_F16: return launch_cluster(persistent_kernel<REG_RIGID, __half, 4>, blocks, cluster, s, p);
+        case REG_F32: return launch_cluster(persistent_kernel<REG_RIGID, float, 2>, blocks, cluster, s, p);
+        case REG_BF16: return launch_cluster(persistent_kernel<REG_RIGID, __nv_bfloat16, 2>, blocks, cluster, s, p);
+        case REG_F16: return launch_cluster(persistent_kernel<REG_RIGID, __half, 2>, blocks, cluster, s, p);
         }
     } else {
         OpKernelFn k = nonrigid_kernel(storage, true, p.unroll);
@@ -2062,9 +2086,9 @@ int persistent_resident_clusters(const Params &p, int storage, int cluster)
         n = resident_clusters(persistent_kernel<kModeMock, float, 8>, cluster, p);
     } else if (p.cfg.mode == REG_RIGID) {
         switch (storage) {
-        case REG_F32: n = resident_clusters(persistent_kernel<REG_RIGID, float, 4>, cluster, p); break;
-        case REG_BF16: n = resident_clusters(persistent_kernel<REG_RIGID, __nv_bfloat16, 4>, cluster, p); break;
-        case REG_F16: n = resident_clusters(persistent_kernel<REG_RIGID, __half, 4>, cluster, p); break;
+        case REG_F32: n = resident_clusters(persistent_kernel<REG_RIGID, float, 2>, cluster, p); break;
+        case REG_BF16: n = resident_clusters(persistent_kernel<REG_RIGID, __nv_bfloat16, 2>, cluster, p); break;
+        case REG_F16: n = resident_clusters(persistent_kernel<REG_RIGID, __half, 2>, cluster, p); break;
         }
     } else {
         OpKernelFn k = nonrigid_kernel(storage, true, p.unroll);
