@@ -35,34 +35,46 @@ constexpr int kNM = 16;        // sums per reduction at most
 constexpr int kMaxCluster = 16; // CTAs per operator at most (non-portable cluster size)
 
 // ------------------------------------------------------------------ shared state
-// Step-controller state (FP64), used by thread 0 of each CTA only: kept in shared memory so
-// it does not occupy registers of every thread.
+// Step-controller state (FP64), used by thread 0 (rigid: warp 0) of each CTA only: kept in shared
+// memory so it does not occupy registers of every thread.
+struct LevelSums {
+    double P, invP, sr, Srr;       // pixels; sum of the reference's shifted samples; S'_RR
+};
+
 struct RigidCtl {
+    LevelSums ls;
     double th[3], tt[3], d[3], dp[3];   // dp: the direction of the last accepted step
-    double E, tau, slope, sr, srr, m0, P, cx, cy, invP, inv_m0;
+    double E, tau, slope, m0, inv_m0;
     double tau_acc;                // length of the last accepted step (along dp)
-    double a, b, rbar, tbar;       // NCC terms at th
     int nrej, iters, evals, stop, rejects, have_prev;
-    double tolg;   // the level's stop tolerance (tol_grad, times tol_coarse above the finest level)
+    double tolg2;  // the level's stop tolerance (tol_grad, times tol_coarse above the finest level), squared
 };
 
 struct FieldCtl {
-    double E, tau, tau_acc, slope, P, Nc, sr, srr, stt, invP, invNc;
-    double a, b, rbar, tbar;      // NCC terms at the current field
-    double ta, tb, trbar, ttbar;  // at the trial field
-    int degen, tdegen;
+    LevelSums ls;
+    double E, tau, tau_acc, slope, invNc, half_lam;   // half_lam: lambda / (2 P)
+    double Eold, slope_old, tau_old;   // of the last accepted step, for its quadratic rule
     int nrej, iters, evals, stop, rejects, have_prev;
-    double tolg;   // the level's stop tolerance (tol_grad, times tol_coarse above the finest level)
+    double tolg2;  // the level's stop tolerance (tol_grad, times tol_coarse above the finest level), squared
 };
+
+// x >= 0, false for a NaN, from the bits: a double-precision compare takes 105 cycles on this GPU, a
+// double-precision operation 64 (an FP32 one 4), so the controller's chains are kept short in both.
+__device__ __forceinline__ bool nonneg(double x)
+{
+    return (unsigned)__double2hiint(x) <= 0x7ff00000u;
+}
 
 // First trial of a line search after an accepted step (Barzilai and Borwein, "Two-point step size
 // gradient methods", 1988, their second step): tau = tau_acc <d_prev, d_prev - d> / |d_prev - d|^2
-// in the flow's metric, given num = <d_prev, d_prev - d> and den = |d_prev - d|^2; without positive
-// curvature the quadratic rule's tau_q stays.  The ratio needs no more than FP32 relative precision.
-__device__ __forceinline__ double bb_tau(double tau_q, double tau_acc, double num, double den)
+// in the flow's metric, given num = <d_prev, d_prev - d> and den = |d_prev - d|^2; false without
+// positive curvature.  The ratio needs no more than FP32 relative precision.
+__device__ __forceinline__ bool bb_tau(double tau_acc, double num, double den, double &tau)
 {
-    if (!(num > 0.0 && den > 0.0)) return tau_q;
-    return tau_acc * num * (double)__frcp_rn((float)den);
+    const float nf = (float)num, df = (float)den;
+    if (!(nf > 0.f && df > 0.f)) return false;
+    tau = tau_acc * num * (double)__frcp_rn(df);
+    return true;
 }
 
 struct Smem {
@@ -153,62 +165,61 @@ __device__ __forceinline__ void cluster_reduce(const float (&hi)[NM], const floa
 
 // ------------------------------------------------------------------ NCC (FP64)
 struct Ncc {
-    double ncc, a, b, rbar, tbar;   // means of the shifted samples
-    double stt;                     // S'_TT
-    int degenerate;
+    double e;                  // 1 - NCC
+    double a, bma;             // dNCC/dTw(x) = a (r - rbar) - b (t - tbar): a and b - a
+    double tbar, dbar;         // mean of t, and tbar - rbar
+    double Stt;
+    bool degenerate;
 };
 
-// NCC = S'_RT / sqrt(S'_RR S'_TT) from shifted sums; dNCC/dTw(x) = a (r - rbar) - b (t - tbar).
-// 1/sqrt(q) for a positive normal q without a double-precision divide or square root (both
-// are long dependent instruction sequences on this GPU's narrow FP64 unit): the hardware
-// reciprocal-square-root approximation, then two Newton-Raphson steps y <- y (3 - q y^2) / 2,
-// each squaring the relative error (about 1e-7 -> 1e-14 -> double rounding).
-__device__ __forceinline__ double rsqrt_nr(double q)
+// 1/sqrt(q) for a positive normal q without a double-precision divide or square root: the hardware
+// reciprocal-square-root approximation y (about 20 bits) and one third-order step, with h = 1 - q y^2
+// y (1 + h/2 + 3/8 h^2), whose error is 5/16 h^3.
+__device__ __forceinline__ double rsqrt_f64(double q)
 {
     double y;
     asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(q));
-#pragma unroll
-    for (int it = 0; it < 2; ++it) {
-        const double t = __dmul_rn(q, __dmul_rn(y, y));
-        y = __dmul_rn(y, __fma_rn(-0.5, t, 1.5));
-    }
-    return y;
+    const double h = __fma_rn(-q, __dmul_rn(y, y), 1.0);
+    return __fma_rn(y, __dmul_rn(h, __fma_rn(0.375, h, 0.5)), y);
 }
 
-// NCC and its gradient coefficients from the shifted sums (invP = 1/P, formed once per level) of r and
-// of the difference e = t - r: sum r, sum e, sum r^2, sum e^2, sum r e.  With S'_TT = S'_RR + 2 S'_RE
-// + S'_EE and S'_RT = S'_RR + S'_RE the rounding of the FP32 sums enters 1 - NCC, about (S'_EE - S'_RE^2
-// / S'_RR) / (2 S'_RR), relative to its own size; sums of t^2 and r t enter it relative to 1, which
-// left 1.8e-8 in an energy of 1e-3 (a noiseless lattice, every run of pixels rounded alike).
-// Explicit round-to-nearest operations keep the result independent of FMA contraction; e = 0 everywhere
-// (T o phi equals R up to the shift: identical inputs) is exactly NCC = 1 with a == b, so the gradient
-// vanishes exactly.
-__device__ Ncc ncc_terms(double P, double invP, double sr, double se, double srr, double see, double sre)
+// NCC and its gradient coefficients from the shifted sums: of r (LevelSums) and of the difference e =
+// t - r: sum e, sum e^2, sum r e.  With S'_TT = S'_RR + 2 S'_RE + S'_EE and S'_RT = S'_RR + S'_RE the
+// rounding of the FP32 sums enters 1 - NCC, about (S'_EE - S'_RE^2 / S'_RR) / (2 S'_RR), relative to its
+// own size; sums of t^2 and r t enter it relative to 1, which left 1.8e-8 in an energy of 1e-3 (a
+// noiseless lattice, every run of pixels rounded alike).  a = 1 / sqrt(S'_RR S'_TT) and b = NCC / S'_TT,
+// so b - a = -a (S'_RE + S'_EE) / S'_TT.  e = 0 everywhere (T o phi equals R up to the shift: identical
+// inputs) is exactly NCC = 1, b = a and tbar = rbar, so the gradient vanishes exactly.
+__device__ __forceinline__ Ncc ncc_terms(const LevelSums &L, double se, double see, double sre)
 {
     Ncc o;
-    const double Srr = __dsub_rn(srr, __dmul_rn(__dmul_rn(sr, sr), invP));
-    const double See = __dsub_rn(see, __dmul_rn(__dmul_rn(se, se), invP));
-    const double Sre = __dsub_rn(sre, __dmul_rn(__dmul_rn(sr, se), invP));
-    const double Srt = __dadd_rn(Srr, Sre);
-    const double Stt = __dadd_rn(Srt, __dadd_rn(Sre, See));
-    o.stt = Stt;
-    o.rbar = __dmul_rn(sr, invP);
-    o.tbar = __dmul_rn(__dadd_rn(sr, se), invP);
-    if (Srr < 1e-12 * P || Stt < 1e-12 * P) {
-        o.ncc = 0.0; o.a = 0.0; o.b = 0.0; o.degenerate = 1;
+    o.dbar = __dmul_rn(se, L.invP);
+    o.tbar = __fma_rn(L.sr, L.invP, o.dbar);
+    const double See = __fma_rn(-se, o.dbar, see), Sre = __fma_rn(-L.sr, o.dbar, sre);
+    const double u = __dadd_rn(Sre, See), Srt = __dadd_rn(L.Srr, Sre);
+    o.Stt = __dadd_rn(Srt, u);
+    o.degenerate = !nonneg(__fma_rn(-1e-12, L.P, L.Srr)) || !nonneg(__fma_rn(-1e-12, L.P, o.Stt));
+    if (o.degenerate) {
+        o.e = 1.0; o.a = 0.0; o.bma = 0.0;
         return o;
     }
-    const double a = rsqrt_nr(__dmul_rn(Srr, Stt));   // 1 / sqrt(S'_rr S'_tt)
+    const double a = rsqrt_f64(__dmul_rn(L.Srr, o.Stt));
     o.a = a;
-    if (Srt == Srr && Srr == Stt) {
-        o.ncc = 1.0;
-        o.b = a;
+    if (Sre == 0.0 && See == 0.0) {
+        o.e = 0.0;
+        o.bma = 0.0;
     } else {
-        o.ncc = __dmul_rn(Srt, a);
-        o.b = __dmul_rn(__dmul_rn(o.ncc, Srr), __dmul_rn(a, a));   // NCC / S'_tt
+        o.e = __fma_rn(-Srt, a, 1.0);
+        o.bma = __dmul_rn(-a, __dmul_rn(__dmul_rn(L.Srr, u), __dmul_rn(a, a)));
     }
-    o.degenerate = 0;
     return o;
+}
+
+// The reference's part of a level's sums.
+__device__ __forceinline__ void set_reference(LevelSums &L, double sr, double srr)
+{
+    L.sr = sr;
+    L.Srr = __fma_rn(-sr, __dmul_rn(sr, L.invP), srr);
 }
 
 // ------------------------------------------------------------------ level access
@@ -438,18 +449,20 @@ __device__ void rigid_pass(const Lvl &L, int r0, int r1, const float *pm, Smem &
 enum Action { kActGrad = 0, kActTrial = 1, kActDone = 2 };
 
 
-__device__ void rigid_params(const double *th, float *pm)
+// Pass parameters of parameter q's value v, written by lanes 0-2 of a warp: cos(alpha) - 1 (without
+// cancellation) and sin(alpha); the fractional and the integer part of Gx and Gy.
+__device__ __forceinline__ void rigid_param(double v, int q, int lane, float *pm)
 {
-    const float a = (float)th[0];
     float h, ch;
-    sincosf(0.5f * a, &h, &ch);
-    pm[0] = -2.f * h * h;            // cos(a) - 1 without cancellation
-    pm[1] = 2.f * h * ch;            // sin(a)
-    const double ix = rint(th[1]), iy = rint(th[2]);
-    pm[2] = (float)(th[1] - ix);
-    pm[3] = (float)(th[2] - iy);
-    pm[4] = (float)fmax(-4.0e6, fmin(4.0e6, ix));
-    pm[5] = (float)fmax(-4.0e6, fmin(4.0e6, iy));
+    sincosf(q == 0 ? 0.5f * (float)v : 0.f, &h, &ch);
+    const double i = rint(v);
+    if (lane == 0) {
+        pm[0] = -2.f * h * h;
+        pm[1] = 2.f * h * ch;
+    } else if (lane < 3) {
+        pm[1 + lane] = (float)(v - i);
+        pm[3 + lane] = fminf(fmaxf((float)i, -4.0e6f), 4.0e6f);
+    }
 }
 
 // Step-size rule of the line search: Armijo backtracking with safeguarded quadratic
@@ -466,69 +479,97 @@ __device__ __forceinline__ double next_tau(double E, double slope, double tau, d
     return accepted ? fmin(fmax(tq, 0.5 * tau), 4.0 * tau) : fmin(fmax(tq, 0.1 * tau), 0.5 * tau);
 }
 
-// Gradient at the point of a pass from its sums and the point's NCC terms: dE/dtheta_k = a sum (t - r)
-// g_k + (b - a) sum t g_k + (a rbar - b tbar) sum g_k; a == b and rbar == tbar give exact zeros.
-__device__ void rigid_gradient(const RigidCtl &k, const double *tot, double *g)
+// Gradient component q at the point of a pass from its sums and the point's NCC terms: dE/dtheta_q = a
+// sum (t - r) g_q + (b - a) sum t g_q + (a rbar - b tbar) sum g_q, the last coefficient being -a (tbar -
+// rbar) - (b - a) tbar; exact zeros for identical frames.
+__device__ __forceinline__ double rigid_gradient(const Ncc &n, const double *tot, int q)
 {
-    const double bma = __dsub_rn(k.b, k.a), kap = __dsub_rn(__dmul_rn(k.a, k.rbar), __dmul_rn(k.b, k.tbar));
-    for (int q = 0; q < 3; ++q) g[q] = k.a * tot[5 + q] + bma * tot[8 + q] + kap * tot[11 + q];
+    const double kap = __fma_rn(-n.bma, n.tbar, -__dmul_rn(n.a, n.dbar));
+    return n.a * tot[5 + q] + n.bma * tot[8 + q] + kap * tot[11 + q];
 }
 
-// Thread-0 controller after a pass at a level's start or at a trial point: the energy there, the Armijo
-// test, and where the point is taken the stop tests, the direction and the next trial.  Returns the
-// next action and writes its parameters.  Same rules as the oracle's level loop.
+// v of lanes 0, 1 and 2 added in that order, in every lane.
+__device__ __forceinline__ double sum3(double v)
+{
+    return (__shfl_sync(0xffffffffu, v, 0) + __shfl_sync(0xffffffffu, v, 1)) + __shfl_sync(0xffffffffu, v, 2);
+}
+
+// Controller after a pass at a level's start or at a trial point: the energy there, the Armijo test, and
+// where the point is taken the stop tests, the direction and the next trial.  Returns the next action
+// and writes its parameters.  Same rules as the oracle's level loop.  Run by one warp: lane q < 3 has
+// parameter q, every lane the scalars (one thread doing all of it took 7,000 of the 19,000 cycles of
+// an iteration at 160x128).
 __device__ int rigid_step(RigidCtl &k, const Config &cfg, const double *tot, bool start, float *pm)
 {
+    const int lane = threadIdx.x & 31, q = min(lane, 2);
     if (start) {
-        k.sr = tot[3];
-        k.srr = tot[4];
+        if (lane == 0) set_reference(k.ls, tot[3], tot[4]);
+        __syncwarp();
     }
-    const Ncc n = ncc_terms(k.P, k.invP, k.sr, tot[0], k.srr, tot[1], tot[2]);
-    const double Et = n.degenerate ? 1.0 : __dsub_rn(1.0, n.ncc);
-    if (!start) {
-        k.evals += 1;
-        if (!(Et <= k.E + cfg.armijo_c * k.tau * k.slope)) {
-            k.rejects += 1;
-            k.nrej += 1;
-            k.tau = next_tau(k.E, k.slope, k.tau, Et, false);
-            if (k.nrej > cfg.max_rejects) { k.stop = REG_STOP_LS; return kActDone; }
-            for (int q = 0; q < 3; ++q) k.tt[q] = k.th[q] + k.tau * k.d[q];
-            rigid_params(k.tt, pm);
-            return kActTrial;
+    const Ncc n = ncc_terms(k.ls, tot[0], tot[1], tot[2]);
+    const double Et = n.e, Eold = k.E, slope_old = k.slope, tau_old = k.tau;
+    double th = k.th[q], d = k.d[q], dp = k.dp[q], tau = k.tau, tau_acc = k.tau_acc;
+    int evals = k.evals + (start ? 0 : 1), iters = k.iters, have_prev = k.have_prev, nrej = k.nrej;
+    bool fresh = start;   // the first point of the level: no step, no previous direction
+    int act = kActTrial;
+    if (!start && !nonneg(Eold + cfg.armijo_c * tau_old * slope_old - Et)) {
+        tau = next_tau(Eold, slope_old, tau_old, Et, false);
+        nrej += 1;
+        if (lane == 0) k.rejects += 1;
+        if (nrej > cfg.max_rejects) {
+            if (lane == 0) k.stop = REG_STOP_LS;
+            act = kActDone;
         }
-        for (int q = 0; q < 3; ++q) { k.th[q] = k.tt[q]; k.dp[q] = k.d[q]; }
-        k.tau_acc = k.tau;
-        k.have_prev = 1;
-        k.iters += 1;
-        k.tau = next_tau(k.E, k.slope, k.tau, Et, true);
-    }
-    const double Eold = k.E;
-    k.E = Et;
-    k.a = n.a; k.b = n.b; k.rbar = n.rbar; k.tbar = n.tbar;
-    if (!start && Eold - Et <= cfg.tol_rel_e * fabs(Eold)) { k.stop = REG_STOP_REL; return kActDone; }
-    double g[3];
-    rigid_gradient(k, tot, g);
-    k.evals += 1;
-    if (k.iters >= cfg.max_iter) { k.stop = REG_STOP_MAXIT; return kActDone; }
-    k.d[0] = -g[0] * k.inv_m0; k.d[1] = -g[1]; k.d[2] = -g[2];
-    k.slope = g[0] * k.d[0] + g[1] * k.d[1] + g[2] * k.d[2];
-    // |g|_M = sqrt(-slope); the tests compare squares (no square root unless the cap applies)
-    const double gn2 = -k.slope;
-    if (!(gn2 >= k.tolg * k.tolg)) { k.stop = REG_STOP_GRAD; return kActDone; }
-    if (k.have_prev) {
-        double num = 0.0, den = 0.0;
-        for (int q = 0; q < 3; ++q) {
-            const double w = q == 0 ? k.m0 : 1.0, y = k.dp[q] - k.d[q];
-            num += w * k.dp[q] * y;
-            den += w * y * y;
+        fresh = false;
+        __syncwarp();
+    } else {
+        if (!start) {
+            th = k.tt[q];
+            dp = d;
+            tau_acc = tau_old;
+            have_prev = 1;
+            iters += 1;
         }
-        k.tau = bb_tau(k.tau, k.tau_acc, num, den);
+        int stop = -1;
+        if (!fresh && nonneg(cfg.tol_rel_e * fabs(Eold) - (Eold - Et))) {
+            stop = REG_STOP_REL;
+            tau = next_tau(Eold, slope_old, tau_old, Et, true);
+        } else {
+            evals += 1;
+            const double im = q == 0 ? k.inv_m0 : 1.0, g = rigid_gradient(n, tot, q);
+            d = -g * im;
+            const double slope = sum3(g * d);
+            // |g|_M = sqrt(-slope); the tests compare squares (no square root unless the cap applies)
+            if (iters >= cfg.max_iter) stop = REG_STOP_MAXIT;
+            else if (!nonneg(-slope - k.tolg2)) stop = REG_STOP_GRAD;
+            else {
+                const double w = q == 0 ? k.m0 : 1.0, y = dp - d;
+                const double num = sum3(w * dp * y), den = sum3(w * y * y);
+                if (!have_prev || !bb_tau(tau_acc, num, den, tau))
+                    tau = start ? tau_old : next_tau(Eold, slope_old, tau_old, Et, true);
+                const double gn2 = -slope;
+                if (!nonneg(cfg.step_cap * cfg.step_cap - tau * tau * gn2)) tau = cfg.step_cap * rsqrt_f64(gn2);
+                nrej = 0;
+            }
+            __syncwarp();
+            if (lane == 0) k.slope = slope;
+        }
+        if (stop >= 0) {
+            if (lane == 0) k.stop = stop;
+            act = kActDone;
+        }
+        __syncwarp();
+        if (lane < 3) { k.th[q] = th; k.d[q] = d; k.dp[q] = dp; }
+        if (lane == 0) { k.E = Et; k.tau_acc = tau_acc; k.iters = iters; k.have_prev = have_prev; }
     }
-    if (k.tau * k.tau * gn2 > cfg.step_cap * cfg.step_cap) k.tau = cfg.step_cap / sqrt(gn2);
-    k.nrej = 0;
-    for (int q = 0; q < 3; ++q) k.tt[q] = k.th[q] + k.tau * k.d[q];
-    rigid_params(k.tt, pm);
-    return kActTrial;
+    if (lane == 0) { k.tau = tau; k.nrej = nrej; k.evals = evals; }
+    if (act == kActTrial) {
+        const double tt = th + tau * d;
+        if (lane < 3) k.tt[q] = tt;
+        rigid_param(tt, q, lane, pm);
+    }
+    __syncwarp();
+    return act;
 }
 
 __device__ __forceinline__ Lvl level_of(const Params &p, int ref, int tmpl, int l)
@@ -578,10 +619,8 @@ __device__ void run_rigid(const Params &p, const OpDesc &op, int op_index, Smem 
         int r0, r1;
         strip_rows(L.H, rank, C, r0, r1);
         if (tid == 0) {
-            k.P = (double)L.W * (double)L.H;
-            k.invP = 1.0 / k.P;
-            k.cx = 0.5 * (L.W - 1);
-            k.cy = 0.5 * (L.H - 1);
+            k.ls.P = (double)L.W * (double)L.H;
+            k.ls.invP = 1.0 / k.ls.P;
             double rho = 0.25 * (L.W + L.H);
             k.m0 = rho * rho;
             k.inv_m0 = 1.0 / k.m0;
@@ -589,10 +628,12 @@ __device__ void run_rigid(const Params &p, const OpDesc &op, int op_index, Smem 
             k.have_prev = 0;
             k.iters = 0; k.evals = 0; k.stop = REG_STOP_MAXIT;
             // a coarse level only supplies the next level's initial guess: a looser stop
-            k.tolg = cfg.tol_grad * (l > 0 ? cfg.tol_coarse : 1.0);
-            rigid_params(k.th, sm.pm);
+            const double tolg = cfg.tol_grad * (l > 0 ? cfg.tol_coarse : 1.0);
+            k.tolg2 = tolg * tolg;
             sm.action = kActTrial;
         }
+        __syncthreads();
+        if (tid < 32) rigid_param(k.th[min(tid, 2)], min(tid, 2), tid, sm.pm);
         for (bool start = true;; start = false) {
             __syncthreads();
             if (sm.action == kActDone) break;
@@ -601,7 +642,10 @@ __device__ void run_rigid(const Params &p, const OpDesc &op, int op_index, Smem 
             for (int q = 0; q < 6; ++q) pm[q] = sm.pm[q];
             if (start) rigid_pass<S, true>(L, r0, r1, pm, sm, buf, cl);
             else rigid_pass<S, false>(L, r0, r1, pm, sm, buf, cl);
-            if (tid == 0) sm.action = rigid_step(k, cfg, sm.tot, start, sm.pm);
+            if (tid < 32) {
+                const int act = rigid_step(k, cfg, sm.tot, start, sm.pm);
+                if (tid == 0) sm.action = act;
+            }
         }
         if (tid == 0) {
             stops[l] = k.stop; iters[l] = k.iters; evals[l] = k.evals;
@@ -1384,27 +1428,17 @@ __device__ void grid_direction(const Grid &G, const Lvl &L, const PassGeom &P, c
     }
 }
 
-__device__ double field_energy(FieldCtl &k, const Config &cfg, const double *tot, bool trial)
-{
-    const Ncc n = ncc_terms(k.P, k.invP, k.sr, tot[0], k.srr, tot[1], tot[2]);
-    k.stt = n.stt;
-    double Ed = n.degenerate ? 1.0 : __dsub_rn(1.0, n.ncc);
-    double E = Ed + 0.5 * cfg.lambda * tot[5] * k.invP;
-    if (trial) { k.ta = n.a; k.tb = n.b; k.trbar = n.rbar; k.ttbar = n.tbar; k.tdegen = n.degenerate; }
-    else { k.a = n.a; k.b = n.b; k.rbar = n.rbar; k.tbar = n.tbar; k.degen = n.degenerate; }
-    return E;
-}
-
 // Parameter slots of the nonrigid passes: gradient coefficients aP, (b - a) P, (a rbar - b tbar) P
 // and lambda; the scalar product's 1/(P var T) and lambda/P; the next trial's step.
 enum FieldParam { kPmA = 0, kPmB = 1, kPmK = 2, kPmLam = 3, kPmDk = 4, kPmRk = 5, kPmTau = 6 };
 
-// Gradient coefficients from the current NCC terms; a == b and rbar == tbar give exact zeros.
-__device__ void field_grad_params(const FieldCtl &k, const Config &cfg, float *pm)
+// Gradient coefficients from a point's NCC terms; exact zeros but aP for identical frames.
+__device__ __forceinline__ void field_grad_params(const Ncc &n, const LevelSums &L, const Config &cfg, float *pm)
 {
-    pm[kPmA] = (float)(k.a * k.P);
-    pm[kPmB] = (float)(__dsub_rn(k.b, k.a) * k.P);
-    pm[kPmK] = (float)(__dsub_rn(__dmul_rn(k.a, k.rbar), __dmul_rn(k.b, k.tbar)) * k.P);
+    const float b = (float)(n.bma * L.P), aP = (float)(n.a * L.P);
+    pm[kPmA] = aP;
+    pm[kPmB] = b;
+    pm[kPmK] = -fmaf(b, (float)n.tbar, aP * (float)n.dbar);
     pm[kPmLam] = (float)cfg.lambda;
 }
 
@@ -1414,29 +1448,30 @@ __device__ void field_grad_params(const FieldCtl &k, const Config &cfg, float *p
 __device__ int field_eval(FieldCtl &k, const Config &cfg, const double *tot, bool start, float *pm, int &accepted)
 {
     accepted = 0;
+    if (start) set_reference(k.ls, tot[3], tot[4]);
+    const Ncc n = ncc_terms(k.ls, tot[0], tot[1], tot[2]);
+    const double Et = __fma_rn(k.half_lam, tot[5], n.e);
     if (start) {
-        k.sr = tot[3]; k.srr = tot[4];
-        k.E = field_energy(k, cfg, tot, false);
+        k.E = Et;
         // the level's scalar product at its initial control values: 1/(P var T) and lambda/P
-        const double vt = k.stt * k.invP;
-        pm[kPmDk] = vt > 0.0 ? (float)(k.invP / vt) : 0.f;
-        pm[kPmRk] = (float)(cfg.lambda * k.invP);
-        field_grad_params(k, cfg, pm);
+        const double vt = n.Stt * k.ls.invP;
+        pm[kPmDk] = vt > 0.0 ? (float)(k.ls.invP / vt) : 0.f;
+        pm[kPmRk] = (float)(2.0 * k.half_lam);
+        field_grad_params(n, k.ls, cfg, pm);
         return kActGrad;
     }
-    const double Et = field_energy(k, cfg, tot, true);
     k.evals += 1;
-    if (Et <= k.E + cfg.armijo_c * k.tau * k.slope) {
+    if (nonneg(k.E + cfg.armijo_c * k.tau * k.slope - Et)) {
         accepted = 1;   // c is advanced by the trial's step
+        field_grad_params(n, k.ls, cfg, pm);
         k.iters += 1;
-        const double Eold = k.E;
+        k.Eold = k.E;
+        k.slope_old = k.slope;
+        k.tau_old = k.tau;
         k.tau_acc = (double)(float)k.tau;   // the step applied: c + (float)tau d
         k.have_prev = 1;
-        k.tau = next_tau(k.E, k.slope, k.tau, Et, true);
         k.E = Et;
-        k.a = k.ta; k.b = k.tb; k.rbar = k.trbar; k.tbar = k.ttbar; k.degen = k.tdegen;
-        if (Eold - Et <= cfg.tol_rel_e * fabs(Eold)) { k.stop = REG_STOP_REL; return kActDone; }
-        field_grad_params(k, cfg, pm);
+        if (nonneg(cfg.tol_rel_e * fabs(k.Eold) - (k.Eold - Et))) { k.stop = REG_STOP_REL; return kActDone; }
         return kActGrad;
     }
     k.rejects += 1;
@@ -1453,14 +1488,18 @@ __device__ int field_grad(FieldCtl &k, const Config &cfg, const double *tot, dou
     k.evals += 1;
     if (k.iters >= cfg.max_iter) { k.stop = REG_STOP_MAXIT; return kActDone; }
     // |g| = sqrt(ss / Nc) and the largest control step dmax: compared squared
-    const double ss = tot[0];
-    k.slope = -ss * k.invNc;
-    if (!(ss * k.invNc >= k.tolg * k.tolg)) { k.stop = REG_STOP_GRAD; return kActDone; }
-    // the metric (mean over control points) is a common factor of the two sums
-    if (k.have_prev) k.tau = bb_tau(k.tau, k.tau_acc, tot[1], tot[2]);
-    if (k.tau * k.tau * dmax2 > cfg.step_cap * cfg.step_cap) k.tau = cfg.step_cap / sqrt(dmax2);
+    const double g2 = tot[0] * k.invNc;
+    k.slope = -g2;
+    if (!nonneg(g2 - k.tolg2)) { k.stop = REG_STOP_GRAD; return kActDone; }
+    // the metric (mean over control points) is a common factor of the two sums; without positive
+    // curvature the quadratic rule of the last step
+    double tau = k.tau;
+    if (k.have_prev && !bb_tau(k.tau_acc, tot[1], tot[2], tau))
+        tau = next_tau(k.Eold, k.slope_old, k.tau_old, k.E, true);
+    if (!nonneg(cfg.step_cap * cfg.step_cap - tau * tau * dmax2)) tau = cfg.step_cap * rsqrt_f64(dmax2);
+    k.tau = tau;
     k.nrej = 0;
-    pm[kPmTau] = (float)k.tau;
+    pm[kPmTau] = (float)tau;
     return kActTrial;
 }
 
@@ -1524,8 +1563,7 @@ __device__ void run_nonrigid(const Params &p, const OpDesc &op, int op_index, Sm
     FieldCtl &k = sm.fctl;
     if (tid == 0) {
         memset(&k, 0, sizeof(k));
-        k.Nc = (double)Nc;
-        k.invNc = 1.0 / k.Nc;
+        k.invNc = 1.0 / (double)Nc;
     }
     int stops[kMaxLevels], iters[kMaxLevels], evals[kMaxLevels];
     for (int l = Lc - 1; l >= 0; --l) {
@@ -1535,13 +1573,15 @@ __device__ void run_nonrigid(const Params &p, const OpDesc &op, int op_index, Sm
         if (cfg.metric == REG_METRIC_MEAN)
             for (int j = tid; j < held; j += kThreads) mt[j] = make_float2(1.f, 1.f);
         if (tid == 0) {
-            k.P = (double)L.W * (double)L.H;
-            k.invP = 1.0 / k.P;
+            k.ls.P = (double)L.W * (double)L.H;
+            k.ls.invP = 1.0 / k.ls.P;
+            k.half_lam = 0.5 * cfg.lambda * k.ls.invP;
             k.tau = cfg.tau0;
             k.have_prev = 0;
             k.iters = 0; k.evals = 0; k.stop = REG_STOP_MAXIT;
             // a coarse level only supplies the next level's initial guess: a looser stop
-            k.tolg = cfg.tol_grad * (l > 0 ? cfg.tol_coarse : 1.0);
+            const double tolg = cfg.tol_grad * (l > 0 ? cfg.tol_coarse : 1.0);
+            k.tolg2 = tolg * tolg;
         }
         __syncthreads();
         for (bool start = true;; start = false) {
@@ -1845,11 +1885,10 @@ __global__ void __launch_bounds__(kThreads) energy_kernel(Params p, const double
         RigidCtl &k = sm.rctl;
         if (tid == 0) {
             memset(&k, 0, sizeof(k));
-            k.P = (double)L.W * L.H;
-            k.invP = 1.0 / k.P;
-            k.th[0] = theta[0]; k.th[1] = theta[1]; k.th[2] = theta[2];
-            rigid_params(k.th, sm.pm);
+            k.ls.P = (double)L.W * L.H;
+            k.ls.invP = 1.0 / k.ls.P;
         }
+        if (tid < 32) rigid_param(theta[min(tid, 2)], min(tid, 2), tid, sm.pm);
         __syncthreads();
         int r0, r1;
         strip_rows(L.H, rank, C, r0, r1);
@@ -1857,10 +1896,10 @@ __global__ void __launch_bounds__(kThreads) energy_kernel(Params p, const double
         for (int q = 0; q < 6; ++q) pm[q] = sm.pm[q];
         rigid_pass<S, true>(L, r0, r1, pm, sm, buf, cl);
         if (first) {
-            const Ncc n = ncc_terms(k.P, k.invP, sm.tot[3], sm.tot[0], sm.tot[4], sm.tot[1], sm.tot[2]);
-            k.a = n.a; k.b = n.b; k.rbar = n.rbar; k.tbar = n.tbar;
-            out[0] = n.degenerate ? 1.0 : __dsub_rn(1.0, n.ncc);
-            rigid_gradient(k, sm.tot, out + 1);
+            set_reference(k.ls, sm.tot[3], sm.tot[4]);
+            const Ncc n = ncc_terms(k.ls, sm.tot[0], sm.tot[1], sm.tot[2]);
+            out[0] = n.e;
+            for (int q = 0; q < 3; ++q) out[1 + q] = rigid_gradient(n, sm.tot, q);
         }
     } else {
         const Grid G{p.gnx, p.gny, p.gs};
@@ -1881,13 +1920,12 @@ __global__ void __launch_bounds__(kThreads) energy_kernel(Params p, const double
         grid_pass<S, true, 2>(L, G, GL, P, B, c, d, 0.f, slots, sm, buf, cl);
         FieldCtl &k = sm.fctl;
         if (tid == 0) {
-            memset(&k, 0, sizeof(k));
-            k.P = (double)L.W * L.H;
-            k.invP = 1.0 / k.P;
-            k.sr = sm.tot[3]; k.srr = sm.tot[4];
-            const double E = field_energy(k, p.cfg, sm.tot, false);
-            if (first) out[0] = E;
-            field_grad_params(k, p.cfg, sm.pm);
+            k.ls.P = (double)L.W * L.H;
+            k.ls.invP = 1.0 / k.ls.P;
+            set_reference(k.ls, sm.tot[3], sm.tot[4]);
+            const Ncc n = ncc_terms(k.ls, sm.tot[0], sm.tot[1], sm.tot[2]);
+            if (first) out[0] = __fma_rn(0.5 * p.cfg.lambda * k.ls.invP, sm.tot[5], n.e);
+            field_grad_params(n, k.ls, p.cfg, sm.pm);
         }
         __syncthreads();
         if (grad_c) {
