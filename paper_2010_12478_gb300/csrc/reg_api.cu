@@ -700,21 +700,22 @@ void note_shape(reg_ctx *ctx, const Params &p, int C)
     ctx->last.ctas_per_sm = p.cfg.mode == REG_NONRIGID ? (p.minb > 0 ? p.minb : 3) : 4;
 }
 
-int pow2_floor(int v)
-{
-    int p = 1;
-    while (p * 2 <= v) p *= 2;
-    return p;
-}
-
-// CTAs per operator for a launch of `n_ops` concurrent operators: enough to fill
-// the GPU twice over (two CTAs per SM), at most 8, unless fixed by the config.
-int auto_cluster(const reg_ctx *ctx, int n_ops)
+// CTAs per operator where about `width` operators run side by side, unless fixed by the config: the
+// largest cluster of which the device holds at least two thirds of `width` at once (two CTAs per SM; of
+// 16-CTA clusters fewer than that fit the GPCs: four fifths), from 16 down to 4.  More CTAs shorten an operator and with it the scan's chains; fewer take less of
+// the time that goes to reductions and steps.  Measured (nonrigid, ms at 16 / 8 / 4 / 2 CTAs): 256 frames
+// of 512x512 (width 50) 24.4 / 16.7 / 21.8 / 33.3; 1,024 frames (width 160) 119 / 74.1 / 69.8 / 84.3;
+// 8 series of 32 at 256x256 (width 81) 15.8 / 7.4 / 5.7 / 7.5; a pair 0.39 / 0.49 / 0.68 / 1.10.  Rigid,
+// 128 frames of 512x512 (width 29): 5.3 / 4.5 / 5.7 / 8.8; 24 of 256x256, a depth at a time: 1.9 / 2.1 /
+// 2.8 / 3.7.  A nonrigid operator has work for no more CTAs than its grid has cell rows.
+int auto_cluster(const reg_ctx *ctx, const Params &p, double width)
 {
     if (ctx->cfg.cluster > 0) return ctx->cfg.cluster;
-    int slots = 2 * ctx->num_sms;
-    int c = pow2_floor(std::max(1, slots / std::max(1, n_ops)));
-    return std::min(8, c);
+    int c = 16;
+    while (c > 4 && width > (c == 16 ? 1.25 : 1.5) * (2 * ctx->num_sms / c)) c /= 2;
+    if (p.cfg.mode == REG_NONRIGID)
+        while (c > 1 && c / 2 >= p.gny - 1) c /= 2;
+    return c;
 }
 
 struct ScanPlan {
@@ -895,7 +896,7 @@ int execute(reg_ctx *ctx, const ScanPlan &plan, Params &p, int exec, const TileS
     if (exec == REG_EXEC_LEVEL) {
         for (int dpt = 0; dpt < n_depth; ++dpt) {
             int b = plan.depth_start[dpt], e = plan.depth_start[dpt + 1];
-            const int C = fit_cluster(p, tuned.cluster > 0 ? tuned.cluster : auto_cluster(ctx, e - b));
+            const int C = fit_cluster(p, tuned.cluster > 0 ? tuned.cluster : auto_cluster(ctx, p, e - b));
             note_shape(ctx, p, C);
             int chunk = std::max(1, e - b);
             for (int q = b; q < e; q += chunk) {
@@ -1059,7 +1060,8 @@ int execute(reg_ctx *ctx, const ScanPlan &plan, Params &p, int exec, const TileS
             long long ms = atoll(t);
             if (ms > 0) p.queue.timeout_ns = ms * 1000 * 1000;
         }
-        const int C = fit_cluster(p, tuned.cluster > 0 ? tuned.cluster : 8);
+        const double width = (double)n_ops / std::max(1, n_depth);
+        const int C = fit_cluster(p, tuned.cluster > 0 ? tuned.cluster : auto_cluster(ctx, p, width));
         note_shape(ctx, p, C);
         int workers = ctx->cfg.workers;
         if (workers <= 0) {
@@ -1546,7 +1548,7 @@ extern "C" int reg_pairwise(reg_ctx_t *ctx, const float *R, const float *T, int 
             CU(cudaStreamSynchronize(s));
         }
     }
-    const int C = fit_cluster(p, ctx->cfg.cluster > 0 ? ctx->cfg.cluster : 8);
+    const int C = fit_cluster(p, auto_cluster(ctx, p, 1.0));
     p.op_base = 0;
     p.unroll = ctx->cfg.unroll;
     p.minb = ctx->cfg.ctas_per_sm;

@@ -222,7 +222,7 @@ extern "C" int reg_pairwise_noalloc(const reg_config_t *cfg, int device, const f
         p.n_nodes = 2;
         p.stats = st;
         p.status = status;
-        const int C = cfg->cluster > 0 ? cfg->cluster : 8;
+        const int C = cfg->cluster > 0 ? cfg->cluster : 16;   // as reg_pairwise
         e = launch_ops(p, cfg->storage, C, 1, s);
         OpStats hst;
         double hth[3];
