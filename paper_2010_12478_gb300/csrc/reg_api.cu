@@ -117,6 +117,17 @@ bool is_device_ptr(const void *p)
     return a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged;
 }
 
+// Memory that kernels on `device` read directly: its own, or managed.
+bool on_device(const void *p, int device)
+{
+    cudaPointerAttributes a;
+    if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return a.type == cudaMemoryTypeManaged || (a.type == cudaMemoryTypeDevice && a.device == device);
+}
+
 using PointerAttrFn = CUresult (*)(void *, CUpointer_attribute, CUdeviceptr);
 PointerAttrFn pointer_attr_fn()
 {
@@ -374,6 +385,7 @@ struct reg_ctx {
     std::vector<int> last_op_nodes;   // node produced by each operator, in per_op order
     DevBuf pick_ids;                  // reg_scan_node_grids: node indices of one request
     DevBuf warp_ws;
+    DevBuf pair;                      // reg_pairwise: its PairBlock
     cudaGraphExec_t graph = nullptr;
     cudaStream_t capture = nullptr;   // graphs are captured here (the caller's stream may be the legacy one)
     uint64_t graph_key = 0;
@@ -639,36 +651,32 @@ int build_pyramids(reg_ctx *ctx, const Geometry &g, const float *frames, int nf,
     return REG_OK;
 }
 
-// Level table for `total` frames (means are read on the device side via a copy).
-int build_level_table(reg_ctx *ctx, const Geometry &g, int total, cudaStream_t s)
+// The context's pyramids as a level table's rows.
+LevelTable level_table(const reg_ctx *ctx, const Geometry &g)
 {
-    const int L = g.levels;
     const size_t sb = storage_bytes(ctx->cfg.storage);
     const int pad = ctx->cfg.mode == REG_NONRIGID ? kPad : 0;
-    std::vector<float> means((size_t)total * L);
-    CU(cudaMemcpyAsync(means.data(), ctx->means.ptr, sizeof(float) * means.size(), cudaMemcpyDeviceToHost, s));
-    CU(cudaStreamSynchronize(s));
-    std::vector<LevelDesc> tab((size_t)total * L);
-    for (int f = 0; f < total; ++f)
-        for (int l = 0; l < L; ++l) {
-            LevelDesc &d = tab[(size_t)f * L + l];
-            const size_t raw = level_elems(g.W[l], g.H[l], pad);
-            d.ptr = (const char *)ctx->pyr[l].ptr + (raw * f + level_origin(g.W[l], pad)) * sb;
-            d.W = g.W[l];
-            d.H = g.H[l];
-            d.pitch = level_pitch(g.W[l], pad);
-            if (pad) {
-                d.rptr = (const char *)ctx->spyr[l].ptr + (size_t)g.W[l] * g.H[l] * sb * f;
-                d.rpitch = g.W[l];
-            } else {
-                d.rptr = d.ptr;
-                d.rpitch = d.pitch;
-            }
-            d.mean = means[(size_t)f * L + l];
-        }
-    CHECK(ctx->level_tab.reserve(sizeof(LevelDesc) * tab.size()));
-    CU(cudaMemcpyAsync(ctx->level_tab.ptr, tab.data(), sizeof(LevelDesc) * tab.size(), cudaMemcpyHostToDevice, s));
-    CU(cudaStreamSynchronize(s));
+    LevelTable t;
+    memset(&t, 0, sizeof(t));
+    t.levels = g.levels;
+    for (int l = 0; l < g.levels; ++l) {
+        t.W[l] = g.W[l];
+        t.H[l] = g.H[l];
+        t.raw[l] = (const char *)ctx->pyr[l].ptr + level_origin(g.W[l], pad) * sb;
+        t.raw_stride[l] = level_elems(g.W[l], g.H[l], pad) * sb;
+        t.pitch[l] = level_pitch(g.W[l], pad);
+        t.ref[l] = pad ? (const char *)ctx->spyr[l].ptr : t.raw[l];
+        t.ref_stride[l] = pad ? (size_t)g.W[l] * g.H[l] * sb : t.raw_stride[l];
+        t.rpitch[l] = pad ? g.W[l] : t.pitch[l];
+    }
+    return t;
+}
+
+// Level table of the first `total` frames.
+int build_level_table(reg_ctx *ctx, const Geometry &g, int total, cudaStream_t s)
+{
+    CHECK(ctx->level_tab.reserve(sizeof(LevelDesc) * (size_t)total * g.levels));
+    CU(launch_level_table(ctx->level_tab.as<LevelDesc>(), level_table(ctx, g), ctx->means.as<float>(), total, s));
     return REG_OK;
 }
 
@@ -791,15 +799,14 @@ int ensure_op_events(reg_ctx *ctx, size_t n)
     return REG_OK;
 }
 
+// The parts of Params that do not depend on where operators and nodes are kept, the control-grid nodes
+// among them.
+int base_params(reg_ctx *ctx, const Geometry &g, int n_frames, int n_nodes, int n_ops, Params &p, cudaStream_t s);
+
 // Allocate node storage and stats; fill Params.
 int prepare_params(reg_ctx *ctx, const Geometry &g, int n_frames, int n_nodes, int n_ops, Params &p, cudaStream_t s)
 {
-    memset(&p, 0, sizeof(p));
-    p.cfg = dev_config(ctx->cfg);
-    p.levels = ctx->level_tab.as<LevelDesc>();
-    p.n_frames = n_frames;
-    p.n_ops = n_ops;
-    p.n_nodes = n_nodes;
+    CHECK(base_params(ctx, g, n_frames, n_nodes, n_ops, p, s));
     CHECK(ctx->ops.reserve(sizeof(OpDesc) * std::max(1, n_ops)));
     p.ops = ctx->ops.as<OpDesc>();
     CHECK(ctx->stats.reserve(sizeof(OpStats) * std::max(1, n_ops)));
@@ -810,6 +817,17 @@ int prepare_params(reg_ctx *ctx, const Geometry &g, int n_frames, int n_nodes, i
     p.status = ctx->status.as<int>();
     CU(cudaMemsetAsync(p.status, 0, sizeof(int) * 4, s));
     CU(cudaMemsetAsync(p.stats, 0, sizeof(OpStats) * std::max(1, n_ops), s));
+    return REG_OK;
+}
+
+int base_params(reg_ctx *ctx, const Geometry &g, int n_frames, int n_nodes, int n_ops, Params &p, cudaStream_t s)
+{
+    memset(&p, 0, sizeof(p));
+    p.cfg = dev_config(ctx->cfg);
+    p.levels = ctx->level_tab.as<LevelDesc>();
+    p.n_frames = n_frames;
+    p.n_ops = n_ops;
+    p.n_nodes = n_nodes;
     if (ctx->cfg.mode == REG_NONRIGID) {
         GridDims gd;
         CHECK(grid_dims(g.W[0], g.H[0], ctx->cfg.grid, g.levels, gd));
@@ -836,11 +854,19 @@ int prepare_params(reg_ctx *ctx, const Geometry &g, int n_frames, int n_nodes, i
     return REG_OK;
 }
 
+int device_status(const int *st);
+
 int check_device_status(reg_ctx *ctx, cudaStream_t s)
 {
     int st[4];
     CU(cudaMemcpyAsync(st, ctx->status.ptr, sizeof(st), cudaMemcpyDeviceToHost, s));
     CU(cudaStreamSynchronize(s));
+    return device_status(st);
+}
+
+// The error a kernel's status word stands for.
+int device_status(const int *st)
+{
     if (st[0] == kDevQueueTimeout) return fail(REG_ETIMEOUT, "device ready-queue wait timed out");
     if (st[0] != 0) return fail(REG_EINVAL, "device rejected an operator descriptor (code %d)", st[0]);
     return REG_OK;
@@ -1520,33 +1546,43 @@ extern "C" int reg_pairwise(reg_ctx_t *ctx, const float *R, const float *T, int 
     CHECK(geometry(W, H, ctx->cfg.levels, g));
     timing_reset(ctx);
     ctx->last_n = 0;   // the node storage of the last scan is reused below
-    const size_t fbytes = sizeof(float) * (size_t)H * pitch;
-    // staged R and T, then (nonrigid) one dense field for the initial guess or the result
-    CHECK(ctx->frames_dev.reserve(2 * fbytes + (nonrigid ? sizeof(float) * 2 * (size_t)W * H : 0)));
-    float *stage = ctx->frames_dev.as<float>();
-    const float *src[2] = {R, T};
-    for (int f = 0; f < 2; ++f) {
-        CU(cudaMemcpyAsync((char *)stage + f * fbytes, src[f], fbytes, cudaMemcpyDefault, s));
+    const size_t fbytes = sizeof(float) * (size_t)H * pitch, fb = sizeof(float) * 2 * (size_t)W * H;
+    // frames and fields in this device's memory are read and written where they are; others go through
+    // a staging buffer: R and T, then (nonrigid) one dense field for the initial guess or the result
+    const bool direct = on_device(R, ctx->device) && on_device(T, ctx->device);
+    const bool in_direct = field_in && on_device(field_in, ctx->device);
+    const bool out_direct = nonrigid && on_device(field_out, ctx->device);
+    const size_t frame_bytes = direct ? 0 : 2 * fbytes;
+    CHECK(ctx->frames_dev.reserve(frame_bytes + (nonrigid && (!out_direct || (field_in && !in_direct)) ? fb : 0)));
+    float *stage = ctx->frames_dev.as<float>(), *stage_u = (float *)((char *)stage + frame_bytes);
+    const float *frames = R;
+    size_t fstride = (size_t)(((intptr_t)T - (intptr_t)R) / (intptr_t)sizeof(float));   // may wrap: added once
+    if (!direct) {
+        CU(cudaMemcpyAsync(stage, R, fbytes, cudaMemcpyDefault, s));
+        CU(cudaMemcpyAsync((char *)stage + fbytes, T, fbytes, cudaMemcpyDefault, s));
+        frames = stage;
+        fstride = (size_t)H * pitch;
     }
-    CHECK(build_pyramids(ctx, g, stage, 2, (size_t)H * pitch, pitch, 0, 2, s));
-    CHECK(build_level_table(ctx, g, 2, s));
+    CHECK(build_pyramids(ctx, g, frames, 2, fstride, pitch, 0, 2, s));
+    CHECK(ctx->level_tab.reserve(sizeof(LevelDesc) * 2 * g.levels));
+    CHECK(ctx->pair.reserve(sizeof(PairBlock)));
+    PairBlock *blk = ctx->pair.as<PairBlock>();
     Params p;
-    CHECK(prepare_params(ctx, g, 2, 2, 1, p, s));
+    CHECK(base_params(ctx, g, 2, 2, 1, p, s));
+    p.ops = &blk->op;
+    p.stats = &blk->stats;
+    p.node_theta = blk->theta;
+    p.status = blk->status;
     const bool has_init = nonrigid ? field_in != nullptr : init != nullptr;
-    OpDesc op{0, 1, -1, -1, 0, has_init ? 1 : -1};
-    CU(cudaMemcpyAsync(ctx->ops.ptr, &op, sizeof(op), cudaMemcpyHostToDevice, s));
-    if (has_init) {
-        if (nonrigid) {
-            // dense initial field -> control values sampled at the control points (node 1)
-            const size_t fb = sizeof(float) * 2 * (size_t)W * H;
-            float *u = (float *)((char *)ctx->frames_dev.ptr + 2 * fbytes);
-            CU(cudaMemcpyAsync(u, field_in, fb, cudaMemcpyDefault, s));
-            CU(launch_grid_from_dense(u, W, H, p.gnx, p.gny, p.gs, p.node_grid + (size_t)p.gnx * p.gny, s));
-        } else {
-            double th[3] = {init->alpha, init->gx, init->gy};
-            CU(cudaMemcpyAsync(p.node_theta + 3, th, sizeof(th), cudaMemcpyHostToDevice, s));
-            CU(cudaStreamSynchronize(s));
-        }
+    const OpDesc op{0, 1, -1, -1, 0, has_init ? 1 : -1};
+    double th0[3] = {0.0, 0.0, 0.0};
+    if (!nonrigid && init) { th0[0] = init->alpha; th0[1] = init->gx; th0[2] = init->gy; }
+    CU(launch_pair_setup(blk, op, th0, ctx->level_tab.as<LevelDesc>(), level_table(ctx, g), ctx->means.as<float>(), s));
+    if (nonrigid && field_in) {
+        // dense initial field -> control values sampled at the control points (node 1)
+        if (!in_direct) CU(cudaMemcpyAsync(stage_u, field_in, fb, cudaMemcpyDefault, s));
+        CU(launch_grid_from_dense(in_direct ? field_in : stage_u, W, H, p.gnx, p.gny, p.gs,
+                                  p.node_grid + (size_t)p.gnx * p.gny, s));
     }
     const int C = fit_cluster(p, auto_cluster(ctx, p, 1.0));
     p.op_base = 0;
@@ -1558,28 +1594,24 @@ extern "C" int reg_pairwise(reg_ctx_t *ctx, const float *R, const float *T, int 
     ctx->op_pairs.push_back({e0, timing_mark(ctx, s)});
     ctx->last.op_launches += 1;
     CU(cudaGetLastError());
-    CHECK(check_device_status(ctx, s));
-    double th[3];
-    OpStats st;
-    CU(cudaMemcpyAsync(th, p.node_theta, sizeof(th), cudaMemcpyDeviceToHost, s));
-    CU(cudaMemcpyAsync(&st, p.stats, sizeof(st), cudaMemcpyDeviceToHost, s));
-    if (nonrigid) {
-        const size_t fb = sizeof(float) * 2 * (size_t)W * H;
-        CHECK(ctx->node_ids.reserve(sizeof(int)));
-        CU(cudaMemsetAsync(ctx->node_ids.ptr, 0, sizeof(int), s));
-        float *u = (float *)((char *)ctx->frames_dev.ptr + 2 * fbytes);
-        CU(launch_grid_dense(p.node_grid, ctx->node_ids.as<int>(), 1, p.gnx, p.gny, p.gs, W, H, u, s));
-        CHECK(copy_out(field_out, u, fb, s));
-    }
+    PairBlock res;
+    CU(cudaMemcpyAsync(&res, blk, offsetof(PairBlock, op), cudaMemcpyDeviceToHost, s));
     CU(cudaStreamSynchronize(s));
+    CHECK(device_status(res.status));
+    if (nonrigid) {
+        float *u = out_direct ? field_out : stage_u;
+        CU(launch_grid_dense(p.node_grid, &blk->node0, 1, p.gnx, p.gny, p.gs, W, H, u, s));
+        if (!out_direct) CHECK(copy_out(field_out, u, fb, s));
+        CU(cudaStreamSynchronize(s));
+    }
     timing_resolve(ctx);
     out->i = 0;
     out->k = 1;
-    out->alpha = (float)th[0];
-    out->gx = (float)th[1];
-    out->gy = (float)th[2];
-    if (stats) memcpy(stats, &st, sizeof(st));
-    if (st.status != kDevOk) return fail(REG_EINVAL, "operator failed on the device (%d)", st.status);
+    out->alpha = (float)res.theta[0];
+    out->gx = (float)res.theta[1];
+    out->gy = (float)res.theta[2];
+    if (stats) memcpy(stats, &res.stats, sizeof(*stats));
+    if (res.stats.status != kDevOk) return fail(REG_EINVAL, "operator failed on the device (%d)", res.stats.status);
     return REG_OK;
 }
 
@@ -1630,12 +1662,20 @@ extern "C" int reg_energy(reg_ctx_t *ctx, const float *R, const float *T, int W,
     int rc = geometry(W, H, 1, g);
     const size_t fbytes = sizeof(float) * (size_t)W * H;
     Params p;
-    if (rc == REG_OK) rc = ctx->frames_dev.reserve(2 * fbytes);
+    const bool direct = on_device(R, ctx->device) && on_device(T, ctx->device);
+    if (rc == REG_OK && !direct) rc = ctx->frames_dev.reserve(2 * fbytes);
     if (rc == REG_OK) {
-        float *stage = ctx->frames_dev.as<float>();
-        cudaMemcpyAsync(stage, R, fbytes, cudaMemcpyDefault, s);
-        cudaMemcpyAsync((char *)stage + fbytes, T, fbytes, cudaMemcpyDefault, s);
-        rc = build_pyramids(ctx, g, stage, 2, (size_t)W * H, W, 0, 2, s);
+        // frames in this device's memory are read where they are (the stride may wrap: it is added once)
+        const float *frames = R;
+        size_t fstride = (size_t)(((intptr_t)T - (intptr_t)R) / (intptr_t)sizeof(float));
+        if (!direct) {
+            float *stage = ctx->frames_dev.as<float>();
+            cudaMemcpyAsync(stage, R, fbytes, cudaMemcpyDefault, s);
+            cudaMemcpyAsync((char *)stage + fbytes, T, fbytes, cudaMemcpyDefault, s);
+            frames = stage;
+            fstride = (size_t)W * H;
+        }
+        rc = build_pyramids(ctx, g, frames, 2, fstride, W, 0, 2, s);
     }
     if (rc == REG_OK) rc = build_level_table(ctx, g, 2, s);
     if (rc == REG_OK) rc = prepare_params(ctx, g, 2, 1, 1, p, s);

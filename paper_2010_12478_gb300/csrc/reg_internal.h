@@ -131,6 +131,28 @@ cudaError_t launch_pyramid(const float *frames, int N, size_t fstride, int W, in
                            int storage, const PyrOut &out, float *means, cudaStream_t s);
 // Kernel launches of one launch_pyramid call.
 int pyramid_launches(int levels, bool means, int pad);
+// Level table of a batch of frames: frame f's row l is that of frame 0, its pointers f strides on, with
+// the level's mean.
+struct LevelTable {
+    int levels;
+    const char *raw[kMaxLevels], *ref[kMaxLevels];         // pixel (0, 0) of frame 0, template and reference role
+    size_t raw_stride[kMaxLevels], ref_stride[kMaxLevels]; // bytes between frames
+    int W[kMaxLevels], H[kMaxLevels], pitch[kMaxLevels], rpitch[kMaxLevels];
+};
+cudaError_t launch_level_table(LevelDesc *tab, const LevelTable &t, const float *means, int frames, cudaStream_t s);
+
+// What one pairwise call needs on the device besides its pyramids, in one block: the operator, its
+// nodes (0 the result, 1 the initial guess), and what comes back to the host (through `status`).
+struct PairBlock {
+    OpStats stats;
+    double theta[6];
+    int status[4];
+    OpDesc op;
+    int node0;         // 0: the dense field is that of node 0
+};
+// Fill the block (statistics and status zero) and the level table of the call's two frames.
+cudaError_t launch_pair_setup(PairBlock *b, const OpDesc &op, const double *init3, LevelDesc *tab, const LevelTable &t,
+                              const float *means, cudaStream_t s);
 // tab[l].mean = means[l] for l < L (a slot's level table rows after its pyramid build).
 cudaError_t launch_set_level_means(LevelDesc *tab, const float *means, int L, cudaStream_t s);
 // CTAs per operator for a launch that asks for `cluster`: more where an operator's control grid does

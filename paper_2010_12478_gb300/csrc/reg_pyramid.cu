@@ -209,6 +209,58 @@ __global__ void __launch_bounds__(kFinishThreads) pyr_finish(Levels<S> L, int pa
     }
 }
 
+// Row i of a level table (frame i / levels).
+__device__ __forceinline__ void level_row(LevelDesc *tab, const LevelTable &t, const float *means, int i)
+{
+    const int f = i / t.levels, l = i - f * t.levels;
+    LevelDesc d;
+    d.ptr = t.raw[l] + (size_t)f * t.raw_stride[l];
+    d.rptr = t.ref[l] + (size_t)f * t.ref_stride[l];
+    d.W = t.W[l];
+    d.H = t.H[l];
+    d.pitch = t.pitch[l];
+    d.rpitch = t.rpitch[l];
+    d.mean = means[i];
+    tab[i] = d;
+}
+
+// Made on the device, the table costs a launch; with the means read back and the rows made by the host it
+// cost two copies and two waits, of a 160x128 pair's call some 40 us.
+__global__ void level_table_kernel(LevelDesc *tab, LevelTable t, const float *means, int rows)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < rows) level_row(tab, t, means, i);
+}
+
+cudaError_t launch_level_table(LevelDesc *tab, const LevelTable &t, const float *means, int frames, cudaStream_t s)
+{
+    const int rows = frames * t.levels;
+    level_table_kernel<<<(rows + 127) / 128, 128, 0, s>>>(tab, t, means, rows);
+    return cudaGetLastError();
+}
+
+__global__ void pair_setup_kernel(PairBlock *b, OpDesc op, double i0, double i1, double i2, LevelDesc *tab, LevelTable t,
+                                  const float *means)
+{
+    if (threadIdx.x < 2 * t.levels) level_row(tab, t, means, threadIdx.x);
+    unsigned *w = reinterpret_cast<unsigned *>(&b->stats);
+    for (int i = threadIdx.x; i < (int)(sizeof(OpStats) / sizeof(unsigned)); i += blockDim.x) w[i] = 0u;
+    if (threadIdx.x == 0) {
+        b->theta[0] = b->theta[1] = b->theta[2] = 0.0;
+        b->theta[3] = i0; b->theta[4] = i1; b->theta[5] = i2;
+        b->status[0] = b->status[1] = b->status[2] = b->status[3] = 0;
+        b->op = op;
+        b->node0 = 0;
+    }
+}
+
+cudaError_t launch_pair_setup(PairBlock *b, const OpDesc &op, const double *init3, LevelDesc *tab, const LevelTable &t,
+                              const float *means, cudaStream_t s)
+{
+    pair_setup_kernel<<<1, 64, 0, s>>>(b, op, init3[0], init3[1], init3[2], tab, t, means);
+    return cudaGetLastError();
+}
+
 // The level means of a freshly built pyramid into its rows of a level table.
 __global__ void set_level_means_kernel(LevelDesc *tab, const float *means, int L)
 {

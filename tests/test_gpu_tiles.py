@@ -131,3 +131,30 @@ def test_a_grid_too_large_for_one_cta_takes_more():
         ctx.pairwise(F[0], F[1], field_out=outs[-1])
         assert ctx.last_timing()["cluster"] >= cluster
     assert float((outs[0] - outs[1]).abs().max()) <= 1e-4
+
+
+@pytest.mark.parametrize("mode", ["rigid", "nonrigid"])
+def test_pair_takes_frames_and_fields_from_anywhere(mode):
+    # device frames and fields are used where they are, anything else is staged: the same result, bit for bit
+    F = synth.make_series(synth.SeriesSpec(2, 90, 101, step=1.5, field_amp=1.0, snr=(10.0, 10.0), seed=3)).frames
+    ctx = B.Context(B.Config(mode=mode))
+    dev = F.cuda()
+    rev = torch.stack([F[1], F[0]]).cuda()   # the template in front of the reference
+    init = torch.full((2, 90, 101), 0.25)
+    runs = []
+    for R, T in ((dev[0], dev[1]), (F[0], F[1]), (F[0].pin_memory(), dev[1]), (rev[1], rev[0])):
+        if mode == "rigid":
+            runs.append(torch.tensor(ctx.pairwise(R, T, init=(0.001, 0.25, 0.25))[1]["theta"], dtype=torch.float64))
+            continue
+        for where in ("cuda", "cpu"):
+            out = torch.empty((2, 90, 101), device=where)
+            ctx.pairwise(R, T, field_in=init.to(where), field_out=out)
+            same = init.to(where).clone()   # the result over the initial guess
+            ctx.pairwise(R, T, field_in=same, field_out=same)
+            runs += [out.cpu(), same.cpu()]
+    assert all(torch.equal(r, runs[0]) for r in runs)
+    if mode == "nonrigid":
+        g = O.grid_for(101, 90)
+        c = torch.zeros((g.ny, g.nx, 2), device="cuda") + 0.3
+        E = [B.Context(B.Config(mode=mode)).energy_grid(R, T, c) for R, T in ((dev[0], dev[1]), (F[0], dev[1]), (rev[1], rev[0]))]
+        assert E[0] == E[1] == E[2]
