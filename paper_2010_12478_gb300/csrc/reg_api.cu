@@ -868,6 +868,7 @@ int check_device_status(reg_ctx *ctx, cudaStream_t s)
 int device_status(const int *st)
 {
     if (st[0] == kDevQueueTimeout) return fail(REG_ETIMEOUT, "device ready-queue wait timed out");
+    if (st[0] == kDevWaitTimeout) return fail(REG_ETIMEOUT, "a wait for the other CTAs of an operator timed out");
     if (st[0] != 0) return fail(REG_EINVAL, "device rejected an operator descriptor (code %d)", st[0]);
     return REG_OK;
 }

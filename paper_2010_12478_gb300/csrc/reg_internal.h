@@ -65,7 +65,7 @@ enum DevStatus : int32_t {
     kDevOk = 0,
     kDevBadOp = 1,       // operator descriptor out of range / non-adjacent
     kDevQueueTimeout = 2, // bounded wait on the ready queue gave up
-    kDevWaitTimeout = 3   // bounded wait on a TMA load (mbarrier) gave up
+    kDevWaitTimeout = 3   // bounded wait on an mbarrier (TMA load, cluster exchange) gave up
 };
 
 // Operator model of a launch beyond REG_RIGID / REG_NONRIGID: the mock operator of reg_mock_scan.

@@ -82,25 +82,114 @@ struct Smem {
     double part[2][kMaxCluster][kNM];   // every CTA's partials, pushed here by each CTA
     double tot[kNM];            // cluster totals
     unsigned wmax[kWarps], pmax[2][kMaxCluster];   // bits of the per-warp and per-CTA maxima
+    unsigned long long xbar[2]; // mbarriers of the exchanges, used in turn
     double tmax;
     float pm[16];               // pass parameters broadcast by thread 0
     int action;
     int idata[4];
+    int fail;                   // an exchange's wait ran out: kDevWaitTimeout
     union {
         RigidCtl rctl;
         FieldCtl fctl;
     };
 };
 
+// ------------------------------------------------------------------ exchanges within a cluster
+// CTAs of a cluster hand each other values by asynchronous stores into the receiver's shared memory
+// that count down bytes on an mbarrier there (st.async), and a receiver waits for the bytes it is due.
+// An exchange is numbered: number n uses barrier and buffers n mod 2.  A CTA sends for n + 2 only after
+// completing n + 1, to which every peer contributes after completing n, so nothing of n + 2 meets
+// anything of n.  A cluster barrier here takes about 2,000 cycles (its release and acquire are fences over
+// global memory), and its acquire drops the SM's L1 lines, so every pass fetched its pixels from L2
+// again (331 cycles a load instead of 75); an exchange takes 500 and leaves them.
+struct Comm {
+    unsigned n;   // number of the next exchange
+};
+
+__device__ __forceinline__ uint32_t smem_addr(const void *p)
+{
+    return (uint32_t)__cvta_generic_to_shared(p);
+}
+
+__device__ __forceinline__ uint32_t peer_addr(const void *p, int rank)
+{
+    uint32_t r;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(smem_addr(p)), "r"(rank));
+    return r;
+}
+
+// Eight (four) bytes to *p in the shared memory of CTA `rank`, counted on its barrier `bar`.
+__device__ __forceinline__ void send8(const void *p, const unsigned long long *bar, int rank, unsigned long long v)
+{
+    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.b64 [%0], %1, [%2];" ::"r"(peer_addr(p, rank)),
+                 "l"(v), "r"(peer_addr(bar, rank))
+                 : "memory");
+}
+
+__device__ __forceinline__ void send8(const void *p, const unsigned long long *bar, int rank, float2 v)
+{
+    send8(p, bar, rank, (unsigned long long)__float_as_uint(v.x) | ((unsigned long long)__float_as_uint(v.y) << 32));
+}
+
+__device__ __forceinline__ void send4(const void *p, const unsigned long long *bar, int rank, unsigned v)
+{
+    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.b32 [%0], %1, [%2];" ::"r"(peer_addr(p, rank)),
+                 "r"(v), "r"(peer_addr(bar, rank))
+                 : "memory");
+}
+
+// One thread, before the cluster's first exchange (a cluster barrier follows).
+__device__ __forceinline__ void comm_init(Smem &sm)
+{
+    for (int i = 0; i < 2; ++i)
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(&sm.xbar[i])) : "memory");
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    sm.fail = 0;
+}
+
+// One thread: this CTA is due `bytes` in exchange n.
+__device__ __forceinline__ void comm_expect(Smem &sm, unsigned n, unsigned bytes)
+{
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_addr(&sm.xbar[n & 1])), "r"(bytes)
+                 : "memory");
+}
+
+// Wait until exchange n has brought what is due; the peers run side by side with this CTA, so it ends,
+// and after two seconds it gives up: sm.fail, and no later exchange of this CTA waits.
+__device__ __forceinline__ void comm_wait(Smem &sm, unsigned n)
+{
+    const uint32_t bar = smem_addr(&sm.xbar[n & 1]), parity = (n >> 1) & 1;
+    unsigned long long t0 = 0;
+    for (unsigned it = 0; *(volatile int *)&sm.fail == 0; ++it) {
+        uint32_t done;
+        asm volatile("{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
+                     : "=r"(done)
+                     : "r"(bar), "r"(parity)
+                     : "memory");
+        if (done) return;
+        if ((it & 63) == 63) {
+            unsigned long long t;
+            asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+            if (t0 == 0) t0 = t;
+            else if (t - t0 > 2000000000ULL) *(volatile int *)&sm.fail = kDevWaitTimeout;
+        }
+    }
+}
+
 // Reduce NM per-thread float-float sums over the cluster into sm.tot, in a fixed order, and with MAXV
-// the largest of a non-negative value into sm.tmax.  Within a warp the sums are exchanged by halves,
-// so a lane carries one of them after log2 steps (9 pair additions for 8 sums instead of 40); the
-// warps', then the CTAs' partials of a sum are shared out over the lanes and folded the same way.
-// Every CTA pushes its partials into every CTA's shared memory (remote stores do not wait; the cluster
-// barrier makes them visible) and adds the same values in the same order: identical totals.
-template <int NM, bool MAXV>
+// the largest of a non-negative value into sm.tmax, by one exchange.  Within a warp the sums are exchanged
+// by halves, so a lane carries one of them after log2 steps (9 pair additions for 8 sums instead of 40);
+// the warps', then the CTAs' partials of a sum are shared out over the lanes and folded the same way.
+// Every CTA sends its partials to every CTA, which adds the same values in the same order: identical
+// totals.  `push` is called by every thread after a barrier of the CTA with the exchange's number, to
+// send more under it; `due`: bytes of such sends that this CTA gets.
+struct NoPush {
+    __device__ void operator()(unsigned) const {}
+};
+template <int NM, bool MAXV, typename Push = NoPush>
 __device__ __forceinline__ void cluster_reduce(const float (&hi)[NM], const float (&lo)[NM], float mx, Smem &sm,
-                                               int &buf, const cg::cluster_group &cl)
+                                               Comm &comm, const cg::cluster_group &cl, unsigned due = 0,
+                                               Push push = Push())
 {
     static_assert(NM <= kNM && kWarps == 8, "reduction slots");
     constexpr int kLog = NM <= 8 ? 3 : 4, N2 = 1 << kLog, kParts = 32 / N2;   // lanes that share a sum
@@ -133,7 +222,10 @@ __device__ __forceinline__ void cluster_reduce(const float (&hi)[NM], const floa
     __syncthreads();
     const int C = cl.num_blocks(), me = cl.block_rank();
     const int m = lane % N2, q = lane / N2;   // warp 0: lane's sum, and which share of its parts
+    const unsigned n = comm.n++, b = n & 1;
+    const unsigned long long *bar = &sm.xbar[b];
     if (w == 0) {
+        if (lane == 0) comm_expect(sm, n, (unsigned)C * (NM * 8 + (MAXV ? 4 : 0)) + due);
         float2 v = sm.warp[q][m];
 #pragma unroll
         for (int k = q + kParts; k < kWarps; k += kParts) ff_add(v.x, v.y, sm.warp[k][m].x, sm.warp[k][m].y);
@@ -142,24 +234,26 @@ __device__ __forceinline__ void cluster_reduce(const float (&hi)[NM], const floa
             const float h2 = __shfl_xor_sync(0xffffffffu, v.x, o), l2 = __shfl_xor_sync(0xffffffffu, v.y, o);
             ff_add(v.x, v.y, h2, l2);
         }
-        const double t = (double)v.x + (double)v.y;
-        for (int r = q; r < C; r += kParts) *cl.map_shared_rank(&sm.part[buf][me][m], r) = t;
+        const unsigned long long t = __double_as_longlong((double)v.x + (double)v.y);
+        if (m < NM)
+            for (int r = q; r < C; r += kParts) send8(&sm.part[b][me][m], bar, r, t);
     } else if (MAXV && w == 1) {
         const unsigned v = __reduce_max_sync(0xffffffffu, lane < kWarps ? sm.wmax[lane] : 0u);
-        if (lane < C) *cl.map_shared_rank(&sm.pmax[buf][me], lane) = v;
+        if (lane < C) send4(&sm.pmax[b][me], bar, lane, v);
     }
-    cl.sync();
+    push(n);
     if (w == 0) {
-        double s = q < C ? sm.part[buf][q][m] : 0.0;
-        for (int r = q + kParts; r < C; r += kParts) s = __dadd_rn(s, sm.part[buf][r][m]);
+        comm_wait(sm, n);
+        double s = q < C && m < NM ? sm.part[b][q][m] : 0.0;
+        for (int r = q + kParts; r < C; r += kParts) s = __dadd_rn(s, m < NM ? sm.part[b][r][m] : 0.0);
 #pragma unroll
         for (int o = N2; o < 32; o <<= 1) s = __dadd_rn(s, __shfl_xor_sync(0xffffffffu, s, o));
         if (lane < N2) sm.tot[m] = s;
-    } else if (MAXV && w == 1) {
-        const unsigned v = __reduce_max_sync(0xffffffffu, lane < C ? sm.pmax[buf][lane] : 0u);
-        if (lane == 0) sm.tmax = (double)__uint_as_float(v);
+        if constexpr (MAXV) {
+            const unsigned v = __reduce_max_sync(0xffffffffu, lane < C ? sm.pmax[b][lane] : 0u);
+            if (lane == 0) sm.tmax = (double)__uint_as_float(v);
+        }
     }
-    buf ^= 1;
     __syncthreads();
 }
 
@@ -289,7 +383,7 @@ constexpr unsigned kRoundBits = 0x4B400000u;
 // keeps its clamped cell; runs that reach the top or bottom edge go row by row through sample_at.
 constexpr int kRigidSums = 14, kRigidRows = 4;   // rows whose loads are in flight together
 template <typename S, bool START>
-__device__ void rigid_pass(const Lvl &L, int r0, int r1, const float *pm, Smem &sm, int &buf,
+__device__ void rigid_pass(const Lvl &L, int r0, int r1, const float *pm, Smem &sm, Comm &comm,
                            const cg::cluster_group &cl)
 {
     constexpr int NS = START ? 5 : 3;
@@ -443,7 +537,7 @@ __device__ void rigid_pass(const Lvl &L, int r0, int r1, const float *pm, Smem &
     }
 #pragma unroll
     for (int i = 0; i < 9; ++i) { hi[5 + i] = gh[i]; lo[5 + i] = gl[i]; }
-    cluster_reduce<kRigidSums, false>(hi, lo, 0.f, sm, buf, cl);
+    cluster_reduce<kRigidSums, false>(hi, lo, 0.f, sm, comm, cl);
 }
 
 enum Action { kActGrad = 0, kActTrial = 1, kActDone = 2 };
@@ -582,13 +676,12 @@ __device__ __forceinline__ Lvl level_of(const Params &p, int ref, int tmpl, int 
 }
 
 template <typename S>
-__device__ void run_rigid(const Params &p, const OpDesc &op, int op_index, Smem &sm,
+__device__ void run_rigid(const Params &p, const OpDesc &op, int op_index, Smem &sm, Comm &comm,
                           const cg::cluster_group &cl)
 {
     const int tid = threadIdx.x;
     const int C = cl.num_blocks(), rank = cl.block_rank();
     const Config &cfg = p.cfg;
-    int buf = 0;
     RigidCtl &k = sm.rctl;
     if (tid == 0) {
         memset(&k, 0, sizeof(k));
@@ -640,11 +733,11 @@ __device__ void run_rigid(const Params &p, const OpDesc &op, int op_index, Smem 
             float pm[6];
 #pragma unroll
             for (int q = 0; q < 6; ++q) pm[q] = sm.pm[q];
-            if (start) rigid_pass<S, true>(L, r0, r1, pm, sm, buf, cl);
-            else rigid_pass<S, false>(L, r0, r1, pm, sm, buf, cl);
+            if (start) rigid_pass<S, true>(L, r0, r1, pm, sm, comm, cl);
+            else rigid_pass<S, false>(L, r0, r1, pm, sm, comm, cl);
             if (tid < 32) {
                 const int act = rigid_step(k, cfg, sm.tot, start, sm.pm);
-                if (tid == 0) sm.action = act;
+                if (tid == 0) sm.action = sm.fail ? (int)kActDone : act;
             }
         }
         if (tid == 0) {
@@ -666,7 +759,7 @@ __device__ void run_rigid(const Params &p, const OpDesc &op, int op_index, Smem 
             st.stop[l] = v ? stops[l] : 0;
         }
         st.rejects = k.rejects;
-        st.status = kDevOk;
+        st.status = sm.fail;
         st.energy = k.E;
         st.theta[0] = o[0]; st.theta[1] = o[1]; st.theta[2] = o[2];
     }
@@ -798,11 +891,12 @@ __host__ __device__ __forceinline__ size_t slot_floats(const PassGeom &P)
 }
 
 // Dynamic shared memory of the nonrigid kernels, in float2 units: c, d, mt (the held rows; mt the
-// flow's scalar product per control point and axis), two staged halo rows of d, then the slots.
+// flow's scalar product per control point and axis), two staged halo rows of d, the sums that the CTA
+// above sends for the first own row, then the slots.
 // With the H1 product mt is the right-hand side of its solve on the whole grid, and the two work
 // grids t and u of the solve lie in the place of the slots, which it has read by then.
 struct GridLayout {
-    int c, d, mt, halo, slots;
+    int c, d, mt, halo, above, slots;
 };
 __host__ __device__ __forceinline__ GridLayout grid_layout(int gnx, int gny, int C, bool h1)
 {
@@ -813,7 +907,8 @@ __host__ __device__ __forceinline__ GridLayout grid_layout(int gnx, int gny, int
     g.d = rows * gnx;
     g.mt = 2 * rows * gnx;
     g.halo = g.mt + (h1 ? gny : rows) * gnx;
-    g.slots = g.halo + 2 * gnx;
+    g.above = g.halo + 2 * gnx;
+    g.slots = g.above + kSlot / 2 * gnx;
     g.slots += g.slots & 1;
     return g;
 }
@@ -925,6 +1020,39 @@ __device__ __forceinline__ float2 bspline2(const TapRow &r0, const TapRow &r1, c
 
 constexpr int kRunRows = 16;   // rows of a straight run at most; half of it is tried next
 
+// Sums of control point (cr0 + i, jx) over the slots that one CTA with nr cell rows wrote: entries
+// first .. first + N - 1, segment by segment and strip by strip.
+template <int N>
+__device__ __forceinline__ void slot_sum(const float *slots, const PassGeom &P, int ncx, int nr, int i, int jx,
+                                         int first, float (&o)[N])
+{
+    const int ga = i > 0 ? (i - 1) / P.m : 0, gb = i < nr ? i / P.m : (nr - 1) / P.m;
+    auto add = [&](int seg, int strip, int row, int pt) {
+        const float *s = slots + (((size_t)(seg * P.nst + strip) * (P.m + 1) + row) * (P.g + 1) + pt) * kSlot + first;
+#pragma unroll
+        for (int k = 0; k < N; k += 2) {
+            const float2 v = *(const float2 *)(s + k);
+            o[k] += v.x;
+            o[k + 1] += v.y;
+        }
+    };
+    const int st = jx / P.g, pt = jx - st * P.g;
+    for (int grp = ga; grp <= gb; ++grp)
+        for (int piece = 0; piece < P.h; ++piece) {
+            const int seg = grp * P.h + piece, row = i - grp * P.m;
+            if (P.sl < 32) {
+                if (pt == 0 && jx > 0) add(seg, st - 1, row, P.g);
+                if (st < P.ns) add(seg, st, row, pt);
+            } else {
+                for (int q = 0; q < P.chunks; ++q) {
+                    if (jx > 0) add(seg, (jx - 1) * P.chunks + q, row, 1);
+                    if (jx < ncx) add(seg, jx * P.chunks + q, row, 0);
+                }
+            }
+            if (P.nst > P.ns && jx >= ncx - 1) add(seg, P.ns, row, jx - (ncx - 1));
+        }
+}
+
 // One pass at c (START: a level's first) or at the trial c + tau d: the moments into sm.tot (e =
 // t - r: 0 sum e, 1 sum e^2, 2 sum r e, with START 3 sum r, 4 sum r^2; 5: sum over control edges of |dct|^2) and the gradient
 // sums into the slots.  The trial values are formed where they are read, fmaf(tau, d_j, c_j), the
@@ -938,8 +1066,8 @@ constexpr int kRunRows = 16;   // rows of a straight run at most; half of it is 
 // float-float.
 template <typename S, bool START, int R>
 __device__ void grid_pass(const Lvl &L, const Grid &G, const GridLvl &GL, const PassGeom &P, const Band &B,
-                          const float2 *c, const float2 *d, float tau, float *slots, Smem &sm, int &buf,
-                          const cg::cluster_group &cl)
+                          const float2 *c, const float2 *d, float tau, float *slots, const float *above, Smem &sm,
+                          Comm &comm, const cg::cluster_group &cl)
 {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int ncx = G.nx - 1, ncy = G.ny - 1, sl = P.sl, pairs = (P.nst + 1) / 2;
@@ -1196,51 +1324,30 @@ __device__ void grid_pass(const Lvl &L, const Grid &G, const GridLvl &GL, const 
         }
         ff_acc(hi[5], lo[5], e);
     }
-    cluster_reduce<6, false>(hi, lo, 0.f, sm, buf, cl);
+    // the last control row's sums, where the CTA below owns that row, go to it
+    constexpr int kPairs = START ? 4 : 3;
+    const unsigned due = B.cr0 > 0 && B.cr0 < B.cr1 ? (unsigned)(G.nx * kPairs) * 8u : 0u;
+    cluster_reduce<6, false>(hi, lo, 0.f, sm, comm, cl, due, [&](unsigned n) {
+        if (!(B.cr0 < B.cr1 && B.own1 < G.ny)) return;
+        for (int t = threadIdx.x; t < G.nx * kPairs; t += kThreads) {
+            const int jx = t / kPairs, i = 2 * (t - jx * kPairs);
+            float v[2] = {0.f, 0.f};
+            slot_sum<2>(slots, P, ncx, B.q, B.q, jx, i, v);
+            send8(above + jx * kSlot + i, &sm.xbar[n & 1], (int)cl.block_rank() + 1, make_float2(v[0], v[1]));
+        }
+    });
 }
 
-// Sums of control point (cr0 + i, jx) over the slots that one CTA with nr cell rows wrote: entries
-// first .. first + N - 1, segment by segment and strip by strip.
-template <int N>
-__device__ __forceinline__ void slot_sum(const float *slots, const PassGeom &P, int ncx, int nr, int i, int jx,
-                                         int first, float (&o)[N])
-{
-    const int ga = i > 0 ? (i - 1) / P.m : 0, gb = i < nr ? i / P.m : (nr - 1) / P.m;
-    auto add = [&](int seg, int strip, int row, int pt) {
-        const float *s = slots + (((size_t)(seg * P.nst + strip) * (P.m + 1) + row) * (P.g + 1) + pt) * kSlot + first;
-#pragma unroll
-        for (int k = 0; k < N; k += 2) {
-            const float2 v = *(const float2 *)(s + k);
-            o[k] += v.x;
-            o[k + 1] += v.y;
-        }
-    };
-    const int st = jx / P.g, pt = jx - st * P.g;
-    for (int grp = ga; grp <= gb; ++grp)
-        for (int piece = 0; piece < P.h; ++piece) {
-            const int seg = grp * P.h + piece, row = i - grp * P.m;
-            if (P.sl < 32) {
-                if (pt == 0 && jx > 0) add(seg, st - 1, row, P.g);
-                if (st < P.ns) add(seg, st, row, pt);
-            } else {
-                for (int q = 0; q < P.chunks; ++q) {
-                    if (jx > 0) add(seg, (jx - 1) * P.chunks + q, row, 1);
-                    if (jx < ncx) add(seg, jx * P.chunks + q, row, 0);
-                }
-            }
-            if (P.nst > P.ns && jx >= ncx - 1) add(seg, P.ns, row, jx - (ncx - 1));
-        }
-}
-
-// The same over the whole grid: this CTA's slots, and at its first row the last partial row of the
-// CTA above.
+// The same over the whole grid: this CTA's slots, and at its first row what the CTA above sent.
 template <int N>
 __device__ __forceinline__ void point_sum(const float *slots, const float *above, const PassGeom &P, const Band &B,
                                           int ncx, int row, int jx, int first, float (&o)[N])
 {
 #pragma unroll
     for (int k = 0; k < N; ++k) o[k] = 0.f;
-    if (row == B.cr0 && above) slot_sum<N>(above, P, ncx, B.q, B.q, jx, first, o);
+    if (row == B.cr0 && row > 0)
+#pragma unroll
+        for (int k = 0; k < N; ++k) o[k] = above[jx * kSlot + first + k];
     slot_sum<N>(slots, P, ncx, B.cr1 - B.cr0, row - B.cr0, jx, first, o);
 }
 
@@ -1320,7 +1427,7 @@ __device__ void h1_solve(const H1Bufs &h, int nx, int ny)
 // axis m = dk sum_x w_j(x)^2 (dT/dp)^2 + rk n_j (dk = 1/(P var T), rk = lambda/P, n_j the neighbours
 // of j), normalised by the mean of all 2 Nc values and floored at 1e-3 of it, written to mt.
 __device__ void grid_metric(const Grid &G, const PassGeom &P, const Band &B, const float *slots, const float *above,
-                            float2 *mt, float dk, float rk, Smem &sm, int &buf, const cg::cluster_group &cl)
+                            float2 *mt, float dk, float rk, Smem &sm, Comm &comm, const cg::cluster_group &cl)
 {
     const int n = (B.own1 - B.cr0) * G.nx;
     float hi[1] = {0.f}, lo[1] = {0.f};
@@ -1333,7 +1440,7 @@ __device__ void grid_metric(const Grid &G, const PassGeom &P, const Band &B, con
         mt[(row - B.h0) * G.nx + jx] = m;
         ff_acc(hi[0], lo[0], m.x + m.y);
     }
-    cluster_reduce<1, false>(hi, lo, 0.f, sm, buf, cl);
+    cluster_reduce<1, false>(hi, lo, 0.f, sm, comm, cl);
     const double mean = sm.tot[0] / (2.0 * (G.nx * G.ny));
     const float inv = mean > 0.0 ? (float)(1.0 / mean) : 0.f;
     for (int j = threadIdx.x; j < n; j += kThreads) {
@@ -1349,7 +1456,7 @@ __device__ void grid_metric(const Grid &G, const PassGeom &P, const Band &B, con
 // sm.tot[1] and |d_old - d|_M^2 in sm.tot[2], max |d_j|^2 in sm.tmax; identical in every CTA.
 __device__ void grid_direction(const Grid &G, const Lvl &L, const PassGeom &P, const Band &B, const float2 *c,
                                float2 *d, float2 *mt, float2 *halo, const float *slots, const float *above,
-                               const float *pm, Smem &sm, int &buf, const cg::cluster_group &cl, const H1Bufs &h1)
+                               const float *pm, Smem &sm, Comm &comm, const cg::cluster_group &cl, const H1Bufs &h1)
 {
     const int Nc = G.nx * G.ny, n = (B.own1 - B.cr0) * G.nx, rank = cl.block_rank();
     const float aP = pm[0], bmaP = pm[1], kappa = pm[2], lam = pm[3];
@@ -1402,25 +1509,29 @@ __device__ void grid_direction(const Grid &G, const Lvl &L, const PassGeom &P, c
         }
         __syncthreads();   // every d_prev was read before d is replaced
         for (int j = threadIdx.x; j < (B.h1 - B.h0) * G.nx; j += kThreads) d[j] = h1.U[B.h0 * G.nx + j];
-        cluster_reduce<3, true>(hi, lo, mx, sm, buf, cl);
+        cluster_reduce<3, true>(hi, lo, mx, sm, comm, cl);
         return;
     }
     // The edge rows go to the neighbours' halo rows (0: the row above the own ones, 1: the row below),
-    // not to their d, which a slower neighbour may still read for its accepted step.
+    // not to their d, which a slower neighbour may still read for its accepted step; they count on the
+    // exchange of the sums below.
+    const unsigned long long *bar = &sm.xbar[comm.n & 1];
+    unsigned due = 0;
+    if (B.cr0 < B.cr1) due = (unsigned)G.nx * 8u * ((B.cr0 > 0 ? 1u : 0u) + (B.own1 < G.ny ? 1u : 0u));
     for (int j = threadIdx.x; j < n; j += kThreads) {
         const int i = j / G.nx, jx = j - i * G.nx, row = B.cr0 + i, k = (row - B.h0) * G.nx + jx;
         const float2 b = rhs(i, jx), mj = mt[k], dold = d[k];
         const float2 dj = make_float2(b.x / mj.x, b.y / mj.y);
         d[k] = dj;
-        if (i == 0 && B.cr0 > 0) *cl.map_shared_rank(halo + G.nx + jx, rank - 1) = dj;
-        if (row == B.cr1 - 1 && B.own1 < G.ny) *cl.map_shared_rank(halo + jx, rank + 1) = dj;
+        if (i == 0 && B.cr0 > 0) send8(halo + G.nx + jx, bar, rank - 1, dj);
+        if (row == B.cr1 - 1 && B.own1 < G.ny) send8(halo + jx, bar, rank + 1, dj);
         const float yx = dold.x - dj.x, yy = dold.y - dj.y;
         ff_acc(hi[0], lo[0], fmaf(mj.x * dj.x, dj.x, mj.y * dj.y * dj.y));
         ff_acc(hi[1], lo[1], fmaf(mj.x * dold.x, yx, mj.y * dold.y * yy));
         ff_acc(hi[2], lo[2], fmaf(mj.x * yx, yx, mj.y * yy * yy));
         mx = fmaxf(mx, fmaf(dj.x, dj.x, dj.y * dj.y));
     }
-    cluster_reduce<3, true>(hi, lo, mx, sm, buf, cl);
+    cluster_reduce<3, true>(hi, lo, mx, sm, comm, cl, due);
     for (int j = threadIdx.x; j < 2 * G.nx; j += kThreads) {
         const bool below = j >= G.nx;
         const int row = below ? B.own1 : B.cr0 - 1;
@@ -1520,7 +1631,7 @@ __device__ __forceinline__ float2 grid_eval_global(const float2 *q, const Grid &
 }
 
 template <typename S, int R>
-__device__ void run_nonrigid(const Params &p, const OpDesc &op, int op_index, Smem &sm, float2 *gbuf,
+__device__ void run_nonrigid(const Params &p, const OpDesc &op, int op_index, Smem &sm, float2 *gbuf, Comm &comm,
                              const cg::cluster_group &cl)
 {
     const int tid = threadIdx.x;
@@ -1535,9 +1646,8 @@ __device__ void run_nonrigid(const Params &p, const OpDesc &op, int op_index, Sm
     const int held = (B.h1 - B.h0) * G.nx, first = B.h0 * G.nx;   // points held, and the first of them
     float2 *c = gbuf + lay.c, *d = gbuf + lay.d, *mt = gbuf + lay.mt, *halo = gbuf + lay.halo;
     float *slots = (float *)(gbuf + lay.slots);
-    const float *above = rank > 0 && B.cr0 < B.cr1 ? cl.map_shared_rank(slots, rank - 1) : nullptr;
+    const float *above = (const float *)(gbuf + lay.above);
     const H1Bufs hb{h1 ? mt : nullptr, (float2 *)slots, (float2 *)slots + Nc, p.h1q, (float)(cfg.sigma * cfg.sigma)};
-    int buf = 0;
     // initial control values (finest px), scaled to the coarsest level
     {
         const float sc = ldexpf(1.f, -(Lc - 1));
@@ -1586,9 +1696,12 @@ __device__ void run_nonrigid(const Params &p, const OpDesc &op, int op_index, Sm
         __syncthreads();
         for (bool start = true;; start = false) {
             const float tau = sm.pm[kPmTau];   // not read by a level's first pass
-            if (start) grid_pass<S, true, R>(L, G, GL, P, B, c, d, 0.f, slots, sm, buf, cl);
-            else grid_pass<S, false, R>(L, G, GL, P, B, c, d, tau, slots, sm, buf, cl);
-            if (tid == 0) sm.action = field_eval(k, cfg, sm.tot, start, sm.pm, sm.idata[0]);
+            if (start) grid_pass<S, true, R>(L, G, GL, P, B, c, d, 0.f, slots, above, sm, comm, cl);
+            else grid_pass<S, false, R>(L, G, GL, P, B, c, d, tau, slots, above, sm, comm, cl);
+            if (tid == 0) {
+                sm.action = field_eval(k, cfg, sm.tot, start, sm.pm, sm.idata[0]);
+                if (sm.fail) sm.action = kActDone;
+            }
             __syncthreads();
             const int act = sm.action;
             if (sm.idata[0]) {
@@ -1605,9 +1718,12 @@ __device__ void run_nonrigid(const Params &p, const OpDesc &op, int op_index, Sm
 #pragma unroll
             for (int q = 0; q < 6; ++q) pm[q] = sm.pm[q];
             if (start && cfg.metric == REG_METRIC_GAUSS_NEWTON)
-                grid_metric(G, P, B, slots, above, mt, pm[kPmDk], pm[kPmRk], sm, buf, cl);
-            grid_direction(G, L, P, B, c, d, mt, halo, slots, above, pm, sm, buf, cl, hb);
-            if (tid == 0) sm.action = field_grad(k, cfg, sm.tot, sm.tmax, sm.pm);
+                grid_metric(G, P, B, slots, above, mt, pm[kPmDk], pm[kPmRk], sm, comm, cl);
+            grid_direction(G, L, P, B, c, d, mt, halo, slots, above, pm, sm, comm, cl, hb);
+            if (tid == 0) {
+                sm.action = field_grad(k, cfg, sm.tot, sm.tmax, sm.pm);
+                if (sm.fail) sm.action = kActDone;
+            }
             __syncthreads();
             if (sm.action == kActDone) break;
         }
@@ -1626,7 +1742,7 @@ __device__ void run_nonrigid(const Params &p, const OpDesc &op, int op_index, Sm
         ff_acc(hi[1], lo[1], v.y);
     }
     __threadfence();   // before the cluster's first CTA publishes the node
-    cluster_reduce<2, false>(hi, lo, 0.f, sm, buf, cl);
+    cluster_reduce<2, false>(hi, lo, 0.f, sm, comm, cl);
     if (tid == 0 && rank == 0) {
         double *th = p.node_theta + 3 * op.out;
         th[0] = 0.0;
@@ -1642,7 +1758,7 @@ __device__ void run_nonrigid(const Params &p, const OpDesc &op, int op_index, Sm
             st.stop[l] = v ? stops[l] : 0;
         }
         st.rejects = k.rejects;
-        st.status = kDevOk;
+        st.status = sm.fail;
         st.energy = k.E;
         st.theta[0] = th[0]; st.theta[1] = th[1]; st.theta[2] = th[2];
     }
@@ -1690,7 +1806,7 @@ __device__ bool op_valid(const Params &p, const OpDesc &op)
 }
 
 template <int MODE, typename S, int U>
-__device__ void run_op(const Params &p, int op_index, Smem &sm, float2 *gbuf, const cg::cluster_group &cl)
+__device__ void run_op(const Params &p, int op_index, Smem &sm, float2 *gbuf, Comm &comm, const cg::cluster_group &cl)
 {
     const OpDesc op = p.ops[op_index];
     if (!op_valid(p, op)) {
@@ -1700,9 +1816,12 @@ __device__ void run_op(const Params &p, int op_index, Smem &sm, float2 *gbuf, co
         }
         return;
     }
-    if constexpr (MODE == REG_RIGID) run_rigid<S>(p, op, op_index, sm, cl);
+    if constexpr (MODE == REG_RIGID) run_rigid<S>(p, op, op_index, sm, comm, cl);
     else if constexpr (MODE == kModeMock) run_mock(p, op, op_index, cl);
-    else run_nonrigid<S, U / 2>(p, op, op_index, sm, gbuf, cl);
+    else run_nonrigid<S, U / 2>(p, op, op_index, sm, gbuf, comm, cl);
+    if constexpr (MODE != kModeMock) {
+        if (threadIdx.x == 0 && sm.fail) atomicCAS(p.status, 0, sm.fail);
+    }
 }
 
 // Batched launch: cluster q of the grid runs operator op_base + q.  MINB: CTAs per SM the register
@@ -1716,8 +1835,11 @@ __global__ void __launch_bounds__(kThreads, MINB) op_kernel(Params p)
     __shared__ Smem sm;
     extern __shared__ __align__(16) float2 gbuf[];   // nonrigid: control grid c, d, ct, gp
     cg::cluster_group cl = cg::this_cluster();
+    Comm comm{0};
+    if (threadIdx.x == 0) comm_init(sm);
+    cl.sync();   // every CTA's barriers are set before a peer sends
     const int q = blockIdx.x / cl.num_blocks();
-    run_op<MODE, S, U>(p, p.op_base + q, sm, gbuf, cl);
+    run_op<MODE, S, U>(p, p.op_base + q, sm, gbuf, comm, cl);
     cl.sync();   // no CTA leaves while a peer may still read its shared memory
 }
 
@@ -1730,6 +1852,8 @@ __global__ void __launch_bounds__(kThreads, MINB) persistent_kernel(Params p)
     extern __shared__ __align__(16) float2 gbuf[];
     cg::cluster_group cl = cg::this_cluster();
     const bool leader = cl.block_rank() == 0 && threadIdx.x == 0;
+    Comm comm{0};
+    if (threadIdx.x == 0) comm_init(sm);   // before the cluster barriers of the first claim
     for (;;) {
         if (leader) {
             // claim the first ready operator of the most urgent non-empty class; every operator
@@ -1825,7 +1949,7 @@ __global__ void __launch_bounds__(kThreads, MINB) persistent_kernel(Params p)
         const int op = *cl.map_shared_rank(&sm.idata[1], 0);
         cl.sync();
         if (op < 0) break;
-        run_op<MODE, S, U>(p, op, sm, gbuf, cl);
+        run_op<MODE, S, U>(p, op, sm, gbuf, comm, cl);
         cl.sync();
         if (cl.block_rank() == 0) {
             // publish the produced node and release its consumers, spread over the CTA's threads (a
@@ -1877,10 +2001,12 @@ __global__ void __launch_bounds__(kThreads) energy_kernel(Params p, const double
     extern __shared__ __align__(16) float2 gbuf[];
     cg::cluster_group cl = cg::this_cluster();
     const int tid = threadIdx.x;
-    int buf = 0;
     const Lvl L = level_of(p, 0, 1, 0);
     const int C = cl.num_blocks(), rank = cl.block_rank();
     const bool first = tid == 0 && rank == 0;
+    Comm comm{0};
+    if (tid == 0) comm_init(sm);
+    cl.sync();
     if constexpr (MODE == REG_RIGID) {
         RigidCtl &k = sm.rctl;
         if (tid == 0) {
@@ -1894,7 +2020,7 @@ __global__ void __launch_bounds__(kThreads) energy_kernel(Params p, const double
         strip_rows(L.H, rank, C, r0, r1);
         float pm[6];
         for (int q = 0; q < 6; ++q) pm[q] = sm.pm[q];
-        rigid_pass<S, true>(L, r0, r1, pm, sm, buf, cl);
+        rigid_pass<S, true>(L, r0, r1, pm, sm, comm, cl);
         if (first) {
             set_reference(k.ls, sm.tot[3], sm.tot[4]);
             const Ncc n = ncc_terms(k.ls, sm.tot[0], sm.tot[1], sm.tot[2]);
@@ -1908,7 +2034,7 @@ __global__ void __launch_bounds__(kThreads) energy_kernel(Params p, const double
         const Band B = grid_band(G, rank, C);
         float2 *c = gbuf + lay.c, *d = gbuf + lay.d, *mt = gbuf + lay.mt, *halo = gbuf + lay.halo;
         float *slots = (float *)(gbuf + lay.slots);
-        const float *above = rank > 0 && B.cr0 < B.cr1 ? cl.map_shared_rank(slots, rank - 1) : nullptr;
+        const float *above = (const float *)(gbuf + lay.above);
         for (int j = tid; j < (B.h1 - B.h0) * G.nx; j += kThreads) {
             c[j] = cgrid[B.h0 * G.nx + j];
             d[j] = make_float2(0.f, 0.f);
@@ -1917,7 +2043,7 @@ __global__ void __launch_bounds__(kThreads) energy_kernel(Params p, const double
         __syncthreads();
         const GridLvl GL = grid_level(G, L, 0);
         const PassGeom P = pass_geom(G.s, G.nx - 1, B.q, L.W > (G.nx - 1) * G.s);
-        grid_pass<S, true, 2>(L, G, GL, P, B, c, d, 0.f, slots, sm, buf, cl);
+        grid_pass<S, true, 2>(L, G, GL, P, B, c, d, 0.f, slots, above, sm, comm, cl);
         FieldCtl &k = sm.fctl;
         if (tid == 0) {
             k.ls.P = (double)L.W * L.H;
@@ -1931,7 +2057,7 @@ __global__ void __launch_bounds__(kThreads) energy_kernel(Params p, const double
         if (grad_c) {
             float pm[4];
             for (int q = 0; q < 4; ++q) pm[q] = sm.pm[q];
-            grid_direction(G, L, P, B, c, d, mt, halo, slots, above, pm, sm, buf, cl, H1Bufs{});
+            grid_direction(G, L, P, B, c, d, mt, halo, slots, above, pm, sm, comm, cl, H1Bufs{});
             // d = -Nc dE/dc (unit scalar product)
             const float s = -1.f / (float)Nc;
             const float2 *own = d + (B.cr0 - B.h0) * G.nx;
