@@ -35,45 +35,59 @@ constexpr int kNM = 16;        // sums per reduction at most
 constexpr int kMaxCluster = 16; // CTAs per operator at most (non-portable cluster size)
 
 // ------------------------------------------------------------------ shared state
-// Step-controller state (FP64), used by thread 0 (rigid: warp 0) of each CTA only: kept in shared
-// memory so it does not occupy registers of every thread.
+// Step-controller state, used by thread 0 (rigid: warp 0) of each CTA only: kept in shared memory so it
+// does not occupy registers of every thread.  Energies, gradients and the tests on them are FP64, step
+// lengths FP32 (the length a step is taken with).  An FP64 instruction, conversions among them, takes 64
+// cycles of its warp on this GPU however many lanes take part, a compare 105, an FP32 one 4: the
+// controllers are written for few FP64 instructions.
 struct LevelSums {
     double P, invP, sr, Srr;       // pixels; sum of the reference's shifted samples; S'_RR
+    double least;                  // a centred sum of squares below this is a constant image
+    float Pf, Srrf, rbar;          // P, S'_RR and the mean of the reference's shifted samples in FP32
 };
 
 struct RigidCtl {
     LevelSums ls;
-    double th[3], tt[3], d[3], dp[3];   // dp: the direction of the last accepted step
-    double E, tau, slope, m0, inv_m0;
-    double tau_acc;                // length of the last accepted step (along dp)
-    int nrej, iters, evals, stop, rejects, have_prev;
+    double th[3], tt[3], d[3];
+    double E, slope, m0, inv_m0;
+    double accept, rel;            // a trial is accepted up to the first energy, and ends the level from the second
     double tolg2;  // the level's stop tolerance (tol_grad, times tol_coarse above the finest level), squared
+    double dp[3];                  // direction of the last accepted step
+    float tau, tau_acc;            // length of the trial step, and of the last accepted one
+    float m0f;                     // m0 in FP32
+    int nrej, iters, evals, stop, rejects, have_prev;
 };
 
 struct FieldCtl {
     LevelSums ls;
-    double E, tau, tau_acc, slope, invNc, half_lam;   // half_lam: lambda / (2 P)
-    double Eold, slope_old, tau_old;   // of the last accepted step, for its quadratic rule
+    double E, ss, invNc, half_lam; // ss: sum_j m_j |d_j|^2; half_lam: lambda / (2 P)
+    double accept, rel;            // a trial is accepted up to the first energy, and ends the level from the second
+    double Eold, ss_old;           // before the last accepted step, for its quadratic rule
+    double tolss;  // the level's stop tolerance (tol_grad, times tol_coarse above the finest level), squared, times Nc
+    float tau, tau_acc;            // length of the trial step, and of the last accepted one
     int nrej, iters, evals, stop, rejects, have_prev;
-    double tolg2;  // the level's stop tolerance (tol_grad, times tol_coarse above the finest level), squared
 };
 
-// x >= 0, false for a NaN, from the bits: a double-precision compare takes 105 cycles on this GPU, a
-// double-precision operation 64 (an FP32 one 4), so the controller's chains are kept short in both.
+// x >= 0, false for a NaN, from the bits.
 __device__ __forceinline__ bool nonneg(double x)
 {
     return (unsigned)__double2hiint(x) <= 0x7ff00000u;
+}
+
+// x >= y for y >= 0, false for a NaN, from the bits (those of non-negative values order as integers).
+__device__ __forceinline__ bool at_least(double x, double y)
+{
+    return __double_as_longlong(x) >= __double_as_longlong(y) && nonneg(x);
 }
 
 // First trial of a line search after an accepted step (Barzilai and Borwein, "Two-point step size
 // gradient methods", 1988, their second step): tau = tau_acc <d_prev, d_prev - d> / |d_prev - d|^2
 // in the flow's metric, given num = <d_prev, d_prev - d> and den = |d_prev - d|^2; false without
 // positive curvature.  The ratio needs no more than FP32 relative precision.
-__device__ __forceinline__ bool bb_tau(double tau_acc, double num, double den, double &tau)
+__device__ __forceinline__ bool bb_tau(float tau_acc, float num, float den, float &tau)
 {
-    const float nf = (float)num, df = (float)den;
-    if (!(nf > 0.f && df > 0.f)) return false;
-    tau = tau_acc * num * (double)__frcp_rn(df);
+    if (!(num > 0.f && den > 0.f)) return false;
+    tau = tau_acc * (num * __frcp_rn(den));
     return true;
 }
 
@@ -83,7 +97,7 @@ struct Smem {
     double tot[kNM];            // cluster totals
     unsigned wmax[kWarps], pmax[2][kMaxCluster];   // bits of the per-warp and per-CTA maxima
     unsigned long long xbar[2]; // mbarriers of the exchanges, used in turn
-    double tmax;
+    float tmax;
     float pm[16];               // pass parameters broadcast by thread 0
     int action;
     int idata[4];
@@ -251,7 +265,7 @@ __device__ __forceinline__ void cluster_reduce(const float (&hi)[NM], const floa
         if (lane < N2) sm.tot[m] = s;
         if constexpr (MAXV) {
             const unsigned v = __reduce_max_sync(0xffffffffu, lane < C ? sm.pmax[b][lane] : 0u);
-            if (lane == 0) sm.tmax = (double)__uint_as_float(v);
+            if (lane == 0) sm.tmax = __uint_as_float(v);
         }
     }
     __syncthreads();
@@ -260,60 +274,55 @@ __device__ __forceinline__ void cluster_reduce(const float (&hi)[NM], const floa
 // ------------------------------------------------------------------ NCC (FP64)
 struct Ncc {
     double e;                  // 1 - NCC
-    double a, bma;             // dNCC/dTw(x) = a (r - rbar) - b (t - tbar): a and b - a
-    double tbar, dbar;         // mean of t, and tbar - rbar
-    double Stt;
-    bool degenerate;
+    double a, u;               // 1 / sqrt(S'_RR S'_TT), S'_RE + S'_EE
+    double dbar, Stt;          // mean of t - r, S'_TT
 };
 
-// 1/sqrt(q) for a positive normal q without a double-precision divide or square root: the hardware
-// reciprocal-square-root approximation y (about 20 bits) and one third-order step, with h = 1 - q y^2
-// y (1 + h/2 + 3/8 h^2), whose error is 5/16 h^3.
-__device__ __forceinline__ double rsqrt_f64(double q)
-{
-    double y;
-    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(q));
-    const double h = __fma_rn(-q, __dmul_rn(y, y), 1.0);
-    return __fma_rn(y, __dmul_rn(h, __fma_rn(0.375, h, 0.5)), y);
-}
-
-// NCC and its gradient coefficients from the shifted sums: of r (LevelSums) and of the difference e =
-// t - r: sum e, sum e^2, sum r e.  With S'_TT = S'_RR + 2 S'_RE + S'_EE and S'_RT = S'_RR + S'_RE the
+// NCC and what its gradient follows from, from the shifted sums: of r (LevelSums) and of the difference
+// e = t - r: sum e, sum e^2, sum r e.  With S'_TT = S'_RR + 2 S'_RE + S'_EE and S'_RT = S'_RR + S'_RE the
 // rounding of the FP32 sums enters 1 - NCC, about (S'_EE - S'_RE^2 / S'_RR) / (2 S'_RR), relative to its
 // own size; sums of t^2 and r t enter it relative to 1, which left 1.8e-8 in an energy of 1e-3 (a
-// noiseless lattice, every run of pixels rounded alike).  a = 1 / sqrt(S'_RR S'_TT) and b = NCC / S'_TT,
-// so b - a = -a (S'_RE + S'_EE) / S'_TT.  e = 0 everywhere (T o phi equals R up to the shift: identical
-// inputs) is exactly NCC = 1, b = a and tbar = rbar, so the gradient vanishes exactly.
+// noiseless lattice, every run of pixels rounded alike).  A constant image has E = 1 and no gradient.
+// 1/sqrt: the hardware approximation y (about 20 bits) and one third-order step, with h = 1 - q y^2
+// y (1 + h/2 + 3/8 h^2), whose error is 5/16 h^3.
 __device__ __forceinline__ Ncc ncc_terms(const LevelSums &L, double se, double see, double sre)
 {
     Ncc o;
     o.dbar = __dmul_rn(se, L.invP);
-    o.tbar = __fma_rn(L.sr, L.invP, o.dbar);
     const double See = __fma_rn(-se, o.dbar, see), Sre = __fma_rn(-L.sr, o.dbar, sre);
-    const double u = __dadd_rn(Sre, See), Srt = __dadd_rn(L.Srr, Sre);
-    o.Stt = __dadd_rn(Srt, u);
-    o.degenerate = !nonneg(__fma_rn(-1e-12, L.P, L.Srr)) || !nonneg(__fma_rn(-1e-12, L.P, o.Stt));
-    if (o.degenerate) {
-        o.e = 1.0; o.a = 0.0; o.bma = 0.0;
-        return o;
-    }
-    const double a = rsqrt_f64(__dmul_rn(L.Srr, o.Stt));
-    o.a = a;
-    if (Sre == 0.0 && See == 0.0) {
-        o.e = 0.0;
-        o.bma = 0.0;
-    } else {
-        o.e = __fma_rn(-Srt, a, 1.0);
-        o.bma = __dmul_rn(-a, __dmul_rn(__dmul_rn(L.Srr, u), __dmul_rn(a, a)));
+    const double Srt = __dadd_rn(L.Srr, Sre);
+    o.u = __dadd_rn(Sre, See);
+    o.Stt = __dadd_rn(Srt, o.u);
+    const double q = __dmul_rn(L.Srr, o.Stt);
+    double y;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(q));
+    const double h = __fma_rn(-q, __dmul_rn(y, y), 1.0);
+    o.a = __fma_rn(y, __dmul_rn(h, __fma_rn(0.375, h, 0.5)), y);
+    o.e = __fma_rn(-Srt, o.a, 1.0);
+    // e = 0 everywhere (T o phi equals R up to the shift: identical inputs) is exactly NCC = 1
+    if ((__double_as_longlong(Sre) | __double_as_longlong(See)) << 1 == 0) o.e = 0.0;
+    if (__double_as_longlong(L.Srr) < __double_as_longlong(L.least) ||
+        __double_as_longlong(o.Stt) < __double_as_longlong(L.least)) {
+        o.e = 1.0; o.a = 0.0;
     }
     return o;
 }
 
-// The reference's part of a level's sums.
+// A level's constants, and the reference's part of its sums (known after the first pass).
+__device__ __forceinline__ void set_level(LevelSums &L, int W, int H)
+{
+    L.P = (double)W * (double)H;
+    L.invP = 1.0 / L.P;
+    L.least = 1e-12 * L.P;
+    L.Pf = (float)L.P;
+}
 __device__ __forceinline__ void set_reference(LevelSums &L, double sr, double srr)
 {
+    const double rbar = __dmul_rn(sr, L.invP);
     L.sr = sr;
-    L.Srr = __fma_rn(-sr, __dmul_rn(sr, L.invP), srr);
+    L.Srr = __fma_rn(-sr, rbar, srr);
+    L.Srrf = (float)L.Srr;
+    L.rbar = (float)rbar;
 }
 
 // ------------------------------------------------------------------ level access
@@ -547,15 +556,16 @@ enum Action { kActGrad = 0, kActTrial = 1, kActDone = 2 };
 // cancellation) and sin(alpha); the fractional and the integer part of Gx and Gy.
 __device__ __forceinline__ void rigid_param(double v, int q, int lane, float *pm)
 {
+    const float vf = (float)v, i = fminf(fmaxf(rintf(vf), -4.0e6f), 4.0e6f);
+    const float frac = (float)(v - (double)i);
     float h, ch;
-    sincosf(q == 0 ? 0.5f * (float)v : 0.f, &h, &ch);
-    const double i = rint(v);
+    sincosf(q == 0 ? 0.5f * vf : 0.f, &h, &ch);
     if (lane == 0) {
         pm[0] = -2.f * h * h;
         pm[1] = 2.f * h * ch;
     } else if (lane < 3) {
-        pm[1 + lane] = (float)(v - i);
-        pm[3 + lane] = fminf(fmaxf((float)i, -4.0e6f), 4.0e6f);
+        pm[1 + lane] = frac;
+        pm[3 + lane] = i;
     }
 }
 
@@ -564,22 +574,24 @@ __device__ __forceinline__ void rigid_param(double v, int q, int lane, float *pm
 // parabola through E(0) = E, E'(0) = slope and E(tau) = Et; a rejected trial retries at tq
 // clamped to [0.1 tau, 0.5 tau], an accepted one starts the next search at tq clamped to
 // [0.5 tau, 4 tau]; without positive curvature the rule halves / doubles.
-__device__ __forceinline__ double next_tau(double E, double slope, double tau, double Et, bool accepted)
+__device__ __forceinline__ float next_tau(double E, double slope, float tau, double Et, bool accepted)
 {
-    const double den = Et - E - slope * tau;
-    if (!(den > 0.0)) return accepted ? 2.0 * tau : 0.5 * tau;
+    const double st = __dmul_rn(slope, (double)tau);
+    const float den = (float)(Et - E - st);
+    if (!(den > 0.f)) return accepted ? 2.f * tau : 0.5f * tau;
     // a step-size estimate needs no more than FP32 relative precision once den is formed
-    const double tq = (-slope * tau * tau) * (double)__frcp_rn((float)(2.0 * den));
-    return accepted ? fmin(fmax(tq, 0.5 * tau), 4.0 * tau) : fmin(fmax(tq, 0.1 * tau), 0.5 * tau);
+    const float tq = -(float)st * tau * __frcp_rn(2.f * den);
+    return accepted ? fminf(fmaxf(tq, 0.5f * tau), 4.f * tau) : fminf(fmaxf(tq, 0.1f * tau), 0.5f * tau);
 }
 
 // Gradient component q at the point of a pass from its sums and the point's NCC terms: dE/dtheta_q = a
-// sum (t - r) g_q + (b - a) sum t g_q + (a rbar - b tbar) sum g_q, the last coefficient being -a (tbar -
-// rbar) - (b - a) tbar; exact zeros for identical frames.
-__device__ __forceinline__ double rigid_gradient(const Ncc &n, const double *tot, int q)
+// sum (t - r) g_q + (b - a) sum t g_q + (a rbar - b tbar) sum g_q, with b = NCC / S'_TT, so b - a = -a^3
+// S'_RR u, and a rbar - b tbar = -a (tbar - rbar) - (b - a) tbar; exact zeros for identical frames.
+__device__ __forceinline__ double rigid_gradient(const LevelSums &L, const Ncc &n, const double *tot, int q)
 {
-    const double kap = __fma_rn(-n.bma, n.tbar, -__dmul_rn(n.a, n.dbar));
-    return n.a * tot[5 + q] + n.bma * tot[8 + q] + kap * tot[11 + q];
+    const double bma = __dmul_rn(__dmul_rn(__dmul_rn(-n.a, n.a), n.a), __dmul_rn(L.Srr, n.u));
+    const double kap = __fma_rn(-bma, __fma_rn(L.sr, L.invP, n.dbar), -__dmul_rn(n.a, n.dbar));
+    return __fma_rn(n.a, tot[5 + q], __fma_rn(bma, tot[8 + q], __dmul_rn(kap, tot[11 + q])));
 }
 
 // v of lanes 0, 1 and 2 added in that order, in every lane.
@@ -591,8 +603,7 @@ __device__ __forceinline__ double sum3(double v)
 // Controller after a pass at a level's start or at a trial point: the energy there, the Armijo test, and
 // where the point is taken the stop tests, the direction and the next trial.  Returns the next action
 // and writes its parameters.  Same rules as the oracle's level loop.  Run by one warp: lane q < 3 has
-// parameter q, every lane the scalars (one thread doing all of it took 7,000 of the 19,000 cycles of
-// an iteration at 160x128).
+// parameter q, every lane the scalars.
 __device__ int rigid_step(RigidCtl &k, const Config &cfg, const double *tot, bool start, float *pm)
 {
     const int lane = threadIdx.x & 31, q = min(lane, 2);
@@ -601,21 +612,20 @@ __device__ int rigid_step(RigidCtl &k, const Config &cfg, const double *tot, boo
         __syncwarp();
     }
     const Ncc n = ncc_terms(k.ls, tot[0], tot[1], tot[2]);
-    const double Et = n.e, Eold = k.E, slope_old = k.slope, tau_old = k.tau;
-    double th = k.th[q], d = k.d[q], dp = k.dp[q], tau = k.tau, tau_acc = k.tau_acc;
-    int evals = k.evals + (start ? 0 : 1), iters = k.iters, have_prev = k.have_prev, nrej = k.nrej;
-    bool fresh = start;   // the first point of the level: no step, no previous direction
-    int act = kActTrial;
-    if (!start && !nonneg(Eold + cfg.armijo_c * tau_old * slope_old - Et)) {
+    const double Et = n.e, Eold = k.E, slope_old = k.slope;
+    const float tau_old = k.tau;
+    double th = k.th[q], d = k.d[q], E = Et, slope = slope_old, accept = k.accept, rel = k.rel;
+    double dp = k.dp[q];
+    float tau = tau_old, tau_acc = k.tau_acc;
+    int evals = k.evals + (start ? 0 : 1), iters = k.iters, have_prev = k.have_prev, nrej = k.nrej, rejects = k.rejects;
+    int stop = -1;
+    const bool taken = start || nonneg(accept - Et);
+    if (!taken) {
+        E = Eold;
         tau = next_tau(Eold, slope_old, tau_old, Et, false);
+        rejects += 1;
         nrej += 1;
-        if (lane == 0) k.rejects += 1;
-        if (nrej > cfg.max_rejects) {
-            if (lane == 0) k.stop = REG_STOP_LS;
-            act = kActDone;
-        }
-        fresh = false;
-        __syncwarp();
+        if (nrej > cfg.max_rejects) stop = REG_STOP_LS;
     } else {
         if (!start) {
             th = k.tt[q];
@@ -624,46 +634,47 @@ __device__ int rigid_step(RigidCtl &k, const Config &cfg, const double *tot, boo
             have_prev = 1;
             iters += 1;
         }
-        int stop = -1;
-        if (!fresh && nonneg(cfg.tol_rel_e * fabs(Eold) - (Eold - Et))) {
+        if (!start && nonneg(Et - rel)) {
             stop = REG_STOP_REL;
-            tau = next_tau(Eold, slope_old, tau_old, Et, true);
         } else {
             evals += 1;
-            const double im = q == 0 ? k.inv_m0 : 1.0, g = rigid_gradient(n, tot, q);
-            d = -g * im;
-            const double slope = sum3(g * d);
-            // |g|_M = sqrt(-slope); the tests compare squares (no square root unless the cap applies)
+            const double g = rigid_gradient(k.ls, n, tot, q);
+            d = q == 0 ? -g * k.inv_m0 : -g;
+            slope = sum3(g * d);
+            // |g|_M = sqrt(-slope); the tests compare squares
             if (iters >= cfg.max_iter) stop = REG_STOP_MAXIT;
-            else if (!nonneg(-slope - k.tolg2)) stop = REG_STOP_GRAD;
+            else if (!at_least(-slope, k.tolg2)) stop = REG_STOP_GRAD;
             else {
-                const double w = q == 0 ? k.m0 : 1.0, y = dp - d;
-                const double num = sum3(w * dp * y), den = sum3(w * y * y);
-                if (!have_prev || !bb_tau(tau_acc, num, den, tau))
-                    tau = start ? tau_old : next_tau(Eold, slope_old, tau_old, Et, true);
-                const double gn2 = -slope;
-                if (!nonneg(cfg.step_cap * cfg.step_cap - tau * tau * gn2)) tau = cfg.step_cap * rsqrt_f64(gn2);
+                if (have_prev) {
+                    const float w = q == 0 ? k.m0f : 1.f, y = (float)(dp - d);
+                    const float a = w * (float)dp * y, b = w * y * y;
+                    const float num = __shfl_sync(0xffffffffu, a, 0) + __shfl_sync(0xffffffffu, a, 1) + __shfl_sync(0xffffffffu, a, 2);
+                    const float den = __shfl_sync(0xffffffffu, b, 0) + __shfl_sync(0xffffffffu, b, 1) + __shfl_sync(0xffffffffu, b, 2);
+                    if (!bb_tau(tau_acc, num, den, tau)) tau = next_tau(Eold, slope_old, tau_old, Et, true);
+                }
+                const float gn2 = (float)-slope, cap = (float)cfg.step_cap;
+                if (tau * tau * gn2 > cap * cap) tau = cap / sqrtf(gn2);
                 nrej = 0;
+                rel = cfg.tol_rel_e == 0.0 ? E : E - cfg.tol_rel_e * fabs(E);
             }
-            __syncwarp();
-            if (lane == 0) k.slope = slope;
         }
-        if (stop >= 0) {
-            if (lane == 0) k.stop = stop;
-            act = kActDone;
-        }
-        __syncwarp();
-        if (lane < 3) { k.th[q] = th; k.d[q] = d; k.dp[q] = dp; }
-        if (lane == 0) { k.E = Et; k.tau_acc = tau_acc; k.iters = iters; k.have_prev = have_prev; }
     }
-    if (lane == 0) { k.tau = tau; k.nrej = nrej; k.evals = evals; }
-    if (act == kActTrial) {
-        const double tt = th + tau * d;
+    __syncwarp();   // every lane has read the state
+    if (stop < 0) {
+        const double taud = (double)tau, tt = __fma_rn(taud, d, th);
+        accept = __fma_rn(cfg.armijo_c * slope, taud, E);
         if (lane < 3) k.tt[q] = tt;
         rigid_param(tt, q, lane, pm);
     }
+    if (lane < 3) { k.th[q] = th; k.d[q] = d; k.dp[q] = dp; }
+    if (lane == 0) {
+        k.E = E; k.slope = slope; k.accept = accept; k.rel = rel;
+        k.tau = tau; k.tau_acc = tau_acc;
+        k.nrej = nrej; k.rejects = rejects; k.iters = iters; k.evals = evals; k.have_prev = have_prev;
+        if (stop >= 0) k.stop = stop;
+    }
     __syncwarp();
-    return act;
+    return stop >= 0 ? kActDone : kActTrial;
 }
 
 __device__ __forceinline__ Lvl level_of(const Params &p, int ref, int tmpl, int l)
@@ -712,12 +723,12 @@ __device__ void run_rigid(const Params &p, const OpDesc &op, int op_index, Smem 
         int r0, r1;
         strip_rows(L.H, rank, C, r0, r1);
         if (tid == 0) {
-            k.ls.P = (double)L.W * (double)L.H;
-            k.ls.invP = 1.0 / k.ls.P;
+            set_level(k.ls, L.W, L.H);
             double rho = 0.25 * (L.W + L.H);
             k.m0 = rho * rho;
             k.inv_m0 = 1.0 / k.m0;
-            k.tau = cfg.tau0;
+            k.m0f = (float)k.m0;
+            k.tau = (float)cfg.tau0;
             k.have_prev = 0;
             k.iters = 0; k.evals = 0; k.stop = REG_STOP_MAXIT;
             // a coarse level only supplies the next level's initial guess: a looser stop
@@ -819,6 +830,22 @@ __host__ __device__ __forceinline__ int band_cells(int gny, int C)
     return (gny - 1 + C - 1) / C;
 }
 
+// Points j = tid, tid + kThreads, ... of rows of nx points as (row, column): the first without a
+// division, and it is the only one of a thread where a band has up to kThreads points.
+struct PointIter {
+    int i0, x0;
+    __device__ __forceinline__ explicit PointIter(int nx)
+    {
+        i0 = (int)threadIdx.x / nx;
+        x0 = (int)threadIdx.x - i0 * nx;
+    }
+    __device__ __forceinline__ static void at(int nx, int j, int &i, int &x)
+    {
+        i = j / nx;
+        x = j - i * nx;
+    }
+};
+
 // The rows of a CTA: cell rows [cr0, cr1); control rows [cr0, own1) are its own (the last band
 // owns the grid's last row too); rows [h0, h1) are held in shared memory.
 struct Band {
@@ -851,9 +878,21 @@ __device__ __forceinline__ Band grid_band(const Grid &G, int rank, int C)
 struct PassGeom {
     int sl, g, chunks;    // cell width, cells per strip, strips per cell (wide cells)
     int ns, nst;          // strips of cells, strips
-    int m, h, ph;         // cell rows per segment, pieces per cell row, pixel rows per piece
-    int nseg;
+    int m, h, ph;         // cell rows per segment, pieces per cell row (a power of two), pixel rows per piece
+    int nseg, hlog;       // segments, log2 of h
+    unsigned rm, rg;      // reciprocals for div20: of m and g
 };
+
+// a / b for a b < 2^20, r = recip20(b): the integer divisions of a pass's set-up take longer than the rows
+// of a small frame.
+__host__ __device__ __forceinline__ unsigned recip20(int b)
+{
+    return (1u << 20) / (unsigned)b + 1u;
+}
+__host__ __device__ __forceinline__ int div20(int a, unsigned r)
+{
+    return (int)(((unsigned)a * r) >> 20);
+}
 
 __host__ __device__ inline PassGeom pass_geom(int sl, int ncx, int q, bool over)
 {
@@ -881,6 +920,9 @@ __host__ __device__ inline PassGeom pass_geom(int sl, int ncx, int q, bool over)
             P.m = 1; P.h = h; P.ph = ph; P.nseg = q * h;
         }
     }
+    P.hlog = P.h == 8 ? 3 : P.h >> 1;
+    P.rm = recip20(P.m);
+    P.rg = recip20(P.g);
     return P;
 }
 
@@ -1026,7 +1068,7 @@ template <int N>
 __device__ __forceinline__ void slot_sum(const float *slots, const PassGeom &P, int ncx, int nr, int i, int jx,
                                          int first, float (&o)[N])
 {
-    const int ga = i > 0 ? (i - 1) / P.m : 0, gb = i < nr ? i / P.m : (nr - 1) / P.m;
+    const int ga = i > 0 ? div20(i - 1, P.rm) : 0, gb = div20(i < nr ? i : nr - 1, P.rm);
     auto add = [&](int seg, int strip, int row, int pt) {
         const float *s = slots + (((size_t)(seg * P.nst + strip) * (P.m + 1) + row) * (P.g + 1) + pt) * kSlot + first;
 #pragma unroll
@@ -1036,8 +1078,9 @@ __device__ __forceinline__ void slot_sum(const float *slots, const PassGeom &P, 
             o[k + 1] += v.y;
         }
     };
-    const int st = jx / P.g, pt = jx - st * P.g;
+    const int st = div20(jx, P.rg), pt = jx - st * P.g;
     for (int grp = ga; grp <= gb; ++grp)
+#pragma unroll 4
         for (int piece = 0; piece < P.h; ++piece) {
             const int seg = grp * P.h + piece, row = i - grp * P.m;
             if (P.sl < 32) {
@@ -1066,8 +1109,8 @@ __device__ __forceinline__ void slot_sum(const float *slots, const PassGeom &P, 
 // float-float.
 template <typename S, bool START, int R>
 __device__ void grid_pass(const Lvl &L, const Grid &G, const GridLvl &GL, const PassGeom &P, const Band &B,
-                          const float2 *c, const float2 *d, float tau, float *slots, const float *above, Smem &sm,
-                          Comm &comm, const cg::cluster_group &cl)
+                          const float2 *c, const float2 *d, float tau, float *slots, const float *above, const PointIter &pi,
+                          Smem &sm, Comm &comm, const cg::cluster_group &cl)
 {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int ncx = G.nx - 1, ncy = G.ny - 1, sl = P.sl, pairs = (P.nst + 1) / 2;
@@ -1088,9 +1131,12 @@ __device__ void grid_pass(const Lvl &L, const Grid &G, const GridLvl &GL, const 
 #pragma unroll
     for (int i = 0; i < NM; ++i) hi2[i] = lo2[i] = a[i] = f2(0.f);
 
-    for (int task = warp; task < pairs * P.nseg; task += kWarps) {
-        const int seg = task / pairs, strip0 = 2 * (task - seg * pairs);
-        const int grp = seg / P.h, piece = seg - grp * P.h;
+    const int kw = sl < 32 ? div20(lane, recip20(sl)) : 0;   // the lane's cell in a strip of whole cells
+    for (int seg = 0, pr = warp;; pr += kWarps) {
+        while (pr >= pairs) { pr -= pairs; ++seg; }
+        if (seg >= P.nseg) break;
+        const int strip0 = 2 * pr;
+        const int grp = seg >> P.hlog, piece = seg & (P.h - 1);
         const int ca = B.cr0 + grp * P.m, cb = min(ca + P.m, B.cr1);
         if (ca >= cb) continue;
         // this lane's column of either strip; an idle lane repeats the last column and counts for nothing
@@ -1101,10 +1147,10 @@ __device__ void grid_pass(const Lvl &L, const Grid &G, const GridLvl &GL, const 
         for (int u = 0; u < 2; ++u) {
             const int strip = strip0 + u;
             const bool over = strip == P.ns;      // the column past the last cell
-            const int cell0 = over ? ncx - 1 : sl < 32 ? strip * P.g : strip / P.chunks;
+            const int cell0 = over ? ncx - 1 : sl < 32 ? strip * P.g : P.chunks == 1 ? strip : strip / P.chunks;
             const int c0 = min(cell0, ncx - 1);
             last[u] = over || sl >= 32 ? 0 : min(P.g, ncx - c0) - 1;
-            kl[u] = over || sl >= 32 ? 0 : lane / sl;
+            kl[u] = over ? 0 : kw;
             const int xs = over ? ncx * sl : sl < 32 ? c0 * sl : c0 * sl + (strip - cell0 * P.chunks) * 32;
             const int xe = over ? L.W : min(L.W, min(c0 * sl + (last[u] + 1) * sl, xs + 32));
             act[u] = strip < P.nst && xs + lane < xe && kl[u] <= last[u];
@@ -1309,8 +1355,10 @@ __device__ void grid_pass(const Lvl &L, const Grid &G, const GridLvl &GL, const 
     {
         float e = 0.f;
         int k = 0;
+        int i = pi.i0, col = pi.x0;
         for (int j = threadIdx.x; j < (B.own1 - B.cr0) * G.nx; j += kThreads) {
-            const int row = B.cr0 + j / G.nx, col = j % G.nx;
+            if (j >= kThreads) PointIter::at(G.nx, j, i, col);
+            const int row = B.cr0 + i;
             const float2 v = ct(row, col);
             if (col + 1 < G.nx) {
                 const float2 w = ct(row, col + 1);
@@ -1427,12 +1475,14 @@ __device__ void h1_solve(const H1Bufs &h, int nx, int ny)
 // axis m = dk sum_x w_j(x)^2 (dT/dp)^2 + rk n_j (dk = 1/(P var T), rk = lambda/P, n_j the neighbours
 // of j), normalised by the mean of all 2 Nc values and floored at 1e-3 of it, written to mt.
 __device__ void grid_metric(const Grid &G, const PassGeom &P, const Band &B, const float *slots, const float *above,
-                            float2 *mt, float dk, float rk, Smem &sm, Comm &comm, const cg::cluster_group &cl)
+                            const PointIter &pi, float2 *mt, float dk, float rk, Smem &sm, Comm &comm, const cg::cluster_group &cl)
 {
     const int n = (B.own1 - B.cr0) * G.nx;
     float hi[1] = {0.f}, lo[1] = {0.f};
+    int i = pi.i0, jx = pi.x0;
     for (int j = threadIdx.x; j < n; j += kThreads) {
-        const int i = j / G.nx, jx = j - i * G.nx, row = B.cr0 + i;
+        if (j >= kThreads) PointIter::at(G.nx, j, i, jx);
+        const int row = B.cr0 + i;
         float s[2];
         point_sum<2>(slots, above, P, B, G.nx - 1, row, jx, 6, s);
         const float nb = (float)((jx > 0) + (jx + 1 < G.nx) + (row > 0) + (row + 1 < G.ny));
@@ -1456,7 +1506,7 @@ __device__ void grid_metric(const Grid &G, const PassGeom &P, const Band &B, con
 // sm.tot[1] and |d_old - d|_M^2 in sm.tot[2], max |d_j|^2 in sm.tmax; identical in every CTA.
 __device__ void grid_direction(const Grid &G, const Lvl &L, const PassGeom &P, const Band &B, const float2 *c,
                                float2 *d, float2 *mt, float2 *halo, const float *slots, const float *above,
-                               const float *pm, Smem &sm, Comm &comm, const cg::cluster_group &cl, const H1Bufs &h1)
+                               const PointIter &pi, const float *pm, Smem &sm, Comm &comm, const cg::cluster_group &cl, const H1Bufs &h1)
 {
     const int Nc = G.nx * G.ny, n = (B.own1 - B.cr0) * G.nx, rank = cl.block_rank();
     const float aP = pm[0], bmaP = pm[1], kappa = pm[2], lam = pm[3];
@@ -1481,8 +1531,9 @@ __device__ void grid_direction(const Grid &G, const Lvl &L, const PassGeom &P, c
         // H1 product: b = -Nc dE/dc into B of every CTA, d = M^-1 b into U by every CTA; then
         // |d|_M^2 = d.b, and for the first trial <d_prev, y>_M, |y|_M^2 with y = d_prev - d, M y
         // taken as the stencil y + s2 Lg y
+        int i = pi.i0, jx = pi.x0;
         for (int j = threadIdx.x; j < n; j += kThreads) {
-            const int i = j / G.nx, jx = j - i * G.nx;
+            if (j >= kThreads) PointIter::at(G.nx, j, i, jx);
             const float2 b = rhs(i, jx);
             for (unsigned r = 0; r < cl.num_blocks(); ++r) *cl.map_shared_rank(h1.B + (B.cr0 + i) * G.nx + jx, r) = b;
         }
@@ -1492,8 +1543,11 @@ __device__ void grid_direction(const Grid &G, const Lvl &L, const PassGeom &P, c
             const float2 a = d[(row - B.h0) * G.nx + jx], b = h1.U[row * G.nx + jx];
             return make_float2(a.x - b.x, a.y - b.y);
         };
+        i = pi.i0;
+        jx = pi.x0;
         for (int j = threadIdx.x; j < n; j += kThreads) {
-            const int i = j / G.nx, jx = j - i * G.nx, row = B.cr0 + i;
+            if (j >= kThreads) PointIter::at(G.nx, j, i, jx);
+            const int row = B.cr0 + i;
             const float2 dj = h1.U[row * G.nx + jx], bj = h1.B[row * G.nx + jx], dold = d[(row - B.h0) * G.nx + jx];
             const float2 y = yv(row, jx);
             float lx = 0.f, ly = 0.f;
@@ -1518,8 +1572,10 @@ __device__ void grid_direction(const Grid &G, const Lvl &L, const PassGeom &P, c
     const unsigned long long *bar = &sm.xbar[comm.n & 1];
     unsigned due = 0;
     if (B.cr0 < B.cr1) due = (unsigned)G.nx * 8u * ((B.cr0 > 0 ? 1u : 0u) + (B.own1 < G.ny ? 1u : 0u));
+    int i = pi.i0, jx = pi.x0;
     for (int j = threadIdx.x; j < n; j += kThreads) {
-        const int i = j / G.nx, jx = j - i * G.nx, row = B.cr0 + i, k = (row - B.h0) * G.nx + jx;
+        if (j >= kThreads) PointIter::at(G.nx, j, i, jx);
+        const int row = B.cr0 + i, k = (row - B.h0) * G.nx + jx;
         const float2 b = rhs(i, jx), mj = mt[k], dold = d[k];
         const float2 dj = make_float2(b.x / mj.x, b.y / mj.y);
         d[k] = dj;
@@ -1543,13 +1599,15 @@ __device__ void grid_direction(const Grid &G, const Lvl &L, const PassGeom &P, c
 // and lambda; the scalar product's 1/(P var T) and lambda/P; the next trial's step.
 enum FieldParam { kPmA = 0, kPmB = 1, kPmK = 2, kPmLam = 3, kPmDk = 4, kPmRk = 5, kPmTau = 6 };
 
-// Gradient coefficients from a point's NCC terms; exact zeros but aP for identical frames.
+// Gradient coefficients from a point's NCC terms: b - a = -a^3 S'_RR u, formed as -(a S'_RR)(a u) a so
+// that no factor leaves the FP32 range; exact zeros but aP for identical frames.
 __device__ __forceinline__ void field_grad_params(const Ncc &n, const LevelSums &L, const Config &cfg, float *pm)
 {
-    const float b = (float)(n.bma * L.P), aP = (float)(n.a * L.P);
+    const float a = (float)n.a, dbar = (float)n.dbar, aP = a * L.Pf;
+    const float b = -(a * L.Srrf) * (a * (float)n.u) * aP;
     pm[kPmA] = aP;
     pm[kPmB] = b;
-    pm[kPmK] = -fmaf(b, (float)n.tbar, aP * (float)n.dbar);
+    pm[kPmK] = -fmaf(b, L.rbar + dbar, aP * dbar);
     pm[kPmLam] = (float)cfg.lambda;
 }
 
@@ -1572,45 +1630,50 @@ __device__ int field_eval(FieldCtl &k, const Config &cfg, const double *tot, boo
         return kActGrad;
     }
     k.evals += 1;
-    if (nonneg(k.E + cfg.armijo_c * k.tau * k.slope - Et)) {
+    if (nonneg(k.accept - Et)) {
         accepted = 1;   // c is advanced by the trial's step
         field_grad_params(n, k.ls, cfg, pm);
         k.iters += 1;
         k.Eold = k.E;
-        k.slope_old = k.slope;
-        k.tau_old = k.tau;
-        k.tau_acc = (double)(float)k.tau;   // the step applied: c + (float)tau d
+        k.ss_old = k.ss;
+        k.tau_acc = k.tau;
         k.have_prev = 1;
         k.E = Et;
-        if (nonneg(cfg.tol_rel_e * fabs(k.Eold) - (k.Eold - Et))) { k.stop = REG_STOP_REL; return kActDone; }
+        if (nonneg(Et - k.rel)) { k.stop = REG_STOP_REL; return kActDone; }
         return kActGrad;
     }
     k.rejects += 1;
     k.nrej += 1;
-    k.tau = next_tau(k.E, k.slope, k.tau, Et, false);
+    const double slope = -k.ss * k.invNc;
+    const float tau = next_tau(k.E, slope, k.tau, Et, false);
+    k.tau = tau;
     if (k.nrej > cfg.max_rejects) { k.stop = REG_STOP_LS; return kActDone; }
-    pm[kPmTau] = (float)k.tau;
+    k.accept = __fma_rn(cfg.armijo_c * slope, (double)tau, k.E);
+    pm[kPmTau] = tau;
     return kActTrial;
 }
 
 // The stop tests at a point whose direction is known, and the first trial's step.
-__device__ int field_grad(FieldCtl &k, const Config &cfg, const double *tot, double dmax2, float *pm)
+__device__ int field_grad(FieldCtl &k, const Config &cfg, const double *tot, float dmax2, float *pm)
 {
     k.evals += 1;
     if (k.iters >= cfg.max_iter) { k.stop = REG_STOP_MAXIT; return kActDone; }
     // |g| = sqrt(ss / Nc) and the largest control step dmax: compared squared
-    const double g2 = tot[0] * k.invNc;
-    k.slope = -g2;
-    if (!nonneg(g2 - k.tolg2)) { k.stop = REG_STOP_GRAD; return kActDone; }
+    const double ss = tot[0];
+    k.ss = ss;
+    if (!at_least(ss, k.tolss)) { k.stop = REG_STOP_GRAD; return kActDone; }
     // the metric (mean over control points) is a common factor of the two sums; without positive
     // curvature the quadratic rule of the last step
-    double tau = k.tau;
-    if (k.have_prev && !bb_tau(k.tau_acc, tot[1], tot[2], tau))
-        tau = next_tau(k.Eold, k.slope_old, k.tau_old, k.E, true);
-    if (!nonneg(cfg.step_cap * cfg.step_cap - tau * tau * dmax2)) tau = cfg.step_cap * rsqrt_f64(dmax2);
+    float tau = k.tau;
+    if (k.have_prev && !bb_tau(k.tau_acc, (float)tot[1], (float)tot[2], tau))
+        tau = next_tau(k.Eold, -k.ss_old * k.invNc, k.tau_acc, k.E, true);
+    const float cap = (float)cfg.step_cap;
+    if (tau * tau * dmax2 > cap * cap) tau = cap / sqrtf(dmax2);
     k.tau = tau;
     k.nrej = 0;
-    pm[kPmTau] = (float)tau;
+    k.accept = __fma_rn(-ss * (cfg.armijo_c * k.invNc), (double)tau, k.E);
+    k.rel = cfg.tol_rel_e == 0.0 ? k.E : k.E - cfg.tol_rel_e * fabs(k.E);
+    pm[kPmTau] = tau;
     return kActTrial;
 }
 
@@ -1643,6 +1706,7 @@ __device__ void run_nonrigid(const Params &p, const OpDesc &op, int op_index, Sm
     const bool h1 = cfg.metric == REG_METRIC_H1;
     const GridLayout lay = grid_layout(G.nx, G.ny, C, h1);
     const Band B = grid_band(G, rank, C);
+    const PointIter pi(G.nx);
     const int held = (B.h1 - B.h0) * G.nx, first = B.h0 * G.nx;   // points held, and the first of them
     float2 *c = gbuf + lay.c, *d = gbuf + lay.d, *mt = gbuf + lay.mt, *halo = gbuf + lay.halo;
     float *slots = (float *)(gbuf + lay.slots);
@@ -1683,21 +1747,20 @@ __device__ void run_nonrigid(const Params &p, const OpDesc &op, int op_index, Sm
         if (cfg.metric == REG_METRIC_MEAN)
             for (int j = tid; j < held; j += kThreads) mt[j] = make_float2(1.f, 1.f);
         if (tid == 0) {
-            k.ls.P = (double)L.W * (double)L.H;
-            k.ls.invP = 1.0 / k.ls.P;
+            set_level(k.ls, L.W, L.H);
             k.half_lam = 0.5 * cfg.lambda * k.ls.invP;
-            k.tau = cfg.tau0;
+            k.tau = (float)cfg.tau0;
             k.have_prev = 0;
             k.iters = 0; k.evals = 0; k.stop = REG_STOP_MAXIT;
             // a coarse level only supplies the next level's initial guess: a looser stop
             const double tolg = cfg.tol_grad * (l > 0 ? cfg.tol_coarse : 1.0);
-            k.tolg2 = tolg * tolg;
+            k.tolss = tolg * tolg * (double)Nc;
         }
         __syncthreads();
         for (bool start = true;; start = false) {
             const float tau = sm.pm[kPmTau];   // not read by a level's first pass
-            if (start) grid_pass<S, true, R>(L, G, GL, P, B, c, d, 0.f, slots, above, sm, comm, cl);
-            else grid_pass<S, false, R>(L, G, GL, P, B, c, d, tau, slots, above, sm, comm, cl);
+            if (start) grid_pass<S, true, R>(L, G, GL, P, B, c, d, 0.f, slots, above, pi, sm, comm, cl);
+            else grid_pass<S, false, R>(L, G, GL, P, B, c, d, tau, slots, above, pi, sm, comm, cl);
             if (tid == 0) {
                 sm.action = field_eval(k, cfg, sm.tot, start, sm.pm, sm.idata[0]);
                 if (sm.fail) sm.action = kActDone;
@@ -1718,8 +1781,8 @@ __device__ void run_nonrigid(const Params &p, const OpDesc &op, int op_index, Sm
 #pragma unroll
             for (int q = 0; q < 6; ++q) pm[q] = sm.pm[q];
             if (start && cfg.metric == REG_METRIC_GAUSS_NEWTON)
-                grid_metric(G, P, B, slots, above, mt, pm[kPmDk], pm[kPmRk], sm, comm, cl);
-            grid_direction(G, L, P, B, c, d, mt, halo, slots, above, pm, sm, comm, cl, hb);
+                grid_metric(G, P, B, slots, above, pi, mt, pm[kPmDk], pm[kPmRk], sm, comm, cl);
+            grid_direction(G, L, P, B, c, d, mt, halo, slots, above, pi, pm, sm, comm, cl, hb);
             if (tid == 0) {
                 sm.action = field_grad(k, cfg, sm.tot, sm.tmax, sm.pm);
                 if (sm.fail) sm.action = kActDone;
@@ -2011,8 +2074,7 @@ __global__ void __launch_bounds__(kThreads) energy_kernel(Params p, const double
         RigidCtl &k = sm.rctl;
         if (tid == 0) {
             memset(&k, 0, sizeof(k));
-            k.ls.P = (double)L.W * L.H;
-            k.ls.invP = 1.0 / k.ls.P;
+            set_level(k.ls, L.W, L.H);
         }
         if (tid < 32) rigid_param(theta[min(tid, 2)], min(tid, 2), tid, sm.pm);
         __syncthreads();
@@ -2025,13 +2087,14 @@ __global__ void __launch_bounds__(kThreads) energy_kernel(Params p, const double
             set_reference(k.ls, sm.tot[3], sm.tot[4]);
             const Ncc n = ncc_terms(k.ls, sm.tot[0], sm.tot[1], sm.tot[2]);
             out[0] = n.e;
-            for (int q = 0; q < 3; ++q) out[1 + q] = rigid_gradient(n, sm.tot, q);
+            for (int q = 0; q < 3; ++q) out[1 + q] = rigid_gradient(k.ls, n, sm.tot, q);
         }
     } else {
         const Grid G{p.gnx, p.gny, p.gs};
         const int Nc = G.nx * G.ny;
         const GridLayout lay = grid_layout(G.nx, G.ny, C, false);
         const Band B = grid_band(G, rank, C);
+        const PointIter pi(G.nx);
         float2 *c = gbuf + lay.c, *d = gbuf + lay.d, *mt = gbuf + lay.mt, *halo = gbuf + lay.halo;
         float *slots = (float *)(gbuf + lay.slots);
         const float *above = (const float *)(gbuf + lay.above);
@@ -2043,11 +2106,10 @@ __global__ void __launch_bounds__(kThreads) energy_kernel(Params p, const double
         __syncthreads();
         const GridLvl GL = grid_level(G, L, 0);
         const PassGeom P = pass_geom(G.s, G.nx - 1, B.q, L.W > (G.nx - 1) * G.s);
-        grid_pass<S, true, 2>(L, G, GL, P, B, c, d, 0.f, slots, above, sm, comm, cl);
+        grid_pass<S, true, 2>(L, G, GL, P, B, c, d, 0.f, slots, above, pi, sm, comm, cl);
         FieldCtl &k = sm.fctl;
         if (tid == 0) {
-            k.ls.P = (double)L.W * L.H;
-            k.ls.invP = 1.0 / k.ls.P;
+            set_level(k.ls, L.W, L.H);
             set_reference(k.ls, sm.tot[3], sm.tot[4]);
             const Ncc n = ncc_terms(k.ls, sm.tot[0], sm.tot[1], sm.tot[2]);
             if (first) out[0] = __fma_rn(0.5 * p.cfg.lambda * k.ls.invP, sm.tot[5], n.e);
@@ -2057,7 +2119,7 @@ __global__ void __launch_bounds__(kThreads) energy_kernel(Params p, const double
         if (grad_c) {
             float pm[4];
             for (int q = 0; q < 4; ++q) pm[q] = sm.pm[q];
-            grid_direction(G, L, P, B, c, d, mt, halo, slots, above, pm, sm, comm, cl, H1Bufs{});
+            grid_direction(G, L, P, B, c, d, mt, halo, slots, above, pi, pm, sm, comm, cl, H1Bufs{});
             // d = -Nc dE/dc (unit scalar product)
             const float s = -1.f / (float)Nc;
             const float2 *own = d + (B.cr0 - B.h0) * G.nx;
