@@ -28,7 +28,9 @@ namespace {
 constexpr int kTW = 64, kTH = 32;          // output tile
 constexpr int kBW = 80, kBH = 40;          // staged source box (tile + margins; kBW % 4 == 0)
 constexpr int kStages = 4;
-constexpr int kConsumers = 8;              // consumer warps; one more warp produces
+constexpr int kConsumers = 8;              // consumer warps; one more warp produces (4 of 8 rows: fewer
+                                           // instructions, 143 us instead of 134, too few warps)
+constexpr int kRows = kTH / kConsumers;    // rows of a tile per consumer warp
 constexpr int kRun = 16;                   // frames summed in FP32 before the float-float fold
 constexpr int kWinX = 12, kWinY = 8;       // control points under a tile (spacing >= 8)
 constexpr int kWThreads = 32 * (kConsumers + 1);
@@ -126,18 +128,48 @@ __device__ __forceinline__ Window window_of(const WarpArgs &a, int x0, int y0)
     return w;
 }
 
+// A producer lane's part of a tile's control window, the same for every frame: up to 3 points (source in a
+// grid, place in the staged window, -1: none), and the two tile columns it interpolates the window's
+// control rows at (cell relative to the window's first, weight).
+struct ProducerLane {
+    int src[3], dst[3];
+    int ix[2];
+    float wx[2];
+};
+
+__device__ __forceinline__ ProducerLane producer_lane(const WarpArgs &a, const Window &w, int x0)
+{
+    const int lane = threadIdx.x & 31;
+    ProducerLane p;
+#pragma unroll
+    for (int t = 0; t < 3; ++t) {
+        const int j = lane + 32 * t, jy = j / w.wx, jx = j - jy * w.wx;
+        const bool has = a.window && j < w.wx * w.wy;
+        p.src[t] = has ? (w.cy0 + jy) * a.nx + w.cx0 + jx : -1;
+        p.dst[t] = jy * kWinX + jx;
+    }
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        // a column past the frame edge uses the last one
+        const float gxf = fminf((float)min(x0 + lane + 32 * h, a.W - 1) * a.inv_s, (float)(a.nx - 1));
+        const int ix = cell_of(gxf, a.nx);
+        p.ix[h] = ix - w.cx0;
+        p.wx[h] = gxf - (float)ix;
+    }
+    return p;
+}
+
 // What the producer needs from global memory for one frame, loaded a frame ahead so that the
 // load latency overlaps the previous frame's work: the rigid parameters, or this lane's share
-// (up to 3 points) of the control window.
+// of the control window.
 struct Prefetch {
     float4 q;
     float2 v[3];
 };
 
-__device__ __forceinline__ Prefetch fetch(const WarpArgs &a, const Window &w, int k)
+__device__ __forceinline__ Prefetch fetch(const WarpArgs &a, const ProducerLane &pl, int k)
 {
     Prefetch f;
-    const int lane = threadIdx.x & 31;
     if (a.mode == REG_RIGID) {
         f.q = a.rigid[k];
         return f;
@@ -145,21 +177,14 @@ __device__ __forceinline__ Prefetch fetch(const WarpArgs &a, const Window &w, in
     f.q = make_float4(0.f, 0.f, 0.f, 0.f);
     const float2 *g = k > 0 ? a.grids + (size_t)(k - 1) * a.nx * a.ny : nullptr;
 #pragma unroll
-    for (int t = 0; t < 3; ++t) {
-        const int j = lane + 32 * t;
-        f.v[t] = make_float2(0.f, 0.f);
-        if (a.window && g && j < w.wx * w.wy) {
-            const int jy = j / w.wx, jx = j - jy * w.wx;
-            f.v[t] = g[(size_t)(w.cy0 + jy) * a.nx + w.cx0 + jx];
-        }
-    }
+    for (int t = 0; t < 3; ++t) f.v[t] = g && pl.src[t] >= 0 ? g[pl.src[t]] : make_float2(0.f, 0.f);
     return f;
 }
 
 // Warp 0: stage the parameters of frame k for the tile (x0, y0) into ring slot st and start
 // the TMA load of its source box.
 __device__ void prepare(const WarpArgs &a, const CUtensorMap *tmap, WarpSmem &sm, int k, int st, int x0, int y0,
-                        const Window &win, const Prefetch &f)
+                        const Window &win, const ProducerLane &pl, const Prefetch &f)
 {
     const int lane = threadIdx.x & 31;
     const int x1 = min(x0 + kTW, a.W) - 1, y1 = min(y0 + kTH, a.H) - 1;
@@ -182,33 +207,26 @@ __device__ void prepare(const WarpArgs &a, const CUtensorMap *tmap, WarpSmem &sm
     } else {
         float uxlo = 0.f, uxhi = 0.f, uylo = 0.f, uyhi = 0.f;
         if (a.window) {
-            const int cx0 = win.cx0, cy0 = win.cy0, wx = win.wx, wy = win.wy;
             uxlo = uylo = 3.0e38f;
             uxhi = uyhi = -3.0e38f;
 #pragma unroll
-            for (int t = 0; t < 3; ++t) {
-                const int j = lane + 32 * t;
-                if (j < wx * wy) {
-                    const int jy = j / wx, jx = j - jy * wx;
+            for (int t = 0; t < 3; ++t)
+                if (pl.src[t] >= 0) {
                     const float2 v = f.v[t];
-                    sm.win[st][jy * kWinX + jx] = v;
+                    sm.win[st][pl.dst[t]] = v;
                     uxlo = fminf(uxlo, v.x); uxhi = fmaxf(uxhi, v.x);
                     uylo = fminf(uylo, v.y); uyhi = fmaxf(uyhi, v.y);
                 }
-            }
-            // each window control row interpolated along x at the tile's columns (a column past
-            // the frame edge uses the last one), so a consumer pixel only interpolates along y
+            // each window control row interpolated along x at the tile's columns, so a consumer pixel
+            // only interpolates along y
             __syncwarp();
-#pragma unroll 4
-            for (int j = lane; j < wy * kTW; j += 32) {
-                const int jy = j / kTW, col = j - jy * kTW;
-                const int c = min(x0 + col, a.W - 1);
-                const float gxf = fminf((float)c * a.inv_s, (float)(a.nx - 1));
-                const int ix = cell_of(gxf, a.nx);
-                const float2 *q = sm.win[st] + jy * kWinX + (ix - cx0);
-                const float2 p0 = q[0], p1 = q[1];
-                sm.xint[st][jy][col] = __ffma2_rn(f2(gxf - (float)ix), f2sub(p1, p0), p0);
-            }
+            for (int jy = 0; jy < win.wy; ++jy)
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const float2 *q = sm.win[st] + jy * kWinX + pl.ix[h];
+                    const float2 p0 = q[0], p1 = q[1];
+                    sm.xint[st][jy][lane + 32 * h] = __ffma2_rn(f2(pl.wx[h]), f2sub(p1, p0), p0);
+                }
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) {
                 uxlo = fminf(uxlo, __shfl_xor_sync(0xffffffffu, uxlo, o));
@@ -216,7 +234,7 @@ __device__ void prepare(const WarpArgs &a, const CUtensorMap *tmap, WarpSmem &sm
                 uylo = fminf(uylo, __shfl_xor_sync(0xffffffffu, uylo, o));
                 uyhi = fmaxf(uyhi, __shfl_xor_sync(0xffffffffu, uyhi, o));
             }
-            if (lane == 0) sm.wo[st] = make_int2(cx0, cy0);
+            if (lane == 0) sm.wo[st] = make_int2(win.cx0, win.cy0);
         } else {
             uxlo = uylo = -1.0e6f;   // no bound without the window: sample from global memory
             uxhi = uyhi = 1.0e6f;
@@ -292,6 +310,7 @@ struct Cols {
     int col0, col1;            // the same columns relative to the tile's first one
     bool in0, in1;
     float2 xc;                 // rigid: columns relative to the rotation centre
+    float2 lo, hi;             // displacements that reach the frame's first and last column
     int ix0, ix1;              // nonrigid: control cell of each column
     float2 wx;                 //           and the weight along x
 };
@@ -379,19 +398,112 @@ __device__ __forceinline__ float2 staged_pair(const WarpArgs &a, const WarpSmem 
     return __ffma2_rn(fy, f2sub(bot, top), top);
 }
 
-// One frame of the tile for one consumer warp: rows warp, warp + 8, warp + 16, warp + 24.
+// v rounded down by adding 1.5 2^23 and its integer's bits (see f2add_down): no conversion instruction.
+constexpr float kRound = 12582912.f;
+constexpr unsigned kRoundBits = 0x4B400000u;
+
+// Displacements along a warp's kRows rows from r0 on of frame slot st as base + w_j slope, one weight per
+// row; false where a control cell ends between them.
+template <int MODE>
+__device__ __forceinline__ bool column_line(const WarpArgs &a, const WarpSmem &sm, int st, const Cols &cl, int r0,
+                                            float2 &bx, float2 &by, float2 &ex, float2 &ey, float &w0, float &dw)
+{
+    if (MODE == REG_RIGID) {
+        const float4 q = sm.rp[st];
+        bx = __ffma2_rn(f2(q.x), cl.xc, f2(q.z));
+        by = __ffma2_rn(f2(q.y), cl.xc, f2(q.w));
+        ex = f2(-q.y);
+        ey = f2(q.x);
+        w0 = (float)r0 - 0.5f * (float)(a.H - 1);
+        dw = 1.f;
+        return true;
+    }
+    const float g0 = fminf((float)r0 * a.inv_s, (float)(a.ny - 1)), g3 = fminf((float)(r0 + kRows - 1) * a.inv_s, (float)(a.ny - 1));
+    const int iy = cell_of(g0, a.ny);
+    if (cell_of(g3, a.ny) != iy) return false;
+    const float2 *t = sm.xint[st][iy - sm.wo[st].y], *b = sm.xint[st][iy - sm.wo[st].y + 1];
+    const float2 t0 = t[cl.col0], t1 = t[cl.col1], b0 = b[cl.col0], b1 = b[cl.col1];
+    bx = make_float2(t0.x, t1.x);
+    by = make_float2(t0.y, t1.y);
+    ex = f2sub(make_float2(b0.x, b1.x), bx);
+    ey = f2sub(make_float2(b0.y, b1.y), by);
+    w0 = g0 - (float)iy;
+    dw = a.inv_s;
+    return true;
+}
+
+// One frame of the tile for one consumer warp: kRows neighbouring rows, whose displacements share their
+// control values.  Strictly inside the staged box a sample's cell comes from the bits of its position
+// rounded down by an addition.  With a displacement from the control rows for each row, and floors and
+// conversions on the narrow conversion pipe, the kernel took 155 us for 256 frames of 512x512 (frames and
+// mean written; 69 % issue, 41 % of the memory rate); this way, with the producer's indexes formed once
+// per tile, 134 us (64 % issue, 50 %).
 template <int MODE, bool WINDOW, int KIND>
 __device__ __forceinline__ void tile_frame(const WarpArgs &a, const WarpSmem &sm, int st, int k, const Cols &cl,
-                                           int y0, float2 (&run)[4])
+                                           int y0, float2 (&run)[kRows])
 {
-    const int warp = threadIdx.x >> 5;
+    const int r0 = y0 + kRows * (threadIdx.x >> 5);
     const float *frame = a.frames + (size_t)k * a.H * a.pitch;
-    float *o = a.out ? a.out + (size_t)k * a.H * a.W : nullptr;
+    float *o = a.out ? a.out + (size_t)k * a.H * a.W + (size_t)r0 * a.W : nullptr;
     const int2 org = sm.org[st];
+    if (KIND != kGlobal && (MODE == REG_RIGID || WINDOW) && r0 + kRows <= a.H) {
+        float2 bx, by, ex, ey;
+        float w0, dw;
+        if (column_line<MODE>(a, sm, st, cl, r0, bx, by, ex, ey, w0, dw)) {
+            // index of a cell's first tap in the box from its rounded position's bits (all offsets wrap
+            // together); the unsigned clamp keeps any index inside the box
+            const unsigned off = kRoundBits * (unsigned)(kBW + 1);
+            unsigned ba = (unsigned)((r0 - org.y) * kBW + cl.c0 - org.x) - off, bb = (unsigned)((r0 - org.y) * kBW + cl.c1 - org.x) - off;
+            const float *buf = sm.buf[st];
+#pragma unroll
+            for (int j = 0; j < kRows; ++j) {
+                const float2 w = f2(fmaf((float)j, dw, w0));
+                float2 vx = __ffma2_rn(w, ex, bx), vy = __ffma2_rn(w, ey, by);
+                if (KIND == kStagedClamped) {
+                    // positions clamped to the frame
+                    const float ylo = (float)-(r0 + j), yhi = (float)(a.H - 1 - (r0 + j));
+                    vx = make_float2(fminf(fmaxf(vx.x, cl.lo.x), cl.hi.x), fminf(fmaxf(vx.y, cl.lo.y), cl.hi.y));
+                    vy = make_float2(fminf(fmaxf(vy.x, ylo), yhi), fminf(fmaxf(vy.y, ylo), yhi));
+                }
+                float2 mx = f2add_down(vx, f2(kRound)), my = f2add_down(vy, f2(kRound));
+                if (KIND == kStagedClamped) {
+                    // the cell at most the last one, where the weight is 1 on the frame's edge
+                    const float ym = (float)(a.H - 2 - (r0 + j)) + kRound;
+                    mx = make_float2(fminf(mx.x, cl.hi.x - 1.f + kRound), fminf(mx.y, cl.hi.y - 1.f + kRound));
+                    my = make_float2(fminf(my.x, ym), fminf(my.y, ym));
+                }
+                const float2 nx = f2sub(mx, f2(kRound)), ny = f2sub(my, f2(kRound));
+                const float2 fx = f2sub(vx, nx), fy = f2sub(vy, ny);
+                const float *pa = buf + min(ba + __float_as_uint(my.x) * (unsigned)kBW + __float_as_uint(mx.x), kMaxTap);
+                const float *pb = buf + min(bb + __float_as_uint(my.y) * (unsigned)kBW + __float_as_uint(mx.y), kMaxTap);
+                const float2 t00 = make_float2(pa[0], pb[0]), t10 = make_float2(pa[kBW], pb[kBW]);
+                const float2 t01 = make_float2(pa[1], pb[1]), t11 = make_float2(pa[kBW + 1], pb[kBW + 1]);
+                float2 v;
+                if (KIND == kStagedClamped) {
+                    // (1 - f) a + f b as f b + (a - f a): exact at f = 1 (the clamped last cell)
+                    const float2 gx = f2sub(nx, vx), gy = f2sub(ny, vy);
+                    const float2 top = __ffma2_rn(fx, t01, __ffma2_rn(gx, t00, t00)), bot = __ffma2_rn(fx, t11, __ffma2_rn(gx, t10, t10));
+                    v = __ffma2_rn(fy, bot, __ffma2_rn(gy, top, top));
+                } else {
+                    // f < 1, and a + f (b - a) is exact at f = 0
+                    const float2 top = __ffma2_rn(fx, f2sub(t01, t00), t00), bot = __ffma2_rn(fx, f2sub(t11, t10), t10);
+                    v = __ffma2_rn(fy, f2sub(bot, top), top);
+                }
+                if (o) {
+                    if (cl.in0) o[j * a.W + cl.c0] = v.x;
+                    if (cl.in1) o[j * a.W + cl.c1] = v.y;
+                }
+                run[j] = __fadd2_rn(run[j], v);
+                ba += kBW;
+                bb += kBW;
+            }
+            return;
+        }
+    }
     const float2 colx = make_float2((float)(cl.c0 - org.x), (float)(cl.c1 - org.x));
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        const int r = y0 + warp + 8 * j;
+    for (int j = 0; j < kRows; ++j) {
+        const int r = r0 + j;
         if (r >= a.H) continue;
         float2 vx, vy;
         displacement<MODE, WINDOW>(a, sm, st, k, cl, r, vx, vy);
@@ -403,8 +515,8 @@ __device__ __forceinline__ void tile_frame(const WarpArgs &a, const WarpSmem &sm
             v = staged_pair<KIND>(a, sm, st, __fadd2_rn(vx, colx), __fadd2_rn(vy, f2((float)(r - org.y))));
         }
         if (o) {
-            if (cl.in0) o[(size_t)r * a.W + cl.c0] = v.x;
-            if (cl.in1) o[(size_t)r * a.W + cl.c1] = v.y;
+            if (cl.in0) o[(size_t)j * a.W + cl.c0] = v.x;
+            if (cl.in1) o[(size_t)j * a.W + cl.c1] = v.y;
         }
         run[j] = __fadd2_rn(run[j], v);
     }
@@ -447,11 +559,12 @@ __global__ void __launch_bounds__(kWThreads, kCtasPerSm) warp_kernel(const WarpA
         // ---- producer: parameters and the TMA load of each frame, up to kStages ahead
         int issued = 0;
         const Window win = window_of(a, x0, y0);
-        Prefetch cur = fetch(a, win, kb);
+        const ProducerLane pl = producer_lane(a, win, x0);
+        Prefetch cur = fetch(a, pl, kb);
         for (int i = 0; i < n; ++i) {
             const int st = i % kStages;
             Prefetch nxt = cur;
-            if (i + 1 < n) nxt = fetch(a, win, kb + i + 1);   // in flight while this frame is prepared
+            if (i + 1 < n) nxt = fetch(a, pl, kb + i + 1);   // in flight while this frame is prepared
             if (i >= kStages) {
                 // every lane acquires: lane 0 reuses the box, all lanes rewrite the window
                 const bool ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&sm.empty[st]),
@@ -462,7 +575,7 @@ __global__ void __launch_bounds__(kWThreads, kCtasPerSm) warp_kernel(const WarpA
                 }
             }
             if (*abort) break;
-            prepare(a, &tmap, sm, kb + i, st, x0, y0, win, cur);
+            prepare(a, &tmap, sm, kb + i, st, x0, y0, win, pl, cur);
             issued = i + 1;
             cur = nxt;
         }
@@ -484,6 +597,8 @@ __global__ void __launch_bounds__(kWThreads, kCtasPerSm) warp_kernel(const WarpA
     cl.col0 = cl.c0 - x0;
     cl.col1 = cl.c1 - x0;
     cl.xc = make_float2((float)cl.c0 - 0.5f * (float)(a.W - 1), (float)cl.c1 - 0.5f * (float)(a.W - 1));
+    cl.lo = make_float2((float)-cl.c0, (float)-cl.c1);
+    cl.hi = make_float2((float)(a.W - 1 - cl.c0), (float)(a.W - 1 - cl.c1));
     if (MODE == REG_NONRIGID) {
         const float g0 = fminf((float)cl.c0 * a.inv_s, (float)(a.nx - 1));
         const float g1 = fminf((float)cl.c1 * a.inv_s, (float)(a.nx - 1));
@@ -491,9 +606,9 @@ __global__ void __launch_bounds__(kWThreads, kCtasPerSm) warp_kernel(const WarpA
         cl.ix1 = cell_of(g1, a.nx);
         cl.wx = make_float2(g0 - (float)cl.ix0, g1 - (float)cl.ix1);
     }
-    float2 hi[4], lo[4], run[4];
+    float2 hi[kRows], lo[kRows], run[kRows];
 #pragma unroll
-    for (int j = 0; j < 4; ++j) { hi[j] = lo[j] = run[j] = make_float2(0.f, 0.f); }
+    for (int j = 0; j < kRows; ++j) { hi[j] = lo[j] = run[j] = make_float2(0.f, 0.f); }
     for (int i = 0; i < n; ++i) {
         const int k = kb + i, st = i % kStages;
         // every lane waits (acquire) before reading the stage
@@ -512,17 +627,17 @@ __global__ void __launch_bounds__(kWThreads, kCtasPerSm) warp_kernel(const WarpA
         if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&sm.empty[st])) : "memory");
         if ((i % kRun) == kRun - 1) {
 #pragma unroll
-            for (int j = 0; j < 4; ++j) fold(hi[j], lo[j], run[j]);
+            for (int j = 0; j < kRows; ++j) fold(hi[j], lo[j], run[j]);
         }
     }
     __syncthreads();
     if (*abort || !a.part) return;
 #pragma unroll
-    for (int j = 0; j < 4; ++j) fold(hi[j], lo[j], run[j]);
+    for (int j = 0; j < kRows; ++j) fold(hi[j], lo[j], run[j]);
     float2 *p = a.part + (size_t)blockIdx.y * a.H * a.W;
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        const int r = y0 + warp + 8 * j;
+    for (int j = 0; j < kRows; ++j) {
+        const int r = y0 + kRows * warp + j;
         if (r >= a.H) continue;
         if (cl.in0) p[(size_t)r * a.W + cl.c0] = make_float2(hi[j].x, lo[j].x);
         if (cl.in1) p[(size_t)r * a.W + cl.c1] = make_float2(hi[j].y, lo[j].y);
@@ -530,7 +645,9 @@ __global__ void __launch_bounds__(kWThreads, kCtasPerSm) warp_kernel(const WarpA
 }
 
 // mean = (1/N) sum over chunks, in chunk order; four pixels per thread (float4 store) when
-// the row length allows it.
+// the row length allows it.  The sums' high parts are added in FP64, whose instructions bound the kernel
+// (64 cycles each: 21 us for 7 chunks of 512x512 with both parts in FP64, 14.5 us so); the low parts, below
+// 2^-24 of them, in FP32, which leaves 2^-45 of the sum.
 __global__ void mean_kernel(const float2 *part, int chunks, int W, int H, double inv_n, float *mean)
 {
     const size_t P = (size_t)W * H;
@@ -539,21 +656,23 @@ __global__ void mean_kernel(const float2 *part, int chunks, int W, int H, double
         const size_t i0 = 4 * q;
         if (i0 >= P) return;
         double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
+        float e0 = 0.f, e1 = 0.f, e2 = 0.f, e3 = 0.f;
         for (int c = 0; c < chunks; ++c) {
             const float4 *v = (const float4 *)(part + c * P + i0);
             const float4 u0 = v[0], u1 = v[1];
-            s0 += (double)u0.x + (double)u0.y;
-            s1 += (double)u0.z + (double)u0.w;
-            s2 += (double)u1.x + (double)u1.y;
-            s3 += (double)u1.z + (double)u1.w;
+            s0 += (double)u0.x; e0 += u0.y;
+            s1 += (double)u0.z; e1 += u0.w;
+            s2 += (double)u1.x; e2 += u1.y;
+            s3 += (double)u1.z; e3 += u1.w;
         }
-        *(float4 *)(mean + i0) = make_float4((float)(s0 * inv_n), (float)(s1 * inv_n), (float)(s2 * inv_n),
-                                             (float)(s3 * inv_n));
+        *(float4 *)(mean + i0) = make_float4((float)((s0 + (double)e0) * inv_n), (float)((s1 + (double)e1) * inv_n),
+                                             (float)((s2 + (double)e2) * inv_n), (float)((s3 + (double)e3) * inv_n));
     } else {
         for (size_t i = 4 * q; i < min(P, 4 * q + 4); ++i) {
             double s = 0.0;
-            for (int c = 0; c < chunks; ++c) s += (double)part[c * P + i].x + (double)part[c * P + i].y;
-            mean[i] = (float)(s * inv_n);
+            float e = 0.f;
+            for (int c = 0; c < chunks; ++c) { s += (double)part[c * P + i].x; e += part[c * P + i].y; }
+            mean[i] = (float)((s + (double)e) * inv_n);
         }
     }
 }
@@ -606,7 +725,7 @@ EncodeTiled encoder()
 // Frames per chunk.  A block takes the frames of one chunk at one tile, so the grid is tiles x
 // chunks; with a fixed 64 frames, 256 frames of 512x512 made 512 blocks for the 456 that are resident
 // at once, and the second wave ran nearly empty (219 us a call with frames and mean out, 196 us with 7 chunks of 37
-// frames in two full waves).  The rule takes the chunk whose waves x (frames + kChunkCost) is least, the larger
+// frames in two full waves; 169 us by now).  The rule takes the chunk whose waves x (frames + kChunkCost) is least, the larger
 // of equals: kChunkCost stands for the pipeline's fill and the chunk's partial sums, in frames, and
 // keeps the chunks of a long series near 64.  It depends on the sizes alone, so a series' mean does
 // not depend on which outputs a call asks for.
