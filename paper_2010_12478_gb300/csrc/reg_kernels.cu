@@ -955,16 +955,20 @@ __host__ __device__ __forceinline__ GridLayout grid_layout(int gnx, int gny, int
     return g;
 }
 
-// Sum 16 per-lane values over aligned segments of SEG lanes by halving exchanges (8 + 4 + 2 + 1
-// shuffles and a butterfly for SEG = 32): on return a lane holds the segment's totals of the values
+// Sum 16 per-lane pairs of values over aligned segments of SEG lanes by halving exchanges (8 + 4 + 2 + 1
+// steps and a butterfly for SEG = 32): on return a lane holds the segment's totals of the values
 // first .. first + 15 / SEG (fixed order, so deterministic).
 template <int SEG> struct SegSum {
     static constexpr int kHeld = SEG >= 16 ? 1 : 16 / SEG;
-    float v[kHeld];
+    float2 v[kHeld];
     int first;
 };
+__device__ __forceinline__ float2 shfl_xor2(float2 v, int o)
+{
+    return make_float2(__shfl_xor_sync(0xffffffffu, v.x, o), __shfl_xor_sync(0xffffffffu, v.y, o));
+}
 template <int SEG>
-__device__ __forceinline__ SegSum<SEG> seg_sum16(float (&v)[16], int lane)
+__device__ __forceinline__ SegSum<SEG> seg_sum16(float2 (&v)[16], int lane)
 {
     SegSum<SEG> o;
     o.first = 0;
@@ -974,12 +978,12 @@ __device__ __forceinline__ SegSum<SEG> seg_sum16(float (&v)[16], int lane)
             const bool up = lane & w;
 #pragma unroll
             for (int k = 0; k < n; ++k) {
-                const float send = up ? v[k] : v[k + n], keep = up ? v[k + n] : v[k];
-                v[k] = keep + __shfl_xor_sync(0xffffffffu, send, w);
+                const float2 send = up ? v[k] : v[k + n], keep = up ? v[k + n] : v[k];
+                v[k] = __fadd2_rn(keep, shfl_xor2(send, w));
             }
             o.first += up ? n : 0;
         } else {
-            v[0] += __shfl_xor_sync(0xffffffffu, v[0], w);
+            v[0] = __fadd2_rn(v[0], shfl_xor2(v[0], w));
         }
     }
 #pragma unroll
@@ -987,48 +991,55 @@ __device__ __forceinline__ SegSum<SEG> seg_sum16(float (&v)[16], int lane)
     return o;
 }
 
-// One control row's sums of a strip into its slots (points 0 .. last + 1 of the strip; slot[p kSlot]).
-// v: the lane's column, already weighted along x: entries 0-7 for the point left of its cell k, 8-15
-// for the point right of it; ncomp entries of each are written.  A point between two cells gets
-// the left cell's share after the right cell's.
+// The emission of a segment's control rows is a chain of shuffles and shared-memory writes that one
+// warp in two per scheduler runs: one strip after the other took 1,000 cycles each, half of a pass over
+// 128x128 pixels; both in one chain of packed additions 230 us -> 217 us for a pair of 128x128 frames, 5.02 ->
+// 4.80 ms for 8 stacks of 32 frames of 256x256.
+// One control row's sums of two strips (.x and .y) into their slots (points 0 .. last + 1 of a strip;
+// slot[p kSlot]).  v: the lane's columns, already weighted along x: entries 0-7 for the point left of its
+// cell k, 8-15 for the point right of it; ncomp entries of each are written, nothing where last < 0.  A
+// point between two cells gets the left cell's share after the right cell's.
 template <int SEG>
-__device__ __forceinline__ void emit_row(float (&v)[16], int lane, int k, int last, float *slot, int ncomp)
+__device__ __forceinline__ void emit_row(float2 (&v)[16], int lane, int k, int2 last, float *s0, float *s1, int ncomp)
 {
     const SegSum<SEG> s = seg_sum16<SEG>(v, lane);
-    const bool writer = k <= last && (SEG < 32 || (lane & 1) == 0);
+    const bool on = SEG < 32 || (lane & 1) == 0;
 #pragma unroll
     for (int i = 0; i < SegSum<SEG>::kHeld; ++i) {
-        const int id = s.first + i, side = id >> 3, comp = id & 7;
-        if (writer && comp < ncomp && (side == 0 || k == last)) slot[(k + side) * kSlot + comp] = s.v[i];
+        const int id = s.first + i, side = id >> 3, comp = id & 7, at = (k + side) * kSlot + comp;
+        const bool w = on && comp < ncomp;
+        if (w && k <= last.x && (side == 0 || k == last.x)) s0[at] = s.v[i].x;
+        if (w && k <= last.y && (side == 0 || k == last.y)) s1[at] = s.v[i].y;
     }
     if (SEG == 32) return;
     __syncwarp();
 #pragma unroll
     for (int i = 0; i < SegSum<SEG>::kHeld; ++i) {
-        const int id = s.first + i, side = id >> 3, comp = id & 7;
-        if (writer && comp < ncomp && side == 1 && k < last) slot[(k + 1) * kSlot + comp] += s.v[i];
+        const int id = s.first + i, side = id >> 3, comp = id & 7, at = (k + 1) * kSlot + comp;
+        if (comp < ncomp && side == 1 && k < last.x) s0[at] += s.v[i].x;
+        if (comp < ncomp && side == 1 && k < last.y) s1[at] += s.v[i].y;
     }
 }
 
-__device__ __forceinline__ void emit_any(int sl, bool whole, float (&v)[16], int lane, int k, int last, float *slot,
-                                         int ncomp)
+__device__ __forceinline__ void emit_any(int sl, float2 (&v)[16], int lane, int k, int2 last, float *s0, float *s1, int ncomp)
 {
-    if (whole) emit_row<32>(v, lane, k, last, slot, ncomp);   // a strip of one cell
-    else if (sl == 16) emit_row<16>(v, lane, k, last, slot, ncomp);
-    else if (sl == 8) emit_row<8>(v, lane, k, last, slot, ncomp);
-    else if (sl == 4) emit_row<4>(v, lane, k, last, slot, ncomp);
-    else if (sl == 2) emit_row<2>(v, lane, k, last, slot, ncomp);
-    else if (sl == 1) emit_row<1>(v, lane, k, last, slot, ncomp);
+    if (sl >= 32) emit_row<32>(v, lane, k, last, s0, s1, ncomp);   // strips of one cell
+    else if (sl == 16) emit_row<16>(v, lane, k, last, s0, s1, ncomp);
+    else if (sl == 8) emit_row<8>(v, lane, k, last, s0, s1, ncomp);
+    else if (sl == 4) emit_row<4>(v, lane, k, last, s0, s1, ncomp);
+    else if (sl == 2) emit_row<2>(v, lane, k, last, s0, s1, ncomp);
+    else if (sl == 1) emit_row<1>(v, lane, k, last, s0, s1, ncomp);
     else
         // a cell width that is no power of two: cell by cell over the whole warp
-        for (int q = 0; q <= last; ++q) {
-            float x[16];
+        for (int q = 0; q <= max(last.x, last.y); ++q) {
+            float2 x[16];
 #pragma unroll
-            for (int i = 0; i < 16; ++i) x[i] = k == q ? v[i] : 0.f;
+            for (int i = 0; i < 16; ++i) x[i] = k == q ? v[i] : f2(0.f);
             const SegSum<32> s = seg_sum16<32>(x, lane);
-            const int side = s.first >> 3, comp = s.first & 7;
-            float *p = slot + (q + side) * kSlot + comp;
-            if ((lane & 1) == 0 && comp < ncomp) *p = side == 0 && q > 0 ? *p + s.v[0] : s.v[0];
+            const int side = s.first >> 3, comp = s.first & 7, at = (q + side) * kSlot + comp;
+            const bool w = (lane & 1) == 0 && comp < ncomp, add = side == 0 && q > 0;
+            if (w && q <= last.x) s0[at] = add ? s0[at] + s.v[0].x : s.v[0].x;
+            if (w && q <= last.y) s1[at] = add ? s1[at] + s.v[0].y : s.v[0].y;
             __syncwarp();
         }
 }
@@ -1069,8 +1080,8 @@ __device__ __forceinline__ void slot_sum(const float *slots, const PassGeom &P, 
                                          int first, float (&o)[N])
 {
     const int ga = i > 0 ? div20(i - 1, P.rm) : 0, gb = div20(i < nr ? i : nr - 1, P.rm);
-    auto add = [&](int seg, int strip, int row, int pt) {
-        const float *s = slots + (((size_t)(seg * P.nst + strip) * (P.m + 1) + row) * (P.g + 1) + pt) * kSlot + first;
+    const int srow = (P.g + 1) * kSlot, sstrip = (P.m + 1) * srow, sseg = P.nst * sstrip;
+    auto add = [&](const float *s) {
 #pragma unroll
         for (int k = 0; k < N; k += 2) {
             const float2 v = *(const float2 *)(s + k);
@@ -1079,21 +1090,27 @@ __device__ __forceinline__ void slot_sum(const float *slots, const PassGeom &P, 
         }
     };
     const int st = div20(jx, P.rg), pt = jx - st * P.g;
-    for (int grp = ga; grp <= gb; ++grp)
+    // the strips that hold the point: where it is the last of one, the first or an inner one of another, and
+    // where it lies beside the column past the last cell
+    const bool narrow = P.sl < 32, over = P.nst > P.ns && jx >= ncx - 1;
+    const bool left = narrow && pt == 0 && jx > 0, own = narrow && st < P.ns;
+    for (int grp = ga; grp <= gb; ++grp) {
+        const float *p = slots + grp * P.h * sseg + (i - grp * P.m) * srow + first;
+        const float *po = p + st * sstrip + pt * kSlot, *pl = po - sstrip + P.g * kSlot;
+        const float *pv = p + P.ns * sstrip + (jx - (ncx - 1)) * kSlot;
 #pragma unroll 4
         for (int piece = 0; piece < P.h; ++piece) {
-            const int seg = grp * P.h + piece, row = i - grp * P.m;
-            if (P.sl < 32) {
-                if (pt == 0 && jx > 0) add(seg, st - 1, row, P.g);
-                if (st < P.ns) add(seg, st, row, pt);
-            } else {
+            if (left) add(pl);
+            if (own) add(po);
+            if (!narrow)
                 for (int q = 0; q < P.chunks; ++q) {
-                    if (jx > 0) add(seg, (jx - 1) * P.chunks + q, row, 1);
-                    if (jx < ncx) add(seg, jx * P.chunks + q, row, 0);
+                    if (jx > 0) add(p + ((jx - 1) * P.chunks + q) * sstrip + kSlot);
+                    if (jx < ncx) add(p + (jx * P.chunks + q) * sstrip);
                 }
-            }
-            if (P.nst > P.ns && jx >= ncx - 1) add(seg, P.ns, row, jx - (ncx - 1));
+            if (over) add(pv);
+            p += sseg; po += sseg; pl += sseg; pv += sseg;
         }
+    }
 }
 
 // One pass at c (START: a level's first) or at the trial c + tau d: the moments into sm.tot (e =
@@ -1140,7 +1157,7 @@ __device__ void grid_pass(const Lvl &L, const Grid &G, const GridLvl &GL, const 
         const int ca = B.cr0 + grp * P.m, cb = min(ca + P.m, B.cr1);
         if (ca >= cb) continue;
         // this lane's column of either strip; an idle lane repeats the last column and counts for nothing
-        int xc[2], cell[2], kl[2], last[2];
+        int xc[2], cell[2], last[2];
         float wx[2];
         bool act[2];
 #pragma unroll
@@ -1150,11 +1167,10 @@ __device__ void grid_pass(const Lvl &L, const Grid &G, const GridLvl &GL, const 
             const int cell0 = over ? ncx - 1 : sl < 32 ? strip * P.g : P.chunks == 1 ? strip : strip / P.chunks;
             const int c0 = min(cell0, ncx - 1);
             last[u] = over || sl >= 32 ? 0 : min(P.g, ncx - c0) - 1;
-            kl[u] = over ? 0 : kw;
             const int xs = over ? ncx * sl : sl < 32 ? c0 * sl : c0 * sl + (strip - cell0 * P.chunks) * 32;
             const int xe = over ? L.W : min(L.W, min(c0 * sl + (last[u] + 1) * sl, xs + 32));
-            act[u] = strip < P.nst && xs + lane < xe && kl[u] <= last[u];
-            cell[u] = c0 + min(kl[u], last[u]);
+            act[u] = strip < P.nst && xs + lane < xe && kw <= last[u];
+            cell[u] = c0 + min(kw, last[u]);
             xc[u] = min(xs + lane, L.W - 1);
             wx[u] = fminf(fmaf(GL.pl, (float)xc[u], GL.off) * GL.scale_inv, (float)ncx) - (float)cell[u];
             if (!act[u]) { xc[u] = min(cell[u] * sl, L.W - 1); wx[u] = 0.f; }
@@ -1314,26 +1330,24 @@ __device__ void grid_pass(const Lvl &L, const Grid &G, const GridLvl &GL, const 
                 ty = by;
             }
             // control row cy: what the cell row above it left and the top sums of the one below
-#pragma unroll 1
-            for (int u = 0; u < 2; ++u) {
-                const int strip = strip0 + u;
-                if (strip >= P.nst) break;
-                const bool on = u ? act[1] : act[0];
-                const float w = u ? wx[1] : wx[0];
-                const float lw = on ? 1.f - w : 0.f, rw = on ? w : 0.f;
-                float v[16];
+            {
+                const float2 rw = make_float2(act[0] ? wx[0] : 0.f, act[1] ? wx[1] : 0.f);
+                const float2 lw = make_float2(act[0] ? 1.f - wx[0] : 0.f, act[1] ? 1.f - wx[1] : 0.f);
+                float2 v[16];
 #pragma unroll
                 for (int i = 0; i < 2; ++i) {
-                    const float f = u ? sF[i].y : sF[i].x, t = u ? sT[i].y : sT[i].x, o = u ? s1[i].y : s1[i].x;
-                    const float m = START ? (u ? sM[i].y : sM[i].x) : 0.f;
-                    v[i] = lw * f; v[8 + i] = rw * f;
-                    v[2 + i] = lw * t; v[10 + i] = rw * t;
-                    v[4 + i] = lw * o; v[12 + i] = rw * o;
-                    v[6 + i] = lw * lw * m; v[14 + i] = rw * rw * m;
+                    v[i] = __fmul2_rn(lw, sF[i]); v[8 + i] = __fmul2_rn(rw, sF[i]);
+                    v[2 + i] = __fmul2_rn(lw, sT[i]); v[10 + i] = __fmul2_rn(rw, sT[i]);
+                    v[4 + i] = __fmul2_rn(lw, s1[i]); v[12 + i] = __fmul2_rn(rw, s1[i]);
+                    v[6 + i] = v[14 + i] = f2(0.f);
+                    if constexpr (START) {
+                        v[6 + i] = __fmul2_rn(__fmul2_rn(lw, lw), sM[i]);
+                        v[14 + i] = __fmul2_rn(__fmul2_rn(rw, rw), sM[i]);
+                    }
                 }
-                float *slot = slots + ((size_t)(seg * P.nst + strip) * (P.m + 1) + (cy - ca)) * (P.g + 1) * kSlot;
-                emit_any(sl, sl >= 32 || strip == P.ns, v, lane, u ? kl[1] : kl[0], u ? last[1] : last[0], slot,
-                         START ? 8 : 6);
+                const int strip = (P.m + 1) * (P.g + 1) * kSlot;
+                float *slot = slots + (seg * P.nst + strip0) * strip + (cy - ca) * (P.g + 1) * kSlot;
+                emit_any(sl, v, lane, kw, make_int2(last[0], strip0 + 1 < P.nst ? last[1] : -1), slot, slot + strip, START ? 8 : 6);
             }
 #pragma unroll
             for (int i = 0; i < 2; ++i) {
