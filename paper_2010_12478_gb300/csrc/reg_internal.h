@@ -98,6 +98,28 @@ struct Queue {
     long long timeout_ns;
 };
 
+// How a pass splits a band's pixels among the warps.  A strip is up to 32 columns: those of g whole cells
+// (32 / sl of them, sl the cell width at the level), or from 32 columns a cell on a chunk of one cell; a
+// column past the last cell, which a frame of 2^k + 1 columns has, is a strip of its own.  A warp's
+// task is two neighbouring strips, a column of each per lane, over the rows of a segment: m cell
+// rows, or one h-th of a cell row.  Every strip of every segment has slots of its own for its sums
+// (m + 1 control rows of g + 1 points, 8 floats each), so no two warps add to one place and the
+// order is fixed.  Long segments are best (a control row inside one is reduced over the lanes once, not
+// twice), short ones where there are too few strips for the warps: the rule takes the least number of
+// rounds x (pixel rows + about two rows' time per reduction) of the splits whose slots fit `room`
+// floats.  Where none does (thousands of chunks), a task is one wide cell, whose chunks a warp walks
+// two at a time and adds up in one strip's slots.
+struct PassGeom {
+    int sl, g, chunks;    // cell width, cells per strip, strips per cell (wide cells)
+    int ns, nst;          // strips of cells with slots, strips with slots
+    int sch;              // strips with slots per wide cell: chunks, or 1 where a task walks them
+    int past;             // the strip past the last cell, counting every chunk
+    int tasks, walk;      // tasks of a segment; pairs of strips a task walks
+    int m, h, ph;         // cell rows per segment, pieces per cell row (a power of two), pixel rows per piece
+    int nseg, hlog;       // segments, log2 of h
+    unsigned rm, rg;      // reciprocals for div20: of m and g
+};
+
 struct Params {
     Config cfg;
     const LevelDesc *levels;   // [n_frames][cfg.levels]
@@ -112,6 +134,7 @@ struct Params {
     int unroll;                // nonrigid passes: pixels in flight per lane (2 or 4; 0 = 4)
     int minb;                  // nonrigid register form as configured (3 or 4; 0 = 3); one kernel serves both
     int gnx, gny, gs;          // nonrigid control grid: points per axis and spacing (finest px)
+    PassGeom geom[kMaxLevels][2];   // nonrigid, set at the launch: per level, without and with columns past the last cell
     int n_nodes;
     OpStats *stats;            // [n_ops]
     int *status;               // kernel status word (first device error)

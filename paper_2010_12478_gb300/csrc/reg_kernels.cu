@@ -20,6 +20,7 @@
 //     values live in shared memory.
 #include <cooperative_groups.h>
 
+#include <algorithm>
 #include <cmath>
 
 #include "reg_internal.h"
@@ -101,6 +102,7 @@ struct Smem {
     float pm[16];               // pass parameters broadcast by thread 0
     int action;
     int idata[4];
+    PassGeom geom;              // of the level
     int fail;                   // an exchange's wait ran out: kDevWaitTimeout
     union {
         RigidCtl rctl;
@@ -866,23 +868,6 @@ __device__ __forceinline__ Band grid_band(const Grid &G, int rank, int C)
     return b;
 }
 
-// How a pass splits a band's pixels among the warps.  A strip is up to 32 columns: those of g = 32 / sl
-// whole cells (sl the cell width at the level), or from 32 columns a cell on a chunk of one cell; a
-// column past the last cell, which a frame of 2^k + 1 columns has, is a strip of its own.  A warp's
-// task is two neighbouring strips, a column of each per lane, over the rows of a segment: m cell
-// rows, or one h-th of a cell row.  Every strip of every segment has slots of its own for its sums
-// (m + 1 control rows of g + 1 points, 8 floats each), so no two warps add to one place and the
-// order is fixed.  Long segments are best (a control row inside one is reduced over the lanes once, not
-// twice), short ones where there are too few strips for the warps: the rule takes the least number of
-// rounds x (pixel rows + about two rows' time per reduction).
-struct PassGeom {
-    int sl, g, chunks;    // cell width, cells per strip, strips per cell (wide cells)
-    int ns, nst;          // strips of cells, strips
-    int m, h, ph;         // cell rows per segment, pieces per cell row (a power of two), pixel rows per piece
-    int nseg, hlog;       // segments, log2 of h
-    unsigned rm, rg;      // reciprocals for div20: of m and g
-};
-
 // a / b for a b < 2^20, r = recip20(b): the integer divisions of a pass's set-up take longer than the rows
 // of a small frame.
 __host__ __device__ __forceinline__ unsigned recip20(int b)
@@ -894,31 +879,47 @@ __host__ __device__ __forceinline__ int div20(int a, unsigned r)
     return (int)(((unsigned)a * r) >> 20);
 }
 
-__host__ __device__ inline PassGeom pass_geom(int sl, int ncx, int q, bool over)
+constexpr int kSlot = 8;   // floats per slot: (t - r, t, 1) x (x, y), then dT^2 x (x, y)
+// The rule of PassGeom.  On the host, once per launch: made by the kernel, per operator and level, it took
+// 16 us of a pair of 128x128 frames.
+//
+// A column's sums run in FP32 over the rows of a segment's cell row.  `exact` takes pieces of at most 8 rows
+// where their slots fit: for a gradient that is a result itself (reg_energy, 512x512), 6.1e-8 of its norm off
+// the 64-bit value instead of 6.8e-8, within a microsecond of a call.
+static PassGeom pass_geom(int sl, int ncx, int q, bool over, int room, bool exact)
 {
     PassGeom P;
     P.sl = sl;
-    P.g = sl < 32 ? 32 / sl : 1;
+    P.g = sl < 32 ? 32 / sl < ncx ? 32 / sl : ncx : 1;
     P.chunks = (sl + 31) / 32;
-    P.ns = sl < 32 ? (ncx + P.g - 1) / P.g : ncx * P.chunks;
-    P.nst = P.ns + (over ? 1 : 0);
-    const int pairs = (P.nst + 1) / 2;
-    int least = -1;
-    for (int k = 1; k < 2 * q; k *= 2) {
-        const int m = (q + k - 1) / k, nseg = (q + m - 1) / m;
-        const int cost = (pairs * nseg + kWarps - 1) / kWarps * (m * sl + 2 * m + 4);
-        if (least < 0 || cost < least) {
-            least = cost;
-            P.m = m; P.h = 1; P.ph = sl; P.nseg = nseg;
+    P.past = sl < 32 ? (ncx + P.g - 1) / P.g : ncx * P.chunks;
+    for (const bool walk : {false, true}) {
+        P.sch = walk ? 1 : P.chunks;
+        P.ns = walk ? ncx : P.past;
+        P.nst = P.ns + (over ? 1 : 0);
+        P.tasks = walk ? P.nst : (P.nst + 1) / 2;
+        P.walk = walk ? (P.chunks + 1) / 2 : 1;
+        int least = -1;
+        const int most = room / ((P.g + 1) * kSlot) / P.nst;   // segments x control rows that fit
+        for (int k = 1; k < 2 * q; k *= 2) {
+            const int m = (q + k - 1) / k, nseg = (q + m - 1) / m;
+            const int cost = (P.tasks * nseg + kWarps - 1) / kWarps * (P.walk * m * sl + 2 * m + 4);
+            if ((least < 0 || cost < least) && nseg * (m + 1) <= most) {
+                least = cost;
+                P.m = m; P.h = 1; P.ph = sl; P.nseg = nseg;
+            }
         }
-    }
-    for (int h = 2; h <= 8 && sl / h >= 2; h *= 2) {
-        const int ph = (sl + h - 1) / h;
-        const int cost = (pairs * q * h + kWarps - 1) / kWarps * (ph + 6);
-        if (cost < least) {
-            least = cost;
-            P.m = 1; P.h = h; P.ph = ph; P.nseg = q * h;
+        for (int h = 2; h <= 8 && sl / h >= 2; h *= 2) {
+            const int ph = (sl + h - 1) / h;
+            const int cost = (P.tasks * q * h + kWarps - 1) / kWarps * (P.walk * ph + 6);
+            if ((least < 0 || cost < least || (exact && P.ph > 8)) && q * h * 2 <= most) {
+                least = cost;
+                P.m = 1; P.h = h; P.ph = ph; P.nseg = q * h;
+            }
         }
+        if (least >= 0) break;
+        P.m = q; P.h = 1; P.ph = sl; P.nseg = 1;   // the fewest slots: they do not fit here, the host refuses
+        if (P.chunks == 1) break;
     }
     P.hlog = P.h == 8 ? 3 : P.h >> 1;
     P.rm = recip20(P.m);
@@ -926,19 +927,21 @@ __host__ __device__ inline PassGeom pass_geom(int sl, int ncx, int q, bool over)
     return P;
 }
 
-constexpr int kSlot = 8;   // floats per slot: (t - r, t, 1) x (x, y), then dT^2 x (x, y)
-__host__ __device__ __forceinline__ size_t slot_floats(const PassGeom &P)
+static size_t slot_floats(const PassGeom &P)
 {
     return (size_t)P.nseg * P.nst * (P.m + 1) * (P.g + 1) * kSlot;
 }
 
+constexpr int kEmitSums = 6, kEmitRow = 36;   // gradient sums of a column; a row of 32 columns, padded against bank conflicts
+constexpr int kEmitFloats = 2 * kEmitSums * kEmitRow;   // a warp's emission: 2 strips' sums
+
 // Dynamic shared memory of the nonrigid kernels, in float2 units: c, d, mt (the held rows; mt the
 // flow's scalar product per control point and axis), two staged halo rows of d, the sums that the CTA
-// above sends for the first own row, then the slots.
+// above sends for the first own row, the warps' rows of an emission, then the slots.
 // With the H1 product mt is the right-hand side of its solve on the whole grid, and the two work
 // grids t and u of the solve lie in the place of the slots, which it has read by then.
 struct GridLayout {
-    int c, d, mt, halo, above, slots;
+    int c, d, mt, halo, above, emits, slots;
 };
 __host__ __device__ __forceinline__ GridLayout grid_layout(int gnx, int gny, int C, bool h1)
 {
@@ -949,99 +952,143 @@ __host__ __device__ __forceinline__ GridLayout grid_layout(int gnx, int gny, int
     g.d = rows * gnx;
     g.mt = 2 * rows * gnx;
     g.halo = g.mt + (h1 ? gny : rows) * gnx;
-    g.above = g.halo + 2 * gnx;
-    g.slots = g.above + kSlot / 2 * gnx;
-    g.slots += g.slots & 1;
+    const int edges = q < gny - 1 ? gnx : 0;   // a band has neighbours
+    g.above = g.halo + 2 * edges;
+    g.emits = g.above + kSlot / 2 * edges;
+    g.emits += g.emits & 1;
+    g.slots = g.emits + kWarps * kEmitFloats / 2;
     return g;
 }
 
-// Sum 16 per-lane pairs of values over aligned segments of SEG lanes by halving exchanges (8 + 4 + 2 + 1
-// steps and a butterfly for SEG = 32): on return a lane holds the segment's totals of the values
-// first .. first + 15 / SEG (fixed order, so deterministic).
-template <int SEG> struct SegSum {
-    static constexpr int kHeld = SEG >= 16 ? 1 : 16 / SEG;
-    float2 v[kHeld];
-    int first;
-};
-__device__ __forceinline__ float2 shfl_xor2(float2 v, int o)
+// Floats that a CTA's shared memory holds as slots beside the rest of the layout and the static part.
+constexpr int kMostSmem = 227 * 1024 - (int)sizeof(Smem) - 256;
+static int slot_room(const GridLayout &g)
 {
-    return make_float2(__shfl_xor_sync(0xffffffffu, v.x, o), __shfl_xor_sync(0xffffffffu, v.y, o));
+    return (kMostSmem - (int)sizeof(float2) * g.slots) / (int)sizeof(float);
 }
-template <int SEG>
-__device__ __forceinline__ SegSum<SEG> seg_sum16(float2 (&v)[16], int lane)
+
+// ------------------------------------------------------------------ a control row's sums
+// The emission of a segment's control row: a lane holds its two columns' sums x (kEmitSums of them per
+// strip; 2 with SQ), which every cell's columns add up to for the point on its left, weighted 1 - w, and
+// on its right, weighted w (SQ: by the squares).  w grows by dw per column from that of the strip's first
+// column, wf, in each cell anew.  The sums go through shared memory: a lane writes its columns, and then
+// has a cell's columns of one sum to itself (with cells of 8 or 16 columns; of 32, half of them), four at
+// a load: right = wf S + dw K, left = wl S + dw L from S = sum x, K = sum k x and L = sum (n - 1 - k) x,
+// wl the last column's 1 - w (S - right has the rounding of S where the left share is small).  Exchanging
+// the lanes' values by halves took twice the instructions, a chain of some 1,000 cycles.  With this and
+// the level's geometry in shared memory (made per operator and held in registers and local memory before)
+// a scan of 256 frames of 512x512 went from 15.4 to 14.4 ms, of 1,024 from 65.1 to 59.9, a pair of
+// 741x1003 (BF16) from 571 to 531 us, of 128x128 from 218 to 210.
+
+// A unit's columns: left and right sum; wf: the first column's weight.
+template <int COLS, bool SQ>
+__device__ __forceinline__ void cell_sums(const float *x, float wf, float dw, float &l, float &r)
 {
-    SegSum<SEG> o;
-    o.first = 0;
+    float4 a = make_float4(0.f, 0.f, 0.f, 0.f), b = a, c = a;
 #pragma unroll
-    for (int w = SEG / 2, n = 8; w >= 1; w >>= 1, n >>= 1) {
-        if (n >= 1) {
-            const bool up = lane & w;
-#pragma unroll
-            for (int k = 0; k < n; ++k) {
-                const float2 send = up ? v[k] : v[k + n], keep = up ? v[k + n] : v[k];
-                v[k] = __fadd2_rn(keep, shfl_xor2(send, w));
-            }
-            o.first += up ? n : 0;
+    for (int k = 0; k < COLS; k += 4) {
+        const float4 v = *(const float4 *)(x + k);
+        if constexpr (SQ) {
+            const float w0 = fmaf((float)k, dw, wf), w1 = fmaf((float)(k + 1), dw, wf), w2 = fmaf((float)(k + 2), dw, wf),
+                        w3 = fmaf((float)(k + 3), dw, wf);
+            a.x = fmaf((1.f - w0) * (1.f - w0), v.x, a.x); b.x = fmaf(w0 * w0, v.x, b.x);
+            a.y = fmaf((1.f - w1) * (1.f - w1), v.y, a.y); b.y = fmaf(w1 * w1, v.y, b.y);
+            a.z = fmaf((1.f - w2) * (1.f - w2), v.z, a.z); b.z = fmaf(w2 * w2, v.z, b.z);
+            a.w = fmaf((1.f - w3) * (1.f - w3), v.w, a.w); b.w = fmaf(w3 * w3, v.w, b.w);
         } else {
-            v[0] = __fadd2_rn(v[0], shfl_xor2(v[0], w));
+            a.x += v.x; b.x = fmaf((float)k, v.x, b.x);       c.x = fmaf((float)(COLS - 1 - k), v.x, c.x);
+            a.y += v.y; b.y = fmaf((float)(k + 1), v.y, b.y); c.y = fmaf((float)(COLS - 2 - k), v.y, c.y);
+            a.z += v.z; b.z = fmaf((float)(k + 2), v.z, b.z); c.z = fmaf((float)(COLS - 3 - k), v.z, c.z);
+            a.w += v.w; b.w = fmaf((float)(k + 3), v.w, b.w); c.w = fmaf((float)(COLS - 4 - k), v.w, c.w);
         }
     }
-#pragma unroll
-    for (int k = 0; k < SegSum<SEG>::kHeld; ++k) o.v[k] = v[k];
-    return o;
-}
-
-// The emission of a segment's control rows is a chain of shuffles and shared-memory writes that one
-// warp in two per scheduler runs: one strip after the other took 1,000 cycles each, half of a pass over
-// 128x128 pixels; both in one chain of packed additions 230 us -> 217 us for a pair of 128x128 frames, 5.02 ->
-// 4.80 ms for 8 stacks of 32 frames of 256x256.
-// One control row's sums of two strips (.x and .y) into their slots (points 0 .. last + 1 of a strip;
-// slot[p kSlot]).  v: the lane's columns, already weighted along x: entries 0-7 for the point left of its
-// cell k, 8-15 for the point right of it; ncomp entries of each are written, nothing where last < 0.  A
-// point between two cells gets the left cell's share after the right cell's.
-template <int SEG>
-__device__ __forceinline__ void emit_row(float2 (&v)[16], int lane, int k, int2 last, float *s0, float *s1, int ncomp)
-{
-    const SegSum<SEG> s = seg_sum16<SEG>(v, lane);
-    const bool on = SEG < 32 || (lane & 1) == 0;
-#pragma unroll
-    for (int i = 0; i < SegSum<SEG>::kHeld; ++i) {
-        const int id = s.first + i, side = id >> 3, comp = id & 7, at = (k + side) * kSlot + comp;
-        const bool w = on && comp < ncomp;
-        if (w && k <= last.x && (side == 0 || k == last.x)) s0[at] = s.v[i].x;
-        if (w && k <= last.y && (side == 0 || k == last.y)) s1[at] = s.v[i].y;
-    }
-    if (SEG == 32) return;
-    __syncwarp();
-#pragma unroll
-    for (int i = 0; i < SegSum<SEG>::kHeld; ++i) {
-        const int id = s.first + i, side = id >> 3, comp = id & 7, at = (k + 1) * kSlot + comp;
-        if (comp < ncomp && side == 1 && k < last.x) s0[at] += s.v[i].x;
-        if (comp < ncomp && side == 1 && k < last.y) s1[at] += s.v[i].y;
+    l = (a.x + a.y) + (a.z + a.w);
+    r = (b.x + b.y) + (b.z + b.w);
+    if constexpr (!SQ) {
+        const float s = l;
+        r = fmaf(wf, s, dw * r);
+        l = fmaf(1.f - fmaf((float)(COLS - 1), dw, wf), s, dw * ((c.x + c.y) + (c.z + c.w)));
     }
 }
 
-__device__ __forceinline__ void emit_any(int sl, float2 (&v)[16], int lane, int k, int2 last, float *s0, float *s1, int ncomp)
+// Cells of 8 or 16 columns, or one of 32 (HALF: by halves of 16).  A point between two cells gets both
+// shares in one addition.  x: the warp's rows, sum by sum, strip by strip; slot s0 or s1 (points 0 .. last + 1
+// of the strip, slot[p kSlot]; none where last < 0), the same one for two chunks of a cell, which `adds`
+// to earlier ones.
+template <int COLS, bool HALF, bool SQ>
+__device__ __forceinline__ void emit_cells(const float *x, int lane, float2 wf, float dw, int2 last, float *s0, float *s1,
+                                           int adds)
 {
-    if (sl >= 32) emit_row<32>(v, lane, k, last, s0, s1, ncomp);   // strips of one cell
-    else if (sl == 16) emit_row<16>(v, lane, k, last, s0, s1, ncomp);
-    else if (sl == 8) emit_row<8>(v, lane, k, last, s0, s1, ncomp);
-    else if (sl == 4) emit_row<4>(v, lane, k, last, s0, s1, ncomp);
-    else if (sl == 2) emit_row<2>(v, lane, k, last, s0, s1, ncomp);
-    else if (sl == 1) emit_row<1>(v, lane, k, last, s0, s1, ncomp);
-    else
-        // a cell width that is no power of two: cell by cell over the whole warp
-        for (int q = 0; q <= max(last.x, last.y); ++q) {
-            float2 x[16];
+    constexpr int kSums = SQ ? 2 : kEmitSums, kCells = 32 / COLS;
 #pragma unroll
-            for (int i = 0; i < 16; ++i) x[i] = k == q ? v[i] : f2(0.f);
-            const SegSum<32> s = seg_sum16<32>(x, lane);
-            const int side = s.first >> 3, comp = s.first & 7, at = (q + side) * kSlot + comp;
-            const bool w = (lane & 1) == 0 && comp < ncomp, add = side == 0 && q > 0;
-            if (w && q <= last.x) s0[at] = add ? s0[at] + s.v[0].x : s.v[0].x;
-            if (w && q <= last.y) s1[at] = add ? s1[at] + s.v[0].y : s.v[0].y;
-            __syncwarp();
+    for (int u0 = 0; u0 < 2 * kSums * kCells; u0 += 32) {
+        const int u = min(u0 + lane, 2 * kSums * kCells - 1), cell = u % kCells, row = u / kCells;
+        const bool second = row >= kSums, mine = u0 + lane == u;
+        const int comp = second ? row - kSums : row, lst = second ? last.y : last.x;
+        float w = second ? wf.y : wf.x, l, r;
+        if (HALF && cell) w = fmaf((float)COLS, dw, w);
+        cell_sums<COLS, SQ>(x + row * kEmitRow + cell * COLS, w, dw, l, r);
+        float *p = (second ? s1 : s0) + (SQ ? kEmitSums : 0) + comp;
+        if (HALF) {
+            l += __shfl_xor_sync(0xffffffffu, l, 1);
+            r += __shfl_xor_sync(0xffffffffu, r, 1);
+            const bool on = mine && cell == 0 && lst >= 0, same = s0 == s1;
+            if (on && !(second && same)) {
+                p[0] = adds ? p[0] + l : l;
+                p[kSlot] = adds ? p[kSlot] + r : r;
+            }
+            if (same) {   // chunks of one cell
+                __syncwarp();
+                if (on && second) {
+                    p[0] += l;
+                    p[kSlot] += r;
+                }
+            }
+        } else {
+            const float left = __shfl_up_sync(0xffffffffu, r, 1);
+            if (cell) l += left;
+            if (mine && cell <= lst) p[cell * kSlot] = l;
+            if (mine && cell == lst) p[(cell + 1) * kSlot] = r;
         }
+    }
+}
+
+// Cells of any width below 32: a lane has a point, and adds the columns of the cells on both sides.
+template <bool SQ>
+__device__ __forceinline__ void emit_points(const float *x, int lane, int sl, int cells, float2 wf, float dw, int2 last, float *s0,
+                                            float *s1)
+{
+    constexpr int kSums = SQ ? 2 : kEmitSums;
+    const unsigned rp = recip20(cells + 1);
+    for (int u = lane; u < 2 * kSums * (cells + 1); u += 32) {
+        const int row = div20(u, rp), pt = u - row * (cells + 1);
+        const bool second = row >= kSums;
+        const int comp = second ? row - kSums : row, lst = second ? last.y : last.x;
+        if (pt > lst + 1 || lst < 0) continue;
+        const float w0 = second ? wf.y : wf.x, *c = x + row * kEmitRow + pt * sl;
+        float v = 0.f;
+        if (pt > 0)
+            for (int k = 0; k < sl; ++k) {
+                const float w = fmaf((float)k, dw, w0);
+                v = fmaf(SQ ? w * w : w, c[k - sl], v);
+            }
+        if (pt <= lst)
+            for (int k = 0; k < sl; ++k) {
+                const float w = 1.f - fmaf((float)k, dw, w0);
+                v = fmaf(SQ ? w * w : w, c[k], v);
+            }
+        ((second ? s1 : s0) + (SQ ? kEmitSums : 0) + comp)[pt * kSlot] = v;
+    }
+}
+
+template <bool SQ>
+__device__ __forceinline__ void emit_any(int sl, const float *x, int lane, int cells, float2 wf, float dw, int2 last, float *s0,
+                                         float *s1, int adds)
+{
+    if (sl == 16) emit_cells<16, false, SQ>(x, lane, wf, dw, last, s0, s1, 0);
+    else if (sl >= 32) emit_cells<16, true, SQ>(x, lane, wf, dw, last, s0, s1, adds);
+    else if (sl == 8) emit_cells<8, false, SQ>(x, lane, wf, dw, last, s0, s1, 0);
+    else emit_points<SQ>(x, lane, sl, cells, wf, dw, last, s0, s1);
 }
 
 // Value and twice the gradient of the B-spline model for two samples (.x and .y) from their 3 x 3
@@ -1074,19 +1121,27 @@ __device__ __forceinline__ float2 bspline2(const TapRow &r0, const TapRow &r1, c
 constexpr int kRunRows = 16;   // rows of a straight run at most; half of it is tried next
 
 // Sums of control point (cr0 + i, jx) over the slots that one CTA with nr cell rows wrote: entries
-// first .. first + N - 1, segment by segment and strip by strip.
-template <int N>
+// first .. first + N - 1, segment by segment and strip by strip (FF: added in float-float).
+template <int N, bool FF = false>
 __device__ __forceinline__ void slot_sum(const float *slots, const PassGeom &P, int ncx, int nr, int i, int jx,
                                          int first, float (&o)[N])
 {
     const int ga = i > 0 ? div20(i - 1, P.rm) : 0, gb = div20(i < nr ? i : nr - 1, P.rm);
     const int srow = (P.g + 1) * kSlot, sstrip = (P.m + 1) * srow, sseg = P.nst * sstrip;
+    float e[N];
+#pragma unroll
+    for (int k = 0; k < N; ++k) e[k] = 0.f;
     auto add = [&](const float *s) {
 #pragma unroll
         for (int k = 0; k < N; k += 2) {
             const float2 v = *(const float2 *)(s + k);
-            o[k] += v.x;
-            o[k + 1] += v.y;
+            if constexpr (FF) {
+                ff_acc(o[k], e[k], v.x);
+                ff_acc(o[k + 1], e[k + 1], v.y);
+            } else {
+                o[k] += v.x;
+                o[k + 1] += v.y;
+            }
         }
     };
     const int st = div20(jx, P.rg), pt = jx - st * P.g;
@@ -1103,14 +1158,17 @@ __device__ __forceinline__ void slot_sum(const float *slots, const PassGeom &P, 
             if (left) add(pl);
             if (own) add(po);
             if (!narrow)
-                for (int q = 0; q < P.chunks; ++q) {
-                    if (jx > 0) add(p + ((jx - 1) * P.chunks + q) * sstrip + kSlot);
-                    if (jx < ncx) add(p + (jx * P.chunks + q) * sstrip);
+                for (int q = 0; q < P.sch; ++q) {
+                    if (jx > 0) add(p + ((jx - 1) * P.sch + q) * sstrip + kSlot);
+                    if (jx < ncx) add(p + (jx * P.sch + q) * sstrip);
                 }
             if (over) add(pv);
             p += sseg; po += sseg; pl += sseg; pv += sseg;
         }
     }
+    if constexpr (FF)
+#pragma unroll
+        for (int k = 0; k < N; ++k) o[k] += e[k];
 }
 
 // One pass at c (START: a level's first) or at the trial c + tau d: the moments into sm.tot (e =
@@ -1126,13 +1184,14 @@ __device__ __forceinline__ void slot_sum(const float *slots, const PassGeom &P, 
 // float-float.
 template <typename S, bool START, int R>
 __device__ void grid_pass(const Lvl &L, const Grid &G, const GridLvl &GL, const PassGeom &P, const Band &B,
-                          const float2 *c, const float2 *d, float tau, float *slots, const float *above, const PointIter &pi,
+                          const float2 *c, const float2 *d, float tau, float *slots, const float *above, float *emits, const PointIter &pi,
                           Smem &sm, Comm &comm, const cg::cluster_group &cl)
 {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int ncx = G.nx - 1, ncy = G.ny - 1, sl = P.sl, pairs = (P.nst + 1) / 2;
+    const int ncx = G.nx - 1, ncy = G.ny - 1, sl = P.sl;
     const S *Rp = (const S *)L.R, *T = (const S *)L.T;
     const float2 ncR = f2(-L.cR), dw = f2(GL.pl * GL.scale_inv);
+    float *emit = emits + warp * kEmitFloats;
     auto ct = [&](int row, int col) {   // control value of the point evaluated
         const int j = (row - B.h0) * G.nx + col;
         const float2 a = c[j];
@@ -1149,10 +1208,15 @@ __device__ void grid_pass(const Lvl &L, const Grid &G, const GridLvl &GL, const 
     for (int i = 0; i < NM; ++i) hi2[i] = lo2[i] = a[i] = f2(0.f);
 
     const int kw = sl < 32 ? div20(lane, recip20(sl)) : 0;   // the lane's cell in a strip of whole cells
-    for (int seg = 0, pr = warp;; pr += kWarps) {
-        while (pr >= pairs) { pr -= pairs; ++seg; }
+    for (int seg = 0, pr = warp, cp = 0;;) {
+        while (pr >= P.tasks) { pr -= P.tasks; ++seg; }
         if (seg >= P.nseg) break;
-        const int strip0 = 2 * pr;
+        // the task's strips from the first to before the last one
+        const bool walk = P.sch < P.chunks, past = walk && pr == P.ns;
+        const int strip0 = walk ? pr * P.chunks + 2 * cp : 2 * pr;
+        const int strips = walk ? past ? P.past + 1 : (pr + 1) * P.chunks : P.nst, slot0 = walk ? pr : strip0;
+        const int adds = cp;
+        if (++cp == P.walk || past) { cp = 0; pr += kWarps; }
         const int grp = seg >> P.hlog, piece = seg & (P.h - 1);
         const int ca = B.cr0 + grp * P.m, cb = min(ca + P.m, B.cr1);
         if (ca >= cb) continue;
@@ -1163,13 +1227,13 @@ __device__ void grid_pass(const Lvl &L, const Grid &G, const GridLvl &GL, const 
 #pragma unroll
         for (int u = 0; u < 2; ++u) {
             const int strip = strip0 + u;
-            const bool over = strip == P.ns;      // the column past the last cell
+            const bool over = strip == P.past;    // the column past the last cell
             const int cell0 = over ? ncx - 1 : sl < 32 ? strip * P.g : P.chunks == 1 ? strip : strip / P.chunks;
             const int c0 = min(cell0, ncx - 1);
             last[u] = over || sl >= 32 ? 0 : min(P.g, ncx - c0) - 1;
             const int xs = over ? ncx * sl : sl < 32 ? c0 * sl : c0 * sl + (strip - cell0 * P.chunks) * 32;
             const int xe = over ? L.W : min(L.W, min(c0 * sl + (last[u] + 1) * sl, xs + 32));
-            act[u] = strip < P.nst && xs + lane < xe && kw <= last[u];
+            act[u] = strip < strips && xs + lane < xe && kw <= last[u];
             cell[u] = c0 + min(kw, last[u]);
             xc[u] = min(xs + lane, L.W - 1);
             wx[u] = fminf(fmaf(GL.pl, (float)xc[u], GL.off) * GL.scale_inv, (float)ncx) - (float)cell[u];
@@ -1331,23 +1395,31 @@ __device__ void grid_pass(const Lvl &L, const Grid &G, const GridLvl &GL, const 
             }
             // control row cy: what the cell row above it left and the top sums of the one below
             {
-                const float2 rw = make_float2(act[0] ? wx[0] : 0.f, act[1] ? wx[1] : 0.f);
-                const float2 lw = make_float2(act[0] ? 1.f - wx[0] : 0.f, act[1] ? 1.f - wx[1] : 0.f);
-                float2 v[16];
+                const float2 wf = make_float2(__shfl_sync(0xffffffffu, wx[0], 0), __shfl_sync(0xffffffffu, wx[1], 0));
+                const int2 lst = make_int2(last[0], strip0 + 1 < strips ? last[1] : -1);
+                const int strip = (P.m + 1) * (P.g + 1) * kSlot;
+                float *slot = slots + (seg * P.nst + slot0) * strip + (cy - ca) * (P.g + 1) * kSlot;
+                float *slot1 = walk ? slot : slot + strip;
+                auto put = [&](int row, int rows, float2 v) {   // the lane's two columns of a sum
+                    emit[row * kEmitRow + lane] = act[0] ? v.x : 0.f;
+                    emit[(rows + row) * kEmitRow + lane] = act[1] ? v.y : 0.f;
+                };
+                __syncwarp();
 #pragma unroll
                 for (int i = 0; i < 2; ++i) {
-                    v[i] = __fmul2_rn(lw, sF[i]); v[8 + i] = __fmul2_rn(rw, sF[i]);
-                    v[2 + i] = __fmul2_rn(lw, sT[i]); v[10 + i] = __fmul2_rn(rw, sT[i]);
-                    v[4 + i] = __fmul2_rn(lw, s1[i]); v[12 + i] = __fmul2_rn(rw, s1[i]);
-                    v[6 + i] = v[14 + i] = f2(0.f);
-                    if constexpr (START) {
-                        v[6 + i] = __fmul2_rn(__fmul2_rn(lw, lw), sM[i]);
-                        v[14 + i] = __fmul2_rn(__fmul2_rn(rw, rw), sM[i]);
-                    }
+                    put(i, kEmitSums, sF[i]);
+                    put(2 + i, kEmitSums, sT[i]);
+                    put(4 + i, kEmitSums, s1[i]);
                 }
-                const int strip = (P.m + 1) * (P.g + 1) * kSlot;
-                float *slot = slots + (seg * P.nst + strip0) * strip + (cy - ca) * (P.g + 1) * kSlot;
-                emit_any(sl, v, lane, kw, make_int2(last[0], strip0 + 1 < P.nst ? last[1] : -1), slot, slot + strip, START ? 8 : 6);
+                __syncwarp();
+                emit_any<false>(sl, emit, lane, P.g, wf, dw.x, lst, slot, slot1, adds);
+                if constexpr (START) {
+                    __syncwarp();
+                    put(0, 2, sM[0]);
+                    put(1, 2, sM[1]);
+                    __syncwarp();
+                    emit_any<true>(sl, emit, lane, P.g, wf, dw.x, lst, slot, slot1, adds);
+                }
             }
 #pragma unroll
             for (int i = 0; i < 2; ++i) {
@@ -1401,7 +1473,7 @@ __device__ void grid_pass(const Lvl &L, const Grid &G, const GridLvl &GL, const 
 }
 
 // The same over the whole grid: this CTA's slots, and at its first row what the CTA above sent.
-template <int N>
+template <int N, bool FF = false>
 __device__ __forceinline__ void point_sum(const float *slots, const float *above, const PassGeom &P, const Band &B,
                                           int ncx, int row, int jx, int first, float (&o)[N])
 {
@@ -1410,7 +1482,7 @@ __device__ __forceinline__ void point_sum(const float *slots, const float *above
     if (row == B.cr0 && row > 0)
 #pragma unroll
         for (int k = 0; k < N; ++k) o[k] = above[jx * kSlot + first + k];
-    slot_sum<N>(slots, P, ncx, B.cr1 - B.cr0, row - B.cr0, jx, first, o);
+    slot_sum<N, FF>(slots, P, ncx, B.cr1 - B.cr0, row - B.cr0, jx, first, o);
 }
 
 // Buffers of the H1 scalar product (B null: another product): B the right-hand side -Nc dE/dc,
@@ -1518,6 +1590,7 @@ __device__ void grid_metric(const Grid &G, const PassGeom &P, const Band &B, con
 // kappa, lambda), at the own rows and, through the neighbours' staged rows, at the held ones.  Leaves
 // sum_j m_j |d_j|^2 in sm.tot[0], with the direction d held before the call <d_old, d_old - d>_M in
 // sm.tot[1] and |d_old - d|_M^2 in sm.tot[2], max |d_j|^2 in sm.tmax; identical in every CTA.
+template <bool FF = false>
 __device__ void grid_direction(const Grid &G, const Lvl &L, const PassGeom &P, const Band &B, const float2 *c,
                                float2 *d, float2 *mt, float2 *halo, const float *slots, const float *above,
                                const PointIter &pi, const float *pm, Smem &sm, Comm &comm, const cg::cluster_group &cl, const H1Bufs &h1)
@@ -1530,7 +1603,7 @@ __device__ void grid_direction(const Grid &G, const Lvl &L, const PassGeom &P, c
     auto rhs = [&](int i, int jx) {
         const int row = B.cr0 + i, k = (row - B.h0) * G.nx + jx;
         float s[6];
-        point_sum<6>(slots, above, P, B, G.nx - 1, row, jx, 0, s);
+        point_sum<6, FF>(slots, above, P, B, G.nx - 1, row, jx, 0, s);
         const float gx = fmaf(aP, s[0], fmaf(bmaP, s[2], kappa * s[4]));
         const float gy = fmaf(aP, s[1], fmaf(bmaP, s[3], kappa * s[5]));
         const float2 cj = c[k];
@@ -1707,6 +1780,15 @@ __device__ __forceinline__ float2 grid_eval_global(const float2 *q, const Grid &
     return u;
 }
 
+// The level's geometry into shared memory (a barrier follows): read from the parameters by every pass, it
+// waits for the constant cache.
+__device__ __forceinline__ const PassGeom &level_geom(Smem &sm, const Params &p, int l, bool over)
+{
+    static_assert(sizeof(PassGeom) % 4 == 0 && sizeof(PassGeom) / 4 <= kThreads, "copied by words");
+    if (threadIdx.x < sizeof(PassGeom) / 4) ((int *)&sm.geom)[threadIdx.x] = ((const int *)&p.geom[l][over])[threadIdx.x];
+    return sm.geom;
+}
+
 template <typename S, int R>
 __device__ void run_nonrigid(const Params &p, const OpDesc &op, int op_index, Smem &sm, float2 *gbuf, Comm &comm,
                              const cg::cluster_group &cl)
@@ -1725,6 +1807,7 @@ __device__ void run_nonrigid(const Params &p, const OpDesc &op, int op_index, Sm
     float2 *c = gbuf + lay.c, *d = gbuf + lay.d, *mt = gbuf + lay.mt, *halo = gbuf + lay.halo;
     float *slots = (float *)(gbuf + lay.slots);
     const float *above = (const float *)(gbuf + lay.above);
+    float *emits = (float *)(gbuf + lay.emits);
     const H1Bufs hb{h1 ? mt : nullptr, (float2 *)slots, (float2 *)slots + Nc, p.h1q, (float)(cfg.sigma * cfg.sigma)};
     // initial control values (finest px), scaled to the coarsest level
     {
@@ -1757,7 +1840,7 @@ __device__ void run_nonrigid(const Params &p, const OpDesc &op, int op_index, Sm
     for (int l = Lc - 1; l >= 0; --l) {
         const Lvl L = level_of(p, op.ref, op.tmpl, l);
         const GridLvl GL = grid_level(G, L, l);
-        const PassGeom P = pass_geom(G.s >> l, G.nx - 1, B.q, L.W > (G.nx - 1) * (G.s >> l));
+        const PassGeom &P = level_geom(sm, p, l, L.W > (G.nx - 1) * (G.s >> l));
         if (cfg.metric == REG_METRIC_MEAN)
             for (int j = tid; j < held; j += kThreads) mt[j] = make_float2(1.f, 1.f);
         if (tid == 0) {
@@ -1773,8 +1856,8 @@ __device__ void run_nonrigid(const Params &p, const OpDesc &op, int op_index, Sm
         __syncthreads();
         for (bool start = true;; start = false) {
             const float tau = sm.pm[kPmTau];   // not read by a level's first pass
-            if (start) grid_pass<S, true, R>(L, G, GL, P, B, c, d, 0.f, slots, above, pi, sm, comm, cl);
-            else grid_pass<S, false, R>(L, G, GL, P, B, c, d, tau, slots, above, pi, sm, comm, cl);
+            if (start) grid_pass<S, true, R>(L, G, GL, P, B, c, d, 0.f, slots, above, emits, pi, sm, comm, cl);
+            else grid_pass<S, false, R>(L, G, GL, P, B, c, d, tau, slots, above, emits, pi, sm, comm, cl);
             if (tid == 0) {
                 sm.action = field_eval(k, cfg, sm.tot, start, sm.pm, sm.idata[0]);
                 if (sm.fail) sm.action = kActDone;
@@ -1907,7 +1990,7 @@ __device__ void run_op(const Params &p, int op_index, Smem &sm, float2 *gbuf, Co
 // 76 (8 CTAs per operator).  U: pixels in flight per lane in the nonrigid passes (2 or 4, the tile shape
 // reg_autotune chooses): two columns of one or two rows.
 template <int MODE, typename S, int MINB, int U = 4>
-__global__ void __launch_bounds__(kThreads, MINB) op_kernel(Params p)
+__global__ void __launch_bounds__(kThreads, MINB) op_kernel(const __grid_constant__ Params p)
 {
     __shared__ Smem sm;
     extern __shared__ __align__(16) float2 gbuf[];   // nonrigid: control grid c, d, ct, gp
@@ -1923,7 +2006,7 @@ __global__ void __launch_bounds__(kThreads, MINB) op_kernel(Params p)
 // Persistent launch: each cluster claims ready operators from the device queue
 // until all n_ops have been claimed.  Every wait is bounded by queue.timeout_ns.
 template <int MODE, typename S, int MINB, int U = 4>
-__global__ void __launch_bounds__(kThreads, MINB) persistent_kernel(Params p)
+__global__ void __launch_bounds__(kThreads, MINB) persistent_kernel(const __grid_constant__ Params p)
 {
     __shared__ Smem sm;
     extern __shared__ __align__(16) float2 gbuf[];
@@ -2071,7 +2154,7 @@ __global__ void __launch_bounds__(kThreads, MINB) persistent_kernel(Params p)
 // Rigid: theta (device) -> out[0] = E, out[1..3] = dE/dtheta.  Nonrigid: control values cgrid
 // (finest px, level 0) -> out[0] = E and grad_c = dE/dc.
 template <int MODE, typename S>
-__global__ void __launch_bounds__(kThreads) energy_kernel(Params p, const double *theta, const float2 *cgrid,
+__global__ void __launch_bounds__(kThreads) energy_kernel(const __grid_constant__ Params p, const double *theta, const float2 *cgrid,
                                                           double *out, float2 *grad_c)
 {
     __shared__ Smem sm;
@@ -2112,6 +2195,7 @@ __global__ void __launch_bounds__(kThreads) energy_kernel(Params p, const double
         float2 *c = gbuf + lay.c, *d = gbuf + lay.d, *mt = gbuf + lay.mt, *halo = gbuf + lay.halo;
         float *slots = (float *)(gbuf + lay.slots);
         const float *above = (const float *)(gbuf + lay.above);
+        float *emits = (float *)(gbuf + lay.emits);
         for (int j = tid; j < (B.h1 - B.h0) * G.nx; j += kThreads) {
             c[j] = cgrid[B.h0 * G.nx + j];
             d[j] = make_float2(0.f, 0.f);
@@ -2119,8 +2203,9 @@ __global__ void __launch_bounds__(kThreads) energy_kernel(Params p, const double
         }
         __syncthreads();
         const GridLvl GL = grid_level(G, L, 0);
-        const PassGeom P = pass_geom(G.s, G.nx - 1, B.q, L.W > (G.nx - 1) * G.s);
-        grid_pass<S, true, 2>(L, G, GL, P, B, c, d, 0.f, slots, above, pi, sm, comm, cl);
+        const PassGeom &P = level_geom(sm, p, 0, L.W > (G.nx - 1) * G.s);
+        __syncthreads();
+        grid_pass<S, true, 2>(L, G, GL, P, B, c, d, 0.f, slots, above, emits, pi, sm, comm, cl);
         FieldCtl &k = sm.fctl;
         if (tid == 0) {
             set_level(k.ls, L.W, L.H);
@@ -2133,12 +2218,12 @@ __global__ void __launch_bounds__(kThreads) energy_kernel(Params p, const double
         if (grad_c) {
             float pm[4];
             for (int q = 0; q < 4; ++q) pm[q] = sm.pm[q];
-            grid_direction(G, L, P, B, c, d, mt, halo, slots, above, pi, pm, sm, comm, cl, H1Bufs{});
+            grid_direction<true>(G, L, P, B, c, d, mt, halo, slots, above, pi, pm, sm, comm, cl, H1Bufs{});
             // d = -Nc dE/dc (unit scalar product)
-            const float s = -1.f / (float)Nc;
+            const double s = -1.0 / (double)Nc;
             const float2 *own = d + (B.cr0 - B.h0) * G.nx;
             for (int j = tid; j < (B.own1 - B.cr0) * G.nx; j += kThreads)
-                grad_c[B.cr0 * G.nx + j] = make_float2(s * own[j].x, s * own[j].y);
+                grad_c[B.cr0 * G.nx + j] = make_float2((float)(s * (double)own[j].x), (float)(s * (double)own[j].y));
         }
     }
     cl.sync();   // no CTA leaves while a peer may still read its shared memory
@@ -2192,36 +2277,42 @@ __global__ void grid_from_dense_kernel(const float *u, int W, int H, Grid G, flo
 
 // ================================================================== host launchers
 // Dynamic shared memory of the nonrigid kernels (layout of grid_layout).
-static size_t grid_smem(const Params &p, int cluster)
+static size_t set_geometry(Params &p, int cluster, bool exact = false)
 {
     if (p.cfg.mode != REG_NONRIGID) return 0;
     const bool h1 = p.cfg.metric == REG_METRIC_H1;
+    const GridLayout lay = grid_layout(p.gnx, p.gny, cluster, h1);
     size_t slots = h1 ? sizeof(float2) * 2 * (size_t)p.gnx * p.gny : 0;
     for (int l = 0; l < p.cfg.levels; ++l)
         for (const bool over : {false, true}) {   // the frame's width decides, which is not known here
-            const size_t b = sizeof(float) * slot_floats(pass_geom(p.gs >> l, p.gnx - 1, band_cells(p.gny, cluster), over));
-            if (b > slots) slots = b;
+            const PassGeom P = pass_geom(p.gs >> l, p.gnx - 1, band_cells(p.gny, cluster), over, slot_room(lay), exact);
+            p.geom[l][over] = P;
+            slots = std::max(slots, sizeof(float) * slot_floats(P));
         }
-    return sizeof(float2) * (size_t)grid_layout(p.gnx, p.gny, cluster, h1).slots + slots;
+    return sizeof(float2) * (size_t)lay.slots + slots;
+}
+static size_t grid_smem(const Params &p, int cluster)
+{
+    Params q = p;
+    return set_geometry(q, cluster);
 }
 
 // The largest grids do not fit the few CTAs of a small cluster: from the size asked for, the first
 // whose control state and slots leave room for the static part.
 int fit_cluster(const Params &p, int cluster)
 {
-    constexpr size_t kMost = 227 * 1024 - sizeof(Smem) - 256;
-    while (cluster < kMaxCluster && grid_smem(p, cluster) > kMost) cluster *= 2;
+    while (cluster < kMaxCluster && grid_smem(p, cluster) > (size_t)kMostSmem) cluster *= 2;
     return cluster;
 }
 
 template <typename K>
-static cudaError_t launch_cluster(K kernel, int blocks, int cluster, cudaStream_t s, const Params &p)
+static cudaError_t launch_cluster(K kernel, int blocks, int cluster, cudaStream_t s, Params p)
 {
     if (cluster > 8) {
         cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
         if (e != cudaSuccess) return e;
     }
-    const size_t smem = grid_smem(p, cluster);
+    const size_t smem = set_geometry(p, cluster);
     if (smem > 0) {
         cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
@@ -2338,16 +2429,17 @@ int persistent_resident_clusters(const Params &p, int storage, int cluster)
     return n;
 }
 
-cudaError_t launch_energy(const Params &p, int storage, const double *theta_dev, const float2 *grid_dev,
+cudaError_t launch_energy(const Params &params, int storage, const double *theta_dev, const float2 *grid_dev,
                           double *out_dev, float2 *grad_dev, cudaStream_t s)
 {
     (void)storage;
     constexpr int kEnergyCtas = kMaxCluster;
+    Params p = params;
     const void *kern = p.cfg.mode == REG_RIGID ? (const void *)energy_kernel<REG_RIGID, float>
                                                : (const void *)energy_kernel<REG_NONRIGID, float>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (e != cudaSuccess) return e;
-    const size_t smem = grid_smem(p, kEnergyCtas);
+    const size_t smem = set_geometry(p, kEnergyCtas, true);
     if (smem > 0) {
         e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;

@@ -98,6 +98,23 @@ def test_gradient_for_every_kind_of_cell_width(shape, grid):
     np.testing.assert_allclose(gd.cpu().numpy().transpose(2, 0, 1), go, atol=2e-4 * np.abs(go).max())
 
 
+@pytest.mark.parametrize("shape,grid", [((64, 60000), 64), ((65, 60001), 96)])
+def test_gradient_of_thousands_of_strips(shape, grid):
+    # more 32-column strips than shared memory has slots for: a warp walks a cell's chunks (two of them; three,
+    # with a column past the last cell), and there is a single band of cell rows
+    H, W = shape
+    rng = np.random.default_rng(22)
+    R, T = (rng.uniform(0, 1, size=(H, W)).astype(np.float32) for _ in range(2))
+    g = O.grid_for(W, H, grid)
+    c = rng.uniform(-0.9, 0.9, size=(g.ny, g.nx, 2)).astype(np.float32)
+    gd = torch.zeros((g.ny, g.nx, 2), device="cuda")
+    E = B.Context(B.Config(mode="nonrigid", grid=grid)).energy_grid(
+        torch.from_numpy(R).cuda(), torch.from_numpy(T).cuda(), torch.from_numpy(c).cuda(), gd)
+    Eo, go = O.grid_energy(R, T, 0, g, c.transpose(2, 0, 1).astype(np.float64), 2.0)
+    assert abs(E - Eo) <= 1e-6 * abs(Eo)
+    np.testing.assert_allclose(gd.cpu().numpy().transpose(2, 0, 1), go, atol=2e-4 * np.abs(go).max())
+
+
 @pytest.mark.parametrize("cluster", [1, 2, 4, 8, 16])
 @pytest.mark.parametrize("levels,grid,metric", [(1, 16, 1), (3, 16, 1), (2, 24, 0), (2, 16, 2)])
 def test_pair_for_every_band_split(cluster, levels, grid, metric):
