@@ -38,6 +38,7 @@ sys.path.insert(0, ROOT)
 
 METRIC = "registered frames/s and operator applications/s at <=0.02 px vs FP64 oracle; stream p50/p99"
 UNIT = "frames/s"
+STOP_REL = 1   # stop code of a level ended by the relative-decrease test
 
 
 def workload_spec(name: str, rank: int, frames: int = 0):
@@ -153,8 +154,8 @@ def peaks():
 
 
 def algorithmic_bytes(stats, H, W, levels, storage_bytes, mode):
-    """Bytes the method must move per step in the operator kernels: every energy
-    evaluation reads the reference and template level once (2 s P_l bytes)."""
+    """Bytes the method must move per step in the operator kernels: every evaluation counted
+    in `stats` reads the reference and template level once (2 s P_l bytes)."""
     total = 0.0
     sizes = []
     h, w = H, W
@@ -165,6 +166,15 @@ def algorithmic_bytes(stats, H, W, levels, storage_bytes, mode):
         for l, ev in enumerate(s["evals"]):
             total += ev * 2 * storage_bytes * sizes[l]
     return total
+
+
+def pixel_passes(stats):
+    """Passes over a level's pixels for the evaluations of `stats`, per operator and level.  One pass
+    gives the energy at a point and the sums its gradient follows from, so a level makes one for its start
+    and one per trial; the evaluations also count the accepted points' gradients, which need none (an
+    accepted point that ends the level by the relative-decrease test has no gradient)."""
+    return [{"evals": [ev - it + (1 if stop == STOP_REL else 0)
+                       for ev, it, stop in zip(s["evals"], s["iters"], s["stop"])]} for s in stats]
 
 
 def pyramid_bytes(N, H, W, levels, storage_bytes, mode):
@@ -750,7 +760,7 @@ def main():
 
     # roofline of the operator kernel
     sb = 4 if cfg.storage == "f32" else 2
-    alg = sum(algorithmic_bytes(st, H, W, cfg.levels, sb, cfg.mode) for st in st_list) / len(st_list)
+    alg = sum(algorithmic_bytes(pixel_passes(st), H, W, cfg.levels, sb, cfg.mode) for st in st_list) / len(st_list)
     kms = sum(t["op_kernel_ms"] for t in tim) / len(tim)
     launches = sum(t["op_launches"] for t in tim) / len(tim)
     peak, peak_src = peaks()
