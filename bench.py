@@ -572,9 +572,8 @@ def mixed_batch(args, dev, world, rank, dist):
         print(json.dumps(line), flush=True)
 
 
-# CTAs per operator and register form for each frame size of c4 (measured on the batched scans:
-# 4 / 3 CTAs per SM for 256^2, 8 / 4 for 512^2, 16 / 3 for 1024^2 took the whole batch from
-# 4,086 to 4,670 frames/s against 16 CTAs for every size)
+# CTAs per operator for each frame size of c4, and the register form as recorded (3 and 4 name the same
+# one): fewer CTAs where more operators run side by side (256^2), more for the large frames
 C4_SHAPE = {256: (4, 3), 512: (8, 4), 1024: (16, 3)}
 
 
