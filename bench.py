@@ -925,7 +925,7 @@ def main():
                          else "fallback 6.8 TB/s",
                          "kernel": f"{kname} (operator kernel)", "algorithmic_bytes_per_step": alg,
                          "kernel_ms_per_step": round(kms, 3), "launches_per_step": launches,
-                         "caveat": "issue-bound, not DRAM-bound: the two pyramids of an operator stay in L2 "
+                         "caveat": "latency-bound, not DRAM-bound: the two pyramids of an operator stay in L2 "
                                    "(see the committed ncu summaries); the algorithmic bytes are read from L2 "
                                    "many times over"},
             "pyramid_roofline": pyramid,

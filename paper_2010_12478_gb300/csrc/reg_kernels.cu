@@ -5,8 +5,8 @@
 //     inside ONE thread-block cluster: every level, every gradient-flow
 //     iteration and every Armijo trial.  The C CTAs of the cluster split the
 //     rows of each pyramid level; their partial sums meet through distributed
-//     shared memory, so an iteration costs cluster barriers and never a
-//     kernel launch or a grid-wide synchronisation.
+//     shared memory, so an iteration costs two exchanges within the cluster (the
+//     rigid model: one) and never a kernel launch or a grid-wide synchronisation.
 //   * Per pixel the work is FP32 (warp, sample, derivative, moment products).
 //     Sums are accumulated per thread in FP32 over runs of 8 pixels, then carried
 //     as float-float pairs (error-free transformations on the FP32 pipes: GB300's
@@ -14,8 +14,9 @@
 //     in FP64 across the cluster.  Reduction order is fixed, so results are bitwise
 //     reproducible for a given cluster size.
 //   * The step controller (NCC from the moments, gradient, Armijo test, step
-//     size, stop rules) is FP64 and runs on thread 0 of every CTA of the
-//     cluster on identical totals, so all CTAs take identical decisions.
+//     size, stop rules) is FP64 and runs on one thread (the rigid model: one
+//     warp) of every CTA of the cluster on identical totals, so all CTAs take
+//     identical decisions.
 //   * Images are read through the read-only path; the nonrigid model's control
 //     values live in shared memory.
 #include <cooperative_groups.h>
@@ -796,12 +797,12 @@ __device__ void run_rigid(const Params &p, const OpDesc &op, int op_index, Smem 
 // the gradient, and a level starts with one pass, which also gives the Gauss-Newton scalar product.
 // The gradient sums of a rejected trial are dropped.  With separate passes a scan of 256 frames of
 // 512x512 took 28.4 ms and a pair 1,031 us (8 CTAs per operator); fused, with two packed columns a lane
-// and sliding windows, 16.5 ms and 513 us, and what bounds the pass is the latency of its loads and of
-// dependent packed steps (39 % issue, 16 warps per SM).
+// and sliding windows, 16.5 ms and 513 us; with the exchanges and emissions below 14.4 ms and 370 us.  What
+// bounds the pass is the latency of its loads and of dependent packed steps (40 % issue, 16 warps per SM).
 //
 // A CTA of the cluster holds the control rows of its own band of cell rows and one row on either
 // side, assembles the gradient at its own rows (the first one with the last partial row of the CTA
-// above, read from its shared memory), and hands the direction of its edge rows to its neighbours.
+// above, which sends it), and hands the direction of its edge rows to its neighbours.
 // With the whole grid in every CTA, each assembled all of it (13,000 cycles of an iteration's 230,000
 // at 512x512, most of one at 128x128) and 26 KB a CTA were taken from the L1 cache.
 
