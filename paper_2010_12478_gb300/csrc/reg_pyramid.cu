@@ -106,7 +106,8 @@ template <typename S> struct Levels {
 // column with kMeanBatch loads in flight), and its first CTA adds the CTAs' sums in rank order.  The
 // split is the same for every batch size, so a frame's means do not depend on the call it is in.
 // One CTA sums at the rate a single SM loads, about 80 us for a 512x512 level: most of the call of a
-// small pair.
+// small pair.  A CTA stores into the first one's shared memory only once every CTA of the cluster is
+// known to run: each arrives at the cluster barrier first and waits there after its sums.
 constexpr int kMeanCtas = 8, kMeanWarps = 8, kMeanBatch = 8;
 template <typename S>
 __global__ void __launch_bounds__(32 * kMeanWarps) level_means(Levels<S> L, float *means, int levels)
@@ -114,6 +115,7 @@ __global__ void __launch_bounds__(32 * kMeanWarps) level_means(Levels<S> L, floa
     __shared__ float2 ws[kMeanWarps];
     __shared__ float2 part[kMeanCtas];
     cg::cluster_group cl = cg::this_cluster();
+    cl.barrier_arrive();
     const int l = blockIdx.y, f = blockIdx.x / kMeanCtas, rank = cl.block_rank();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int W = L.W[l], H = L.H[l], pitch = L.pitch[l];
@@ -137,6 +139,7 @@ __global__ void __launch_bounds__(32 * kMeanWarps) level_means(Levels<S> L, floa
     }
     if (lane == 0) ws[warp] = make_float2(hi, lo);
     __syncthreads();
+    cl.barrier_wait();
     if (threadIdx.x == 0) {
         float h = 0.f, l2 = 0.f;
         for (int k = 0; k < kMeanWarps; ++k) ff_add(h, l2, ws[k].x, ws[k].y);

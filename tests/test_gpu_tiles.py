@@ -175,3 +175,22 @@ def test_pair_takes_frames_and_fields_from_anywhere(mode):
         c = torch.zeros((g.ny, g.nx, 2), device="cuda") + 0.3
         E = [B.Context(B.Config(mode=mode)).energy_grid(R, T, c) for R, T in ((dev[0], dev[1]), (F[0], dev[1]), (rev[1], rev[0]))]
         assert E[0] == E[1] == E[2]
+
+
+@pytest.mark.parametrize("mode", ["rigid", "nonrigid"])
+def test_level_means_of_levels_with_fewer_rows_than_ctas(mode):
+    # most CTAs that sum a level's mean have no row of it and reach the exchange at once: many frames side by
+    # side, the coarsest level 2 x 2 pixels.  A frame's means, and with them a pair's result, do not depend on
+    # the launch they are in: identical frames give identical operators, at the energy of a pair on its own
+    pair = synth.make_series(synth.SeriesSpec(2, 8, 7, step=0.5, snr=(10.0, 10.0), seed=5)).frames
+    F = torch.cat([pair] * 256).contiguous().cuda()
+    cfg = B.Config(mode=mode, levels=3, max_iter=3)
+    ctx = B.Context(cfg)
+    out = torch.empty((2, 8, 7), device="cuda")
+    _, one = ctx.pairwise(F[0], F[1], field_out=out if mode == "nonrigid" else None)
+    for _ in range(4):
+        _, st = ctx.scan(F, exec="level")
+        assert {s["energy"] for s in st[:len(F) - 1:2]} == {st[0]["energy"]}
+        assert {s["energy"] for s in st[1:len(F) - 1:2]} == {st[1]["energy"]}
+    # another cluster size, another order of the sums: the relative energy bar of the parity tests
+    assert abs(one["energy"] - st[0]["energy"]) <= 1e-5 * max(abs(one["energy"]), 1e-2)
