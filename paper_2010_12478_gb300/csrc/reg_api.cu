@@ -117,9 +117,11 @@ bool is_device_ptr(const void *p)
     return a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged;
 }
 
-// Memory that kernels on `device` read directly: its own, or managed.
-bool on_device(const void *p, int device)
+// Floats that kernels on `device` take where they are: its own memory, or managed, at a float's
+// alignment.  Anything else is copied first, and a copy takes any address.
+bool in_place(const void *p, int device)
 {
+    if ((uintptr_t)p % alignof(float) != 0) return false;
     cudaPointerAttributes a;
     if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
         cudaGetLastError();
@@ -1551,9 +1553,9 @@ extern "C" int reg_pairwise(reg_ctx_t *ctx, const float *R, const float *T, int 
     const size_t fbytes = sizeof(float) * (size_t)H * pitch, fb = sizeof(float) * 2 * (size_t)W * H;
     // frames and fields in this device's memory are read and written where they are; others go through
     // a staging buffer: R and T, then (nonrigid) one dense field for the initial guess or the result
-    const bool direct = on_device(R, ctx->device) && on_device(T, ctx->device);
-    const bool in_direct = field_in && on_device(field_in, ctx->device);
-    const bool out_direct = nonrigid && on_device(field_out, ctx->device);
+    const bool direct = in_place(R, ctx->device) && in_place(T, ctx->device);
+    const bool in_direct = field_in && in_place(field_in, ctx->device);
+    const bool out_direct = nonrigid && in_place(field_out, ctx->device);
     const size_t frame_bytes = direct ? 0 : 2 * fbytes;
     CHECK(ctx->frames_dev.reserve(frame_bytes + (nonrigid && (!out_direct || (field_in && !in_direct)) ? fb : 0)));
     float *stage = ctx->frames_dev.as<float>(), *stage_u = (float *)((char *)stage + frame_bytes);
@@ -1664,7 +1666,7 @@ extern "C" int reg_energy(reg_ctx_t *ctx, const float *R, const float *T, int W,
     int rc = geometry(W, H, 1, g);
     const size_t fbytes = sizeof(float) * (size_t)W * H;
     Params p;
-    const bool direct = on_device(R, ctx->device) && on_device(T, ctx->device);
+    const bool direct = in_place(R, ctx->device) && in_place(T, ctx->device);
     if (rc == REG_OK && !direct) rc = ctx->frames_dev.reserve(2 * fbytes);
     if (rc == REG_OK) {
         // frames in this device's memory are read where they are (the stride may wrap: it is added once)

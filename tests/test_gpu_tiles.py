@@ -194,3 +194,40 @@ def test_level_means_of_levels_with_fewer_rows_than_ctas(mode):
         assert {s["energy"] for s in st[1:len(F) - 1:2]} == {st[1]["energy"]}
     # another cluster size, another order of the sums: the relative energy bar of the parity tests
     assert abs(one["energy"] - st[0]["energy"]) <= 1e-5 * max(abs(one["energy"]), 1e-2)
+
+
+class _At:
+    """Floats at any byte of a device buffer, as a caller's packed record may hold them."""
+
+    def __init__(self, a, off):
+        self.shape = a.shape
+        raw = a.contiguous().view(torch.uint8).reshape(-1)
+        self.buf = torch.zeros(raw.numel() + 16, dtype=torch.uint8, device="cuda")
+        self.at = self.buf[off:off + raw.numel()]
+        self.at.copy_(raw)
+
+    def data_ptr(self):
+        return self.at.data_ptr()
+
+    def is_contiguous(self):
+        return True
+
+    def floats(self):
+        return self.at.clone().view(torch.float32).reshape(self.shape).cpu()
+
+
+@pytest.mark.parametrize("off", [1, 2, 6, 4])
+def test_frames_and_fields_off_a_floats_alignment_are_staged(off):
+    # the kernels load floats: device memory off their alignment goes through the staging copy, as host memory
+    # does; frames a fraction of a float apart do too
+    F = synth.make_series(synth.SeriesSpec(2, 40, 37, step=1.0, field_amp=0.5, snr=(10.0, 10.0), seed=6)).frames.cuda()
+    init = torch.full((2, 40, 37), 0.25, device="cuda")
+    for R, T in ((_At(F[0], off), _At(F[1], off)), (F[0], _At(F[1], off)), (_At(F[0], off), F[1])):
+        ctx = B.Context(B.Config(mode="rigid"))
+        assert ctx.pairwise(R, T)[1] == ctx.pairwise(F[0], F[1])[1]
+        assert ctx.energy_rigid(R, T, [0.01, 0.2, 0.1])[0] == ctx.energy_rigid(F[0], F[1], [0.01, 0.2, 0.1])[0]
+        ctx = B.Context(B.Config(mode="nonrigid"))
+        want, got = torch.empty((2, 40, 37), device="cuda"), _At(torch.zeros((2, 40, 37), device="cuda"), off)
+        ctx.pairwise(F[0], F[1], field_in=init, field_out=want)
+        ctx.pairwise(R, T, field_in=_At(init, off), field_out=got)
+        assert torch.equal(got.floats(), want.cpu())
