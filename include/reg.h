@@ -44,7 +44,9 @@
  *     environment overrides it), and reg_scan then returns REG_ETIMEOUT with the
  *     context still usable.  For tests, REG_FAULT_INJECT=stuck_op in the
  *     environment makes one operator of the next persistent reg_scan wait for
- *     an input that never arrives.
+ *     an input that never arrives.  The CTAs of an operator wait for each other
+ *     two seconds at most (REG_EXCHANGE_TIMEOUT_MS); REG_FAULT_INJECT=mute_cta
+ *     keeps an operator's last CTA from sending, so that they wait in vain.
  */
 #ifndef REG_H
 #define REG_H
@@ -61,7 +63,7 @@ extern "C" {
 #define REG_EINVAL   -1   /* bad argument (size, pointer, mode, adjacency of B's inputs) */
 #define REG_ENOMEM   -2   /* device or host allocation failed */
 #define REG_EBUDGET  -3   /* stream admission refused: memory budget or slots full; retry later */
-#define REG_ETIMEOUT -4   /* a bounded wait gave up (device queue or host poll) */
+#define REG_ETIMEOUT -4   /* a bounded wait gave up (device queue, an operator's CTAs for each other, host poll) */
 #define REG_ECUDA    -5   /* CUDA runtime error, or no usable GPU */
 #define REG_ESTATE   -6   /* object used in the wrong state */
 
@@ -212,7 +214,8 @@ void reg_ctx_destroy(reg_ctx_t *ctx);
  *   field_out  REG_NONRIGID result field [2][H][W] (host or device); may be NULL
  *              for REG_RIGID.
  *   stats      optional (host).
- * Errors: REG_EINVAL (W or H < 2 at the coarsest level, pitch < W, NULL R/T/out). */
+ * Errors: REG_EINVAL (W or H < 2 at the coarsest level, pitch < W, NULL R/T/out), REG_ETIMEOUT
+ * (the operator's CTAs waited two seconds for each other: no result). */
 int reg_pairwise(reg_ctx_t *ctx, const float *R, const float *T, int W, int H, int pitch,
                  const reg_elem_t *init, const float *field_in,
                  reg_elem_t *out, float *field_out, reg_stats_t *stats, void *stream);
@@ -230,7 +233,8 @@ int reg_pairwise(reg_ctx_t *ctx, const float *R, const float *T, int W, int H, i
  *   per_op     optional host array of (N-1) + (#B operators of the schedule)
  *              stats, leaves first, then the B operators in DAG order
  *              (reg_scan_work() gives the count).
- * Errors: REG_EINVAL, REG_ENOMEM, REG_ECUDA, REG_ETIMEOUT (persistent queue). */
+ * Errors: REG_EINVAL, REG_ENOMEM, REG_ECUDA, REG_ETIMEOUT (persistent
+ * queue, or an operator as in reg_pairwise). */
 int reg_scan(reg_ctx_t *ctx, const float *frames, int N, int W, int H, int pitch,
              int schedule, int exec, reg_elem_t *out, float *fields_out,
              reg_stats_t *per_op, void *stream);
@@ -330,7 +334,7 @@ int reg_scan_dag(int schedule, int n, int32_t *left, int32_t *right, int32_t *ou
  *   stream   a stream of `device` (REG_EINVAL otherwise), or NULL.
  * Errors: REG_EINVAL for a nonrigid or otherwise invalid config, sizes beyond the
  * limit (with a message naming it), host, foreign-device or NULL pointers, a stream
- * of another device; REG_ECUDA for CUDA failures.
+ * of another device; REG_ETIMEOUT as reg_pairwise; REG_ECUDA for CUDA failures.
  * The first call for a device resolves the array's device address
  * (cudaGetSymbolAddress) with that device current.  The call waits for `stream`
  * several times (the level means come back to the host between the pyramid and the
@@ -356,7 +360,8 @@ int reg_pyramid(reg_ctx_t *ctx, const float *frame, int W, int H, int pitch,
  *   REG_NONRIGID: grid_values: control values [ny][nx] (x, y) pairs, device;
  *                 grad_values: dE/dc in the same layout, device, optional.
  *                 lambda and grid spacing from the context configuration.
- *   energy (host): E. */
+ *   energy (host): E.
+ * Errors: REG_EINVAL, REG_ECUDA, REG_ETIMEOUT (as reg_pairwise; energy and grad are not written). */
 int reg_energy(reg_ctx_t *ctx, const float *R, const float *T, int W, int H,
                const double *theta, const float *grid_values, double *energy,
                double *grad, float *grad_values, void *stream);
@@ -406,7 +411,8 @@ int reg_stream_grids(reg_stream_t *s, float *ring, int capacity);
 
 /* Collect up to `max` finished results in submission order; waits up to
  * timeout_us for at least one (0 = do not wait).  *n_out = number written.
- * REG_ETIMEOUT if none finished in time (n_out = 0). */
+ * REG_ETIMEOUT if none finished in time (n_out = 0).  REG_ECUDA once a launch failed or an operator's CTAs
+ * gave up waiting for each other: what finished before is still returned, nothing after it will be. */
 int reg_stream_poll(reg_stream_t *s, reg_result_t *out, int max, int *n_out, int timeout_us);
 
 /* Finish all submitted frames and release the stream. */

@@ -806,6 +806,13 @@ int ensure_op_events(reg_ctx *ctx, size_t n)
 // among them.
 int base_params(reg_ctx *ctx, const Geometry &g, int n_frames, int n_nodes, int n_ops, Params &p, cudaStream_t s);
 
+// A launch's status words, and what reg_energy's kernel reads and writes beside them.
+struct StatusBlock {
+    int status[4];
+    double energy[4];   // E and, rigid, its gradient
+    double theta[3];
+};
+
 // Allocate node storage and stats; fill Params.
 int prepare_params(reg_ctx *ctx, const Geometry &g, int n_frames, int n_nodes, int n_ops, Params &p, cudaStream_t s)
 {
@@ -816,7 +823,7 @@ int prepare_params(reg_ctx *ctx, const Geometry &g, int n_frames, int n_nodes, i
     p.stats = ctx->stats.as<OpStats>();
     CHECK(ctx->node_theta.reserve(sizeof(double) * 3 * std::max(1, n_nodes)));
     p.node_theta = ctx->node_theta.as<double>();
-    CHECK(ctx->status.reserve(sizeof(int) * 4));
+    CHECK(ctx->status.reserve(sizeof(StatusBlock)));
     p.status = ctx->status.as<int>();
     CU(cudaMemsetAsync(p.status, 0, sizeof(int) * 4, s));
     CU(cudaMemsetAsync(p.stats, 0, sizeof(OpStats) * std::max(1, n_ops), s));
@@ -958,6 +965,7 @@ int execute(reg_ctx *ctx, const ScanPlan &plan, Params &p, int exec, const TileS
         // The graph bakes in the kernel arguments (workspace pointers, config) and the
         // dependency edges; the descriptors themselves are read from device memory when it runs.
         p.op_base = 0;
+        set_exchange_limits(p);
         uint64_t key = fnv1a(&p, sizeof(p), 1469598103934665603ULL);
         key = fnv1a(plan.ops.data(), sizeof(OpDesc) * plan.ops.size(), key);
         int hdr[4] = {C, storage, ctx->cfg.mode, n_ops};
@@ -1683,18 +1691,18 @@ extern "C" int reg_energy(reg_ctx_t *ctx, const float *R, const float *T, int W,
     }
     if (rc == REG_OK) rc = build_level_table(ctx, g, 2, s);
     if (rc == REG_OK) rc = prepare_params(ctx, g, 2, 1, 1, p, s);
-    if (rc == REG_OK) rc = ctx->tmp.reserve(sizeof(double) * 8);
     if (rc == REG_OK) {
-        double *dv = ctx->tmp.as<double>();
-        if (!nonrigid) cudaMemcpyAsync(dv + 4, theta, sizeof(double) * 3, cudaMemcpyHostToDevice, s);
-        cudaError_t e = launch_energy(p, REG_F32, dv + 4, (const float2 *)grid_values, dv, (float2 *)grad_values, s);
-        double res[4] = {0, 0, 0, 0};
-        if (e == cudaSuccess) e = cudaMemcpyAsync(res, dv, sizeof(res), cudaMemcpyDeviceToHost, s);
+        StatusBlock *blk = ctx->status.as<StatusBlock>(), res;
+        if (!nonrigid) cudaMemcpyAsync(blk->theta, theta, sizeof(double) * 3, cudaMemcpyHostToDevice, s);
+        cudaError_t e = launch_energy(p, REG_F32, blk->theta, (const float2 *)grid_values, blk->energy,
+                                      (float2 *)grad_values, s);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(&res, blk, offsetof(StatusBlock, theta), cudaMemcpyDeviceToHost, s);
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
         if (e != cudaSuccess) rc = fail(REG_ECUDA, "energy kernel: %s", cudaGetErrorString(e));
-        else {
-            *energy = res[0];
-            if (grad && !nonrigid) { grad[0] = res[1]; grad[1] = res[2]; grad[2] = res[3]; }
+        else rc = device_status(res.status);
+        if (rc == REG_OK) {
+            *energy = res.energy[0];
+            if (grad && !nonrigid) { grad[0] = res.energy[1]; grad[1] = res.energy[2]; grad[2] = res.energy[3]; }
         }
     }
     ctx->cfg = saved;

@@ -138,6 +138,8 @@ struct Params {
     int n_nodes;
     OpStats *stats;            // [n_ops]
     int *status;               // kernel status word (first device error)
+    long long wait_ns;         // set at the launch: limit of a wait for the other CTAs of an operator,
+    int mute;                  // and whether a test keeps an operator's last CTA from sending
     Queue queue;               // persistent executor only
 };
 
@@ -181,6 +183,8 @@ cudaError_t launch_set_level_means(LevelDesc *tab, const float *means, int L, cu
 // CTAs per operator for a launch that asks for `cluster`: more where an operator's control grid does
 // not fit the shared memory of so few.
 int fit_cluster(const Params &p, int cluster);
+// The launchers set wait_ns and mute by this; a caller that compares Params of two launches does so first.
+void set_exchange_limits(Params &p);
 cudaError_t launch_ops(const Params &p, int storage, int cluster, int n_launch_ops,
                        cudaStream_t s);
 cudaError_t launch_persistent(const Params &p, int storage, int cluster, int workers,

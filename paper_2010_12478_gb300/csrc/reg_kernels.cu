@@ -23,6 +23,8 @@
 
 #include <algorithm>
 #include <cmath>
+#include <cstdlib>
+#include <cstring>
 
 #include "reg_internal.h"
 #include "reg_dev.cuh"
@@ -104,7 +106,9 @@ struct Smem {
     int action;
     int idata[4];
     PassGeom geom;              // of the level
+    long long wait_ns;          // limit of an exchange's wait
     int fail;                   // an exchange's wait ran out: kDevWaitTimeout
+    int mute;                   // sends nothing (Params::mute)
     union {
         RigidCtl rctl;
         FieldCtl fctl;
@@ -156,27 +160,41 @@ __device__ __forceinline__ void send4(const void *p, const unsigned long long *b
 }
 
 // One thread, before the cluster's first exchange (a cluster barrier follows).
-__device__ __forceinline__ void comm_init(Smem &sm)
+__device__ __forceinline__ void comm_init(Smem &sm, const Params &p, const cg::cluster_group &cl)
 {
     for (int i = 0; i < 2; ++i)
         asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(&sm.xbar[i])) : "memory");
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    sm.wait_ns = p.wait_ns;
     sm.fail = 0;
+    sm.mute = p.mute && cl.block_rank() + 1 == cl.num_blocks();
+}
+
+// A CTA that has given up neither waits nor sends in any later exchange: a peer that lacks its part gives up
+// too, instead of taking a later one for it, and no barrier gets an arrival beyond the one of its phase.
+// The same in every thread of a CTA between two barriers.
+__device__ __forceinline__ bool comm_quiet(const Smem &sm)
+{
+    return sm.fail != 0 || sm.mute != 0;
 }
 
 // One thread: this CTA is due `bytes` in exchange n.
 __device__ __forceinline__ void comm_expect(Smem &sm, unsigned n, unsigned bytes)
 {
+    if (sm.fail != 0) return;
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_addr(&sm.xbar[n & 1])), "r"(bytes)
                  : "memory");
 }
 
-// Wait until exchange n has brought what is due; the peers run side by side with this CTA, so it ends,
-// and after two seconds it gives up: sm.fail, and no later exchange of this CTA waits.
+// Wait until exchange n has brought what is due; the peers run side by side with this CTA, so it ends.  After
+// sm.wait_ns of waiting it gives up: sm.fail, which the operator's status and the launch's status word report.
+// The time between two looks at the clock counts for kWaitStep at most, so a process that was suspended does not
+// give up on what is on its way.
+constexpr unsigned long long kWaitStep = 50000000ULL;
 __device__ __forceinline__ void comm_wait(Smem &sm, unsigned n)
 {
     const uint32_t bar = smem_addr(&sm.xbar[n & 1]), parity = (n >> 1) & 1;
-    unsigned long long t0 = 0;
+    unsigned long long last = 0, spent = 0;
     for (unsigned it = 0; *(volatile int *)&sm.fail == 0; ++it) {
         uint32_t done;
         asm volatile("{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
@@ -184,11 +202,12 @@ __device__ __forceinline__ void comm_wait(Smem &sm, unsigned n)
                      : "r"(bar), "r"(parity)
                      : "memory");
         if (done) return;
-        if ((it & 63) == 63) {
+        if ((it & 15) == 15) {
             unsigned long long t;
             asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-            if (t0 == 0) t0 = t;
-            else if (t - t0 > 2000000000ULL) *(volatile int *)&sm.fail = kDevWaitTimeout;
+            if (last != 0) spent += min(t - last, kWaitStep);
+            last = t;
+            if (spent >= (unsigned long long)sm.wait_ns) *(volatile int *)&sm.fail = kDevWaitTimeout;
         }
     }
 }
@@ -211,6 +230,7 @@ __device__ __forceinline__ void cluster_reduce(const float (&hi)[NM], const floa
     static_assert(NM <= kNM && kWarps == 8, "reduction slots");
     constexpr int kLog = NM <= 8 ? 3 : 4, N2 = 1 << kLog, kParts = 32 / N2;   // lanes that share a sum
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+    const bool quiet = comm_quiet(sm);   // before this exchange's wait
     float h[N2], l[N2];
 #pragma unroll
     for (int m = 0; m < N2; ++m) { h[m] = m < NM ? hi[m] : 0.f; l[m] = m < NM ? lo[m] : 0.f; }
@@ -252,13 +272,13 @@ __device__ __forceinline__ void cluster_reduce(const float (&hi)[NM], const floa
             ff_add(v.x, v.y, h2, l2);
         }
         const unsigned long long t = __double_as_longlong((double)v.x + (double)v.y);
-        if (m < NM)
+        if (m < NM && !quiet)
             for (int r = q; r < C; r += kParts) send8(&sm.part[b][me][m], bar, r, t);
     } else if (MAXV && w == 1) {
         const unsigned v = __reduce_max_sync(0xffffffffu, lane < kWarps ? sm.wmax[lane] : 0u);
-        if (lane < C) send4(&sm.pmax[b][me], bar, lane, v);
+        if (lane < C && !quiet) send4(&sm.pmax[b][me], bar, lane, v);
     }
-    push(n);
+    if (!quiet) push(n);
     if (w == 0) {
         comm_wait(sm, n);
         double s = q < C && m < NM ? sm.part[b][q][m] : 0.0;
@@ -1597,6 +1617,7 @@ __device__ void grid_direction(const Grid &G, const Lvl &L, const PassGeom &P, c
                                const PointIter &pi, const float *pm, Smem &sm, Comm &comm, const cg::cluster_group &cl, const H1Bufs &h1)
 {
     const int Nc = G.nx * G.ny, n = (B.own1 - B.cr0) * G.nx, rank = cl.block_rank();
+    const bool quiet = comm_quiet(sm);
     const float aP = pm[0], bmaP = pm[1], kappa = pm[2], lam = pm[3];
     const float scale = -(float)Nc / ((float)L.W * (float)L.H);
     float hi[3] = {0.f, 0.f, 0.f}, lo[3] = {0.f, 0.f, 0.f}, mx = 0.f;
@@ -1619,13 +1640,20 @@ __device__ void grid_direction(const Grid &G, const Lvl &L, const PassGeom &P, c
         // H1 product: b = -Nc dE/dc into B of every CTA, d = M^-1 b into U by every CTA; then
         // |d|_M^2 = d.b, and for the first trial <d_prev, y>_M, |y|_M^2 with y = d_prev - d, M y
         // taken as the stencil y + s2 Lg y
+        // an exchange of its own; every CTA sends every other one at least a word, as exchanges rely on
+        const unsigned xn = comm.n++, C = cl.num_blocks();
+        const unsigned long long *xb = &sm.xbar[xn & 1];
+        if (threadIdx.x == 0) comm_expect(sm, xn, (unsigned)Nc * 8u + C * 4u);
+        if (threadIdx.x < C && !quiet) send4(&sm.pmax[xn & 1][rank], xb, threadIdx.x, 0u);
         int i = pi.i0, jx = pi.x0;
         for (int j = threadIdx.x; j < n; j += kThreads) {
             if (j >= kThreads) PointIter::at(G.nx, j, i, jx);
             const float2 b = rhs(i, jx);
-            for (unsigned r = 0; r < cl.num_blocks(); ++r) *cl.map_shared_rank(h1.B + (B.cr0 + i) * G.nx + jx, r) = b;
+            if (!quiet)
+                for (unsigned r = 0; r < C; ++r) send8(h1.B + (B.cr0 + i) * G.nx + jx, xb, r, b);
         }
-        cl.sync();   // B is complete, and no CTA reads another's slots any more (T and U lie there)
+        if (threadIdx.x < 32) comm_wait(sm, xn);
+        __syncthreads();   // B is complete, and this CTA's slots have been read (T and U lie there)
         h1_solve(h1, G.nx, G.ny);
         auto yv = [&](int row, int jx) {
             const float2 a = d[(row - B.h0) * G.nx + jx], b = h1.U[row * G.nx + jx];
@@ -1667,8 +1695,8 @@ __device__ void grid_direction(const Grid &G, const Lvl &L, const PassGeom &P, c
         const float2 b = rhs(i, jx), mj = mt[k], dold = d[k];
         const float2 dj = make_float2(b.x / mj.x, b.y / mj.y);
         d[k] = dj;
-        if (i == 0 && B.cr0 > 0) send8(halo + G.nx + jx, bar, rank - 1, dj);
-        if (row == B.cr1 - 1 && B.own1 < G.ny) send8(halo + jx, bar, rank + 1, dj);
+        if (i == 0 && B.cr0 > 0 && !quiet) send8(halo + G.nx + jx, bar, rank - 1, dj);
+        if (row == B.cr1 - 1 && B.own1 < G.ny && !quiet) send8(halo + jx, bar, rank + 1, dj);
         const float yx = dold.x - dj.x, yy = dold.y - dj.y;
         ff_acc(hi[0], lo[0], fmaf(mj.x * dj.x, dj.x, mj.y * dj.y * dj.y));
         ff_acc(hi[1], lo[1], fmaf(mj.x * dold.x, yx, mj.y * dold.y * yy));
@@ -1997,11 +2025,11 @@ __global__ void __launch_bounds__(kThreads, MINB) op_kernel(const __grid_constan
     extern __shared__ __align__(16) float2 gbuf[];   // nonrigid: control grid c, d, ct, gp
     cg::cluster_group cl = cg::this_cluster();
     Comm comm{0};
-    if (threadIdx.x == 0) comm_init(sm);
+    if (threadIdx.x == 0) comm_init(sm, p, cl);
     cl.sync();   // every CTA's barriers are set before a peer sends
     const int q = blockIdx.x / cl.num_blocks();
     run_op<MODE, S, U>(p, p.op_base + q, sm, gbuf, comm, cl);
-    cl.sync();   // no CTA leaves while a peer may still read its shared memory
+    cl.sync();   // no CTA leaves while a peer may still send to it
 }
 
 // Persistent launch: each cluster claims ready operators from the device queue
@@ -2014,7 +2042,7 @@ __global__ void __launch_bounds__(kThreads, MINB) persistent_kernel(const __grid
     cg::cluster_group cl = cg::this_cluster();
     const bool leader = cl.block_rank() == 0 && threadIdx.x == 0;
     Comm comm{0};
-    if (threadIdx.x == 0) comm_init(sm);   // before the cluster barriers of the first claim
+    if (threadIdx.x == 0) comm_init(sm, p, cl);   // before the cluster barriers of the first claim
     for (;;) {
         if (leader) {
             // claim the first ready operator of the most urgent non-empty class; every operator
@@ -2166,7 +2194,7 @@ __global__ void __launch_bounds__(kThreads) energy_kernel(const __grid_constant_
     const int C = cl.num_blocks(), rank = cl.block_rank();
     const bool first = tid == 0 && rank == 0;
     Comm comm{0};
-    if (tid == 0) comm_init(sm);
+    if (tid == 0) comm_init(sm, p, cl);
     cl.sync();
     if constexpr (MODE == REG_RIGID) {
         RigidCtl &k = sm.rctl;
@@ -2227,7 +2255,8 @@ __global__ void __launch_bounds__(kThreads) energy_kernel(const __grid_constant_
                 grad_c[B.cr0 * G.nx + j] = make_float2((float)(s * (double)own[j].x), (float)(s * (double)own[j].y));
         }
     }
-    cl.sync();   // no CTA leaves while a peer may still read its shared memory
+    if (tid == 0 && sm.fail) atomicCAS(p.status, 0, sm.fail);
+    cl.sync();   // no CTA leaves while a peer may still send to it
 }
 
 // Composition of two control grids at the control points (standalone entry point).
@@ -2306,9 +2335,24 @@ int fit_cluster(const Params &p, int cluster)
     return cluster;
 }
 
+// Limit of an exchange's wait, two seconds: the CTAs of a cluster run side by side, and a pass over the largest
+// frame takes milliseconds.  Host-side fault injection for tests: REG_FAULT_INJECT=mute_cta keeps an operator's
+// last CTA from sending, so that the waits run out; REG_EXCHANGE_TIMEOUT_MS shortens them.
+void set_exchange_limits(Params &p)
+{
+    p.wait_ns = 2000000000LL;
+    if (const char *t = getenv("REG_EXCHANGE_TIMEOUT_MS")) {
+        const long long ms = atoll(t);
+        if (ms > 0) p.wait_ns = ms * 1000000LL;
+    }
+    const char *inj = getenv("REG_FAULT_INJECT");
+    p.mute = inj && strcmp(inj, "mute_cta") == 0;
+}
+
 template <typename K>
 static cudaError_t launch_cluster(K kernel, int blocks, int cluster, cudaStream_t s, Params p)
 {
+    set_exchange_limits(p);
     if (cluster > 8) {
         cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
         if (e != cudaSuccess) return e;
@@ -2436,6 +2480,7 @@ cudaError_t launch_energy(const Params &params, int storage, const double *theta
     (void)storage;
     constexpr int kEnergyCtas = kMaxCluster;
     Params p = params;
+    set_exchange_limits(p);
     const void *kern = p.cfg.mode == REG_RIGID ? (const void *)energy_kernel<REG_RIGID, float>
                                                : (const void *)energy_kernel<REG_NONRIGID, float>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);

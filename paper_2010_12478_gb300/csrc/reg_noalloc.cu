@@ -236,6 +236,10 @@ extern "C" int reg_pairwise_noalloc(const reg_config_t *cfg, int device, const f
             rc = noalloc_fail(REG_ECUDA, "operator kernel failed");
             break;
         }
+        if (hstatus[0] == kDevWaitTimeout) {
+            rc = noalloc_fail(REG_ETIMEOUT, "a wait for the other CTAs of the operator timed out");
+            break;
+        }
         if (hstatus[0] != 0 || hst.status != kDevOk) {
             rc = noalloc_fail(REG_EINVAL, "the operator kernel rejected its descriptor");
             break;

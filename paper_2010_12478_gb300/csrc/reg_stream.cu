@@ -258,7 +258,11 @@ void advance(Service *sv, reg_stream *s)
             sl->launched[0] = true;
         }
         for (int o = 0; o < kOpsPerSlot; ++o)
-            if (sl->launched[o] && !sl->fin[o] && done(sl->ev[o])) sl->fin[o] = true;
+            if (sl->launched[o] && !sl->fin[o] && done(sl->ev[o])) {
+                sl->fin[o] = true;
+                // an operator whose CTAs lost each other has no result, nor has any that builds on it
+                if (s->h_stats[op_of(i, o)].status == kDevWaitTimeout) { s->error = REG_ECUDA; return; }
+            }
         // windows W_lev(i), lev = 1..m, for i >= 2^lev
         for (int lev = 1; lev <= m; ++lev) {
             if (sl->launched[lev] || i < (1LL << lev)) continue;

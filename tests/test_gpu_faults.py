@@ -94,3 +94,106 @@ def test_autotune_tunes_the_nonrigid_tile_shape_and_uses_it(tmp_path):
     ctx4 = B.Context(B.Config(mode="nonrigid", unroll=2))
     ctx4.autotune(F, exec="persistent")
     assert ctx4.tuned_shape(tuple(F.shape), "persistent")["unroll"] == 2
+
+
+@pytest.fixture
+def mute_cta(monkeypatch):
+    """An operator's last CTA sends nothing (host-side injection): every wait for it runs out after 50 ms."""
+    def on():
+        monkeypatch.setenv("REG_FAULT_INJECT", "mute_cta")
+        monkeypatch.setenv("REG_EXCHANGE_TIMEOUT_MS", "50")
+
+    def off():
+        monkeypatch.delenv("REG_FAULT_INJECT")
+        monkeypatch.delenv("REG_EXCHANGE_TIMEOUT_MS")
+    return on, off
+
+
+def _pair(n=2):
+    return synth.make_series(synth.SeriesSpec(n, 70, 81, step=1.0, field_amp=0.5, snr=(10.0, 10.0), seed=12)).frames.cuda()
+
+
+def _times_out(call):
+    t0 = time.time()
+    with pytest.raises(B.RegError) as e:
+        call()
+    assert e.value.code == B.REG_ETIMEOUT
+    assert time.time() - t0 < 10.0
+
+
+@pytest.mark.parametrize("mode,metric", [("rigid", 1), ("nonrigid", 1), ("nonrigid", 0), ("nonrigid", 2)])
+@pytest.mark.parametrize("cluster", [1, 4, 16])
+def test_a_silent_cta_is_reported_by_pairs_and_scans(mute_cta, mode, metric, cluster):
+    on, off = mute_cta
+    F = _pair(5)
+    ctx = B.Context(B.Config(mode=mode, metric=metric, cluster=cluster, max_iter=3))
+    out = torch.empty((2, 70, 81), device="cuda") if mode == "nonrigid" else None
+    pair = lambda: ctx.pairwise(F[0], F[1], field_out=out)
+    scan = lambda exec: ctx.scan(F, exec=exec)[0]
+    good, goods = pair(), {e: scan(e) for e in ("level", "persistent", "graph", "plain")}
+    on()
+    _times_out(pair)
+    for e in goods:
+        _times_out(lambda: scan(e))
+    off()
+    assert pair() == good
+    for e in goods:
+        assert scan(e) == goods[e]
+
+
+def test_a_silent_cta_is_reported_by_energies(mute_cta):
+    on, off = mute_cta
+    F = _pair()
+    rigid, field = B.Context(B.Config()), B.Context(B.Config(mode="nonrigid"))
+    nx, ny, _ = B.grid_dims(81, 70)
+    c = torch.zeros((ny, nx, 2), device="cuda")
+    calls = [lambda: rigid.energy_rigid(F[0], F[1], [0.01, 0.3, -0.2])[0], lambda: field.energy_grid(F[0], F[1], c),
+             lambda: field.energy_grid(F[0], F[1], c, torch.zeros_like(c))]
+    good = [f() for f in calls]
+    on()
+    for f in calls:
+        _times_out(f)
+    off()
+    assert [f() for f in calls] == good
+
+
+def test_a_silent_cta_is_reported_by_the_allocation_free_call(mute_cta):
+    on, off = mute_cta
+    F = _pair()
+    cfg = B.Config(max_iter=3)
+    good = B.pairwise_noalloc(cfg, F[0], F[1])
+    on()
+    _times_out(lambda: B.pairwise_noalloc(cfg, F[0], F[1]))
+    off()
+    assert B.pairwise_noalloc(cfg, F[0], F[1]) == good
+
+
+@pytest.mark.parametrize("mode", ["rigid", "nonrigid"])
+def test_a_silent_cta_ends_a_stream(mute_cta, mode):
+    # f_0's result (the identity) comes, then the error: no later result builds on an operator that failed
+    on, off = mute_cta
+    F = _pair(3)
+    ctx = B.Context(B.Config(mode=mode, max_iter=3))
+    on()
+    s = B.Stream(ctx, 81, 70)
+    for k in range(3):
+        s.submit(F[k], k)
+    got, code = [], None
+    t0 = time.time()
+    while code is None and time.time() - t0 < 10.0:
+        try:
+            got += s.poll(timeout_us=100000)
+        except B.RegError as e:
+            code = e.code
+    off()
+    assert code == B.REG_ECUDA
+    assert [r["frame_id"] for r in got] in ([0], [])   # the poll that raises drops what it returned
+    s.close()
+    s = B.Stream(ctx, 81, 70)
+    for k in range(3):
+        s.submit(F[k], k)
+    got, t0 = [], time.time()
+    while len(got) < 3 and time.time() - t0 < 10.0:
+        got += s.poll(timeout_us=100000)
+    s.close()
+    assert [r["frame_id"] for r in got] == [0, 1, 2] and all(r["status"] == 0 for r in got)
