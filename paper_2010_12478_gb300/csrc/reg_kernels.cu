@@ -190,6 +190,10 @@ __device__ __forceinline__ void comm_expect(Smem &sm, unsigned n, unsigned bytes
 // sm.wait_ns of waiting it gives up: sm.fail, which the operator's status and the launch's status word report.
 // The time between two looks at the clock counts for kWaitStep at most, so a process that was suspended does not
 // give up on what is on its way.
+// The wait acquires at cluster scope, as it orders the peers' stores before the reads that follow (a CTA's other
+// threads, by the barrier after it); at its default scope, its own CTA, the memory model orders nothing of a
+// peer's.  It costs 1.6 % over the timed calls (a rigid scan of 24 frames 848 -> 918 us, a pair of 512x512 276 ->
+// 280, scans of hundreds of frames nothing).
 constexpr unsigned long long kWaitStep = 50000000ULL;
 __device__ __forceinline__ void comm_wait(Smem &sm, unsigned n)
 {
@@ -197,7 +201,7 @@ __device__ __forceinline__ void comm_wait(Smem &sm, unsigned n)
     unsigned long long last = 0, spent = 0;
     for (unsigned it = 0; *(volatile int *)&sm.fail == 0; ++it) {
         uint32_t done;
-        asm volatile("{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
+        asm volatile("{\n .reg .pred p;\n mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
                      : "=r"(done)
                      : "r"(bar), "r"(parity)
                      : "memory");
