@@ -961,8 +961,12 @@ constexpr int kEmitSums = 6, kEmitRow = 36;   // gradient sums of a column; a ro
 constexpr int kEmitFloats = 2 * kEmitSums * kEmitRow;   // a warp's emission: 2 strips' sums
 
 // Dynamic shared memory of the nonrigid kernels, in float2 units: c, d, mt (the held rows; mt the
-// flow's scalar product per control point and axis), two staged halo rows of d, the sums that the CTA
-// above sends for the first own row, the warps' rows of an emission, then the slots.
+// flow's scalar product per control point and axis), the sums that the CTA above sends for the first own
+// row, the warps' rows of an emission, then the slots.  Two staged halo rows of d lie in the place of the
+// emissions: a neighbour sends them after a pass's exchange, to which this CTA contributed behind its last
+// emission, and they are read before its next pass.  Without that the 3-row grids of 858 to 892 points a row
+// (frames of 28,000 x 50 at a spacing of 32), which grid_dims takes, had no split that fits 16 CTAs; now every
+// grid that it takes has one.
 // With the H1 product mt is the right-hand side of its solve on the whole grid, and the two work
 // grids t and u of the solve lie in the place of the slots, which it has read by then.
 struct GridLayout {
@@ -976,12 +980,13 @@ __host__ __device__ __forceinline__ GridLayout grid_layout(int gnx, int gny, int
     g.c = 0;
     g.d = rows * gnx;
     g.mt = 2 * rows * gnx;
-    g.halo = g.mt + (h1 ? gny : rows) * gnx;
     const int edges = q < gny - 1 ? gnx : 0;   // a band has neighbours
-    g.above = g.halo + 2 * edges;
+    g.above = g.mt + (h1 ? gny : rows) * gnx;
     g.emits = g.above + kSlot / 2 * edges;
     g.emits += g.emits & 1;
-    g.slots = g.emits + kWarps * kEmitFloats / 2;
+    g.halo = g.emits;
+    const int warps = kWarps * kEmitFloats / 2;
+    g.slots = g.emits + (warps > 2 * edges ? warps : 2 * edges);
     return g;
 }
 

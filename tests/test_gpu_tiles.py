@@ -231,3 +231,32 @@ def test_frames_and_fields_off_a_floats_alignment_are_staged(off):
         ctx.pairwise(F[0], F[1], field_in=init, field_out=want)
         ctx.pairwise(R, T, field_in=_At(init, off), field_out=got)
         assert torch.equal(got.floats(), want.cpu())
+
+
+@pytest.mark.parametrize("grid,past,metric", [(32, 0, 1), (32, 1, 1), (32, 1, 2), (17, 1, 1), (40, 1, 0)])
+def test_the_largest_accepted_grid_of_three_rows(grid, past, metric):
+    # 892 x 3 control points, the most that reg_grid_dims takes at three rows, with and without a column past the
+    # last cell, cells of a strip each and of two chunks: two bands of one cell row in 16 CTAs
+    W, H = 891 * grid + past, 2 * grid + past
+    assert B.grid_dims(W, H, grid, 1)[:2] == (892, 3)
+    rng = np.random.default_rng(31)
+    R = rng.uniform(0, 1, size=(H, W)).astype(np.float32)
+    T = (0.5 * (R + np.roll(R, 1, axis=1))).astype(np.float32)
+    dR, dT = torch.from_numpy(R).cuda(), torch.from_numpy(T).cuda()
+    g = O.grid_for(W, H, grid)
+    c = rng.uniform(-0.9, 0.9, size=(g.ny, g.nx, 2)).astype(np.float32)
+    gd = torch.zeros((g.ny, g.nx, 2), device="cuda")
+    E = B.Context(B.Config(mode="nonrigid", levels=1, grid=grid)).energy_grid(dR, dT, torch.from_numpy(c).cuda(), gd)
+    Eo, go = O.grid_energy(R, T, 0, g, c.transpose(2, 0, 1).astype(np.float64), 2.0)
+    assert abs(E - Eo) <= 1e-6 * abs(Eo)
+    np.testing.assert_allclose(gd.cpu().numpy().transpose(2, 0, 1), go, atol=2e-4 * np.abs(go).max())
+    # one accepted step from the identity, as in test_pair_for_every_band_split
+    cfg = B.Config(mode="nonrigid", levels=1, grid=grid, metric=metric, max_iter=1)
+    out = torch.empty((2, H, W), device="cuda")
+    _, st = B.Context(cfg).pairwise(dR, dT, field_out=out)
+    oc = O.Config(levels=1, max_iter=1, max_rejects=cfg.max_rejects, tol_grad=cfg.tol_grad, tol_rel_e=cfg.tol_rel_e,
+                  armijo_c=cfg.armijo_c, tau0=cfg.tau0, step_cap=cfg.step_cap, lam=cfg.lam, mode="nonrigid", grid=grid,
+                  metric=metric, sigma=cfg.sigma, tol_coarse=cfg.tol_coarse)
+    c_o, st_o = O.register_nonrigid(O.pyramid(R, 1), O.pyramid(T, 1), None, oc)
+    assert O.max_px_error(out.cpu().numpy(), c_o, H, W, "nonrigid", grid) <= 1e-3
+    assert st["iters"] == list(st_o.iters) and abs(st["energy"] - st_o.energy) <= 1e-6 * abs(st_o.energy)
