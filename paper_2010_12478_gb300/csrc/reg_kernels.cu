@@ -310,8 +310,6 @@ struct Ncc {
 // rounding of the FP32 sums enters 1 - NCC, about (S'_EE - S'_RE^2 / S'_RR) / (2 S'_RR), relative to its
 // own size; sums of t^2 and r t enter it relative to 1, which left 1.8e-8 in an energy of 1e-3 (a
 // noiseless lattice, every run of pixels rounded alike).  A constant image has E = 1 and no gradient.
-// 1/sqrt: the hardware approximation y (about 20 bits) and one third-order step, with h = 1 - q y^2
-// y (1 + h/2 + 3/8 h^2), whose error is 5/16 h^3.
 __device__ __forceinline__ Ncc ncc_terms(const LevelSums &L, double se, double see, double sre)
 {
     Ncc o;
@@ -320,11 +318,7 @@ __device__ __forceinline__ Ncc ncc_terms(const LevelSums &L, double se, double s
     const double Srt = __dadd_rn(L.Srr, Sre);
     o.u = __dadd_rn(Sre, See);
     o.Stt = __dadd_rn(Srt, o.u);
-    const double q = __dmul_rn(L.Srr, o.Stt);
-    double y;
-    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(q));
-    const double h = __fma_rn(-q, __dmul_rn(y, y), 1.0);
-    o.a = __fma_rn(y, __dmul_rn(h, __fma_rn(0.375, h, 0.5)), y);
+    o.a = rsqrt(__dmul_rn(L.Srr, o.Stt));
     o.e = __fma_rn(-Srt, o.a, 1.0);
     // e = 0 everywhere (T o phi equals R up to the shift: identical inputs) is exactly NCC = 1
     if ((__double_as_longlong(Sre) | __double_as_longlong(See)) << 1 == 0) o.e = 0.0;
