@@ -40,14 +40,12 @@ constexpr int kMaxCluster = 16; // CTAs per operator at most (non-portable clust
 
 // ------------------------------------------------------------------ shared state
 // Step-controller state, used by thread 0 (rigid: warp 0) of each CTA only: kept in shared memory so it
-// does not occupy registers of every thread.  Energies, gradients and the tests on them are FP64, step
-// lengths FP32 (the length a step is taken with).  An FP64 instruction, conversions among them, takes 64
-// cycles of its warp on this GPU however many lanes take part, a compare 105, an FP32 one 4: the
+// does not occupy registers of every thread.  All of it is FP64.  An FP64 instruction, conversions among them,
+// takes 64 cycles of its warp on this GPU however many lanes take part, a compare 105, an FP32 one 4: the
 // controllers are written for few FP64 instructions.
 struct LevelSums {
     double P, invP, sr, Srr;       // pixels; sum of the reference's shifted samples; S'_RR
     double least;                  // a centred sum of squares below this is a constant image
-    float Pf, Srrf, rbar;          // P, S'_RR and the mean of the reference's shifted samples in FP32
 };
 
 struct RigidCtl {
@@ -57,8 +55,7 @@ struct RigidCtl {
     double accept, rel;            // a trial is accepted up to the first energy, and ends the level from the second
     double tolg2;  // the level's stop tolerance (tol_grad, times tol_coarse above the finest level), squared
     double dp[3];                  // direction of the last accepted step
-    float tau, tau_acc;            // length of the trial step, and of the last accepted one
-    float m0f;                     // m0 in FP32
+    double tau, tau_acc;           // length of the trial step, and of the last accepted one
     int nrej, iters, evals, stop, rejects, have_prev;
 };
 
@@ -68,7 +65,7 @@ struct FieldCtl {
     double accept, rel;            // a trial is accepted up to the first energy, and ends the level from the second
     double Eold, ss_old;           // before the last accepted step, for its quadratic rule
     double tolss;  // the level's stop tolerance (tol_grad, times tol_coarse above the finest level), squared, times Nc
-    float tau, tau_acc;            // length of the trial step, and of the last accepted one
+    double tau, tau_acc;           // length of the trial step, and of the last accepted one as it was taken (FP32)
     int nrej, iters, evals, stop, rejects, have_prev;
 };
 
@@ -88,10 +85,10 @@ __device__ __forceinline__ bool at_least(double x, double y)
 // gradient methods", 1988, their second step): tau = tau_acc <d_prev, d_prev - d> / |d_prev - d|^2
 // in the flow's metric, given num = <d_prev, d_prev - d> and den = |d_prev - d|^2; false without
 // positive curvature.  The ratio needs no more than FP32 relative precision.
-__device__ __forceinline__ bool bb_tau(float tau_acc, float num, float den, float &tau)
+__device__ __forceinline__ bool bb_tau(double tau_acc, double num, double den, double &tau)
 {
-    if (!(num > 0.f && den > 0.f)) return false;
-    tau = tau_acc * (num * __frcp_rn(den));
+    if (!(num > 0.0 && den > 0.0)) return false;
+    tau = tau_acc * num * (double)__frcp_rn((float)den);
     return true;
 }
 
@@ -335,15 +332,12 @@ __device__ __forceinline__ void set_level(LevelSums &L, int W, int H)
     L.P = (double)W * (double)H;
     L.invP = 1.0 / L.P;
     L.least = 1e-12 * L.P;
-    L.Pf = (float)L.P;
 }
 __device__ __forceinline__ void set_reference(LevelSums &L, double sr, double srr)
 {
     const double rbar = __dmul_rn(sr, L.invP);
     L.sr = sr;
     L.Srr = __fma_rn(-sr, rbar, srr);
-    L.Srrf = (float)L.Srr;
-    L.rbar = (float)rbar;
 }
 
 // ------------------------------------------------------------------ level access
@@ -595,14 +589,13 @@ __device__ __forceinline__ void rigid_param(double v, int q, int lane, float *pm
 // parabola through E(0) = E, E'(0) = slope and E(tau) = Et; a rejected trial retries at tq
 // clamped to [0.1 tau, 0.5 tau], an accepted one starts the next search at tq clamped to
 // [0.5 tau, 4 tau]; without positive curvature the rule halves / doubles.
-__device__ __forceinline__ float next_tau(double E, double slope, float tau, double Et, bool accepted)
+__device__ __forceinline__ double next_tau(double E, double slope, double tau, double Et, bool accepted)
 {
-    const double st = __dmul_rn(slope, (double)tau);
-    const float den = (float)(Et - E - st);
-    if (!(den > 0.f)) return accepted ? 2.f * tau : 0.5f * tau;
+    const double st = __dmul_rn(slope, tau), den = Et - E - st;
+    if (!(den > 0.0)) return accepted ? 2.0 * tau : 0.5 * tau;
     // a step-size estimate needs no more than FP32 relative precision once den is formed
-    const float tq = -(float)st * tau * __frcp_rn(2.f * den);
-    return accepted ? fminf(fmaxf(tq, 0.5f * tau), 4.f * tau) : fminf(fmaxf(tq, 0.1f * tau), 0.5f * tau);
+    const double tq = -st * tau * (double)__frcp_rn((float)(2.0 * den));
+    return accepted ? fmin(fmax(tq, 0.5 * tau), 4.0 * tau) : fmin(fmax(tq, 0.1 * tau), 0.5 * tau);
 }
 
 // Gradient component q at the point of a pass from its sums and the point's NCC terms: dE/dtheta_q = a
@@ -634,10 +627,10 @@ __device__ int rigid_step(RigidCtl &k, const Config &cfg, const double *tot, boo
     }
     const Ncc n = ncc_terms(k.ls, tot[0], tot[1], tot[2]);
     const double Et = n.e, Eold = k.E, slope_old = k.slope;
-    const float tau_old = k.tau;
+    const double tau_old = k.tau;
     double th = k.th[q], d = k.d[q], E = Et, slope = slope_old, accept = k.accept, rel = k.rel;
     double dp = k.dp[q];
-    float tau = tau_old, tau_acc = k.tau_acc;
+    double tau = tau_old, tau_acc = k.tau_acc;
     int evals = k.evals + (start ? 0 : 1), iters = k.iters, have_prev = k.have_prev, nrej = k.nrej, rejects = k.rejects;
     int stop = -1;
     const bool taken = start || nonneg(accept - Et);
@@ -667,14 +660,10 @@ __device__ int rigid_step(RigidCtl &k, const Config &cfg, const double *tot, boo
             else if (!at_least(-slope, k.tolg2)) stop = REG_STOP_GRAD;
             else {
                 if (have_prev) {
-                    const float w = q == 0 ? k.m0f : 1.f, y = (float)(dp - d);
-                    const float a = w * (float)dp * y, b = w * y * y;
-                    const float num = __shfl_sync(0xffffffffu, a, 0) + __shfl_sync(0xffffffffu, a, 1) + __shfl_sync(0xffffffffu, a, 2);
-                    const float den = __shfl_sync(0xffffffffu, b, 0) + __shfl_sync(0xffffffffu, b, 1) + __shfl_sync(0xffffffffu, b, 2);
-                    if (!bb_tau(tau_acc, num, den, tau)) tau = next_tau(Eold, slope_old, tau_old, Et, true);
+                    const double y = dp - d, wy = q == 0 ? k.m0 * y : y;
+                    if (!bb_tau(tau_acc, sum3(dp * wy), sum3(y * wy), tau)) tau = next_tau(Eold, slope_old, tau_old, Et, true);
                 }
-                const float gn2 = (float)-slope, cap = (float)cfg.step_cap;
-                if (tau * tau * gn2 > cap * cap) tau = cap / sqrtf(gn2);
+                if (tau * tau * -slope > cfg.step_cap * cfg.step_cap) tau = cfg.step_cap / sqrt(-slope);
                 nrej = 0;
                 rel = cfg.tol_rel_e == 0.0 ? E : E - cfg.tol_rel_e * fabs(E);
             }
@@ -682,8 +671,8 @@ __device__ int rigid_step(RigidCtl &k, const Config &cfg, const double *tot, boo
     }
     __syncwarp();   // every lane has read the state
     if (stop < 0) {
-        const double taud = (double)tau, tt = __fma_rn(taud, d, th);
-        accept = __fma_rn(cfg.armijo_c * slope, taud, E);
+        const double tt = __fma_rn(tau, d, th);
+        accept = __fma_rn(cfg.armijo_c * slope, tau, E);
         if (lane < 3) k.tt[q] = tt;
         rigid_param(tt, q, lane, pm);
     }
@@ -748,8 +737,7 @@ __device__ void run_rigid(const Params &p, const OpDesc &op, int op_index, Smem 
             double rho = 0.25 * (L.W + L.H);
             k.m0 = rho * rho;
             k.inv_m0 = 1.0 / k.m0;
-            k.m0f = (float)k.m0;
-            k.tau = (float)cfg.tau0;
+            k.tau = cfg.tau0;
             k.have_prev = 0;
             k.iters = 0; k.evals = 0; k.stop = REG_STOP_MAXIT;
             // a coarse level only supplies the next level's initial guess: a looser stop
@@ -1718,15 +1706,15 @@ __device__ void grid_direction(const Grid &G, const Lvl &L, const PassGeom &P, c
 // and lambda; the scalar product's 1/(P var T) and lambda/P; the next trial's step.
 enum FieldParam { kPmA = 0, kPmB = 1, kPmK = 2, kPmLam = 3, kPmDk = 4, kPmRk = 5, kPmTau = 6 };
 
-// Gradient coefficients from a point's NCC terms: b - a = -a^3 S'_RR u, formed as -(a S'_RR)(a u) a so
-// that no factor leaves the FP32 range; exact zeros but aP for identical frames.
+// Gradient coefficients from a point's NCC terms, b - a = -a^3 S'_RR u: formed in FP64, rounded once; exact
+// zeros but aP for identical frames.
 __device__ __forceinline__ void field_grad_params(const Ncc &n, const LevelSums &L, const Config &cfg, float *pm)
 {
-    const float a = (float)n.a, dbar = (float)n.dbar, aP = a * L.Pf;
-    const float b = -(a * L.Srrf) * (a * (float)n.u) * aP;
-    pm[kPmA] = aP;
-    pm[kPmB] = b;
-    pm[kPmK] = -fmaf(b, L.rbar + dbar, aP * dbar);
+    const double aP = __dmul_rn(n.a, L.P);
+    const double b = -__dmul_rn(__dmul_rn(n.a, L.Srr), __dmul_rn(__dmul_rn(n.a, n.u), aP));
+    pm[kPmA] = (float)aP;
+    pm[kPmB] = (float)b;
+    pm[kPmK] = (float)-__fma_rn(b, __fma_rn(L.sr, L.invP, n.dbar), __dmul_rn(aP, n.dbar));
     pm[kPmLam] = (float)cfg.lambda;
 }
 
@@ -1755,7 +1743,7 @@ __device__ int field_eval(FieldCtl &k, const Config &cfg, const double *tot, boo
         k.iters += 1;
         k.Eold = k.E;
         k.ss_old = k.ss;
-        k.tau_acc = k.tau;
+        k.tau_acc = (double)(float)k.tau;
         k.have_prev = 1;
         k.E = Et;
         if (nonneg(Et - k.rel)) { k.stop = REG_STOP_REL; return kActDone; }
@@ -1764,11 +1752,11 @@ __device__ int field_eval(FieldCtl &k, const Config &cfg, const double *tot, boo
     k.rejects += 1;
     k.nrej += 1;
     const double slope = -k.ss * k.invNc;
-    const float tau = next_tau(k.E, slope, k.tau, Et, false);
+    const double tau = next_tau(k.E, slope, k.tau, Et, false);
     k.tau = tau;
     if (k.nrej > cfg.max_rejects) { k.stop = REG_STOP_LS; return kActDone; }
-    k.accept = __fma_rn(cfg.armijo_c * slope, (double)tau, k.E);
-    pm[kPmTau] = tau;
+    k.accept = __fma_rn(cfg.armijo_c * slope, tau, k.E);
+    pm[kPmTau] = (float)tau;
     return kActTrial;
 }
 
@@ -1783,16 +1771,15 @@ __device__ int field_grad(FieldCtl &k, const Config &cfg, const double *tot, flo
     if (!at_least(ss, k.tolss)) { k.stop = REG_STOP_GRAD; return kActDone; }
     // the metric (mean over control points) is a common factor of the two sums; without positive
     // curvature the quadratic rule of the last step
-    float tau = k.tau;
-    if (k.have_prev && !bb_tau(k.tau_acc, (float)tot[1], (float)tot[2], tau))
-        tau = next_tau(k.Eold, -k.ss_old * k.invNc, k.tau_acc, k.E, true);
-    const float cap = (float)cfg.step_cap;
-    if (tau * tau * dmax2 > cap * cap) tau = cap / sqrtf(dmax2);
+    double tau = k.tau;
+    if (k.have_prev && !bb_tau(k.tau_acc, tot[1], tot[2], tau))
+        tau = next_tau(k.Eold, -k.ss_old * k.invNc, k.tau, k.E, true);
+    if (tau * tau * (double)dmax2 > cfg.step_cap * cfg.step_cap) tau = cfg.step_cap / sqrt((double)dmax2);
     k.tau = tau;
     k.nrej = 0;
-    k.accept = __fma_rn(-ss * (cfg.armijo_c * k.invNc), (double)tau, k.E);
+    k.accept = __fma_rn(-ss * (cfg.armijo_c * k.invNc), tau, k.E);
     k.rel = cfg.tol_rel_e == 0.0 ? k.E : k.E - cfg.tol_rel_e * fabs(k.E);
-    pm[kPmTau] = tau;
+    pm[kPmTau] = (float)tau;
     return kActTrial;
 }
 
@@ -1878,7 +1865,7 @@ __device__ void run_nonrigid(const Params &p, const OpDesc &op, int op_index, Sm
         if (tid == 0) {
             set_level(k.ls, L.W, L.H);
             k.half_lam = 0.5 * cfg.lambda * k.ls.invP;
-            k.tau = (float)cfg.tau0;
+            k.tau = cfg.tau0;
             k.have_prev = 0;
             k.iters = 0; k.evals = 0; k.stop = REG_STOP_MAXIT;
             // a coarse level only supplies the next level's initial guess: a looser stop

@@ -260,3 +260,14 @@ def test_the_largest_accepted_grid_of_three_rows(grid, past, metric):
     c_o, st_o = O.register_nonrigid(O.pyramid(R, 1), O.pyramid(T, 1), None, oc)
     assert O.max_px_error(out.cpu().numpy(), c_o, H, W, "nonrigid", grid) <= 1e-3
     assert st["iters"] == list(st_o.iters) and abs(st["energy"] - st_o.energy) <= 1e-6 * abs(st_o.energy)
+
+
+@pytest.mark.parametrize("cap", [1e-3, 3.7e-4])
+def test_a_capped_step_has_the_caps_length_in_64_bits(cap):
+    # the step controller works in FP64: a first step that the cap shortens has exactly its length in the flow's
+    # metric, a few roundings of 1.1e-16 (a length held in FP32 is off by up to 6e-8)
+    F = synth.make_series(synth.SeriesSpec(2, 96, 110, step=1.0, snr=(10.0, 10.0), seed=15)).frames.cuda()
+    _, st = B.Context(B.Config(levels=1, max_iter=1, step_cap=cap)).pairwise(F[0], F[1])
+    a, x, y = st["theta"]
+    assert st["iters"] == [1] and st["rejects"] == 0
+    assert abs(np.sqrt((0.25 * (96 + 110) * a) ** 2 + x * x + y * y) / cap - 1.0) <= 1e-13
