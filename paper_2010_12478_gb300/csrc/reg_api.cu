@@ -645,10 +645,10 @@ int build_pyramids(reg_ctx *ctx, const Geometry &g, const float *frames, int nf,
             o.smooth[l] = (char *)ctx->spyr[l].ptr + o.smooth_stride[l] * sb * first;
         }
     }
-    CHECK(ctx->means.reserve(sizeof(float) * (size_t)total * L));
+    CHECK(ctx->means.reserve(sizeof(LevelStat) * (size_t)total * L));
     int e0 = timing_mark(ctx, s);
     CU(launch_pyramid(frames, nf, fstride, g.W[0], g.H[0], pitch, L, ctx->cfg.storage, o,
-                      ctx->means.as<float>() + (size_t)first * L, s));
+                      ctx->means.as<LevelStat>() + (size_t)first * L, s));
     ctx->pyr_pairs.push_back({e0, timing_mark(ctx, s)});
     ctx->last.pyramid_launches += pyramid_launches(L, true, o.pad);
     return REG_OK;
@@ -679,7 +679,7 @@ LevelTable level_table(const reg_ctx *ctx, const Geometry &g)
 int build_level_table(reg_ctx *ctx, const Geometry &g, int total, cudaStream_t s)
 {
     CHECK(ctx->level_tab.reserve(sizeof(LevelDesc) * (size_t)total * g.levels));
-    CU(launch_level_table(ctx->level_tab.as<LevelDesc>(), level_table(ctx, g), ctx->means.as<float>(), total, s));
+    CU(launch_level_table(ctx->level_tab.as<LevelDesc>(), level_table(ctx, g), ctx->means.as<LevelStat>(), total, s));
     return REG_OK;
 }
 
@@ -1590,7 +1590,7 @@ extern "C" int reg_pairwise(reg_ctx_t *ctx, const float *R, const float *T, int 
     const OpDesc op{0, 1, -1, -1, 0, has_init ? 1 : -1};
     double th0[3] = {0.0, 0.0, 0.0};
     if (!nonrigid && init) { th0[0] = init->alpha; th0[1] = init->gx; th0[2] = init->gy; }
-    CU(launch_pair_setup(blk, op, th0, ctx->level_tab.as<LevelDesc>(), level_table(ctx, g), ctx->means.as<float>(), s));
+    CU(launch_pair_setup(blk, op, th0, ctx->level_tab.as<LevelDesc>(), level_table(ctx, g), ctx->means.as<LevelStat>(), s));
     if (nonrigid && field_in) {
         // dense initial field -> control values sampled at the control points (node 1)
         if (!in_direct) CU(cudaMemcpyAsync(stage_u, field_in, fb, cudaMemcpyDefault, s));

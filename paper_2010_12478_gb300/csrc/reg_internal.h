@@ -20,7 +20,13 @@ struct LevelDesc {
                         // at the pixel centres (nonrigid model)
     int W, H, pitch;    // pitch of ptr, in elements
     int rpitch;         // pitch of rptr, in elements
-    float mean;         // level mean (FP32 shift constant of the moment sums)
+    float mean, sd;     // the level's (LevelStat)
+};
+
+// Mean of a level's samples, the shift constant of its moment sums, and their standard deviation, which only
+// scales one image to the other where the sums are formed (a few digits do).
+struct LevelStat {
+    float mean, sd;
 };
 
 // Pyramid layout.  The nonrigid model samples the quadratic B-spline of a level's samples
@@ -151,20 +157,20 @@ struct TileShape {
 
 // Host launchers (reg_kernels.cu).
 // Pyramids of N frames (frame f at frames + f * fstride, rows of `pitch`) into the layout `out`
-// (storage-typed); means[f * levels + l] = mean of level l of frame f (or null).
+// (storage-typed); means[f * levels + l] = those of level l of frame f (or null).
 cudaError_t launch_pyramid(const float *frames, int N, size_t fstride, int W, int H, int pitch, int levels,
-                           int storage, const PyrOut &out, float *means, cudaStream_t s);
+                           int storage, const PyrOut &out, LevelStat *means, cudaStream_t s);
 // Kernel launches of one launch_pyramid call.
 int pyramid_launches(int levels, bool means, int pad);
 // Level table of a batch of frames: frame f's row l is that of frame 0, its pointers f strides on, with
-// the level's mean.
+// the level's mean and standard deviation.
 struct LevelTable {
     int levels;
     const char *raw[kMaxLevels], *ref[kMaxLevels];         // pixel (0, 0) of frame 0, template and reference role
     size_t raw_stride[kMaxLevels], ref_stride[kMaxLevels]; // bytes between frames
     int W[kMaxLevels], H[kMaxLevels], pitch[kMaxLevels], rpitch[kMaxLevels];
 };
-cudaError_t launch_level_table(LevelDesc *tab, const LevelTable &t, const float *means, int frames, cudaStream_t s);
+cudaError_t launch_level_table(LevelDesc *tab, const LevelTable &t, const LevelStat *means, int frames, cudaStream_t s);
 
 // What one pairwise call needs on the device besides its pyramids, in one block: the operator, its
 // nodes (0 the result, 1 the initial guess), and what comes back to the host (through `status`).
@@ -177,9 +183,9 @@ struct PairBlock {
 };
 // Fill the block (statistics and status zero) and the level table of the call's two frames.
 cudaError_t launch_pair_setup(PairBlock *b, const OpDesc &op, const double *init3, LevelDesc *tab, const LevelTable &t,
-                              const float *means, cudaStream_t s);
-// tab[l].mean = means[l] for l < L (a slot's level table rows after its pyramid build).
-cudaError_t launch_set_level_means(LevelDesc *tab, const float *means, int L, cudaStream_t s);
+                              const LevelStat *means, cudaStream_t s);
+// tab[l].mean and sd = means[l] for l < L (a slot's level table rows after its pyramid build).
+cudaError_t launch_set_level_means(LevelDesc *tab, const LevelStat *means, int L, cudaStream_t s);
 // CTAs per operator for a launch that asks for `cluster`: more where an operator's control grid does
 // not fit the shared memory of so few.
 int fit_cluster(const Params &p, int cluster);

@@ -45,6 +45,7 @@ constexpr int kMaxCluster = 16; // CTAs per operator at most (non-portable clust
 // controllers are written for few FP64 instructions.
 struct LevelSums {
     double P, invP, sr, Srr;       // pixels; sum of the reference's shifted samples; S'_RR
+    double gam;                    // scale of the reference in the difference e = t - gam r
     double least;                  // a centred sum of squares below this is a constant image
 };
 
@@ -298,38 +299,44 @@ __device__ __forceinline__ void cluster_reduce(const float (&hi)[NM], const floa
 // ------------------------------------------------------------------ NCC (FP64)
 struct Ncc {
     double e;                  // 1 - NCC
-    double a, u;               // 1 / sqrt(S'_RR S'_TT), S'_RE + S'_EE
-    double dbar, Stt;          // mean of t - r, S'_TT
+    double a, u;               // 1 / sqrt(S'_RR S'_TT), gam S'_RE + S'_EE
+    double Srt, Stt, ebar;     // S'_RT, S'_TT, mean of e
 };
 
 // NCC and what its gradient follows from, from the shifted sums: of r (LevelSums) and of the difference
-// e = t - r: sum e, sum e^2, sum r e.  With S'_TT = S'_RR + 2 S'_RE + S'_EE and S'_RT = S'_RR + S'_RE the
-// rounding of the FP32 sums enters 1 - NCC, about (S'_EE - S'_RE^2 / S'_RR) / (2 S'_RR), relative to its
-// own size; sums of t^2 and r t enter it relative to 1, which left 1.8e-8 in an energy of 1e-3 (a
-// noiseless lattice, every run of pixels rounded alike).  A constant image has E = 1 and no gradient.
+// e = t - gam r: sum e, sum e^2, sum r e.  Each image is shifted by its own mean, and gam is the ratio of their
+// standard deviations (level_gain), so e is small wherever the images match up to the gain and offset that NCC
+// does not see.  With S'_RT = gam S'_RR + S'_RE and S'_TT = gam S'_RT + u, u = gam S'_RE + S'_EE, the rounding of
+// the FP32 sums enters 1 - NCC, about (S'_EE - S'_RE^2 / S'_RR) / (2 S'_TT), relative to its own size; sums of t^2
+// and r t, or of t - r at another gain or offset, enter it relative to 1.  Restated on the host (512x512
+// lattices and noise, 1 - NCC from 7e-6 to 1): off by 1e-13 to 1e-8 at any gain and offset; t - r with one shift
+// 3e-13 to 1e-8 at equal ones, but 1e-7 at gains of 3 and 1/5 and 1e-4 at an offset of 100 times the contrast; sums of t^2 and
+// r t with every product's rounding kept 1e-9 to 1e-8, 2e-6 and 1e-5.  A constant image has E = 1 and no gradient.
 __device__ __forceinline__ Ncc ncc_terms(const LevelSums &L, double se, double see, double sre)
 {
     Ncc o;
-    o.dbar = __dmul_rn(se, L.invP);
-    const double See = __fma_rn(-se, o.dbar, see), Sre = __fma_rn(-L.sr, o.dbar, sre);
-    const double Srt = __dadd_rn(L.Srr, Sre);
-    o.u = __dadd_rn(Sre, See);
-    o.Stt = __dadd_rn(Srt, o.u);
+    o.ebar = __dmul_rn(se, L.invP);
+    const double See = __fma_rn(-se, o.ebar, see), Sre = __fma_rn(-L.sr, o.ebar, sre);
+    o.Srt = __fma_rn(L.gam, L.Srr, Sre);
+    o.u = __fma_rn(L.gam, Sre, See);
+    o.Stt = __fma_rn(L.gam, o.Srt, o.u);
     o.a = rsqrt(__dmul_rn(L.Srr, o.Stt));
-    o.e = __fma_rn(-Srt, o.a, 1.0);
-    // e = 0 everywhere (T o phi equals R up to the shift: identical inputs) is exactly NCC = 1
+    o.e = __fma_rn(-o.Srt, o.a, 1.0);
+    // e = 0 everywhere (T o phi equals R up to gain and offset: identical inputs) is exactly NCC = 1
     if ((__double_as_longlong(Sre) | __double_as_longlong(See)) << 1 == 0) o.e = 0.0;
+    // a constant template has no deviation at all (gam 0), whatever its samples between the pixels round to
     if (__double_as_longlong(L.Srr) < __double_as_longlong(L.least) ||
-        __double_as_longlong(o.Stt) < __double_as_longlong(L.least)) {
+        __double_as_longlong(o.Stt) < __double_as_longlong(L.least) || __double_as_longlong(L.gam) == 0) {
         o.e = 1.0; o.a = 0.0;
     }
     return o;
 }
 
 // A level's constants, and the reference's part of its sums (known after the first pass).
-__device__ __forceinline__ void set_level(LevelSums &L, int W, int H)
+__device__ __forceinline__ void set_level(LevelSums &L, int W, int H, float gam)
 {
     L.P = (double)W * (double)H;
+    L.gam = gam;
     L.invP = 1.0 / L.P;
     L.least = 1e-12 * L.P;
 }
@@ -344,7 +351,8 @@ __device__ __forceinline__ void set_reference(LevelSums &L, double sr, double sr
 struct Lvl {
     const void *R, *T;
     int W, H, Rp, Tp;
-    float cR;   // shift constant (mean of the reference level)
+    float cR, cT;   // shift constants: the levels' means
+    float gam;      // level_gain
 };
 
 __device__ __forceinline__ void strip_rows(int H, int rank, int C, int &r0, int &r1)
@@ -395,10 +403,10 @@ constexpr unsigned kRoundBits = 0x4B400000u;
 
 // ================================================================== rigid
 // One pass over a level's rows [r0, r1) at (cos(alpha) - 1, sin(alpha), translation) gives the moments
-// of the energy and the sums the gradient follows from: with the shifted samples t = T(phi(x)) - cR,
-// r = R(x) - cR, F = P dE/dTw = aP (t - r) + (b - a) P t + kappa as in the nonrigid pass, and g_k =
-// grad T(phi(x)) . dphi/dtheta_k, k = alpha, Gx, Gy.  Sums in sm.tot, e = t - r: 0 sum e, 1 sum e^2,
-// 2 sum r e, with START (a level's first pass) 3 sum r, 4 sum r^2; 5 + k sum e g_k; 8 + k sum t g_k;
+// of the energy and the sums the gradient follows from: with the shifted samples t = T(phi(x)) - cT,
+// r = R(x) - cR, e = t - gam r, dE/dTw = b e + c r + kappa as in the nonrigid pass, and g_k =
+// grad T(phi(x)) . dphi/dtheta_k, k = alpha, Gx, Gy.  Sums in sm.tot: 0 sum e, 1 sum e^2,
+// 2 sum r e, with START (a level's first pass) 3 sum r, 4 sum r^2; 5 + k sum e g_k; 8 + k sum r g_k;
 // 11 + k sum g_k.
 //
 // Two columns a lane in packed steps, as in the nonrigid pass: a warp's task is 64 columns over a
@@ -417,7 +425,7 @@ __device__ void rigid_pass(const Lvl &L, int r0, int r1, const float *pm, Smem &
     const int gix = (int)pm[4], giy = (int)pm[5];
     const float cx = 0.5f * (float)(L.W - 1), cy = 0.5f * (float)(L.H - 1);
     const S *R = (const S *)L.R, *T = (const S *)L.T;
-    const float2 ncR = f2(-L.cR), one = f2(1.f);
+    const float2 ncR = f2(-L.cR), ncT = f2(-L.cT), ngam = f2(-L.gam), one = f2(1.f);
     float2 mh[NS], ml[NS], m[NS];   // moments: float-float sums and the current run, per column
     float gh[9], gl[9];             // gradient sums: float-float, and the current run
     float2 g[9];
@@ -459,10 +467,10 @@ __device__ void rigid_pass(const Lvl &L, int r0, int r1, const float *pm, Smem &
             vy = __ffma2_rn(f2(sa), xc, f2(fmaf(cm1, yc, gfy)));
         };
         auto pixel = [&](float2 tw, float2 dx, float2 dy, float2 rv, float yc) {
-            const float2 t = __fadd2_rn(tw, ncR), r = __fadd2_rn(rv, ncR), F = f2sub(t, r);
-            m[0] = __fadd2_rn(m[0], F);
-            m[1] = __ffma2_rn(F, F, m[1]);
-            m[2] = __ffma2_rn(r, F, m[2]);
+            const float2 r = __fadd2_rn(rv, ncR), e = __ffma2_rn(ngam, r, __fadd2_rn(tw, ncT));
+            m[0] = __fadd2_rn(m[0], e);
+            m[1] = __ffma2_rn(e, e, m[1]);
+            m[2] = __ffma2_rn(r, e, m[2]);
             if constexpr (START) {
                 m[3] = __fadd2_rn(m[3], r);
                 m[4] = __ffma2_rn(r, r, m[4]);
@@ -472,8 +480,8 @@ __device__ void rigid_pass(const Lvl &L, int r0, int r1, const float *pm, Smem &
             const float2 q[3] = {__ffma2_rn(dy, py, __fmul2_rn(dx, px)), dx, dy};
 #pragma unroll
             for (int i = 0; i < 3; ++i) {
-                g[i] = __ffma2_rn(F, q[i], g[i]);
-                g[3 + i] = __ffma2_rn(t, q[i], g[3 + i]);
+                g[i] = __ffma2_rn(e, q[i], g[i]);
+                g[3 + i] = __ffma2_rn(r, q[i], g[3 + i]);
                 g[6 + i] = __fadd2_rn(g[6 + i], q[i]);
             }
         };
@@ -598,14 +606,27 @@ __device__ __forceinline__ double next_tau(double E, double slope, double tau, d
     return accepted ? fmin(fmax(tq, 0.5 * tau), 4.0 * tau) : fmin(fmax(tq, 0.1 * tau), 0.5 * tau);
 }
 
-// Gradient component q at the point of a pass from its sums and the point's NCC terms: dE/dtheta_q = a
-// sum (t - r) g_q + (b - a) sum t g_q + (a rbar - b tbar) sum g_q, with b = NCC / S'_TT, so b - a = -a^3
-// S'_RR u, and a rbar - b tbar = -a (tbar - rbar) - (b - a) tbar; exact zeros for identical frames.
+// Coefficients of the gradient of 1 - NCC: dE/dTw(x) = b (t - tbar) - a (r - rbar) = b e + c r + kappa with
+// b = NCC / S'_TT, c = gam b - a = -a u / S'_TT, kappa = -(b ebar + c rbar); 1 / S'_TT = a^2 S'_RR.  c and kappa are
+// exact zeros for identical frames.
+struct GradCoef {
+    double b, c, kappa;
+};
+__device__ __forceinline__ GradCoef grad_coef(const LevelSums &L, const Ncc &n)
+{
+    const double w = __dmul_rn(__dmul_rn(n.a, n.a), __dmul_rn(n.a, L.Srr));
+    GradCoef o;
+    o.b = __dmul_rn(w, n.Srt);
+    o.c = -__dmul_rn(w, n.u);
+    o.kappa = -__fma_rn(o.b, n.ebar, __dmul_rn(o.c, __dmul_rn(L.sr, L.invP)));
+    return o;
+}
+
+// Gradient component q at the point of a pass from its sums and the point's NCC terms.
 __device__ __forceinline__ double rigid_gradient(const LevelSums &L, const Ncc &n, const double *tot, int q)
 {
-    const double bma = __dmul_rn(__dmul_rn(__dmul_rn(-n.a, n.a), n.a), __dmul_rn(L.Srr, n.u));
-    const double kap = __fma_rn(-bma, __fma_rn(L.sr, L.invP, n.dbar), -__dmul_rn(n.a, n.dbar));
-    return __fma_rn(n.a, tot[5 + q], __fma_rn(bma, tot[8 + q], __dmul_rn(kap, tot[11 + q])));
+    const GradCoef k = grad_coef(L, n);
+    return __fma_rn(k.b, tot[5 + q], __fma_rn(k.c, tot[8 + q], __dmul_rn(k.kappa, tot[11 + q])));
 }
 
 // v of lanes 0, 1 and 2 added in that order, in every lane.
@@ -687,12 +708,21 @@ __device__ int rigid_step(RigidCtl &k, const Config &cfg, const double *tot, boo
     return stop >= 0 ? kActDone : kActTrial;
 }
 
+// Scale of a reference of standard deviation sr to a template of st; any value gives the same NCC up to rounding,
+// 1 where there is none (a constant reference, samples that are not finite).
+__device__ __forceinline__ float level_gain(float sr, float st)
+{
+    const float g = st / sr;
+    return sr >= 1e-6f && g <= 1e30f ? g : 1.f;
+}
+
 __device__ __forceinline__ Lvl level_of(const Params &p, int ref, int tmpl, int l)
 {
     const LevelDesc &a = p.levels[ref * p.cfg.levels + l];
     const LevelDesc &b = p.levels[tmpl * p.cfg.levels + l];
     Lvl L;
-    L.R = a.rptr; L.T = b.ptr; L.W = a.W; L.H = a.H; L.Rp = a.rpitch; L.Tp = b.pitch; L.cR = a.mean;
+    L.R = a.rptr; L.T = b.ptr; L.W = a.W; L.H = a.H; L.Rp = a.rpitch; L.Tp = b.pitch;
+    L.cR = a.mean; L.cT = b.mean; L.gam = level_gain(a.sd, b.sd);
     return L;
 }
 
@@ -733,7 +763,7 @@ __device__ void run_rigid(const Params &p, const OpDesc &op, int op_index, Smem 
         int r0, r1;
         strip_rows(L.H, rank, C, r0, r1);
         if (tid == 0) {
-            set_level(k.ls, L.W, L.H);
+            set_level(k.ls, L.W, L.H, L.gam);
             double rho = 0.25 * (L.W + L.H);
             k.m0 = rho * rho;
             k.inv_m0 = 1.0 / k.m0;
@@ -793,12 +823,11 @@ __device__ void run_rigid(const Params &p, const OpDesc &op, int op_index, Smem 
 //
 // One pass over a level's pixels gives everything an evaluation needs: the moments of the energy
 // and, per control point, the sums from which the gradient follows once the moments are known.
-// With F = P dE/dTw = aP (t - r) + (b - a) P t + kappa (r, t the shifted samples, kappa =
-// (a rbar - b tbar) P), the gradient of the data term is
-//     sum_x w_j F dT/dp = aP sum w_j (t - r) dT/dp + (b - a) P sum w_j t dT/dp + kappa sum w_j dT/dp,
-// three sums per point and axis that do not depend on the moments.  The second coefficient is
-// small where the energy is (b = NCC sqrt(S'_rr / S'_tt) a), so the split loses no precision to
-// cancellation; identical frames give t - r = 0, b = a and kappa = 0 exactly.  An accepted trial
+// With dE/dTw = b e + c r + kappa (e = t - gam r and r the shifted samples, ncc_terms; b, c, kappa:
+// grad_coef), the gradient of the data term is
+//     b sum_x w_j e dT/dp + c sum w_j r dT/dp + kappa sum w_j dT/dp,
+// three sums per point and axis that do not depend on the moments.  c is small where the energy is, so the
+// split loses no precision to cancellation; identical frames give e = 0, c = 0 and kappa = 0 exactly.  An accepted trial
 // (three in four and more) thus costs one pass over the pixels, not one for the energy and one for
 // the gradient, and a level starts with one pass, which also gives the Gauss-Newton scalar product.
 // The gradient sums of a rejected trial are dropped.  With separate passes a scan of 256 frames of
@@ -886,7 +915,7 @@ __host__ __device__ __forceinline__ int div20(int a, unsigned r)
     return (int)(((unsigned)a * r) >> 20);
 }
 
-constexpr int kSlot = 8;   // floats per slot: (t - r, t, 1) x (x, y), then dT^2 x (x, y)
+constexpr int kSlot = 8;   // floats per slot: (e, r, 1) x (x, y), then dT^2 x (x, y)
 // The rule of PassGeom.  On the host, once per launch: made by the kernel, per operator and level, it took
 // 16 us of a pair of 128x128 frames.
 //
@@ -1184,7 +1213,7 @@ __device__ __forceinline__ void slot_sum(const float *slots, const PassGeom &P, 
 }
 
 // One pass at c (START: a level's first) or at the trial c + tau d: the moments into sm.tot (e =
-// t - r: 0 sum e, 1 sum e^2, 2 sum r e, with START 3 sum r, 4 sum r^2; 5: sum over control edges of |dct|^2) and the gradient
+// t - gam r: 0 sum e, 1 sum e^2, 2 sum r e, with START 3 sum r, 4 sum r^2; 5: sum over control edges of |dct|^2) and the gradient
 // sums into the slots.  The trial values are formed where they are read, fmaf(tau, d_j, c_j), the
 // expression an accepted step stores into c.
 //
@@ -1202,7 +1231,7 @@ __device__ void grid_pass(const Lvl &L, const Grid &G, const GridLvl &GL, const 
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int ncx = G.nx - 1, ncy = G.ny - 1, sl = P.sl;
     const S *Rp = (const S *)L.R, *T = (const S *)L.T;
-    const float2 ncR = f2(-L.cR), dw = f2(GL.pl * GL.scale_inv);
+    const float2 ncR = f2(-L.cR), ncT = f2(-L.cT), ngam = f2(-L.gam), dw = f2(GL.pl * GL.scale_inv);
     float *emit = emits + warp * kEmitFloats;
     auto ct = [&](int row, int col) {   // control value of the point evaluated
         const int j = (row - B.h0) * G.nx + col;
@@ -1257,9 +1286,9 @@ __device__ void grid_pass(const Lvl &L, const Grid &G, const GridLvl &GL, const 
             ty = make_float2(fmaf(wx[0], p1.y - p0.y, p0.y), fmaf(wx[1], q1.y - q0.y, q0.y));
         };
         const S *ra = Rp + xc[0], *rb = Rp + xc[1];
-        float2 sF[4], sT[4], s1[4], sM[4];   // top x, top y, bottom x, bottom y
+        float2 sE[4], sR[4], s1[4], sM[4];   // top x, top y, bottom x, bottom y
 #pragma unroll
-        for (int i = 0; i < 4; ++i) sF[i] = sT[i] = s1[i] = sM[i] = f2(0.f);
+        for (int i = 0; i < 4; ++i) sE[i] = sR[i] = s1[i] = sM[i] = f2(0.f);
         float2 tx, ty;
         column(ca, tx, ty);
         auto flush = [&]() {
@@ -1272,11 +1301,10 @@ __device__ void grid_pass(const Lvl &L, const Grid &G, const GridLvl &GL, const 
         // one pixel of either column; wy: the weight of the control row below
         auto pixel = [&](const TapRow &t0, const TapRow &t1, const TapRow &t2, float2 fx, float2 fy, float2 r, float2 wy) {
             float2 dx2, dy2;
-            const float2 t = __fadd2_rn(bspline2(t0, t1, t2, fx, fy, dx2, dy2), ncR);
-            const float2 F = f2sub(t, r);
-            a[0] = __fadd2_rn(a[0], F);
-            a[1] = __ffma2_rn(F, F, a[1]);
-            a[2] = __ffma2_rn(r, F, a[2]);
+            const float2 e = __ffma2_rn(ngam, r, __fadd2_rn(bspline2(t0, t1, t2, fx, fy, dx2, dy2), ncT));
+            a[0] = __fadd2_rn(a[0], e);
+            a[1] = __ffma2_rn(e, e, a[1]);
+            a[2] = __ffma2_rn(r, e, a[2]);
             if constexpr (START) {
                 a[3] = __fadd2_rn(a[3], r);
                 a[4] = __ffma2_rn(r, r, a[4]);
@@ -1285,8 +1313,8 @@ __device__ void grid_pass(const Lvl &L, const Grid &G, const GridLvl &GL, const 
             const float2 g[4] = {__fmul2_rn(wt, dx2), __fmul2_rn(wt, dy2), __fmul2_rn(wb, dx2), __fmul2_rn(wb, dy2)};
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
-                sF[i] = __ffma2_rn(F, g[i], sF[i]);
-                sT[i] = __ffma2_rn(t, g[i], sT[i]);
+                sE[i] = __ffma2_rn(e, g[i], sE[i]);
+                sR[i] = __ffma2_rn(r, g[i], sR[i]);
                 s1[i] = __fadd2_rn(s1[i], g[i]);
                 if constexpr (START) sM[i] = __ffma2_rn(g[i], g[i], sM[i]);
             }
@@ -1419,8 +1447,8 @@ __device__ void grid_pass(const Lvl &L, const Grid &G, const GridLvl &GL, const 
                 __syncwarp();
 #pragma unroll
                 for (int i = 0; i < 2; ++i) {
-                    put(i, kEmitSums, sF[i]);
-                    put(2 + i, kEmitSums, sT[i]);
+                    put(i, kEmitSums, sE[i]);
+                    put(2 + i, kEmitSums, sR[i]);
                     put(4 + i, kEmitSums, s1[i]);
                 }
                 __syncwarp();
@@ -1435,8 +1463,8 @@ __device__ void grid_pass(const Lvl &L, const Grid &G, const GridLvl &GL, const 
             }
 #pragma unroll
             for (int i = 0; i < 2; ++i) {
-                sF[i] = sF[2 + i]; sF[2 + i] = f2(0.f);
-                sT[i] = sT[2 + i]; sT[2 + i] = f2(0.f);
+                sE[i] = sE[2 + i]; sE[2 + i] = f2(0.f);
+                sR[i] = sR[2 + i]; sR[2 + i] = f2(0.f);
                 s1[i] = s1[2 + i]; s1[2 + i] = f2(0.f);
                 sM[i] = sM[2 + i]; sM[2 + i] = f2(0.f);
             }
@@ -1598,8 +1626,8 @@ __device__ void grid_metric(const Grid &G, const PassGeom &P, const Band &B, con
 }
 
 // The descent direction d = -M^-1 grad E at c with the scalar product mt, from the pass's gradient
-// sums: dE/dc_j = (1/P) [aP sF + bmaP sT + kappa s1 + lambda sum_nbrs (c_j - c_k)] (pm: aP, (b - a) P,
-// kappa, lambda), at the own rows and, through the neighbours' staged rows, at the held ones.  Leaves
+// sums: dE/dc_j = (1/P) [bP sE + cP sR + kP s1 + lambda sum_nbrs (c_j - c_k)] (pm: b P, c P, kappa P,
+// lambda), at the own rows and, through the neighbours' staged rows, at the held ones.  Leaves
 // sum_j m_j |d_j|^2 in sm.tot[0], with the direction d held before the call <d_old, d_old - d>_M in
 // sm.tot[1] and |d_old - d|_M^2 in sm.tot[2], max |d_j|^2 in sm.tmax; identical in every CTA.
 template <bool FF = false>
@@ -1609,7 +1637,7 @@ __device__ void grid_direction(const Grid &G, const Lvl &L, const PassGeom &P, c
 {
     const int Nc = G.nx * G.ny, n = (B.own1 - B.cr0) * G.nx, rank = cl.block_rank();
     const bool quiet = comm_quiet(sm);
-    const float aP = pm[0], bmaP = pm[1], kappa = pm[2], lam = pm[3];
+    const float bP = pm[0], cP = pm[1], kP = pm[2], lam = pm[3];
     const float scale = -(float)Nc / ((float)L.W * (float)L.H);
     float hi[3] = {0.f, 0.f, 0.f}, lo[3] = {0.f, 0.f, 0.f}, mx = 0.f;
     // -Nc dE/dc at own point j (row i of the own rows)
@@ -1617,8 +1645,8 @@ __device__ void grid_direction(const Grid &G, const Lvl &L, const PassGeom &P, c
         const int row = B.cr0 + i, k = (row - B.h0) * G.nx + jx;
         float s[6];
         point_sum<6, FF>(slots, above, P, B, G.nx - 1, row, jx, 0, s);
-        const float gx = fmaf(aP, s[0], fmaf(bmaP, s[2], kappa * s[4]));
-        const float gy = fmaf(aP, s[1], fmaf(bmaP, s[3], kappa * s[5]));
+        const float gx = fmaf(bP, s[0], fmaf(cP, s[2], kP * s[4]));
+        const float gy = fmaf(bP, s[1], fmaf(cP, s[3], kP * s[5]));
         const float2 cj = c[k];
         float lx = 0.f, ly = 0.f;
         if (jx > 0)         { const float2 v = c[k - 1];    lx += cj.x - v.x; ly += cj.y - v.y; }
@@ -1702,19 +1730,17 @@ __device__ void grid_direction(const Grid &G, const Lvl &L, const PassGeom &P, c
     }
 }
 
-// Parameter slots of the nonrigid passes: gradient coefficients aP, (b - a) P, (a rbar - b tbar) P
+// Parameter slots of the nonrigid passes: gradient coefficients b P, c P, kappa P (grad_coef)
 // and lambda; the scalar product's 1/(P var T) and lambda/P; the next trial's step.
-enum FieldParam { kPmA = 0, kPmB = 1, kPmK = 2, kPmLam = 3, kPmDk = 4, kPmRk = 5, kPmTau = 6 };
+enum FieldParam { kPmB = 0, kPmC = 1, kPmK = 2, kPmLam = 3, kPmDk = 4, kPmRk = 5, kPmTau = 6 };
 
-// Gradient coefficients from a point's NCC terms, b - a = -a^3 S'_RR u: formed in FP64, rounded once; exact
-// zeros but aP for identical frames.
+// The coefficients times P, formed in FP64 and rounded once.
 __device__ __forceinline__ void field_grad_params(const Ncc &n, const LevelSums &L, const Config &cfg, float *pm)
 {
-    const double aP = __dmul_rn(n.a, L.P);
-    const double b = -__dmul_rn(__dmul_rn(n.a, L.Srr), __dmul_rn(__dmul_rn(n.a, n.u), aP));
-    pm[kPmA] = (float)aP;
-    pm[kPmB] = (float)b;
-    pm[kPmK] = (float)-__fma_rn(b, __fma_rn(L.sr, L.invP, n.dbar), __dmul_rn(aP, n.dbar));
+    const GradCoef k = grad_coef(L, n);
+    pm[kPmB] = (float)__dmul_rn(k.b, L.P);
+    pm[kPmC] = (float)__dmul_rn(k.c, L.P);
+    pm[kPmK] = (float)__dmul_rn(k.kappa, L.P);
     pm[kPmLam] = (float)cfg.lambda;
 }
 
@@ -1863,7 +1889,7 @@ __device__ void run_nonrigid(const Params &p, const OpDesc &op, int op_index, Sm
         if (cfg.metric == REG_METRIC_MEAN)
             for (int j = tid; j < held; j += kThreads) mt[j] = make_float2(1.f, 1.f);
         if (tid == 0) {
-            set_level(k.ls, L.W, L.H);
+            set_level(k.ls, L.W, L.H, L.gam);
             k.half_lam = 0.5 * cfg.lambda * k.ls.invP;
             k.tau = cfg.tau0;
             k.have_prev = 0;
@@ -2190,7 +2216,7 @@ __global__ void __launch_bounds__(kThreads) energy_kernel(const __grid_constant_
         RigidCtl &k = sm.rctl;
         if (tid == 0) {
             memset(&k, 0, sizeof(k));
-            set_level(k.ls, L.W, L.H);
+            set_level(k.ls, L.W, L.H, L.gam);
         }
         if (tid < 32) rigid_param(theta[min(tid, 2)], min(tid, 2), tid, sm.pm);
         __syncthreads();
@@ -2227,7 +2253,7 @@ __global__ void __launch_bounds__(kThreads) energy_kernel(const __grid_constant_
         grid_pass<S, true, 2>(L, G, GL, P, B, c, d, 0.f, slots, above, emits, pi, sm, comm, cl);
         FieldCtl &k = sm.fctl;
         if (tid == 0) {
-            set_level(k.ls, L.W, L.H);
+            set_level(k.ls, L.W, L.H, L.gam);
             set_reference(k.ls, sm.tot[3], sm.tot[4]);
             const Ncc n = ncc_terms(k.ls, sm.tot[0], sm.tot[1], sm.tot[2]);
             if (first) out[0] = __fma_rn(0.5 * p.cfg.lambda * k.ls.invP, sm.tot[5], n.e);

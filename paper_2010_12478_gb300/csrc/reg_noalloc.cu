@@ -37,6 +37,7 @@ constexpr size_t kOffTheta = kOffStats + 256 * ((sizeof(OpStats) + 255) / 256);
 constexpr size_t kOffStatus = kOffTheta + 256;
 constexpr size_t kOffMeans = kOffStatus + 256;
 constexpr size_t kScratchBytes = kOffMeans + 256;
+static_assert(2 * kMaxLevels * sizeof(LevelStat) <= 256, "the last record's room");
 
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kScratchBytes];
 
@@ -144,7 +145,7 @@ extern "C" int reg_pairwise_noalloc(const reg_config_t *cfg, int device, const f
         OpStats *st = (OpStats *)(base + kOffStats);
         double *theta = (double *)(base + kOffTheta);
         int *status = (int *)(base + kOffStatus);
-        float *means = (float *)(base + kOffMeans);
+        LevelStat *means = (LevelStat *)(base + kOffMeans);
 
         // the array keeps the previous call's contents: clear what must start at zero
         cudaError_t e = cudaMemsetAsync(st, 0, sizeof(OpStats), s);
@@ -167,9 +168,9 @@ extern "C" int reg_pairwise_noalloc(const reg_config_t *cfg, int device, const f
         if (e == cudaSuccess)
             e = launch_pyramid(T, 1, (size_t)H * pitch, W, H, pitch, cfg->levels, cfg->storage, ot,
                                means + cfg->levels, s);
-        float hmeans[2 * kMaxLevels];
+        LevelStat hmeans[2 * kMaxLevels];
         if (e == cudaSuccess)
-            e = cudaMemcpyAsync(hmeans, means, sizeof(float) * 2 * cfg->levels, cudaMemcpyDeviceToHost, s);
+            e = cudaMemcpyAsync(hmeans, means, sizeof(LevelStat) * 2 * cfg->levels, cudaMemcpyDeviceToHost, s);
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
         if (e != cudaSuccess) {
             cudaGetLastError();
@@ -186,7 +187,8 @@ extern "C" int reg_pairwise_noalloc(const reg_config_t *cfg, int device, const f
                 d.H = Hl[l];
                 d.pitch = Wl[l];
                 d.rpitch = Wl[l];
-                d.mean = hmeans[f * cfg->levels + l];
+                d.mean = hmeans[f * cfg->levels + l].mean;
+                d.sd = hmeans[f * cfg->levels + l].sd;
             }
         OpDesc hop{0, 1, -1, -1, 0, init ? 1 : -1};
         double hinit[3] = {init ? init->alpha : 0.0, init ? init->gx : 0.0, init ? init->gy : 0.0};

@@ -101,7 +101,19 @@ template <typename S> struct Levels {
     int nxb[kMaxLevels], nsb[kMaxLevels];   // pyr_finish: column blocks of the model, and its blocks
 };
 
-// Mean of every level of each frame, a deterministic float-float sum: a cluster of kMeanCtas CTAs
+// Samples counted, their mean and sum of squared deviations; the union of two sets by Chan, Golub and LeVeque,
+// "Updating formulae and a pairwise algorithm for computing sample variances", 1979: no cancellation, whatever
+// the mean.
+struct Spread {
+    float n, mean, dev;
+};
+__device__ __forceinline__ Spread joined(Spread a, Spread b)
+{
+    const float n = a.n + b.n, d = b.mean - a.mean, w = n > 0.f ? b.n / n : 0.f;
+    return Spread{n, fmaf(d, w, a.mean), a.dev + b.dev + d * d * (a.n * w)};
+}
+
+// Mean and standard deviation of every level of each frame; the mean a deterministic float-float sum: a cluster of kMeanCtas CTAs
 // sums the rows of one level (a warp takes every kMeanCtas * kMeanWarps-th row, a lane every 32nd
 // column with kMeanBatch loads in flight), and its first CTA adds the CTAs' sums in rank order.  The
 // split is the same for every batch size, so a frame's means do not depend on the call it is in.
@@ -110,10 +122,11 @@ template <typename S> struct Levels {
 // known to run: each arrives at the cluster barrier first and waits there after its sums.
 constexpr int kMeanCtas = 8, kMeanWarps = 8, kMeanBatch = 8;
 template <typename S>
-__global__ void __launch_bounds__(32 * kMeanWarps) level_means(Levels<S> L, float *means, int levels)
+__global__ void __launch_bounds__(32 * kMeanWarps) level_means(Levels<S> L, LevelStat *means, int levels)
 {
     __shared__ float2 ws[kMeanWarps];
     __shared__ float2 part[kMeanCtas];
+    __shared__ Spread wsp[kMeanWarps], spart[kMeanCtas];
     cg::cluster_group cl = cg::this_cluster();
     cl.barrier_arrive();
     const int l = blockIdx.y, f = blockIdx.x / kMeanCtas, rank = cl.block_rank();
@@ -121,35 +134,50 @@ __global__ void __launch_bounds__(32 * kMeanWarps) level_means(Levels<S> L, floa
     const int W = L.W[l], H = L.H[l], pitch = L.pitch[l];
     const S *img = L.lvl[l] + (size_t)f * L.stride[l];
     float hi = 0.f, lo = 0.f;
+    float x0 = 0.f, n = 0.f, s1 = 0.f, s2 = 0.f;   // the lane's first sample, and its samples' differences from it
     for (int r = rank * kMeanWarps + warp; r < H; r += kMeanCtas * kMeanWarps) {
         const S *row = img + (size_t)r * pitch;
         for (int c0 = lane; c0 < W; c0 += 32 * kMeanBatch) {
             float x[kMeanBatch], a = 0.f;
 #pragma unroll
             for (int k = 0; k < kMeanBatch; ++k) x[k] = c0 + 32 * k < W ? ldS<S>(row + c0 + 32 * k) : 0.f;
+            if (n == 0.f) x0 = x[0];
 #pragma unroll
-            for (int k = 0; k < kMeanBatch; ++k) a += x[k];
+            for (int k = 0; k < kMeanBatch; ++k) {
+                a += x[k];
+                const float d = c0 + 32 * k < W ? x[k] - x0 : 0.f;
+                s1 += d;
+                s2 = fmaf(d, d, s2);
+            }
+            n += (float)min(kMeanBatch, (W - c0 + 31) / 32);
             ff_acc(hi, lo, a);
         }
     }
+    const float m1 = n > 0.f ? s1 / n : 0.f;
+    Spread sp{n, x0 + m1, fmaxf(fmaf(-s1, m1, s2), 0.f)};
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) {
         const float h2 = __shfl_xor_sync(0xffffffffu, hi, off), l2 = __shfl_xor_sync(0xffffffffu, lo, off);
         ff_add(hi, lo, h2, l2);
+        sp = joined(sp, Spread{__shfl_xor_sync(0xffffffffu, sp.n, off), __shfl_xor_sync(0xffffffffu, sp.mean, off),
+                               __shfl_xor_sync(0xffffffffu, sp.dev, off)});
     }
-    if (lane == 0) ws[warp] = make_float2(hi, lo);
+    if (lane == 0) { ws[warp] = make_float2(hi, lo); wsp[warp] = sp; }
     __syncthreads();
     cl.barrier_wait();
     if (threadIdx.x == 0) {
         float h = 0.f, l2 = 0.f;
         for (int k = 0; k < kMeanWarps; ++k) ff_add(h, l2, ws[k].x, ws[k].y);
         *cl.map_shared_rank(&part[rank], 0) = make_float2(h, l2);
+        for (int k = 1; k < kMeanWarps; ++k) sp = joined(sp, wsp[k]);
+        *cl.map_shared_rank(&spart[rank], 0) = sp;
     }
     cl.sync();
     if (rank == 0 && threadIdx.x == 0) {
         float h = 0.f, l2 = 0.f;
         for (int k = 0; k < kMeanCtas; ++k) ff_add(h, l2, part[k].x, part[k].y);
-        means[(size_t)f * levels + l] = (float)(((double)h + (double)l2) / ((double)W * (double)H));
+        for (int k = 1; k < kMeanCtas; ++k) sp = joined(sp, spart[k]);
+        means[(size_t)f * levels + l] = LevelStat{(float)(((double)h + (double)l2) / ((double)W * (double)H)), sqrtf(sp.dev / sp.n)};
     }
 }
 
@@ -164,12 +192,12 @@ __global__ void __launch_bounds__(32 * kMeanWarps) level_means(Levels<S> L, floa
 // bottom bands first, then the left and right ones.
 constexpr int kSmoothRows = 16, kFinishThreads = 128;
 template <typename S>
-__global__ void __launch_bounds__(kFinishThreads) pyr_finish(Levels<S> L, int pad, const float *means, int levels)
+__global__ void __launch_bounds__(kFinishThreads) pyr_finish(Levels<S> L, int pad, const LevelStat *means, int levels)
 {
     const int l = blockIdx.y;
     const int W = L.W[l], H = L.H[l], pitch = L.pitch[l];
     S *lvl = L.lvl[l] + blockIdx.z * L.stride[l];
-    const S edge = toS<S>(means[(size_t)blockIdx.z * levels + l]);
+    const S edge = toS<S>(means[(size_t)blockIdx.z * levels + l].mean);
     if ((int)blockIdx.x >= L.nsb[l]) {
         const int bands = 2 * pad * pitch, sides = 2 * pad * H;
         const int t = ((int)blockIdx.x - L.nsb[l]) * kFinishThreads + threadIdx.x;
@@ -213,7 +241,7 @@ __global__ void __launch_bounds__(kFinishThreads) pyr_finish(Levels<S> L, int pa
 }
 
 // Row i of a level table (frame i / levels).
-__device__ __forceinline__ void level_row(LevelDesc *tab, const LevelTable &t, const float *means, int i)
+__device__ __forceinline__ void level_row(LevelDesc *tab, const LevelTable &t, const LevelStat *means, int i)
 {
     const int f = i / t.levels, l = i - f * t.levels;
     LevelDesc d;
@@ -223,19 +251,20 @@ __device__ __forceinline__ void level_row(LevelDesc *tab, const LevelTable &t, c
     d.H = t.H[l];
     d.pitch = t.pitch[l];
     d.rpitch = t.rpitch[l];
-    d.mean = means[i];
+    d.mean = means[i].mean;
+    d.sd = means[i].sd;
     tab[i] = d;
 }
 
 // Made on the device, the table costs a launch; with the means read back and the rows made by the host it
 // cost two copies and two waits, of a 160x128 pair's call some 40 us.
-__global__ void level_table_kernel(LevelDesc *tab, LevelTable t, const float *means, int rows)
+__global__ void level_table_kernel(LevelDesc *tab, LevelTable t, const LevelStat *means, int rows)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i < rows) level_row(tab, t, means, i);
 }
 
-cudaError_t launch_level_table(LevelDesc *tab, const LevelTable &t, const float *means, int frames, cudaStream_t s)
+cudaError_t launch_level_table(LevelDesc *tab, const LevelTable &t, const LevelStat *means, int frames, cudaStream_t s)
 {
     const int rows = frames * t.levels;
     level_table_kernel<<<(rows + 127) / 128, 128, 0, s>>>(tab, t, means, rows);
@@ -243,7 +272,7 @@ cudaError_t launch_level_table(LevelDesc *tab, const LevelTable &t, const float 
 }
 
 __global__ void pair_setup_kernel(PairBlock *b, OpDesc op, double i0, double i1, double i2, LevelDesc *tab, LevelTable t,
-                                  const float *means)
+                                  const LevelStat *means)
 {
     if (threadIdx.x < 2 * t.levels) level_row(tab, t, means, threadIdx.x);
     unsigned *w = reinterpret_cast<unsigned *>(&b->stats);
@@ -258,20 +287,20 @@ __global__ void pair_setup_kernel(PairBlock *b, OpDesc op, double i0, double i1,
 }
 
 cudaError_t launch_pair_setup(PairBlock *b, const OpDesc &op, const double *init3, LevelDesc *tab, const LevelTable &t,
-                              const float *means, cudaStream_t s)
+                              const LevelStat *means, cudaStream_t s)
 {
     pair_setup_kernel<<<1, 64, 0, s>>>(b, op, init3[0], init3[1], init3[2], tab, t, means);
     return cudaGetLastError();
 }
 
 // The level means of a freshly built pyramid into its rows of a level table.
-__global__ void set_level_means_kernel(LevelDesc *tab, const float *means, int L)
+__global__ void set_level_means_kernel(LevelDesc *tab, const LevelStat *means, int L)
 {
     const int l = threadIdx.x;
-    if (l < L) tab[l].mean = means[l];
+    if (l < L) { tab[l].mean = means[l].mean; tab[l].sd = means[l].sd; }
 }
 
-cudaError_t launch_set_level_means(LevelDesc *tab, const float *means, int L, cudaStream_t s)
+cudaError_t launch_set_level_means(LevelDesc *tab, const LevelStat *means, int L, cudaStream_t s)
 {
     set_level_means_kernel<<<1, 32, 0, s>>>(tab, means, L);
     return cudaGetLastError();
@@ -284,7 +313,7 @@ int pyramid_launches(int levels, bool means, int pad)
 
 template <typename S>
 static cudaError_t pyramid_t(const float *frames, int N, size_t fstride, int W, int H, int pitch, int levels,
-                             const PyrOut &o, float *means, cudaStream_t s)
+                             const PyrOut &o, LevelStat *means, cudaStream_t s)
 {
     Levels<S> L = {};
     int w = W, h = H, most = 0;
@@ -335,7 +364,7 @@ static cudaError_t pyramid_t(const float *frames, int N, size_t fstride, int W, 
 }
 
 cudaError_t launch_pyramid(const float *frames, int N, size_t fstride, int W, int H, int pitch, int levels,
-                           int storage, const PyrOut &out, float *means, cudaStream_t s)
+                           int storage, const PyrOut &out, LevelStat *means, cudaStream_t s)
 {
     if (out.pad != 0) {
         // the smoothed levels read the 3x3 window of a bordered level; the border holds the mean

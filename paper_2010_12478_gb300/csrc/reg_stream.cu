@@ -74,7 +74,7 @@ struct reg_stream {
     float *stage[2] = {};        // fp32 frames being copied in (two, used in turn)
     cudaEvent_t stage_free[2] = {};   // the pyramid build that read stage[b] is done
     int next_stage = 0;
-    float *means = nullptr;      // level means of the frame being staged
+    LevelStat *means = nullptr;  // of the frame being staged
     LevelDesc *table = nullptr;  // [kSlots + 1][L]; slot 0 holds f_0
     OpDesc *ops = nullptr;       // [2 (kSlots + 1)]: A of slot s at 2s, B at 2s + 1
     OpStats *stats = nullptr;
@@ -453,7 +453,7 @@ extern "C" int reg_stream_open(reg_ctx_t *ctx, int W, int H, reg_stream_t **out)
         if (ok && pad) ok = cudaMalloc(&s->spyr[l], (size_t)Wl[l] * Hl[l] * sb * (kSlots + 1)) == cudaSuccess;
     }
     for (int b = 0; b < 2 && ok; ++b) ok = cudaMalloc(&s->stage[b], sizeof(float) * (size_t)W * H) == cudaSuccess;
-    ok = ok && cudaMalloc(&s->means, sizeof(float) * kMaxLevels) == cudaSuccess;
+    ok = ok && cudaMalloc(&s->means, sizeof(LevelStat) * kMaxLevels) == cudaSuccess;
     ok = ok && cudaMalloc(&s->table, sizeof(LevelDesc) * (kSlots + 1) * c.levels) == cudaSuccess;
     ok = ok && cudaMalloc(&s->ops, sizeof(OpDesc) * nops) == cudaSuccess;
     ok = ok && cudaMalloc(&s->stats, sizeof(OpStats) * nops) == cudaSuccess;

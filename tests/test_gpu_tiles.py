@@ -271,3 +271,74 @@ def test_a_capped_step_has_the_caps_length_in_64_bits(cap):
     a, x, y = st["theta"]
     assert st["iters"] == [1] and st["rejects"] == 0
     assert abs(np.sqrt((0.25 * (96 + 110) * a) ** 2 + x * x + y * y) / cap - 1.0) <= 1e-13
+
+
+def _lattice(shift, period=13.3, n=512):
+    y, x = np.mgrid[0:n, 0:n].astype(np.float64)
+    return 0.5 + 0.2 * np.cos(2 * np.pi * (x + shift) / period) + 0.2 * np.cos(2 * np.pi * (y + 0.5 * shift) / period)
+
+
+def _ncc_energy(R, T):
+    # 1 - NCC of two images pixel by pixel, in extended precision (sums of FP64 products in FP64, as the oracle's,
+    # are off by 1e-5 of an energy of 7e-6 at an offset of 25 times the contrast)
+    r, t = (v.astype(np.longdouble) - v.astype(np.longdouble).mean() for v in (R, T))
+    return float(1 - (r * t).sum() / np.sqrt((r * r).sum() * (t * t).sum()))
+
+
+@pytest.mark.parametrize("shift", [0.01, 0.1])
+@pytest.mark.parametrize("gain,offset", [(1.0, 0.0), (1.3, 0.0), (3.0, 0.0), (0.2, 0.0), (1.0, 5.0), (-1.0, 0.0), (1.3, -5.0)])
+def test_small_energies_at_any_gain_and_offset(shift, gain, offset):
+    # 1 - NCC does not see gain and offset, and its rounding must not either.  At the identity the rigid model's
+    # samples are the pixels, so only the sums round: relative to the energy, as the difference that is summed is as
+    # small as the energy (the bar of the energies, 1e-6).  The nonrigid model's samples round to 6e-8 of their own
+    # value, 1e-4 of the difference at E = 7e-6, at random over the pixels: a few 1e-6 of the energy
+    R = _lattice(0.0).astype(np.float32)
+    T = (gain * _lattice(shift) + offset).astype(np.float32)
+    dR, dT = torch.from_numpy(R).cuda(), torch.from_numpy(T).cuda()
+    E, _ = B.Context(B.Config()).energy_rigid(dR, dT, [0.0, 0.0, 0.0])
+    Ex = _ncc_energy(R, T)
+    assert abs(E - Ex) <= 1e-6 * Ex
+    if abs(offset) > 1.0:
+        return
+    g = O.grid_for(512, 512)
+    c = np.zeros((g.ny, g.nx, 2), np.float32)
+    gd = torch.zeros((g.ny, g.nx, 2), device="cuda")
+    E = B.Context(B.Config(mode="nonrigid")).energy_grid(dR, dT, torch.from_numpy(c).cuda(), gd)
+    Eo, go = O.grid_energy(R, T, 0, g, c.transpose(2, 0, 1).astype(np.float64), 2.0)
+    assert abs(E - Eo) <= 1e-5 * abs(Eo)
+    np.testing.assert_allclose(gd.cpu().numpy().transpose(2, 0, 1), go, atol=2e-4 * np.abs(go).max())
+
+
+@pytest.mark.parametrize("mode", ["rigid", "nonrigid"])
+@pytest.mark.parametrize("gain,offset", [(3.0, 0.0), (0.25, 2.0)])
+def test_pairs_of_different_gain_and_offset_match_the_oracle(mode, gain, offset):
+    F = synth.make_series(synth.SeriesSpec(2, 120, 131, step=1.0, field_amp=1.0, snr=(10.0, 10.0), seed=8)).frames.numpy()
+    R, T = F[0], (gain * F[1] + offset).astype(np.float32)
+    cfg = B.Config(mode=mode)
+    out = torch.empty((2, 120, 131), device="cuda") if mode == "nonrigid" else None
+    _, st = B.Context(cfg).pairwise(torch.from_numpy(R).cuda(), torch.from_numpy(T).cuda(), field_out=out)
+    oc = O.Config(levels=cfg.levels, max_iter=cfg.max_iter, max_rejects=cfg.max_rejects, tol_grad=cfg.tol_grad,
+                  tol_rel_e=cfg.tol_rel_e, armijo_c=cfg.armijo_c, tau0=cfg.tau0, step_cap=cfg.step_cap, lam=cfg.lam,
+                  mode=mode, metric=cfg.metric, sigma=cfg.sigma, tol_coarse=cfg.tol_coarse)
+    Rp, Tp = O.pyramid(R, cfg.levels), O.pyramid(T, cfg.levels)
+    p_o, st_o = O.register_nonrigid(Rp, Tp, None, oc) if mode == "nonrigid" else O.register_rigid(Rp, Tp, np.zeros(3), oc)
+    got = out.cpu().numpy() if mode == "nonrigid" else np.array(st["theta"])
+    assert O.max_px_error(got, p_o, 120, 131, mode) <= 0.02
+    assert abs(st["energy"] - st_o.energy) <= 1e-5 * abs(st_o.energy)
+
+
+@pytest.mark.parametrize("value", [0.0, 0.5, 0.3, -7.1, 1000.3])
+@pytest.mark.parametrize("which", ["template", "reference", "both"])
+def test_a_constant_image_has_energy_one_and_no_gradient(value, which):
+    rng = np.random.default_rng(3)
+    img = torch.from_numpy(rng.uniform(0, 1, size=(128, 117)).astype(np.float32)).cuda()
+    const = torch.full_like(img, value)
+    R = const if which != "template" else img
+    T = const if which != "reference" else img
+    E, g = B.Context(B.Config()).energy_rigid(R, T, [0.01, 0.37, -2.21])
+    assert E == 1.0 and not g.any()
+    nx, ny, _ = B.grid_dims(117, 128)
+    c = torch.zeros((ny, nx, 2), device="cuda") + 0.37   # a translation: no regulariser
+    gd = torch.ones_like(c)
+    E = B.Context(B.Config(mode="nonrigid")).energy_grid(R, T, c, gd)
+    assert E == 1.0 and not gd.any()
