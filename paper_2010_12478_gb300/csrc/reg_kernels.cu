@@ -82,6 +82,12 @@ __device__ __forceinline__ bool at_least(double x, double y)
     return __double_as_longlong(x) >= __double_as_longlong(y) && nonneg(x);
 }
 
+// x < y for a finite x and y > 0, false for a NaN of either sign, from the bits.
+__device__ __forceinline__ bool below(double x, double y)
+{
+    return __double_as_longlong(x) < __double_as_longlong(y) && ((unsigned)__double2hiint(x) & 0x7fffffffu) < 0x7ff00000u;
+}
+
 // First trial of a line search after an accepted step (Barzilai and Borwein, "Two-point step size
 // gradient methods", 1988, their second step): tau = tau_acc <d_prev, d_prev - d> / |d_prev - d|^2
 // in the flow's metric, given num = <d_prev, d_prev - d> and den = |d_prev - d|^2; false without
@@ -325,8 +331,7 @@ __device__ __forceinline__ Ncc ncc_terms(const LevelSums &L, double se, double s
     // e = 0 everywhere (T o phi equals R up to gain and offset: identical inputs) is exactly NCC = 1
     if ((__double_as_longlong(Sre) | __double_as_longlong(See)) << 1 == 0) o.e = 0.0;
     // a constant template has no deviation at all (gam 0), whatever its samples between the pixels round to
-    if (__double_as_longlong(L.Srr) < __double_as_longlong(L.least) ||
-        __double_as_longlong(o.Stt) < __double_as_longlong(L.least) || __double_as_longlong(L.gam) == 0) {
+    if (below(L.Srr, L.least) || below(o.Stt, L.least) || __double_as_longlong(L.gam) == 0) {
         o.e = 1.0; o.a = 0.0;
     }
     return o;

@@ -342,3 +342,25 @@ def test_a_constant_image_has_energy_one_and_no_gradient(value, which):
     gd = torch.ones_like(c)
     E = B.Context(B.Config(mode="nonrigid")).energy_grid(R, T, c, gd)
     assert E == 1.0 and not gd.any()
+
+
+@pytest.mark.parametrize("bad", [float("nan"), float("inf"), -float("inf"), "f16"])
+@pytest.mark.parametrize("which", ["template", "reference", "both"])
+@pytest.mark.parametrize("mode", ["rigid", "nonrigid"])
+def test_samples_that_are_not_finite_are_no_constant_image(mode, which, bad):
+    # one pixel that is not finite, or that FP16 storage cannot hold: the energy is NaN (not that of a constant
+    # image), and no step is taken
+    F = synth.make_series(synth.SeriesSpec(2, 64, 70, step=1.0, snr=(10.0, 10.0), seed=2)).frames.cuda()
+    R, T = F[0].clone(), F[1].clone()
+    for img in ([R] if which == "reference" else [T] if which == "template" else [R, T]):
+        img[30, 33] = 1e6 if bad == "f16" else bad
+    nx, ny, _ = B.grid_dims(70, 64)
+    if bad != "f16":
+        ctx = B.Context(B.Config(mode=mode))
+        E = ctx.energy_rigid(R, T, [0.0, 0.3, 0.2])[0] if mode == "rigid" else ctx.energy_grid(
+            R, T, torch.full((ny, nx, 2), 0.3, device="cuda"))
+        assert np.isnan(E)
+    for cluster in (1, 16):
+        out = torch.empty((2, 64, 70), device="cuda") if mode == "nonrigid" else None
+        _, st = B.Context(B.Config(mode=mode, cluster=cluster, storage="f16" if bad == "f16" else "f32")).pairwise(R, T, field_out=out)
+        assert np.isnan(st["energy"]) and st["iters"] == [0, 0]
