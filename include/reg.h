@@ -274,8 +274,8 @@ int reg_scan_node_grids(reg_ctx_t *ctx, const int32_t *ops, int n, float *grids_
  * registered to the first one, then the series is averaged].
  *   out_k(x) = f_k(phi_{0,k}(x)), k = 0..N-1 (phi_{0,0} = identity), bilinear
  *   with clamp-to-edge, the sampling of the operator; mean(x) = (1/N) sum_k out_k(x),
- *   summed per chunk of at most 64 frames with compensation and over chunks in FP64 (the
- *   compensation's low parts in FP32), in a fixed order (bitwise reproducible).
+ *   summed per chunk of at most 64 frames with compensation and over chunks in FP64, in
+ *   a fixed order (bitwise reproducible).
  *   frames   device fp32 [N][H][pitch], N >= 1.
  *   elems    REG_RIGID: the N-1 prefixes from reg_scan (host or device), element
  *            k-1 = phi_{0,k}.  Ignored for REG_NONRIGID.

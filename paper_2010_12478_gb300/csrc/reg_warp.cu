@@ -644,10 +644,8 @@ __global__ void __launch_bounds__(kWThreads, kCtasPerSm) warp_kernel(const WarpA
     }
 }
 
-// mean = (1/N) sum over chunks, in chunk order; four pixels per thread (float4 store) when
-// the row length allows it.  The sums' high parts are added in FP64, whose instructions bound the kernel
-// (64 cycles each: 21 us for 7 chunks of 512x512 with both parts in FP64, 14.5 us so); the low parts, below
-// 2^-24 of them, in FP32, which leaves 2^-45 of the sum.
+// mean = (1/N) sum over chunks in FP64, in chunk order; four pixels per thread (float4 store) when
+// the row length allows it.
 __global__ void mean_kernel(const float2 *part, int chunks, int W, int H, double inv_n, float *mean)
 {
     const size_t P = (size_t)W * H;
@@ -656,23 +654,21 @@ __global__ void mean_kernel(const float2 *part, int chunks, int W, int H, double
         const size_t i0 = 4 * q;
         if (i0 >= P) return;
         double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
-        float e0 = 0.f, e1 = 0.f, e2 = 0.f, e3 = 0.f;
         for (int c = 0; c < chunks; ++c) {
             const float4 *v = (const float4 *)(part + c * P + i0);
             const float4 u0 = v[0], u1 = v[1];
-            s0 += (double)u0.x; e0 += u0.y;
-            s1 += (double)u0.z; e1 += u0.w;
-            s2 += (double)u1.x; e2 += u1.y;
-            s3 += (double)u1.z; e3 += u1.w;
+            s0 += (double)u0.x + (double)u0.y;
+            s1 += (double)u0.z + (double)u0.w;
+            s2 += (double)u1.x + (double)u1.y;
+            s3 += (double)u1.z + (double)u1.w;
         }
-        *(float4 *)(mean + i0) = make_float4((float)((s0 + (double)e0) * inv_n), (float)((s1 + (double)e1) * inv_n),
-                                             (float)((s2 + (double)e2) * inv_n), (float)((s3 + (double)e3) * inv_n));
+        *(float4 *)(mean + i0) = make_float4((float)(s0 * inv_n), (float)(s1 * inv_n), (float)(s2 * inv_n),
+                                             (float)(s3 * inv_n));
     } else {
         for (size_t i = 4 * q; i < min(P, 4 * q + 4); ++i) {
             double s = 0.0;
-            float e = 0.f;
-            for (int c = 0; c < chunks; ++c) { s += (double)part[c * P + i].x; e += part[c * P + i].y; }
-            mean[i] = (float)((s + (double)e) * inv_n);
+            for (int c = 0; c < chunks; ++c) s += (double)part[c * P + i].x + (double)part[c * P + i].y;
+            mean[i] = (float)(s * inv_n);
         }
     }
 }
