@@ -723,9 +723,9 @@ EncodeTiled encoder()
 // at once, and the second wave ran nearly empty (219 us a call with frames and mean out, 196 us with 7 chunks of 37
 // frames in two full waves; 169 us by now).  The rule takes the chunk whose waves x (frames + kChunkCost) is least, the larger
 // of equals: kChunkCost stands for the pipeline's fill and the chunk's partial sums, in frames, and
-// keeps the chunks of a long series near 64.  It depends on the sizes alone, so a series' mean does
-// not depend on which outputs a call asks for.
-constexpr int kMaxChunk = 64, kChunkCost = 4;
+// keeps the chunks of a long series near 64, of those whose number a grid's y extent holds.  It depends on
+// the sizes and the GPU's number of SMs, so a series' mean does not depend on which outputs a call asks for.
+constexpr int kMaxChunk = 64, kChunkCost = 4, kMostChunks = 65535;
 static int warp_chunk_frames(int N, int W, int H)
 {
     int dev = 0, sms = 0;
@@ -736,7 +736,9 @@ static int warp_chunk_frames(int N, int W, int H)
     int best = top;
     long long least = -1;
     for (int c = top; c >= 1; --c) {
-        const long long blocks = tiles * ((N + c - 1) / c), cost = (blocks + slots - 1) / slots * (c + kChunkCost);
+        const int chunks = N / c + (N % c != 0);
+        if (chunks > kMostChunks) break;
+        const long long blocks = tiles * chunks, cost = (blocks + slots - 1) / slots * (c + kChunkCost);
         if (least < 0 || cost < least) {
             least = cost;
             best = c;

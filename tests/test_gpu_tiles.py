@@ -364,3 +364,13 @@ def test_samples_that_are_not_finite_are_no_constant_image(mode, which, bad):
         out = torch.empty((2, 64, 70), device="cuda") if mode == "nonrigid" else None
         _, st = B.Context(B.Config(mode=mode, cluster=cluster, storage="f16" if bad == "f16" else "f32")).pairwise(R, T, field_out=out)
         assert np.isnan(st["energy"]) and st["iters"] == [0, 0]
+
+
+def test_registered_mean_of_the_longest_series():
+    # 64 frames for each of the 65,535 chunks that a launch's grid holds: a shorter chunk would make more of them
+    N = 64 * 65535
+    g = torch.Generator(device="cuda").manual_seed(3)
+    F = torch.rand((N, 2, 2), device="cuda", generator=g)
+    mean = torch.empty((2, 2), device="cuda")
+    B.Context(B.Config(mode="nonrigid", levels=1)).warp(F, grids=torch.zeros((N - 1, 2, 2, 2), device="cuda"), mean=mean)
+    assert float((mean.double() - F.double().mean(dim=0)).abs().max()) <= 1e-5
