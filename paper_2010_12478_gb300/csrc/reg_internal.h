@@ -123,7 +123,7 @@ struct PassGeom {
     int tasks, walk;      // tasks of a segment; pairs of strips a task walks
     int m, h, ph;         // cell rows per segment, pieces per cell row (a power of two), pixel rows per piece
     int nseg, hlog;       // segments, log2 of h
-    unsigned rm, rg;      // reciprocals for div20: of m and g
+    unsigned rm, rg;      // reciprocals for div31: of m and g
 };
 
 struct Params {

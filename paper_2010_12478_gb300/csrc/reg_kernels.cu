@@ -909,15 +909,16 @@ __device__ __forceinline__ Band grid_band(const Grid &G, int rank, int C)
     return b;
 }
 
-// a / b for a b < 2^20, r = recip20(b): the integer divisions of a pass's set-up take longer than the rows
-// of a small frame.
-__host__ __device__ __forceinline__ unsigned recip20(int b)
+// a / b for a b < 2^31, r = recip31(b): the integer divisions of a pass's set-up take longer than the rows
+// of a small frame.  A quotient's rounding is a / 2^31 at most, below 1 / b.  (With 20 bits a band of 1,205 cell
+// rows, which two CTAs hold of a 2 x 2,410 grid, was beyond it.)
+__host__ __device__ __forceinline__ unsigned recip31(int b)
 {
-    return (1u << 20) / (unsigned)b + 1u;
+    return (1u << 31) / (unsigned)b + 1u;
 }
-__host__ __device__ __forceinline__ int div20(int a, unsigned r)
+__host__ __device__ __forceinline__ int div31(int a, unsigned r)
 {
-    return (int)(((unsigned)a * r) >> 20);
+    return (int)(((unsigned long long)(unsigned)a * r) >> 31);
 }
 
 constexpr int kSlot = 8;   // floats per slot: (e, r, 1) x (x, y), then dT^2 x (x, y)
@@ -963,8 +964,8 @@ static PassGeom pass_geom(int sl, int ncx, int q, bool over, int room, bool exac
         if (P.chunks == 1) break;
     }
     P.hlog = P.h == 8 ? 3 : P.h >> 1;
-    P.rm = recip20(P.m);
-    P.rg = recip20(P.g);
+    P.rm = recip31(P.m);
+    P.rg = recip31(P.g);
     return P;
 }
 
@@ -1105,9 +1106,9 @@ __device__ __forceinline__ void emit_points(const float *x, int lane, int sl, in
                                             float *s1)
 {
     constexpr int kSums = SQ ? 2 : kEmitSums;
-    const unsigned rp = recip20(cells + 1);
+    const unsigned rp = recip31(cells + 1);
     for (int u = lane; u < 2 * kSums * (cells + 1); u += 32) {
-        const int row = div20(u, rp), pt = u - row * (cells + 1);
+        const int row = div31(u, rp), pt = u - row * (cells + 1);
         const bool second = row >= kSums;
         const int comp = second ? row - kSums : row, lst = second ? last.y : last.x;
         if (pt > lst + 1 || lst < 0) continue;
@@ -1172,7 +1173,7 @@ template <int N, bool FF = false>
 __device__ __forceinline__ void slot_sum(const float *slots, const PassGeom &P, int ncx, int nr, int i, int jx,
                                          int first, float (&o)[N])
 {
-    const int ga = i > 0 ? div20(i - 1, P.rm) : 0, gb = div20(i < nr ? i : nr - 1, P.rm);
+    const int ga = i > 0 ? div31(i - 1, P.rm) : 0, gb = div31(i < nr ? i : nr - 1, P.rm);
     const int srow = (P.g + 1) * kSlot, sstrip = (P.m + 1) * srow, sseg = P.nst * sstrip;
     float e[N];
 #pragma unroll
@@ -1190,7 +1191,7 @@ __device__ __forceinline__ void slot_sum(const float *slots, const PassGeom &P, 
             }
         }
     };
-    const int st = div20(jx, P.rg), pt = jx - st * P.g;
+    const int st = div31(jx, P.rg), pt = jx - st * P.g;
     // the strips that hold the point: where it is the last of one, the first or an inner one of another, and
     // where it lies beside the column past the last cell
     const bool narrow = P.sl < 32, over = P.nst > P.ns && jx >= ncx - 1;
@@ -1253,7 +1254,7 @@ __device__ void grid_pass(const Lvl &L, const Grid &G, const GridLvl &GL, const 
 #pragma unroll
     for (int i = 0; i < NM; ++i) hi2[i] = lo2[i] = a[i] = f2(0.f);
 
-    const int kw = sl < 32 ? div20(lane, recip20(sl)) : 0;   // the lane's cell in a strip of whole cells
+    const int kw = sl < 32 ? div31(lane, recip31(sl)) : 0;   // the lane's cell in a strip of whole cells
     for (int seg = 0, pr = warp, cp = 0;;) {
         while (pr >= P.tasks) { pr -= P.tasks; ++seg; }
         if (seg >= P.nseg) break;

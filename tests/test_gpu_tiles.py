@@ -374,3 +374,27 @@ def test_registered_mean_of_the_longest_series():
     mean = torch.empty((2, 2), device="cuda")
     B.Context(B.Config(mode="nonrigid", levels=1)).warp(F, grids=torch.zeros((N - 1, 2, 2, 2), device="cuda"), mean=mean)
     assert float((mean.double() - F.double().mean(dim=0)).abs().max()) <= 1e-5
+
+
+@pytest.mark.parametrize("H,grid", [(38545, 16), (38577, 16), (9637, 4)])
+def test_pair_of_a_tall_frame_in_two_bands(H, grid):
+    # 2,410 control rows of 2 points: two CTAs hold bands of 1,205 cell rows in one segment, the longest there is;
+    # 2,412 rows take four CTAs
+    W = grid + 1
+    assert B.grid_dims(W, H, grid, 1)[0] == 2 and 2410 <= B.grid_dims(W, H, grid, 1)[1] <= 2412
+    rng = np.random.default_rng(17)
+    R = rng.uniform(0, 1, size=(H, W)).astype(np.float32)
+    T = (0.5 * (R + np.roll(R, 1, axis=0))).astype(np.float32)
+    outs = []
+    for cluster in (2, 16):
+        ctx = B.Context(B.Config(mode="nonrigid", levels=1, grid=grid, max_iter=1, cluster=cluster))
+        outs.append(torch.empty((2, H, W), device="cuda"))
+        _, st = ctx.pairwise(torch.from_numpy(R).cuda(), torch.from_numpy(T).cuda(), field_out=outs[-1])
+        assert ctx.last_timing()["cluster"] == (4 if H == 38577 and cluster == 2 else cluster)
+    cfg = B.Config()
+    oc = O.Config(levels=1, max_iter=1, max_rejects=cfg.max_rejects, tol_grad=cfg.tol_grad, tol_rel_e=cfg.tol_rel_e,
+                  armijo_c=cfg.armijo_c, tau0=cfg.tau0, step_cap=cfg.step_cap, lam=cfg.lam, mode="nonrigid", grid=grid,
+                  metric=cfg.metric, sigma=cfg.sigma, tol_coarse=cfg.tol_coarse)
+    c_o, st_o = O.register_nonrigid(O.pyramid(R, 1), O.pyramid(T, 1), None, oc)
+    for out in outs:   # one accepted step, as in test_pair_for_every_band_split
+        assert O.max_px_error(out.cpu().numpy(), c_o, H, W, "nonrigid", grid) <= 1e-3
