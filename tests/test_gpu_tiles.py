@@ -398,3 +398,27 @@ def test_pair_of_a_tall_frame_in_two_bands(H, grid):
     c_o, st_o = O.register_nonrigid(O.pyramid(R, 1), O.pyramid(T, 1), None, oc)
     for out in outs:   # one accepted step, as in test_pair_for_every_band_split
         assert O.max_px_error(out.cpu().numpy(), c_o, H, W, "nonrigid", grid) <= 1e-3
+
+
+@pytest.mark.parametrize("exec", ["level", "plain", "graph", "persistent"])
+def test_scans_and_streams_of_a_grid_too_large_for_one_cta_take_two(exec):
+    # 65 x 65 points need 292 KB in one CTA and 178 KB in each of two: asked for one, every executor and a stream
+    # take two, with the results of two
+    F = synth.make_series(synth.SeriesSpec(3, 513, 513, step=1.0, field_amp=1.0, snr=(10.0, 10.0), seed=9), device="cuda").frames
+    els = {}
+    for cluster in (1, 2):
+        ctx = B.Context(B.Config(mode="nonrigid", grid=8, cluster=cluster, max_iter=2))
+        els[cluster] = ctx.scan(F, schedule="sequential", exec=exec)[0]
+        assert ctx.last_timing()["cluster"] == 2
+    assert els[1] == els[2]
+    if exec == "plain":
+        s = B.Stream(B.Context(B.Config(mode="nonrigid", grid=8, cluster=1, max_iter=2)), 513, 513)
+        for k in range(3):
+            assert s.submit(F[k], k) == B.REG_OK
+        got = []
+        for _ in range(100):
+            got += s.poll(timeout_us=100000)
+            if len(got) == 3:
+                break
+        s.close()
+        assert [r["elem"] for r in got[1:]] == els[2] and all(r["status"] == 0 for r in got)
