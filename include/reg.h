@@ -464,8 +464,8 @@ typedef struct {
     double  leaf_ms, dag_ms;   /* REG_EXEC_SPLIT_PHASES with timing: device time of the A phase and
                                   of the B phase (same method as op_kernel_ms) */
     int32_t cluster;           /* launch shape of the last operator launch: CTAs per operator, */
-    int32_t unroll;            /* energy-pass pixels per lane (0 for REG_RIGID), */
-    int32_t ctas_per_sm;       /* and the register form */
+    int32_t unroll;            /* pixels in flight per lane (0 for REG_RIGID), */
+    int32_t ctas_per_sm;       /* and the register form as recorded */
     int32_t h2d_path;          /* host frames staged by: 0 none (device frames), 1 cudaMemcpyAsync,
                                   2 the SMs reading mapped page-locked memory */
     double  h2d_ms;            /* with timing: device time of that staging (0 for device frames) */

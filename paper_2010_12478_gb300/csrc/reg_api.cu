@@ -711,7 +711,8 @@ void note_shape(reg_ctx *ctx, const Params &p, int C)
     ctx->last.ctas_per_sm = p.cfg.mode == REG_NONRIGID ? (p.minb > 0 ? p.minb : 3) : 4;
 }
 
-// CTAs per operator where about `width` operators run side by side, unless fixed by the config: the
+// CTAs per operator where about `width` operators run side by side (for a whole DAG the average over its depths,
+// which the timings below are for too), unless fixed by the config: the
 // largest cluster of which the device holds at least two thirds of `width` at once (two CTAs per SM; of
 // 16-CTA clusters fewer than that fit the GPCs: four fifths), from 16 down to 4.  More CTAs shorten an
 // operator and with it the scan's chains; fewer take less of the time that goes to reductions and steps.
@@ -923,6 +924,11 @@ int launch_plain(reg_ctx *ctx, const ScanPlan &plan, const Params &p, int C, cud
     return REG_OK;
 }
 
+// CTAs per operator of the executors that launch operators one by one: how many of them run side by side follows
+// from the streams, not from a width.  Scans at 4 / 8 / 16 CTAs (plain; the graph within 5 %), ms: rigid 24 frames of
+// 256x256 1.11 / 0.91 / 0.83, 128 of 512x512 4.0 / 3.1 / 3.9; nonrigid 2.16 / 1.77 / 1.76 and 10.9 / 7.8 / 9.1.
+constexpr int kLaunchCluster = 8;
+
 // Execute the planned operators.
 int execute(reg_ctx *ctx, const ScanPlan &plan, Params &p, int exec, const TileShape &tuned, cudaStream_t s)
 {
@@ -950,7 +956,7 @@ int execute(reg_ctx *ctx, const ScanPlan &plan, Params &p, int exec, const TileS
     if (exec == REG_EXEC_PLAIN) {
         CHECK(ensure_pool(ctx));
         CHECK(ensure_op_events(ctx, n_ops));
-        const int C = fit_cluster(p, tuned.cluster > 0 ? tuned.cluster : 8);
+        const int C = fit_cluster(p, tuned.cluster > 0 ? tuned.cluster : kLaunchCluster);
         note_shape(ctx, p, C);
         const int t0 = timing_mark(ctx, s);
         CHECK(launch_plain(ctx, plan, p, C, s));
@@ -961,7 +967,7 @@ int execute(reg_ctx *ctx, const ScanPlan &plan, Params &p, int exec, const TileS
     if (exec == REG_EXEC_GRAPH) {
         CHECK(ensure_pool(ctx));
         CHECK(ensure_op_events(ctx, n_ops));
-        const int C = fit_cluster(p, tuned.cluster > 0 ? tuned.cluster : 8);
+        const int C = fit_cluster(p, tuned.cluster > 0 ? tuned.cluster : kLaunchCluster);
         note_shape(ctx, p, C);
         // The graph bakes in the kernel arguments (workspace pointers, config) and the
         // dependency edges; the descriptors themselves are read from device memory when it runs.

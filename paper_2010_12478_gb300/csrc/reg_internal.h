@@ -149,8 +149,8 @@ struct Params {
     Queue queue;               // persistent executor only
 };
 
-// Launch shape of the operator kernels (0 = not chosen): CTAs per operator, energy-pass pixels
-// per lane, and register form.
+// Launch shape of the operator kernels (0 = not chosen): CTAs per operator, pixels in flight per lane, and the
+// register form as recorded.
 struct TileShape {
     int cluster = 0, unroll = 0, minb = 0;
 };

@@ -373,7 +373,7 @@ constexpr int kFast = 8;   // pixels of a thread in one FP32 run before the floa
 // position keeps the FP32 fractional part exact to the precision of the offset, not
 // of the absolute coordinate.  Cell choice and clamping follow floor(p) clamped to
 // [0, W-2]; the derivative along a clamped axis (p < 0 or p > W-1) is 0.
-template <typename S, bool DERIV>
+template <typename S>
 __device__ __forceinline__ float sample_at(const S *T, int W, int H, int Tp, int xi, int yi, float vx, float vy,
                                            float &dtx, float &dty)
 {
@@ -393,10 +393,8 @@ __device__ __forceinline__ float sample_at(const S *T, int W, int H, int Tp, int
     float gx = 1.f - fx, gy = 1.f - fy;
     float top = fmaf(fx, t01, gx * t00);
     float bot = fmaf(fx, t11, gx * t10);
-    if (DERIV) {
-        dtx = clx ? 0.f : fmaf(fy, t11 - t10, gy * (t01 - t00));
-        dty = cly ? 0.f : (bot - top);
-    }
+    dtx = clx ? 0.f : fmaf(fy, t11 - t10, gy * (t01 - t00));
+    dty = cly ? 0.f : (bot - top);
     return fmaf(fy, bot, gy * top);
 }
 
@@ -555,8 +553,8 @@ __device__ void rigid_pass(const Lvl &L, int r0, int r1, const float *pm, Smem &
                 for (int k = 0; k < n; ++k) {
                     float2 vx, vy, dx, dy, tw;
                     shift(y + k, vx, vy, yc);
-                    tw.x = sample_at<S, true>(T, L.W, L.H, L.Tp, xa + gix, y + k + giy, vx.x, vy.x, dx.x, dy.x);
-                    tw.y = sample_at<S, true>(T, L.W, L.H, L.Tp, xb + gix, y + k + giy, vx.y, vy.y, dx.y, dy.y);
+                    tw.x = sample_at<S>(T, L.W, L.H, L.Tp, xa + gix, y + k + giy, vx.x, vy.x, dx.x, dy.x);
+                    tw.y = sample_at<S>(T, L.W, L.H, L.Tp, xb + gix, y + k + giy, vx.y, vy.y, dx.y, dy.y);
                     pixel(tw, dx, dy, make_float2(ldS<S>(pa), ldS<S>(pb)), yc);
                     pa += L.Rp; pb += L.Rp;
                 }
@@ -2044,7 +2042,7 @@ template <int MODE, typename S, int MINB, int U = 4>
 __global__ void __launch_bounds__(kThreads, MINB) op_kernel(const __grid_constant__ Params p)
 {
     __shared__ Smem sm;
-    extern __shared__ __align__(16) float2 gbuf[];   // nonrigid: control grid c, d, ct, gp
+    extern __shared__ __align__(16) float2 gbuf[];   // nonrigid: grid_layout
     cg::cluster_group cl = cg::this_cluster();
     Comm comm{0};
     if (threadIdx.x == 0) comm_init(sm, p, cl);
@@ -2200,8 +2198,8 @@ __global__ void __launch_bounds__(kThreads, MINB) persistent_kernel(const __grid
 }
 
 // Energy/gradient at a given deformation for a single pair, on one cluster of kEnergyCtas CTAs that
-// split the rows as the operator's do.  It is bound by the latency of the two passes over the pair: with
-// a single CTA a call took 801 us for 512x512 (nonrigid), with 16 it takes 126 us.
+// split the rows as the operator's do.  It is bound by latency: one pass over the pair, and the call's
+// launches.  A call took 801 us for 512x512 (nonrigid) with a single CTA, 126 with 16 in two passes, and takes 79.
 // Rigid: theta (device) -> out[0] = E, out[1..3] = dE/dtheta.  Nonrigid: control values cgrid
 // (finest px, level 0) -> out[0] = E and grad_c = dE/dc.
 template <int MODE, typename S>
