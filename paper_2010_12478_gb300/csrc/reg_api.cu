@@ -716,10 +716,10 @@ void note_shape(reg_ctx *ctx, const Params &p, int C)
 // largest cluster of which the device holds at least two thirds of `width` at once (two CTAs per SM; of
 // 16-CTA clusters fewer than that fit the GPCs: four fifths), from 16 down to 4.  More CTAs shorten an
 // operator and with it the scan's chains; fewer take less of the time that goes to reductions and steps.
-// Measured (nonrigid, ms at 16 / 8 / 4 / 2 CTAs): 256 frames of 512x512 (width 50) 20.1 / 14.4 / 18.8 / 30.5;
-// 1,024 frames (width 160) 98.2 / 63.8 / 60.0 / 74.2; 8 series of 32 at 256x256 (width 81) 11.3 / 5.6 / 4.7 /
-// 6.4; a pair 0.28 / 0.37 / 0.54 / 0.90.  Rigid, 128 frames of 512x512 (width 29): 4.5 / 4.0 / 5.2 / 8.4; 24
-// of 256x256, a depth at a time: 1.3 / 1.5 / 1.7 / 2.5.  A nonrigid operator has work for no more CTAs than
+// Measured (nonrigid, ms at 16 / 8 / 4 / 2 CTAs): 256 frames of 512x512 (width 50) 20.2 / 13.9 / 18.1 / 28.2;
+// 1,024 frames (width 160) 83.1 / 53.6 / 50.8 / 58.5; 8 series of 32 at 256x256 (width 81) 12.4 / 6.1 / 4.9 /
+// 6.6; a pair 0.31 / 0.39 / 0.58 / 1.00.  Rigid, 128 frames of 512x512 (width 29): 5.0 / 4.3 / 5.5 / 8.6; 24
+// of 256x256, a depth at a time: 1.1 / 1.2 / 1.5 / 2.0.  A nonrigid operator has work for no more CTAs than
 // its grid has cell rows.
 int auto_cluster(const reg_ctx *ctx, const Params &p, double width)
 {

@@ -126,7 +126,7 @@ struct Smem {
 // completing n + 1, to which every peer contributes after completing n, so nothing of n + 2 meets
 // anything of n.  A cluster barrier here takes about 2,000 cycles (its release and acquire are fences over
 // global memory), and its acquire drops the SM's L1 lines, so every pass fetched its pixels from L2
-// again (331 cycles a load instead of 75); an exchange takes 500 and leaves them.
+// again (331 cycles a load instead of 75); an exchange takes 500, and comm_wait's acquire some more.
 struct Comm {
     unsigned n;   // number of the next exchange
 };
@@ -835,7 +835,7 @@ __device__ void run_rigid(const Params &p, const OpDesc &op, int op_index, Smem 
 // the gradient, and a level starts with one pass, which also gives the Gauss-Newton scalar product.
 // The gradient sums of a rejected trial are dropped.  With separate passes a scan of 256 frames of
 // 512x512 took 28.4 ms and a pair 1,031 us (8 CTAs per operator); fused, with two packed columns a lane
-// and sliding windows, 16.5 ms and 513 us; with the exchanges and emissions below 14.4 ms and 370 us.  What
+// and sliding windows, 16.5 ms and 513 us; with the exchanges and emissions below 13.9 ms and 390 us.  What
 // bounds the pass is the latency of its loads and of dependent packed steps (40 % issue, 16 warps per SM).
 //
 // A CTA of the cluster holds the control rows of its own band of cell rows and one row on either
@@ -925,7 +925,7 @@ constexpr int kSlot = 8;   // floats per slot: (e, r, 1) x (x, y), then dT^2 x (
 //
 // A column's sums run in FP32 over the rows of a segment's cell row.  `exact` takes pieces of at most 8 rows
 // where their slots fit: for a gradient that is a result itself (reg_energy, 512x512), 6.1e-8 of its norm off
-// the 64-bit value instead of 6.8e-8, within a microsecond of a call.
+// the 64-bit value instead of 6.8e-8 when it was chosen (5.1e-8 to 5.8e-8 now), within a microsecond of a call.
 static PassGeom pass_geom(int sl, int ncx, int q, bool over, int room, bool exact)
 {
     PassGeom P;

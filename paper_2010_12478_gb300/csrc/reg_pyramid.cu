@@ -119,7 +119,8 @@ __device__ __forceinline__ Spread joined(Spread a, Spread b)
 // split is the same for every batch size, so a frame's means do not depend on the call it is in.
 // One CTA sums at the rate a single SM loads, about 80 us for a 512x512 level: most of the call of a
 // small pair.  A CTA stores into the first one's shared memory only once every CTA of the cluster is
-// known to run: each arrives at the cluster barrier first and waits there after its sums.
+// known to run: each arrives at the cluster barrier first and waits there after its sums.  The deviation's
+// sums ride on the same loads: with the passes' use of them, 2.7 of the 97 us of a 160x128 pair.
 constexpr int kMeanCtas = 8, kMeanWarps = 8, kMeanBatch = 8;
 template <typename S>
 __global__ void __launch_bounds__(32 * kMeanWarps) level_means(Levels<S> L, LevelStat *means, int levels)

@@ -721,7 +721,7 @@ EncodeTiled encoder()
 // Frames per chunk.  A block takes the frames of one chunk at one tile, so the grid is tiles x
 // chunks; with a fixed 64 frames, 256 frames of 512x512 made 512 blocks for the 456 that are resident
 // at once, and the second wave ran nearly empty (219 us a call with frames and mean out, 196 us with 7 chunks of 37
-// frames in two full waves; 169 us by now).  The rule takes the chunk whose waves x (frames + kChunkCost) is least, the larger
+// frames in two full waves; 181 us by now).  The rule takes the chunk whose waves x (frames + kChunkCost) is least, the larger
 // of equals: kChunkCost stands for the pipeline's fill and the chunk's partial sums, in frames, and
 // keeps the chunks of a long series near 64, of those whose number a grid's y extent holds.  It depends on
 // the sizes and the GPU's number of SMs, so a series' mean does not depend on which outputs a call asks for.
