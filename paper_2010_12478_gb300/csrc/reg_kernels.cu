@@ -2107,28 +2107,27 @@ __global__ void __launch_bounds__(kThreads, MINB) persistent_kernel(const __grid
             for (; kClassQueue && Q.n_class > 1;) {
                 if (*vc >= p.n_ops) break;
                 // every class's head and tail in one round of loads; the first class with a ready
-                // operator is claimed with an atomic on its head (no compare-and-swap: under
-                // contention a worker may draw a slot past the tail, which a later release of that
-                // class fills; a draw past the class's last operator is void)
+                // operator is claimed by a compare-and-swap on its head, which never passes the tail
+                // (with a plain addition, workers that lost a race sat on slots that a later release
+                // of that class fills, while ready operators of other classes waited for a worker: the
+                // B operators of 4,096 frames of 512x512 on 4 CTAs took 360 ms, in one run of ten 450 to
+                // 880)
                 int hs[kQueueClasses], ts[kQueueClasses];
 #pragma unroll
                 for (int c = 0; c < kQueueClasses; ++c) hs[c] = c < Q.n_class ? vh[c] : 0;
 #pragma unroll
                 for (int c = 0; c < kQueueClasses; ++c) ts[c] = c < Q.n_class ? vt[c] : 0;
                 int slot = -1;
-                bool void_draw = false;
 #pragma unroll
                 for (int c = 0; c < kQueueClasses; ++c)
-                    if (slot < 0 && !void_draw && hs[c] < ts[c]) {
-                        const int h = atomicAdd(Q.head + c, 1);
-                        if (h < Q.class_off[c + 1] - Q.class_off[c]) slot = Q.class_off[c] + h;
-                        else void_draw = true;   // the class is used up: look again at once
+                    for (int h = hs[c]; slot < 0 && h < ts[c];) {
+                        const int was = atomicCAS(Q.head + c, h, h + 1);
+                        if (was == h) slot = Q.class_off[c] + h;
+                        h = was;
                     }
-                if (void_draw) continue;
                 if (slot >= 0) {
                     atomicAdd(Q.claimed, 1);
-                    // the releaser bumps the tail before it writes the slot; a slot drawn past the
-                    // tail is written by a later release of its class
+                    // the releaser bumps the tail before it writes the slot
                     while ((op = vs[slot]) < 0) {
                         unsigned long long now;
                         asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(now));
