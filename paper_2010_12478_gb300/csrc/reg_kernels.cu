@@ -2148,7 +2148,7 @@ __global__ void __launch_bounds__(kThreads, MINB) persistent_kernel(const __grid
                     break;
                 }
                 __nanosleep(ns);
-                if (ns < 1024) ns *= 2;
+                if (ns < 256) ns *= 2;   // at 1,024 a rigid scan of 128 frames of 512x512 takes 1 % longer
             }
             __threadfence();
             sm.idata[1] = op;
